@@ -382,10 +382,8 @@ DQGAN_API uint64_t dqgan_launch_count(const dqgan_handle* h);
  * on a device looks up the array's device address (cudaGetSymbolAddress) and
  * keeps it for the life of the process: make that first call before any
  * stream capture, and do not reset the device while the library is loaded.
- * The kernels rewrite the array's counts, prefixes and candidates in full on
- * every call, so nothing needs clearing; the one word that carries over from
- * call to call is the previous call's candidate threshold, which only
- * decides how much work the first pass saves and never changes a result.
+ * The kernels rewrite what they read of the array on every call, so nothing
+ * needs clearing and nothing carries over from call to call.
  * All calls share the array: calls whose work overlaps on the GPU (other
  * streams, other host threads) race and give wrong results.
  * Returns DQGAN_OK, DQGAN_ERR_INVALID_ARG (sizes beyond the limit, NULL or

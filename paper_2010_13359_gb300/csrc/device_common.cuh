@@ -204,11 +204,15 @@ __device__ __forceinline__ float server_out(const ServerArgs& s, float w, float 
 // as the blocks of the kernel before it in the stream exit, instead of after
 // the whole grid has drained.  Each kernel first waits for that grid to
 // complete (its writes visible); it reads and writes nothing before the
-// wait.  No kernel triggers its dependents early: that let the next grid's
+// wait (one exception, which states why: the top-k form kernel).  No kernel
+// that fills the GPU triggers its dependents early: that let the next grid's
 // blocks sit waiting on the SMs, and measured up to a third slower per step
 // (compress and server alternating on the 25M-parameter workload) against
 // 1-9 % faster without it.  Without the attribute the wait is a no-op.
 __device__ __forceinline__ void dq_pdl_enter() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Lets the next grid's blocks be scheduled now (after every block of this
+// one has called it or exited).
+__device__ __forceinline__ void dq_pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // Index checks of the checked build (compiled with -DDQGAN_CHECK_BOUNDS):
 // dq_in_bounds(cond, err) is cond, and when cond is false it also sets

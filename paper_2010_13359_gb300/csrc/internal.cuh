@@ -129,23 +129,33 @@ constexpr int kSignSegBoxWords = 36;
 // d >= 32 and w 16-byte aligned.
 bool encode_params_map(float* w, int64_t d, int32_t box_rows, CUtensorMap* out);
 
-// Launches `kern` as a programmatic dependent launch (see dq_pdl_enter in
-// device_common.cuh: every kernel launched this way waits for its
-// predecessor's grid before touching memory).  Returns the launch status.
+// Launches `kern`, in clusters of `cluster` blocks along x, as a programmatic
+// dependent launch (see dq_pdl_enter in device_common.cuh: every kernel
+// launched this way waits for its predecessor's grid before touching
+// memory).  Returns the launch status.
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
-                              Args&&... args) {
+inline cudaError_t launch_pdl_cluster(void (*kern)(KArgs...), int cluster, dim3 grid, dim3 block, size_t smem,
+                                      cudaStream_t stream, Args&&... args) {
   cudaLaunchConfig_t lc = {};
   lc.gridDim = grid;
   lc.blockDim = block;
   lc.dynamicSmemBytes = smem;
   lc.stream = stream;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)cluster;
+  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
   lc.attrs = attr;
-  lc.numAttrs = 1;
+  lc.numAttrs = cluster > 1 ? 2 : 1;
   return cudaLaunchKernelEx(&lc, kern, std::forward<Args>(args)...);
+}
+
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
+                              Args&&... args) {
+  return launch_pdl_cluster(kern, 1, grid, block, smem, stream, std::forward<Args>(args)...);
 }
 
 // Kernel launchers: each enqueues its kernels on `stream`, adds the number of
@@ -160,10 +170,7 @@ cudaError_t launch_identity_compress(const CompressArgs& a, bool keep_h, cudaStr
 
 // Scratch of the top-k path: `rows` rows (one per local worker) and the
 // server's tables for `nworkers` messages (none for 0).  A row needs no
-// clearing between calls: every call rewrites its tile counts, tile prefixes
-// and candidates in full.  Only the row's last state word carries over -- the
-// candidate threshold of the worker's previous call (0 before the first),
-// which decides how much work the first pass saves and never a result.  The
+// clearing between calls: every call rewrites what it reads of it.  The
 // server's per-index worker masks (up to 64 workers) must be zero when the
 // scratch is created; each server call clears the masks it set.
 size_t topk_scratch_bytes(int64_t d, int32_t rows, int32_t nworkers);

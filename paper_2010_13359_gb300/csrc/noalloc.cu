@@ -24,7 +24,7 @@ namespace dq {
 namespace {
 
 // Largest d the fixed scratch supports, and the scratch itself (8.75 MiB;
-// the one scratch row of a top-k worker at that d takes 8.01 MiB).  Both
+// the one scratch row of a top-k worker at that d takes 8.22 MiB).  Both
 // numbers are the ones dqgan.h states.
 constexpr int64_t kNoAllocMaxD = DQGAN_NOALLOC_MAX_D;
 constexpr size_t kNoAllocScratchBytes = (size_t)DQGAN_NOALLOC_SCRATCH_BYTES;
@@ -85,11 +85,8 @@ extern "C" int dqgan_topk_compress_noalloc(const float* g, float* e, void* out_m
   }
 
   cudaStream_t stream = reinterpret_cast<cudaStream_t>(cuda_stream);
-  // No clearing: the top-k kernels rewrite the tile counts, tile prefixes and
-  // candidates of the row in full on every call.  The one word that carries
-  // over is the candidate threshold of the previous call (zero in the array
-  // as loaded, i.e. none); it decides how much work the first pass saves and
-  // never changes a result, whatever d and k the previous call had.
+  // No clearing: the top-k kernels rewrite what they read of the row on every
+  // call, so nothing carries over, whatever d and k the previous call had.
   dq::CompressArgs a{};
   a.g = g;
   a.g_stride = 0;

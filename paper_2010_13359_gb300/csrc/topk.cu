@@ -4,30 +4,32 @@
 // (ties to the lower index), send them as (u32 index, f32 value) records in
 // ascending index order, and keep e_j = p_j - p_j (+0) at the kept entries
 // and e_j = p_j elsewhere.  |p_j| is ordered by its bit pattern with the sign
-// cleared (a 31-bit key), so the k-th largest key T is found by a three-digit
-// radix select (11 + 10 + 10 bits) without sorting.
+// cleared (a 31-bit key), so the k-th largest key T is found by counting,
+// without sorting.
 //
-// Two kernels per call, one pass over the dense vectors:
-//   1. form (tiles of 4096 elements): p -> e in place, h (optional), and the
-//      tile's candidates -- the elements whose key is at least a threshold
-//      tau carried over from the worker's previous call (15/16 of its T) --
-//      written in index order to the tile's slot, with the tile's count.
-//   2. select-and-compact, one cluster of 8 CTAs per worker.  The candidates
-//      are split evenly over the 8 CTAs (by their index order, through a
-//      prefix of the tile counts); each CTA histograms the top, then the
-//      middle, then the low digit of its share, the cluster sums each
-//      histogram through distributed shared memory, and every CTA selects
-//      the same T and the number `need` of keys equal to T that are kept
-//      (the lowest indices).  If T >= tau, every key >= T was a candidate
-//      and T is exact; otherwise (first call, or T fell below the carried
-//      threshold) each CTA histograms the top digit over its tiles of p,
-//      re-extracts the elements whose top digit reaches the selected one,
-//      and the selection is repeated.  Kept records are then written at
-//      position (number of keys > T before it) + min(number of keys == T
-//      before it, need), the per-CTA counts taken from the CTA's own
-//      histograms.
-// The carried threshold only decides how much work the first pass saves the
-// second; the result is the same bit for bit either way.
+// Small problems (chip_ctas): one kernel, 1, 8 or 16 CTAs per worker that keep
+// p on chip.  Large ones: five kernels, one pass over the dense vectors:
+//   1. sample (8 blocks per worker): p at 65,536 elements spread over the
+//      vector; tau, a key that rather more than k of the d keys reach (1.3 k
+//      for k = d / 100), is read off their ranks.
+//   2. form (tiles of 4096 elements): p, h (optional), and the tile's
+//      candidates -- the elements whose key is at least tau -- written in
+//      index order to the tile's slot, with the tile's count.  e is written
+//      as if every candidate were kept.
+//   3. count: the candidates in 2048 bins relative to tau.
+//   4. resolve: the counts give T's bin; the keys in the bin are counted one
+//      by one and listed, those above it per group of tiles.
+//   5. emit: T and the number of keys equal to T that are kept (the lowest
+//      indices), the groups' places among the records, and the kept records,
+//      at (number of keys > T before it) + min(number of keys == T before it,
+//      the number kept); a candidate that is not kept gets its e_j = p_j (and
+//      h_j) back.
+// With k candidates or more T >= tau, so every key >= T was a candidate and T
+// is exact.  With fewer (the sample sat where p is larger than elsewhere)
+// steps 4 and 5 put e back, take the candidates again from the top digits of
+// all of p, and select among those.  tau only decides how much work the first
+// pass saves; the result is the same bit for bit.  Nothing carries over from
+// call to call.
 //
 // Server: w_j -= (sum over workers of the value recorded for j, absent
 // workers as +0, in the library's pairwise order) / M at the indices some
@@ -39,6 +41,7 @@
 // records of each 256-index tile start, and one thread per record searches
 // the other workers' records of its tile.
 #include <atomic>
+#include <cmath>
 
 #include <cooperative_groups.h>
 
@@ -53,38 +56,76 @@ namespace cg = cooperative_groups;
 constexpr int kTile = 4096;                                   // elements per tile
 constexpr int kFormThreads = 256;                             // threads of a form block
 constexpr int kFormRows = kTile / (4 * kFormThreads);         // float4 rows per form thread
-constexpr int kCluster = 8;                                   // CTAs per worker in the select kernel
 constexpr int kSelThreads = 512;                              // threads of a select CTA
-constexpr int kSelRows = kTile / (4 * kSelThreads);           // float4 rows per select thread
-constexpr int kBins0 = 2048, kBins1 = 1024;                   // 11-bit, then 10-bit digits
-constexpr int kStateWords = 32;
-constexpr int kChunkTiles = 2048;                             // tile prefixes a select CTA holds at once
-constexpr int kCacheCap = 20480;                              // candidates a select CTA keeps on chip
-constexpr int kBatch = 8;                                     // candidate loads in flight per thread
+constexpr int kSelWarps = kSelThreads / 32;
+constexpr int kFineShift = 12, kFineBins = 1792;              // bins of 4096 keys from tau up (7/8 of a binade)
+constexpr int kBins = kFineBins + 256;                        // first round: then one bin per exponent
+constexpr int kBins2 = 1 << kFineShift;                       // second round
+constexpr int kTopBins = 2048;                                // bins of 2^20 keys
+constexpr int kMaxGroups = 8192;                              // groups of tiles per worker, at most
+constexpr int kChipThreads = 1024;                            // CTAs that keep their part of p on chip
+constexpr int kGroup = 64;                                    // bins per coarse count
+constexpr int kChipMax = 49152;                               // parameters of a part, at most
+constexpr int kStateWords = 64;
+constexpr int kFirst = 4, kBatch = 8;                         // rows of 32 candidates a warp loads at once
+constexpr int kSampBlocks = 8;                                // sample blocks per worker
+constexpr int kSampThreads = 512;
+constexpr int kSampRuns = 8192;                               // sampled runs of 8 elements
+constexpr int kSamples = 8 * kSampRuns;
+constexpr int kSampBits = 14;                                 // key bits a block's estimate is resolved to
 constexpr int kSrvTile = 256;                                 // indices per server tile
 constexpr int kSrvThreads = 256;
-constexpr uint32_t kTauValid = 0x80000000u;                   // flag bit of the carried threshold word
 
-// State words.  ST_TAU (the carried threshold: kTauValid | key, or 0 for
-// none) is the last word, so that a caller may clear the others and keep it.
-enum : int { ST_TAU = kStateWords - 1 };
+// State words of a scratch row: the sample blocks' estimates of tau, then
+// what one step of a call leaves for the next.
+enum : int {
+  ST_TAU = 0,
+  ST_TICKET = kSampBlocks,    // finished CTAs of steps 4 and 5
+  ST_LISTED = ST_TICKET + 2,  // keys of T's bin put into the list so far
+  ST_PLACED,                  // step 4 finds T and the groups' places as well
+  ST_SHORT,                   // too few candidates
+  ST_BIN,                     // T's first-round bin
+  ST_REST,                    // k less the keys above it
+  ST_T,
+  ST_NEED,                    // keys equal to T that are kept
+  ST_TAU2                     // tau of a row with too few candidates
+};
 
 __host__ __device__ constexpr int64_t tiles_of(int64_t d) { return (d + kTile - 1) / kTile; }
 __host__ __device__ constexpr int64_t round64(int64_t x) { return (x + 63) / 64 * 64; }
 
-// Per-worker scratch, in u32 words: state | tile counts | the 8 CTAs'
-// private tile-prefix arrays (nt + 1 each) | candidate slots (kTile uint2
-// per tile).
+// Keys of T's bin a row lists: far more than it holds unless very many keys
+// are nearly equal (about 0.0005 k ln-slopes of the distribution at T).
+__host__ __device__ constexpr uint32_t list_cap(int64_t d) { return (uint32_t)(8192 + d / 128); }
+
+// Steps 3 to 5 take a worker's tiles in at most kMaxGroups groups of 2^shift
+// consecutive ones (one tile each up to d = 2^25).
+__host__ __device__ constexpr int group_shift(int64_t d) {
+  int s = 0;
+  while (((tiles_of(d) - 1) >> s) + 1 > kMaxGroups) ++s;
+  return s;
+}
+__host__ __device__ constexpr int groups_of(int64_t d) { return (int)(((tiles_of(d) - 1) >> group_shift(d)) + 1); }
+
+// Per-worker scratch, in u32 words: state | first- and second-round counts |
+// tile counts | the groups' counts or places (uint2) | the list of T's bin
+// (uint2) | candidate slots (kTile uint2 per tile).  Step 1 clears the
+// state's counters and the round counts; the rest is rewritten by every call
+// before it is read.
+constexpr int64_t kHistWords = kBins + kBins2;
 __host__ __device__ constexpr int64_t head_words(int64_t d) {
-  return round64(kStateWords + tiles_of(d) + kCluster * (tiles_of(d) + 1));
+  return kStateWords + kHistWords + round64(tiles_of(d)) + 2 * kMaxGroups + round64(2 * (int64_t)list_cap(d));
 }
 __host__ __device__ constexpr int64_t row_words(int64_t d) { return head_words(d) + 2 * tiles_of(d) * kTile; }
 __host__ __device__ constexpr int64_t srv_tiles(int64_t d) { return (d + kSrvTile - 1) / kSrvTile; }
 
 struct RowScratch {
   uint32_t* state;
+  uint32_t* hist;
+  uint32_t* hist2;
   uint32_t* cnt;
-  uint32_t* gpre;  // kCluster arrays of nt + 1 words
+  uint2* before;
+  uint2* list;
   uint2* cand;
 };
 
@@ -92,42 +133,41 @@ __device__ __forceinline__ RowScratch row_scratch(void* base, int64_t d, int row
   uint32_t* p = reinterpret_cast<uint32_t*>(base) + (int64_t)row * row_words(d);
   RowScratch r;
   r.state = p;
-  r.cnt = r.state + kStateWords;
-  r.gpre = r.cnt + tiles_of(d);
+  r.hist = r.state + kStateWords;
+  r.hist2 = r.hist + kBins;
+  r.cnt = r.hist2 + kBins2;
+  r.before = reinterpret_cast<uint2*>(r.cnt + round64(tiles_of(d)));
+  r.list = r.before + kMaxGroups;
   r.cand = reinterpret_cast<uint2*>(p + head_words(d));
   return r;
 }
 
 __device__ __forceinline__ uint32_t key_of(float v) { return __float_as_uint(v) & 0x7FFFFFFFu; }
+// tau of the call under way: the mean of the sample blocks' estimates.
+__device__ __forceinline__ uint32_t call_tau(const uint32_t* state) {
+  static_assert(kSampBlocks == 8 && ST_TAU == 0, "two loads of four estimates, an eighth of each");
+  const uint4 a = __ldcg(reinterpret_cast<const uint4*>(state)), b = __ldcg(reinterpret_cast<const uint4*>(state) + 1);
+  return (a.x >> 3) + (a.y >> 3) + (a.z >> 3) + (a.w >> 3) + (b.x >> 3) + (b.y >> 3) + (b.z >> 3) + (b.w >> 3);
+}
 __device__ __forceinline__ uint32_t key_bits(uint32_t bits) { return bits & 0x7FFFFFFFu; }
 
-// hist[bin] += 1 for each lane of `mask` (the lanes that call it together)
-// with `valid`: lanes with the same bin are counted by one atomic.  (The
-// candidates of a call lie within a few binades above the carried threshold,
-// so their top digits fall into a few bins, and plain per-lane atomics on
-// them serialise.)
-__device__ __forceinline__ void warp_hist_add(uint32_t* hist, uint32_t bin, bool valid, unsigned mask) {
-  const unsigned peers = __match_any_sync(mask, valid ? bin : 0xFFFFFFFFu);
-  if (valid && (int)(threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(hist + bin, (uint32_t)__popc(peers));
-}
-
 // Block-wide exclusive scan of one value per thread; *total gets the sum.
-// `warp_sums` is shared memory of NT/32 words.  Two barriers.
-template <int NT>
-__device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t* total, uint32_t* warp_sums) {
+// `warp_sums` is shared memory of NT/32 values.  Two barriers.
+template <int NT, typename T>
+__device__ __forceinline__ T block_exclusive_scan(T v, T* total, T* warp_sums) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  uint32_t x = v;
+  T x = v;
 #pragma unroll
   for (int off = 1; off < 32; off <<= 1) {
-    const uint32_t y = __shfl_up_sync(kFullMask, x, off);
+    const T y = __shfl_up_sync(kFullMask, x, off);
     if (lane >= off) x += y;
   }
   if (lane == 31) warp_sums[warp] = x;
   __syncthreads();
-  uint32_t before = 0, sum = 0;
+  T before = 0, sum = 0;
 #pragma unroll
   for (int w = 0; w < NT / 32; ++w) {
-    const uint32_t s = warp_sums[w];
+    const T s = warp_sums[w];
     if (w < warp) before += s;
     sum += s;
   }
@@ -136,51 +176,13 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t* t
   return before + x - v;
 }
 
-// Block-wide sum of one value per thread (two barriers).
-template <int NT>
-__device__ __forceinline__ uint32_t block_sum(uint32_t v, uint32_t* warp_sums) {
-  uint32_t total;
-  block_exclusive_scan<NT>(v, &total, warp_sums);
-  return total;
-}
-
-// Digit selection in a shared-memory histogram of BINS counts: the digit b
-// with count(> b) < k_rem <= count(>= b); *digit = b, *krem = k_rem -
-// count(> b) (shared-memory outputs, valid after the call for all threads;
-// left as they were when no digit qualifies).
-template <int NT, int BINS>
-__device__ void block_select(const uint32_t* hist, uint32_t k_rem, uint32_t* digit, uint32_t* krem,
-                             uint32_t* warp_sums) {
-  constexpr int kPer = BINS / NT;  // bins per thread, taken in descending digit order
-  static_assert(kPer >= 1 && kPer * NT == BINS, "bins must be a multiple of the block size");
-  uint32_t cnt[kPer];
-  uint32_t local = 0;
-#pragma unroll
-  for (int q = 0; q < kPer; ++q) {
-    cnt[q] = hist[BINS - 1 - ((int)threadIdx.x * kPer + q)];
-    local += cnt[q];
-  }
-  uint32_t total;
-  uint32_t cum = block_exclusive_scan<NT>(local, &total, warp_sums);
-#pragma unroll
-  for (int q = 0; q < kPer; ++q) {
-    if (cum < k_rem && k_rem <= cum + cnt[q]) {
-      *digit = (uint32_t)(BINS - 1 - ((int)threadIdx.x * kPer + q));
-      *krem = k_rem - cum;
-    }
-    cum += cnt[q];
-  }
-  __syncthreads();
-}
-
 // Writes one tile's flagged elements to its candidate slot in index order.
-// Element order in the tile: row i, thread t, component q is tile offset
-// 4 * (i * NT + t) + q.  Per lane and row at most 4 flags, per warp and row
-// at most 128, so the R <= 4 row counts share one 32-bit warp scan (8 bits
+// Element order in the tile: thread t, component q is tile offset 4 (i NT + t)
+// + q for row i < R.  Per lane and row at most 4 flags, per warp and row at
+// most 128, so the R <= 4 row counts share one 32-bit warp scan (8 bits
 // each).  `totals` is shared memory of NT/32 words.  Returns the tile's
-// count (in every thread); one barrier, two when `reuse` (the caller writes
-// `totals` again afterwards).
-template <int NT, int R, bool REUSE>
+// count (in every thread); two barriers.
+template <int NT, int R>
 __device__ __forceinline__ uint32_t write_tile_candidates(const float (&v)[R][4], const uint32_t (&cmask)[R],
                                                           int64_t tile0, uint2* slot, uint32_t* totals,
                                                           uint32_t* err) {
@@ -220,23 +222,103 @@ __device__ __forceinline__ uint32_t write_tile_candidates(const float (&v)[R][4]
         }
     }
   }
-  if constexpr (REUSE) __syncthreads();
+  __syncthreads();
   return done;
 }
 
+// First-round bin of a candidate: 1792 bins of 4096 keys from tau up, then
+// the key's exponent.  The k-th largest key lies within 7/8 of a binade of
+// tau unless the sample was far off, so that two rounds give it exactly.
+__device__ __forceinline__ uint32_t first_bin(uint32_t key, uint32_t tau) {
+  const uint32_t r = key - tau;
+  return r < ((uint32_t)kFineBins << kFineShift) ? r >> kFineShift : (uint32_t)kFineBins + (key >> 23);
+}
+
 // ---------------------------------------------------------------------------
-// 1. p = fl(fl(eta g) + e) into e; h = fl(fl(eta g) + p) (corrected at the kept
-// entries by the second kernel); candidates with key >= the carried
-// threshold (none without one).  Element order in a tile: row i,
+// 1. tau from a sample.  The vector's whole 8-element runs are cut into
+// kSampRuns equal strata, and one run of each is read, at a place in the
+// stratum that a multiplicative hash picks (so that no period of the vector
+// lines up with the sample).  Block b of a worker takes the strata b, b + 8,
+// ... and writes the largest key of kSampBits leading bits that at least
+// `rank` of its samples reach.  The caller's rank is an eighth of the expected
+// one of the k-th largest key, r = k kSamples / d, plus seven standard
+// deviations sqrt(r) of a binomial count (2.5, when the eight elements of a
+// run are always large together); tau is the mean of the blocks' estimates, which varies
+// about as little as one estimate from all samples would, and the blocks need
+// not wait for one another.  rank = 0: no sample, tau = 0.  Latency is all
+// that counts here: 8 loads of 16 bytes in flight per thread, then a bisection
+// over samples in registers.  The blocks also clear the row's counts.  They
+// let the form kernel start at once: it loads its first tiles meanwhile.
+// ---------------------------------------------------------------------------
+__global__ void __launch_bounds__(kSampThreads) topk_sample_kernel(const CompressArgs a, uint32_t rank, void* scratch) {
+  dq_pdl_enter();
+  dq_pdl_release();
+  constexpr int kHalves = 2 * kSampRuns / kSampBlocks / kSampThreads;  // half runs (float4) per thread
+  __shared__ uint32_t count[kSampBits];
+  const int row = blockIdx.y;
+  const int worker = a.worker0 + row;
+  const float* g = a.g + (int64_t)row * a.g_stride;
+  const float* e = a.e + (int64_t)(worker - a.row0) * a.ld;
+  const RowScratch rs = row_scratch(scratch, a.d, worker - a.row0);
+  for (int i = blockIdx.x * kSampThreads + threadIdx.x; i < kHistWords; i += kSampBlocks * kSampThreads) rs.hist[i] = 0;
+  if (blockIdx.x == 0 && threadIdx.x < 3) rs.state[ST_TICKET + threadIdx.x] = 0;
+  static_assert(ST_LISTED == ST_TICKET + 2, "three counters");
+  if (rank == 0) {
+    if (threadIdx.x == 0) rs.state[ST_TAU + blockIdx.x] = 0;
+    return;
+  }
+  if (threadIdx.x < kSampBits) count[threadIdx.x] = 0;
+  const int64_t runs = a.d >> 3;  // >= kSampRuns
+  float4 gv[kHalves], ev[kHalves];
+#pragma unroll
+  for (int i = 0; i < kHalves; ++i) {
+    const uint32_t s = (uint32_t)(i * (kSampThreads / 2) + (threadIdx.x >> 1)) * kSampBlocks + blockIdx.x;
+    const int64_t lo = runs * s / kSampRuns, hi = runs * (s + 1) / kSampRuns;
+    const int64_t at = lo + __umulhi(s * 0x9E3779B1u, (uint32_t)(hi - lo));
+    const int64_t j = 8 * at + 4 * (threadIdx.x & 1);
+    gv[i] = __ldcs(reinterpret_cast<const float4*>(g + j));
+    ev[i] = __ldcs(reinterpret_cast<const float4*>(e + j));
+  }
+  uint32_t key[kHalves][4];
+#pragma unroll
+  for (int i = 0; i < kHalves; ++i) {
+    key[i][0] = key_of(ef_p(a.lr, gv[i].x, ev[i].x));
+    key[i][1] = key_of(ef_p(a.lr, gv[i].y, ev[i].y));
+    key[i][2] = key_of(ef_p(a.lr, gv[i].z, ev[i].z));
+    key[i][3] = key_of(ef_p(a.lr, gv[i].w, ev[i].w));
+  }
+  __syncthreads();
+  uint32_t tau = 0;
+#pragma unroll 1
+  for (int it = 0; it < kSampBits; ++it) {
+    const uint32_t trial = tau | (1u << (30 - it));
+    uint32_t n = 0;
+#pragma unroll
+    for (int i = 0; i < kHalves; ++i)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) n += key[i][q] >= trial ? 1u : 0u;
+    n = __reduce_add_sync(kFullMask, n);
+    if ((threadIdx.x & 31) == 0) atomicAdd(&count[it], n);
+    __syncthreads();
+    if (count[it] >= rank) tau = trial;
+  }
+  if (threadIdx.x == 0) rs.state[ST_TAU + blockIdx.x] = tau;
+}
+
+// ---------------------------------------------------------------------------
+// 2. p = fl(fl(eta g) + e); e = p, or p - p at a candidate (key >= tau), and
+// h = fl(fl(eta g) + e); the select kernel corrects both at the candidates
+// that are not kept, a fraction of them.  Element order in a tile: row i,
 // thread t, component q is tile offset 4 * (i * 256 + t) + q, so warp w of
 // row i covers the 128 consecutive offsets of group g = 8 i + w.  Candidate
 // values wait in shared memory (flagged in a bitmask) until the block's one
 // barrier; then each warp writes its groups' candidates to the tile's slot
-// in index order.
+// in index order.  (Adding them to the row's counts here instead of in a
+// step of their own took the kernel from 0.74 to 1.6 ms at 16 x 25M, k = d /
+// 100: the additions meet in the few cache lines of the bins just above tau.)
 // ---------------------------------------------------------------------------
 template <bool KEEP_H>
-__global__ void __launch_bounds__(kFormThreads, 6) topk_form_kernel(const CompressArgs a, void* scratch) {
-  dq_pdl_enter();
+__global__ void __launch_bounds__(kFormThreads, 4) topk_form_kernel(const CompressArgs a, void* scratch) {
   constexpr int kGroups = kTile / 128;
   __shared__ float vstage[kTile];
   __shared__ uint32_t flags[kTile / 32];
@@ -247,32 +329,45 @@ __global__ void __launch_bounds__(kFormThreads, 6) topk_form_kernel(const Compre
   float* e = a.e + (int64_t)(worker - a.row0) * a.ld;
   float* h = KEEP_H ? a.h + (int64_t)(worker - a.row0) * a.ld : nullptr;
   RowScratch rs = row_scratch(scratch, a.d, worker - a.row0);
-  const uint32_t tau_word = rs.state[ST_TAU];
-  const bool has_tau = (tau_word & kTauValid) != 0;
-  const uint32_t tau = tau_word & 0x7FFFFFFFu;
   const int64_t tile = blockIdx.x;
   const int64_t tile0 = tile * kTile;
+  // The tile's g and e before the wait for the sample: every block of the
+  // sample kernel let this one start only after its own wait, when the grids
+  // before it had completed, and it writes neither (read from L2, where those
+  // grids' writes are).
+  float4 gr[kFormRows], er[kFormRows];
+#pragma unroll
+  for (int i = 0; i < kFormRows; ++i) {
+    const int64_t j = tile0 + 4 * (i * kFormThreads + (int)threadIdx.x);
+    gr[i] = er[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (j + 3 < a.d) {
+      gr[i] = __ldcg(reinterpret_cast<const float4*>(g + j));
+      er[i] = __ldcg(reinterpret_cast<const float4*>(e + j));
+    }
+  }
+  dq_pdl_enter();
+  const uint32_t tau = call_tau(rs.state);
 #pragma unroll
   for (int i = 0; i < kFormRows; ++i) {
     const int off = 4 * (i * kFormThreads + (int)threadIdx.x);
     const int64_t j = tile0 + off;
-    float v[4];
-    int nvalid = 0;
+    float v[4], en[4];
+    uint32_t bits = 0;
     if (j + 3 < a.d) {
-      const float4 gv = __ldcs(reinterpret_cast<const float4*>(g + j));
-      const float4 ev = __ldcs(reinterpret_cast<const float4*>(e + j));
-      const float gq[4] = {gv.x, gv.y, gv.z, gv.w};
-      const float eq[4] = {ev.x, ev.y, ev.z, ev.w};
+      const float gq[4] = {gr[i].x, gr[i].y, gr[i].z, gr[i].w};
+      const float eq[4] = {er[i].x, er[i].y, er[i].z, er[i].w};
       float hv[4];
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const float s = __fmul_rn(a.lr, gq[q]);
         v[q] = __fadd_rn(s, eq[q]);
-        hv[q] = __fadd_rn(s, v[q]);
+        const bool c = key_of(v[q]) >= tau;
+        if (c) bits |= 1u << q;
+        en[q] = c ? __fsub_rn(v[q], v[q]) : v[q];
+        hv[q] = __fadd_rn(s, en[q]);
       }
-      __stcs(reinterpret_cast<float4*>(e + j), make_float4(v[0], v[1], v[2], v[3]));
+      __stcs(reinterpret_cast<float4*>(e + j), make_float4(en[0], en[1], en[2], en[3]));
       if constexpr (KEEP_H) __stcs(reinterpret_cast<float4*>(h + j), make_float4(hv[0], hv[1], hv[2], hv[3]));
-      nvalid = 4;
     } else {
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
@@ -280,23 +375,17 @@ __global__ void __launch_bounds__(kFormThreads, 6) topk_form_kernel(const Compre
         if (j + q < a.d) {
           const float s = __fmul_rn(a.lr, g[j + q]);
           v[q] = __fadd_rn(s, e[j + q]);
-          e[j + q] = v[q];
-          if constexpr (KEEP_H) h[j + q] = __fadd_rn(s, v[q]);
-          nvalid = q + 1;
+          const bool c = key_of(v[q]) >= tau;
+          if (c) bits |= 1u << q;
+          en[q] = c ? __fsub_rn(v[q], v[q]) : v[q];
+          e[j + q] = en[q];
+          if constexpr (KEEP_H) h[j + q] = __fadd_rn(s, en[q]);
         }
       }
     }
-    uint32_t bits = 0;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      if (q < nvalid) {
-        const uint32_t key = key_of(v[q]);
-        if (has_tau && key >= tau) {
-          bits |= 1u << q;
-          vstage[off + q] = v[q];
-        }
-      }
-    }
+    for (int q = 0; q < 4; ++q)
+      if ((bits >> q) & 1u) vstage[off + q] = v[q];
     // 8 lanes' 4 flag bits form one 32-bit word of the tile's bitmask
     uint32_t word = bits << (4 * (lane & 7));
     word |= __shfl_xor_sync(kFullMask, word, 1);
@@ -345,578 +434,705 @@ __global__ void __launch_bounds__(kFormThreads, 6) topk_form_kernel(const Compre
 }
 
 // ---------------------------------------------------------------------------
-// 2. Select T over the candidates and write the kept records (a cluster of
-// kCluster CTAs per worker).
+// 3-5. Select T over the candidates and write the kept records: three grids of
+// a.nworkers rows of CTAs, a warp per group of tiles, groups dealt out over
+// the row's warps in turn (so that a stretch of the vector that holds most of
+// the candidates is shared by all of them).  What a step has to know of the
+// whole worker every CTA works out for itself from the counts of the step
+// before, which costs less than a step between them.  (A cluster of 8 or 16
+// CTAs per worker, with the counts summed through distributed shared memory,
+// took as long while the share of a CTA fits on chip, and twice as long for
+// 16 workers with 250,000 records each: 14 clusters of 16 fit at a time.)
 // ---------------------------------------------------------------------------
-struct SelectSmem {
-  uint32_t hist_t[kBins0];          // this CTA's top-digit histogram (read by the cluster)
-  uint32_t hist_a[kBins1];          // this CTA's middle-digit histogram (read by the cluster)
-  uint32_t hist_b[kBins1];          // this CTA's low-digit histogram (read by the cluster)
-  uint32_t full[kBins0];            // a whole histogram (top digit; then the cluster's sums)
-  uint32_t tpre[kChunkTiles + 1];   // candidate prefix at the chunk's tiles
-  uint32_t warp_sums[kSelThreads / 32];
-  uint32_t sel[6];
-  uint32_t pre_t[kBins0];           // the same three histograms summed over the CTAs of lower rank
-  uint32_t pre_a[kBins1];
-  uint32_t pre_b[kBins1];
-  uint32_t span[2];                 // first and last tile overlapping this CTA's share
-  uint2 cache[kCacheCap];           // this CTA's share of the candidates, when it fits
+struct SelectTask {
+  const CompressArgs& a;
+  RowScratch rs;
+  int64_t k;
+  int64_t nt;
+  int groups, shift;
+  float* e;
+  float* h;
+  const float* g;
+  uint2* rec;
+  int warp0, nwarps;  // this warp's first group, and the stride
+  int rows;           // rows of 32 candidates of a tile worth loading before its count is known
 };
 
-// Tile counts a select thread holds in registers (all tiles, when nt fits).
-constexpr int kRegTiles = 4;
+__device__ __forceinline__ SelectTask select_task(const CompressArgs& a, int64_t k, int rows, void* scratch) {
+  const int row = blockIdx.y;
+  const int worker = a.worker0 + row;
+  const int64_t at = (int64_t)(worker - a.row0) * a.ld;
+  return SelectTask{a, row_scratch(scratch, a.d, worker - a.row0), k, tiles_of(a.d), groups_of(a.d), group_shift(a.d),
+                    a.e + at, a.h ? a.h + at : nullptr, a.g + (int64_t)row * a.g_stride,
+                    reinterpret_cast<uint2*>(a.msg + (int64_t)row * a.msg_stride),
+                    (int)blockIdx.x * kSelWarps + (int)(threadIdx.x >> 5), (int)gridDim.x * kSelWarps, rows};
+}
 
-// The tile of candidate f: the largest i < n with tpre[i] <= f (tpre
-// non-decreasing, tpre[0] <= f < tpre[n]; an empty tile repeats its
-// successor's prefix, so the tile found holds f), in a fixed number of
-// halving steps (n <= kChunkTiles).  Used where the share is not kept on
-// chip; filling the on-chip copy uses the tile map instead (a search per
-// candidate, with the lanes reading scattered prefixes, conflicts in the
-// shared-memory banks).
-__device__ __forceinline__ int tile_of(const uint32_t* tpre, int n, uint32_t f) {
-  int lo = 0;
+// A tile's count and first rows of 32 candidates, loaded together (a slot has
+// kTile entries, whatever the count) and ahead of their use.
+struct TileAhead {
+  uint32_t n;
+  uint2 c[kFirst];
+};
+
+__device__ __forceinline__ TileAhead load_tile(const SelectTask& s, int64_t t) {
+  TileAhead x;
+  x.n = 0;
+  if (t < s.nt) {
+    const uint2* slot = s.rs.cand + t * kTile + (threadIdx.x & 31);
+    x.n = __ldcg(s.rs.cnt + t);
 #pragma unroll
-  for (int step = kChunkTiles / 2; step >= 1; step >>= 1) {
-    const int mid = lo + step;
-    if (mid < n && tpre[mid] <= f) lo = mid;
+    for (int u = 0; u < kFirst; ++u) x.c[u] = u < s.rows ? __ldcg(slot + 32 * u) : make_uint2(0u, 0u);
   }
-  return lo;
+  return x;
 }
 
-// Candidate f (prefix coordinates of tpre) of the chunk starting at tile tc0.
-__device__ __forceinline__ uint2 chunk_candidate(const uint2* cand, const uint32_t* tpre, int n, int64_t tc0,
-                                                 uint32_t f) {
-  const int i = tile_of(tpre, n, f);
-  return cand[(tc0 + i) * kTile + (f - tpre[i])];
+__device__ __forceinline__ TileAhead load_first(const SelectTask& s) {
+  return load_tile(s, (int64_t)s.warp0 << s.shift);
 }
 
-// Sums the cluster's copies of one histogram into sm.full[0, BINS), and
-// those of the CTAs of lower rank than this one into pre[0, BINS) (from which
-// the CTA's first record position follows).  The cluster barrier publishes
-// every CTA's counts; each histogram buffer is written once per selection
-// round, so no barrier is needed after the reads.
-template <int BINS>
-__device__ __forceinline__ void cluster_sum(cg::cluster_group& cluster, uint32_t* local, uint32_t* pre,
-                                            int rank, SelectSmem& sm) {
-  cluster.sync();
-  for (int i = threadIdx.x; i < BINS; i += kSelThreads) {
-    uint32_t s = 0, below = 0;
+// This warp's groups of tiles in turn, each tile's candidates in index order:
+// start(group), row(candidate, valid) for rows of 32, finish(group), by the
+// whole warp.  `cur` is the first tile; the next one loads while a tile is
+// worked on.
+template <typename Start, typename Row, typename Finish>
+__device__ __forceinline__ void walk(const SelectTask& s, TileAhead cur, Start&& start, Row&& row, Finish&& finish) {
+  const int lane = threadIdx.x & 31;
+  const int64_t mask = ((int64_t)1 << s.shift) - 1;
+  for (int64_t t = (int64_t)s.warp0 << s.shift; t < s.nt;) {
+    const int group = (int)(t >> s.shift);
+    int64_t next = t + 1;
+    const bool ends = (next & mask) == 0 || next >= s.nt;
+    if (ends) next = (int64_t)(group + s.nwarps) << s.shift;
+    const TileAhead ahead = load_tile(s, next);
+    if ((t & mask) == 0) start(group);
 #pragma unroll
-    for (int r = 0; r < kCluster; ++r) {
-      const uint32_t x = cluster.map_shared_rank(local, r)[i];
-      if (r < rank) below += x;
-      s += x;
+    for (int u = 0; u < kFirst; ++u)
+      if (u < s.rows && 32 * u < cur.n) row(cur.c[u], 32 * u + lane < cur.n);
+    const uint2* slot = s.rs.cand + t * kTile + lane;
+    for (uint32_t o = 32 * s.rows; o < cur.n; o += 32 * kBatch) {
+      uint2 c[kBatch];
+#pragma unroll
+      for (int u = 0; u < kBatch; ++u) {
+        c[u] = make_uint2(0u, 0u);
+        if (o + 32 * u + lane < cur.n) c[u] = __ldcg(slot + o + 32 * u);
+      }
+#pragma unroll
+      for (int u = 0; u < kBatch; ++u)
+        if (o + 32 * u < cur.n) row(c[u], o + 32 * u + lane < cur.n);
     }
-    sm.full[i] = s;
-    pre[i] = below;
+    if (ends) finish(group);
+    t = next;
+    cur = ahead;
   }
+}
+
+constexpr int kOwnList = 512;  // keys of T's bin a CTA collects before it adds them to the row's list
+
+template <int NT>
+struct SelectSmem {
+  alignas(16) uint32_t hist[kBins2];  // this CTA's counts
+  uint64_t scan[NT / 32];
+  uint32_t warp_sums[NT / 32];
+  uint32_t found[3];
+  uint32_t ticket;
+  uint32_t listed;
+  uint2 list[NT == kSelThreads ? kOwnList : 1];
+};
+
+// The bin b of BINS counts with count(> b) < k_rem <= count(>= b), k_rem -
+// count(> b) and count(b), in sm.found (as they were when there are fewer).
+// Returns the sum of all counts.  GLOBAL: counts other CTAs have added to.
+template <int NT, int BINS, bool GLOBAL>
+__device__ __forceinline__ uint32_t find_bin(SelectSmem<NT>& sm, const uint32_t* counts, uint32_t k_rem) {
+  constexpr int kPer = BINS / NT;  // bins per thread, from the top down
+  static_assert(kPer * NT == BINS, "whole bins per thread");
+  const int first = BINS - ((int)threadIdx.x + 1) * kPer;
+  uint32_t cnt[kPer], sum = 0;
+  if constexpr (GLOBAL && kPer % 4 == 0) {
+#pragma unroll
+    for (int q = 0; q < kPer; q += 4) {
+      const uint4 x = __ldcg(reinterpret_cast<const uint4*>(counts + first + q));
+      cnt[q] = x.x;
+      cnt[q + 1] = x.y;
+      cnt[q + 2] = x.z;
+      cnt[q + 3] = x.w;
+    }
+  } else {
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) cnt[q] = GLOBAL ? __ldcg(counts + first + q) : counts[first + q];
+  }
+#pragma unroll
+  for (int q = 0; q < kPer; ++q) sum += cnt[q];
+  uint32_t total;
+  uint32_t cum = block_exclusive_scan<NT>(sum, &total, sm.warp_sums);
+#pragma unroll
+  for (int q = kPer - 1; q >= 0; --q) {
+    if (cum < k_rem && k_rem - cum <= cnt[q]) {
+      sm.found[0] = (uint32_t)(first + q);
+      sm.found[1] = k_rem - cum;
+      sm.found[2] = cnt[q];
+    }
+    cum += cnt[q];
+  }
+  __syncthreads();
+  return total;
+}
+
+template <int NT>
+__device__ __forceinline__ void clear_hist(SelectSmem<NT>& sm, int bins) {
+  for (int i = threadIdx.x; i < bins; i += NT) sm.hist[i] = 0;
   __syncthreads();
 }
 
-template <bool KEEP_H>
-__global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kSelThreads, 1)
-topk_select_kernel(const CompressArgs a, int64_t k, void* scratch) {
-  // launched as a programmatic dependent of the form kernel: its tile counts,
-  // candidates and p are complete and visible after this wait
+// Whether every CTA of the row has come here: told to all threads of the one
+// that comes last, which then sees what the others wrote before.
+__device__ __forceinline__ bool last_of_row(SelectSmem<kSelThreads>& sm, uint32_t* ticket) {
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) sm.ticket = atomicAdd(ticket, 1u);
+  __syncthreads();
+  const bool last = sm.ticket == gridDim.x - 1;
+  if (last) __threadfence();
+  return last;
+}
+
+__device__ __forceinline__ void add_hist(const SelectSmem<kSelThreads>& sm, uint32_t* row_hist, int bins) {
+  __syncthreads();
+  for (int i = threadIdx.x; i < bins; i += kSelThreads) {
+    const uint32_t n = sm.hist[i];
+    if (n) atomicAdd(row_hist + i, n);
+  }
+}
+
+// e_j = p_j (and h_j) again at a candidate that is not kept.
+__device__ __forceinline__ void put_back(const SelectTask& s, uint2 c) {
+  const float p = __uint_as_float(c.y);
+  s.e[c.x] = p;
+  if (s.h) s.h[c.x] = __fadd_rn(__fmul_rn(s.a.lr, s.g[c.x]), p);
+}
+
+__device__ __forceinline__ void put_on_list(const SelectTask& s, uint2 x) {
+  const uint32_t at = atomicAdd(s.rs.state + ST_LISTED, 1u);
+  if (dq_in_bounds(at < list_cap(s.a.d), s.a.err)) s.rs.list[at] = x;
+}
+
+// The second round over this task's groups, into sm.hist: the 4096 keys of
+// the first round's bin, or (T is far above tau) the next 12 bits of the
+// exponent's keys.  Also each group's number of keys above the bin, and
+// (`listing`: the first round's count says that they fit) the row's list of
+// the keys in it.
+__device__ __forceinline__ void count_second(SelectSmem<kSelThreads>& sm, const SelectTask& s, const TileAhead& first,
+                                             uint32_t tau, uint32_t bin, bool listing) {
+  if (threadIdx.x == 0) sm.listed = 0;
+  clear_hist(sm, kBins2);
+  const int lane = threadIdx.x & 31;
+  const bool fine = bin < (uint32_t)kFineBins;
+  uint32_t above = 0, in_group = 0;
+  walk(
+      s, first, [&](int group) { above = 0, in_group = (uint32_t)group; },
+      [&](uint2 c, bool valid) {
+        const uint32_t key = key_bits(c.y);
+        const uint32_t b = first_bin(key, tau);
+        above += valid && b > bin ? 1u : 0u;
+        const bool in = valid && b == bin;
+        if (in) {  // rare: about one candidate in 500
+          atomicAdd(&sm.hist[(fine ? key - tau : key >> 11) & (kBins2 - 1)], 1u);
+          if (listing) {
+            const uint32_t at = atomicAdd(&sm.listed, 1u);
+            if (at < (uint32_t)kOwnList) sm.list[at] = make_uint2(in_group, key);
+            else put_on_list(s, make_uint2(in_group, key));
+          }
+        }
+      },
+      [&](int group) {
+        above = __reduce_add_sync(kFullMask, above);
+        if (lane == 0) s.rs.before[group] = make_uint2(above, 0u);
+      });
+  __syncthreads();
+  const uint32_t own = min(sm.listed, (uint32_t)kOwnList);
+  if (!own) return;
+  if (threadIdx.x == 0) sm.ticket = atomicAdd(s.rs.state + ST_LISTED, own);
+  __syncthreads();
+  const uint32_t cap = list_cap(s.a.d);
+  for (uint32_t i = threadIdx.x; i < own; i += kSelThreads)
+    if (dq_in_bounds(sm.ticket + i < cap, s.a.err)) s.rs.list[sm.ticket + i] = sm.list[i];
+}
+
+__device__ __forceinline__ void count_first(SelectSmem<kSelThreads>& sm, const SelectTask& s, const TileAhead& first,
+                                            uint32_t tau) {
+  clear_hist(sm, kBins);
+  walk(
+      s, first, [](int) {},
+      [&](uint2 c, bool valid) {
+        if (valid) atomicAdd(&sm.hist[first_bin(key_bits(c.y), tau)], 1u);
+      },
+      [](int) {});
+}
+
+// One CTA, after the second round's counts of the whole row are in: T and the
+// number of keys equal to it that are kept (into the state), and for each
+// group the numbers of keys above and equal to T in the groups before it.
+template <bool GLOBAL>
+__device__ __forceinline__ void resolve_row(SelectSmem<kSelThreads>& sm, const SelectTask& s, uint32_t tau,
+                                            uint32_t bin, uint32_t k_rem, bool listing, const uint32_t* counts) {
+  find_bin<kSelThreads, kBins2, GLOBAL>(sm, counts, k_rem);
+  const uint32_t digit = sm.found[0];
+  k_rem = sm.found[1];
+  __syncthreads();
+  const uint32_t listed = listing ? __ldcg(s.rs.state + ST_LISTED) : 0u;
+  // body(group, key) over the row's keys in the bin: from the list, or (very
+  // many keys are nearly equal) from all candidates
+  auto for_listed = [&](auto&& body) {
+    if (listing) {
+      for (uint32_t i = threadIdx.x; i < listed; i += kSelThreads) {
+        const uint2 x = __ldcg(s.rs.list + i);
+        body((int)x.x, x.y);
+      }
+    } else {
+      SelectTask all = s;
+      all.warp0 = threadIdx.x >> 5;
+      all.nwarps = kSelWarps;
+      int in_group = 0;
+      walk(
+          all, load_first(all), [&](int group) { in_group = group; },
+          [&](uint2 c, bool valid) {
+            const uint32_t key = key_bits(c.y);
+            if (valid && first_bin(key, tau) == bin) body(in_group, key);
+          },
+          [](int) {});
+    }
+  };
+  uint32_t T;
+  if (bin < (uint32_t)kFineBins) {
+    T = tau + (bin << kFineShift) + digit;
+  } else {  // the last 11 bits
+    const uint32_t high = ((bin - kFineBins) << 12) | digit;
+    clear_hist(sm, 2048);
+    for_listed([&](int, uint32_t key) {
+      if ((key >> 11) == high) atomicAdd(&sm.hist[key & 2047u], 1u);
+    });
+    __syncthreads();
+    find_bin<kSelThreads, 2048, false>(sm, sm.hist, k_rem);
+    T = (high << 11) | sm.found[0];
+    k_rem = sm.found[1];
+  }
+  for_listed([&](int group, uint32_t key) {
+    if (key > T) atomicAdd(&s.rs.before[group].x, 1u);
+    if (key == T) atomicAdd(&s.rs.before[group].y, 1u);
+  });
+  __threadfence();
+  __syncthreads();
+  constexpr int kPer = kMaxGroups / kSelThreads;
+  uint64_t sum = 0, total;  // keys above T | keys equal to T << 32, both below 2^32
+  for (int q = 0; q < kPer; ++q) {
+    const int i = (int)threadIdx.x * kPer + q;
+    const uint2 v = i < s.groups ? __ldcg(s.rs.before + i) : make_uint2(0u, 0u);
+    sum += (uint64_t)v.x | (uint64_t)v.y << 32;
+  }
+  uint64_t p = block_exclusive_scan<kSelThreads>(sum, &total, sm.scan);
+  for (int q = 0; q < kPer; ++q) {
+    const int i = (int)threadIdx.x * kPer + q;
+    if (i < s.groups) {
+      const uint2 v = __ldcg(s.rs.before + i);
+      s.rs.before[i] = make_uint2((uint32_t)p, (uint32_t)(p >> 32));
+      p += (uint64_t)v.x | (uint64_t)v.y << 32;
+    }
+  }
+  if (threadIdx.x == 0) {
+    s.rs.state[ST_T] = T;
+    s.rs.state[ST_NEED] = k_rem;
+  }
+}
+
+// The records of this task's groups, and e and h at the candidates not kept;
+// place(group): the numbers of keys above and equal to T before it.
+template <typename Place>
+__device__ __forceinline__ void emit_groups(const SelectTask& s, const TileAhead& first, uint32_t T, uint32_t need,
+                                            Place&& place) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t lt = (1u << lane) - 1u;
+  uint2 before = make_uint2(0u, 0u);
+  walk(
+      s, first, [&](int group) { before = place(group); },
+      [&](uint2 c, bool valid) {
+        const uint32_t key = key_bits(c.y);
+        const uint32_t gts = __ballot_sync(kFullMask, valid && key > T);
+        const uint32_t eqs = __ballot_sync(kFullMask, valid && key == T);
+        const uint32_t tie = before.y + __popc(eqs & lt);
+        if (valid) {
+          if (key > T || (key == T && tie < need)) {
+            const uint32_t pos = before.x + __popc(gts & lt) + min(tie, need);
+            if (dq_in_bounds(pos < (uint64_t)s.k, s.a.err)) s.rec[pos] = c;  // always true; keeps the write inside
+          } else {
+            put_back(s, c);
+          }
+        }
+        before.x += __popc(gts);
+        before.y += __popc(eqs);
+      },
+      [](int) {});
+}
+
+// 3. First round.
+__global__ void __launch_bounds__(kSelThreads, 2) topk_count_kernel(const CompressArgs a, int rows, void* scratch) {
   dq_pdl_enter();
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  SelectSmem& sm = *reinterpret_cast<SelectSmem*>(smem_raw);
+  __shared__ SelectSmem<kSelThreads> sm;
+  const SelectTask s = select_task(a, 0, rows, scratch);
+  count_first(sm, s, load_first(s), call_tau(s.rs.state));
+  add_hist(sm, s.rs.hist, kBins);
+}
+
+// 4. T's bin from the first-round counts, then the second round.  Where the
+// bin holds more keys than the list or T is far above tau, the row's last CTA
+// (a ticket counter; no CTA waits for another) goes on to T and the groups'
+// places; else every CTA of step 5 finds them.  For a row with too few
+// candidates instead: e as it is without any, and the top digit of all of p,
+// from which the last CTA takes a new tau.
+__global__ void __launch_bounds__(kSelThreads, 2) topk_resolve_kernel(const CompressArgs a, int64_t k, int rows, void* scratch) {
+  dq_pdl_enter();
+  __shared__ SelectSmem<kSelThreads> sm;
+  const SelectTask s = select_task(a, k, rows, scratch);
+  const TileAhead first = load_first(s);
+  const uint32_t n = find_bin<kSelThreads, kBins, true>(sm, s.rs.hist, (uint32_t)k);
+  const bool too_few = (int64_t)n < k;
+  const uint32_t bin = sm.found[0], rest = sm.found[1];
+  const bool listing = sm.found[2] <= list_cap(a.d);
+  const bool placed = bin >= (uint32_t)kFineBins || !listing;
+  __syncthreads();
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    s.rs.state[ST_PLACED] = placed ? 1u : 0u;
+    s.rs.state[ST_SHORT] = too_few ? 1u : 0u;
+    s.rs.state[ST_BIN] = bin;
+    s.rs.state[ST_REST] = rest;
+  }
+  if (!too_few) {
+    const uint32_t tau = call_tau(s.rs.state);
+    count_second(sm, s, first, tau, bin, listing);
+    add_hist(sm, s.rs.hist2, kBins2);
+    if (!placed || !last_of_row(sm, s.rs.state + ST_TICKET)) return;
+    resolve_row<true>(sm, s, tau, bin, rest, listing, s.rs.hist2);
+    return;
+  }
+  clear_hist(sm, kTopBins);
+  for (int64_t t = blockIdx.x; t < s.nt; t += gridDim.x) {
+    const uint32_t m = __ldcg(s.rs.cnt + t);
+    for (uint32_t i = threadIdx.x; i < m; i += kSelThreads) put_back(s, __ldcg(s.rs.cand + t * kTile + i));
+    __syncthreads();
+    const int64_t end = min64((t + 1) * kTile, a.d);
+    for (int64_t j = t * kTile + threadIdx.x; j < end; j += kSelThreads) atomicAdd(&sm.hist[key_of(s.e[j]) >> 20], 1u);
+  }
+  add_hist(sm, s.rs.hist2, kTopBins);
+  if (!last_of_row(sm, s.rs.state + ST_TICKET)) return;
+  find_bin<kSelThreads, kTopBins, true>(sm, s.rs.hist2, (uint32_t)k);
+  if (threadIdx.x == 0) s.rs.state[ST_TAU2] = sm.found[0] << 20;
+}
+
+// 5. T from the second-round counts, the groups' places from their counts and
+// the list, and the records.  For a row with too few candidates: the
+// candidates again, from the new tau up, and the last CTA selects among them
+// by itself.
+__global__ void __launch_bounds__(kSelThreads, 2) topk_emit_kernel(const CompressArgs a, int64_t k, int rows, void* scratch) {
+  dq_pdl_enter();
+  __shared__ SelectSmem<kSelThreads> sm;
+  extern __shared__ uint32_t places[];
+  SelectTask s = select_task(a, k, rows, scratch);
+  const TileAhead first = load_first(s);
+  const uint32_t listed = s.rs.state[ST_LISTED];
+  const uint2 early = s.rs.list[threadIdx.x];  // (the list holds at least 8192)
+  auto placed = [&](int group) { return __ldcg(s.rs.before + group); };
+  if (!s.rs.state[ST_SHORT]) {
+    if (s.rs.state[ST_PLACED]) {
+      emit_groups(s, first, s.rs.state[ST_T], s.rs.state[ST_NEED], placed);
+      return;
+    }
+    uint32_t* gt = places;
+    uint32_t* eq = places + s.groups;
+    for (int i = threadIdx.x; i < s.groups; i += kSelThreads) {
+      gt[i] = s.rs.before[i].x;
+      eq[i] = 0;
+    }
+    find_bin<kSelThreads, kBins2, true>(sm, s.rs.hist2, s.rs.state[ST_REST]);
+    const uint32_t T = call_tau(s.rs.state) + (s.rs.state[ST_BIN] << kFineShift) + sm.found[0], need = sm.found[1];
+    for (uint32_t i = threadIdx.x; i < listed; i += kSelThreads) {
+      const uint2 x = i < (uint32_t)kSelThreads ? early : s.rs.list[i];
+      if (x.y > T) atomicAdd(gt + x.x, 1u);
+      if (x.y == T) atomicAdd(eq + x.x, 1u);
+    }
+    __syncthreads();
+    // exclusive prefix of both; an odd number of groups per thread keeps the
+    // threads' shared-memory accesses on different banks
+    const int per = ((s.groups + kSelThreads - 1) / kSelThreads) | 1;
+    const int i0 = min((int)threadIdx.x * per, s.groups), i1 = min(i0 + per, s.groups);
+    uint64_t sum = 0, total;  // keys above T | keys equal to T << 32, both below 2^32
+    for (int i = i0; i < i1; ++i) sum += (uint64_t)gt[i] | (uint64_t)eq[i] << 32;
+    uint64_t p = block_exclusive_scan<kSelThreads>(sum, &total, sm.scan);
+    for (int i = i0; i < i1; ++i) {
+      const uint64_t v = (uint64_t)gt[i] | (uint64_t)eq[i] << 32;
+      gt[i] = (uint32_t)p;
+      eq[i] = (uint32_t)(p >> 32);
+      p += v;
+    }
+    __syncthreads();
+    emit_groups(s, first, T, need, [&](int group) { return make_uint2(gt[group], eq[group]); });
+    return;
+  }
+  const uint32_t tau = s.rs.state[ST_TAU2];
+  for (int64_t t = blockIdx.x; t < s.nt; t += gridDim.x) {
+    constexpr int kRows = kTile / (4 * kSelThreads);
+    float v[kRows][4];
+    uint32_t cmask[kRows];
+#pragma unroll
+    for (int i = 0; i < kRows; ++i) {
+      const int64_t j = t * kTile + 4 * ((int64_t)i * kSelThreads + threadIdx.x);
+      cmask[i] = 0;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        v[i][q] = 0.f;
+        if (j + q < a.d) {
+          v[i][q] = s.e[j + q];
+          if (key_of(v[i][q]) >= tau) {
+            cmask[i] |= 1u << q;
+            const float en = __fsub_rn(v[i][q], v[i][q]);
+            s.e[j + q] = en;
+            if (s.h) s.h[j + q] = __fadd_rn(__fmul_rn(a.lr, s.g[j + q]), en);
+          }
+        }
+      }
+    }
+    const uint32_t n = write_tile_candidates<kSelThreads, kRows>(v, cmask, t * kTile, s.rs.cand + t * kTile,
+                                                                 sm.warp_sums, a.err);
+    if (threadIdx.x == 0) s.rs.cnt[t] = n;
+  }
+  if (!last_of_row(sm, s.rs.state + ST_TICKET + 1)) return;
+  s.warp0 = threadIdx.x >> 5;
+  s.nwarps = kSelWarps;
+  count_first(sm, s, load_first(s), tau);
+  __syncthreads();
+  find_bin<kSelThreads, kBins, false>(sm, sm.hist, (uint32_t)k);
+  const uint32_t bin = sm.found[0], rest = sm.found[1];
+  const bool listing = sm.found[2] <= list_cap(a.d);
+  __syncthreads();
+  count_second(sm, s, load_first(s), tau, bin, listing);
+  __threadfence();
+  __syncthreads();
+  resolve_row<false>(sm, s, tau, bin, rest, listing, sm.hist);
+  __threadfence();
+  __syncthreads();
+  emit_groups(s, load_first(s), __ldcg(s.rs.state + ST_T), __ldcg(s.rs.state + ST_NEED), placed);
+}
+
+// ---------------------------------------------------------------------------
+// The whole step of a worker in one launch, by C CTAs (one cluster) that keep
+// p on chip: CTA r has the r-th part of the vector.  The digits of T (11 + 10
+// + 10 bits) come from three counting rounds, the cluster's counts read
+// through distributed shared memory; then e, h and the records, a warp per
+// stretch of consecutive elements.  At these sizes launches and memory
+// latency are most of the time.
+// ---------------------------------------------------------------------------
+struct ChipSmem {
+  uint32_t hist[2048 + 1024 + 1024];            // the rounds' counts (read by the cluster)
+  uint32_t coarse[(2048 + 1024 + 1024) / kGroup];  // sums of kGroup bins (read by the cluster)
+  uint32_t found[3][4];                          // per round: bin, rest of k, lower ranks' keys above the bin and in it
+  uint32_t warp_gt[kChipThreads / 32], warp_eq[kChipThreads / 32];
+};
+
+// Elements of a CTA's part: a multiple of 4.
+__host__ __device__ constexpr int64_t chip_part(int64_t d, int ctas) { return ((d + ctas - 1) / ctas + 3) / 4 * 4; }
+
+// One warp: the bin b of the cluster's summed counts with count(> b) < k_rem
+// <= count(>= b): first its group, from every CTA's group sums, then the bin,
+// from every CTA's counts of the group.  out: b, k_rem - count(> b), and the
+// counts of the CTAs of lower rank in the bins above b and in b.
+template <int C, int BINS>
+__device__ __forceinline__ void cluster_find(uint32_t* hist, uint32_t* coarse, uint32_t k_rem, int rank, uint32_t* out) {
+  constexpr int G = BINS / kGroup;
+  static_assert(G <= 32 && kGroup == 64, "a group per lane, two bins per lane");
   cg::cluster_group cluster = cg::this_cluster();
-  const int rank = (int)cluster.block_rank();
+  const int lane = threadIdx.x & 31;
+  // the inclusive sums of two values from lane 0 up
+  auto scan = [&](uint32_t& x, uint32_t& y) {
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const uint32_t a = __shfl_up_sync(kFullMask, x, off), b = __shfl_up_sync(kFullMask, y, off);
+      if (lane >= off) {
+        x += a;
+        y += b;
+      }
+    }
+  };
+  uint32_t all = 0, low = 0;  // of group G - 1 - lane
+  if (lane < G) {
+#pragma unroll
+    for (int r = 0; r < C; ++r) {
+      const uint32_t* at = coarse + G - 1 - lane;
+      const uint32_t x = C == 1 ? *at : *cluster.map_shared_rank(at, r);
+      if (r < rank) low += x;
+      all += x;
+    }
+  }
+  uint32_t cum = all, cum_low = low;
+  scan(cum, cum_low);
+  const uint32_t hit = __ballot_sync(kFullMask, cum - all < k_rem && k_rem <= cum);
+  const int src = hit ? __ffs(hit) - 1 : 0;
+  const uint32_t above = __shfl_sync(kFullMask, cum - all, src), above_low = __shfl_sync(kFullMask, cum_low - low, src);
+  // bins 63 - 2 lane (y) and 62 - 2 lane (x) of the group
+  const uint32_t bin = (uint32_t)(G - 1 - src) * kGroup + kGroup - 2 - 2 * lane;
+  uint2 n = make_uint2(0u, 0u), m = n;
+#pragma unroll
+  for (int r = 0; r < C; ++r) {
+    const uint2* at = reinterpret_cast<const uint2*>(hist + bin);
+    const uint2 x = C == 1 ? *at : *cluster.map_shared_rank(at, r);
+    if (r < rank) {
+      m.x += x.x;
+      m.y += x.y;
+    }
+    n.x += x.x;
+    n.y += x.y;
+  }
+  cum = n.x + n.y;
+  cum_low = m.x + m.y;
+  scan(cum, cum_low);
+  cum += above - n.x - n.y;  // keys above this lane's two bins
+  cum_low += above_low - m.x - m.y;
+  if (cum < k_rem && k_rem - cum <= n.y) {
+    out[0] = bin + 1;
+    out[1] = k_rem - cum;
+    out[2] = cum_low;
+    out[3] = m.y;
+  } else if (cum + n.y < k_rem && k_rem - cum - n.y <= n.x) {
+    out[0] = bin;
+    out[1] = k_rem - cum - n.y;
+    out[2] = cum_low + m.y;
+    out[3] = m.x;
+  }
+}
+
+template <int C, bool KEEP_H>
+__global__ void __launch_bounds__(kChipThreads, 1) topk_chip_kernel(const CompressArgs a, int64_t k) {
+  dq_pdl_enter();
+  extern __shared__ __align__(16) float p[];
+  __shared__ __align__(16) ChipSmem sm;
+  constexpr int kWarps = kChipThreads / 32;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int rank = blockIdx.x;
   const int row = blockIdx.y;
   const int worker = a.worker0 + row;
-  float* e = a.e + (int64_t)(worker - a.row0) * a.ld;
-  float* h = KEEP_H ? a.h + (int64_t)(worker - a.row0) * a.ld : nullptr;
-  const float* g = a.g + (int64_t)row * a.g_stride;
+  const int64_t part = chip_part(a.d, C);
+  const int64_t first = min64(a.d, part * rank);
+  const int d = (int)(min64(a.d, first + part) - first);  // elements of this part
+  const float* g = a.g + (int64_t)row * a.g_stride + first;
+  float* e = a.e + (int64_t)(worker - a.row0) * a.ld + first;
+  float* h = KEEP_H ? a.h + (int64_t)(worker - a.row0) * a.ld + first : nullptr;
   uint2* rec = reinterpret_cast<uint2*>(a.msg + (int64_t)row * a.msg_stride);
-  RowScratch rs = row_scratch(scratch, a.d, worker - a.row0);
-  const int64_t nt = tiles_of(a.d);
-  uint32_t* gpre = rs.gpre + (int64_t)rank * (nt + 1);  // this CTA's private prefix array
-  const uint32_t tau_word = rs.state[ST_TAU];
-  const uint32_t tau = tau_word & 0x7FFFFFFFu;
-  bool fast = (tau_word & kTauValid) != 0;
-  const bool reg_tiles = nt <= (int64_t)kSelThreads * kRegTiles;
-
-  // the first pass's tile counts
-  uint32_t cnt_r[kRegTiles];
+  for (int i = threadIdx.x; i < 4096; i += kChipThreads) sm.hist[i] = 0;
+  __syncthreads();
+  // p, and the counts of its top 11 bits
+  constexpr int kLoads = 4;  // loads of 16 bytes of each vector in flight
+  for (int j0 = 4 * threadIdx.x; j0 < d; j0 += 4 * kLoads * kChipThreads) {
+    float4 gv[kLoads], ev[kLoads];
 #pragma unroll
-  for (int q = 0; q < kRegTiles; ++q) {
-    const int64_t t = (int64_t)threadIdx.x * kRegTiles + q;
-    cnt_r[q] = (fast && reg_tiles && t < nt) ? rs.cnt[t] : 0u;
-  }
-  uint32_t b0 = 0;  // top digit of T
-
-  // This CTA's share: candidates [F0, F1) in prefix coordinates, lying in
-  // tiles [ta, tb).  With one chunk, sm.tpre[i] is the prefix at tile ta + i.
-  int64_t ta = 0, tb = 0;
-  uint32_t F0 = 0, F1 = 0;
-  bool one_chunk = true, cached = false;
-  uint32_t lo1 = 0, hi1 = 0;  // the share's bounds when it is one chunk
-
-  // Loads the prefix of tiles [tc0, tc0 + n] from gpre into sm.tpre.
-  auto load_chunk = [&](int64_t tc0, int n) {
-    for (int i = threadIdx.x; i <= n; i += kSelThreads) sm.tpre[i] = gpre[tc0 + i];
-    __syncthreads();
-  };
-
-  const int64_t t0 = nt * rank / kCluster, t1 = nt * (rank + 1) / kCluster;  // this CTA's tiles
-
-  auto set_up = [&]() {
-    if (fast && reg_tiles) {
-      // the tile counts are in registers: one scan gives every prefix
-      uint32_t local = 0;
-#pragma unroll
-      for (int q = 0; q < kRegTiles; ++q) local += cnt_r[q];
-      uint32_t N;
-      const uint32_t ex = block_exclusive_scan<kSelThreads>(local, &N, sm.warp_sums);
-      F0 = (uint32_t)((uint64_t)N * rank / kCluster);
-      F1 = (uint32_t)((uint64_t)N * (rank + 1) / kCluster);
-      if (threadIdx.x == 0) {
-        sm.span[0] = 0xFFFFFFFFu;
-        sm.span[1] = 0;
+    for (int i = 0; i < kLoads; ++i) {
+      const int j = j0 + 4 * i * kChipThreads;
+      if (j + 3 < d) {
+        gv[i] = __ldcs(reinterpret_cast<const float4*>(g + j));
+        ev[i] = __ldcs(reinterpret_cast<const float4*>(e + j));
       }
-      __syncthreads();
-      uint32_t p = ex;
+    }
 #pragma unroll
-      for (int q = 0; q < kRegTiles; ++q) {
-        const uint32_t t = threadIdx.x * kRegTiles + q;
-        if (cnt_r[q] > 0 && p < F1 && p + cnt_r[q] > F0) {
-          atomicMin(&sm.span[0], t);
-          atomicMax(&sm.span[1], t);
-        }
-        p += cnt_r[q];
-      }
-      __syncthreads();
-      if (F0 < F1) {
-        ta = sm.span[0];
-        tb = (int64_t)sm.span[1] + 1;
+    for (int i = 0; i < kLoads; ++i) {
+      const int j = j0 + 4 * i * kChipThreads;
+      float v[4];
+      if (j + 3 < d) {
+        v[0] = ef_p(a.lr, gv[i].x, ev[i].x);
+        v[1] = ef_p(a.lr, gv[i].y, ev[i].y);
+        v[2] = ef_p(a.lr, gv[i].z, ev[i].z);
+        v[3] = ef_p(a.lr, gv[i].w, ev[i].w);
+        *reinterpret_cast<float4*>(p + j) = make_float4(v[0], v[1], v[2], v[3]);
       } else {
-        ta = tb = 0;
-      }
-      p = ex;
 #pragma unroll
-      for (int q = 0; q < kRegTiles; ++q) {
-        const int64_t t = (int64_t)threadIdx.x * kRegTiles + q;
-        if (t >= ta && t < tb) sm.tpre[t - ta] = p;
-        p += cnt_r[q];
-        if (t + 1 == tb) sm.tpre[tb - ta] = p;
+        for (int q = 0; q < 4; ++q)
+          if (j + q < d) p[j + q] = v[q] = ef_p(a.lr, g[j + q], e[j + q]);
       }
-      __syncthreads();
-      one_chunk = true;
-    } else if (fast) {
-      // all tiles' prefix through this CTA's private array in global memory
-      uint32_t N = 0;
-      for (int64_t base = 0; base < nt; base += kSelThreads) {
-        const int64_t t = base + threadIdx.x;
-        N += block_sum<kSelThreads>(t < nt ? rs.cnt[t] : 0u, sm.warp_sums);
-      }
-      F0 = (uint32_t)((uint64_t)N * rank / kCluster);
-      F1 = (uint32_t)((uint64_t)N * (rank + 1) / kCluster);
-      if (threadIdx.x == 0) {
-        sm.span[0] = 0xFFFFFFFFu;
-        sm.span[1] = 0;
-      }
-      __syncthreads();
-      uint32_t run = 0;
-      for (int64_t base = 0; base < nt; base += kSelThreads) {
-        const int64_t t = base + threadIdx.x;
-        const uint32_t c = t < nt ? rs.cnt[t] : 0u;
-        uint32_t total;
-        const uint32_t p = run + block_exclusive_scan<kSelThreads>(c, &total, sm.warp_sums);
-        if (t < nt) {
-          gpre[t] = p;
-          if (c > 0 && p < F1 && p + c > F0) {
-            atomicMin(&sm.span[0], (uint32_t)t);
-            atomicMax(&sm.span[1], (uint32_t)t);
-          }
-        }
-        run += total;
-      }
-      if (threadIdx.x == 0) gpre[nt] = run;
-      __syncthreads();
-      if (F0 < F1) {
-        ta = sm.span[0];
-        tb = (int64_t)sm.span[1] + 1;
-      } else {
-        ta = tb = 0;
-      }
-      one_chunk = (tb - ta) <= kChunkTiles;
-      if (one_chunk && tb > ta) load_chunk(ta, (int)(tb - ta));
-    } else {
-      // re-extract this CTA's tiles from p: every element with top digit >= b0
-      for (int64_t t = t0; t < t1; ++t) {
-        const int64_t tile0 = t * kTile;
-        float v[kSelRows][4];
-        uint32_t cmask[kSelRows];
 #pragma unroll
-        for (int i = 0; i < kSelRows; ++i) {
-          const int64_t j = tile0 + 4 * ((int64_t)i * kSelThreads + threadIdx.x);
-          cmask[i] = 0;
-          if (j + 3 < a.d) {
-            const float4 x = *reinterpret_cast<const float4*>(e + j);
-            v[i][0] = x.x; v[i][1] = x.y; v[i][2] = x.z; v[i][3] = x.w;
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-              if ((key_of(v[i][q]) >> 20) >= b0) cmask[i] |= 1u << q;
-          } else {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              v[i][q] = (j + q < a.d) ? e[j + q] : 0.f;
-              if (j + q < a.d && (key_of(v[i][q]) >> 20) >= b0) cmask[i] |= 1u << q;
-            }
-          }
-        }
-        const uint32_t n = write_tile_candidates<kSelThreads, kSelRows, true>(v, cmask, tile0,
-                                                                              rs.cand + t * kTile, sm.warp_sums, a.err);
-        if (threadIdx.x == 0) rs.cnt[t] = n;
-      }
-      __syncthreads();
-      // prefix of this CTA's own tiles, from 0
-      uint32_t run = 0;
-      for (int64_t base = t0; base < t1; base += kSelThreads) {
-        const int64_t t = base + threadIdx.x;
-        const uint32_t c = t < t1 ? rs.cnt[t] : 0u;
-        uint32_t total;
-        const uint32_t p = run + block_exclusive_scan<kSelThreads>(c, &total, sm.warp_sums);
-        if (t < t1) gpre[t] = p;
-        run += total;
-      }
-      if (threadIdx.x == 0) gpre[t1] = run;
-      __syncthreads();
-      ta = t0;
-      tb = t1;
-      F0 = 0;
-      F1 = run;
-      one_chunk = (tb - ta) <= kChunkTiles;
-      if (one_chunk && tb > ta) load_chunk(ta, (int)(tb - ta));
-    }
-    cached = false;
-    lo1 = hi1 = 0;
-    if (one_chunk && tb > ta) {
-      lo1 = max(F0, sm.tpre[0]);
-      hi1 = min(F1, sm.tpre[tb - ta]);
-      cached = hi1 - lo1 <= (uint32_t)kCacheCap;
-    }
-  };
-
-  // Runs body(candidate) over this CTA's share, kBatch loads in flight per
-  // thread; with `fill`, also keeps the share on chip.
-  // (body(candidate, valid) is called by every thread of the block the same
-  // number of times, so it may use warp collectives.)
-  auto for_each = [&](auto&& body, bool fill) {
-    if (fill) {
-      // The share becomes the on-chip copy (cached: one chunk of tiles
-      // [ta, tb), candidates [lo1, hi1)).  First every candidate slot gets
-      // its tile: each tile with candidates in the share marks its first
-      // slot with its number, and a block-wide running maximum over the
-      // slots carries each mark forward (the marks grow with the slot).  The
-      // cost does not depend on how the candidates spread over the tiles,
-      // and the loads below need no search.
-      const int n = (int)(tb - ta);
-      const uint32_t S = hi1 - lo1;
-      for (uint32_t f = threadIdx.x; f < S; f += kSelThreads) sm.cache[f].x = 0u;
-      __syncthreads();
-      for (int i = threadIdx.x; i < n; i += kSelThreads) {
-        const uint32_t a0 = sm.tpre[i], a1 = sm.tpre[i + 1];
-        if (a0 < a1 && a1 > lo1 && a0 < hi1) sm.cache[max(a0, lo1) - lo1].x = (uint32_t)i;
-      }
-      __syncthreads();
-      const uint32_t per = (S + kSelThreads - 1) / kSelThreads;
-      const uint32_t g0 = min(threadIdx.x * per, S), g1 = min(g0 + per, S);
-      uint32_t run = 0;
-      for (uint32_t f = g0; f < g1; ++f) run = max(run, sm.cache[f].x);
-      // exclusive running maximum over the threads' runs
-      {
-        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-        uint32_t x = run;
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-          const uint32_t y = __shfl_up_sync(kFullMask, x, off);
-          if (lane >= off) x = max(x, y);
-        }
-        if (lane == 31) sm.warp_sums[warp] = x;
-        __syncthreads();
-        uint32_t before = 0;
-#pragma unroll
-        for (int w = 0; w < kSelThreads / 32; ++w)
-          if (w < warp) before = max(before, sm.warp_sums[w]);
-        const uint32_t up = __shfl_up_sync(kFullMask, x, 1);
-        run = max(before, lane > 0 ? up : 0u);
-        __syncthreads();
-      }
-      for (uint32_t f = g0; f < g1; ++f) {
-        run = max(run, sm.cache[f].x);
-        sm.cache[f].x = run;
-      }
-      __syncthreads();
-      for (uint32_t base = lo1; base < hi1; base += kSelThreads * kBatch) {
-        uint2 c[kBatch];
-#pragma unroll
-        for (int u = 0; u < kBatch; ++u) {
-          const uint32_t f = base + u * kSelThreads + threadIdx.x;
-          c[u] = make_uint2(0u, 0u);
-          if (f < hi1) {
-            const uint32_t i = sm.cache[f - lo1].x;
-            c[u] = rs.cand[(ta + i) * kTile + (f - sm.tpre[i])];
-          }
-        }
-#pragma unroll
-        for (int u = 0; u < kBatch; ++u) {
-          const uint32_t f = base + u * kSelThreads + threadIdx.x;
-          if (f < hi1) sm.cache[f - lo1] = c[u];
-          body(c[u], f < hi1);
-        }
-      }
-      __syncthreads();
-      return;
-    }
-    if (cached) {
-      for (uint32_t base = lo1; base < hi1; base += kSelThreads) {
-        const uint32_t f = base + threadIdx.x;
-        body(f < hi1 ? sm.cache[f - lo1] : make_uint2(0u, 0u), f < hi1);
-      }
-      return;
-    }
-    for (int64_t tc0 = ta; tc0 < tb; tc0 += kChunkTiles) {
-      const int n = (int)min64(kChunkTiles, tb - tc0);
-      if (!one_chunk) load_chunk(tc0, n);
-      const uint32_t lo = max(F0, sm.tpre[0]), hi = min(F1, sm.tpre[n]);
-      for (uint32_t base = lo; base < hi; base += kSelThreads * kBatch) {
-        uint2 c[kBatch];
-#pragma unroll
-        for (int u = 0; u < kBatch; ++u) {
-          const uint32_t f = base + u * kSelThreads + threadIdx.x;
-          c[u] = (f < hi) ? chunk_candidate(rs.cand, sm.tpre, n, tc0, f) : make_uint2(0u, 0u);
-        }
-#pragma unroll
-        for (int u = 0; u < kBatch; ++u) {
-          const uint32_t f = base + u * kSelThreads + threadIdx.x;
-          if (fill && f < hi) sm.cache[f - lo] = c[u];
-          body(c[u], f < hi);
-        }
-      }
-      if (!one_chunk) __syncthreads();  // sm.tpre is reloaded for the next chunk
-    }
-  };
-
-  // Histogram of the top digit over all of p in this CTA's tiles.
-  auto histogram_p = [&]() {
-    for (int64_t t = t0; t < t1; ++t) {
-#pragma unroll
-      for (int i = 0; i < kSelRows; ++i) {
-        const int64_t j = t * kTile + 4 * ((int64_t)i * kSelThreads + threadIdx.x);
-        float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (j + 3 < a.d) {
-          x = *reinterpret_cast<const float4*>(e + j);
-        } else {
-          if (j < a.d) x.x = e[j];
-          if (j + 1 < a.d) x.y = e[j + 1];
-          if (j + 2 < a.d) x.z = e[j + 2];
-        }
-        // (all of p: its top digits spread over many bins, so plain atomics)
-        if (j < a.d) atomicAdd(&sm.hist_t[key_of(x.x) >> 20], 1u);
-        if (j + 1 < a.d) atomicAdd(&sm.hist_t[key_of(x.y) >> 20], 1u);
-        if (j + 2 < a.d) atomicAdd(&sm.hist_t[key_of(x.z) >> 20], 1u);
-        if (j + 3 < a.d) atomicAdd(&sm.hist_t[key_of(x.w) >> 20], 1u);
-      }
-    }
-    __syncthreads();
-  };
-
-  uint32_t T = 0, need = 0;
-  for (int attempt = 0; attempt < 2; ++attempt) {
-    if (attempt > 0) cluster.sync();  // every CTA is done reading the first round's histograms
-    for (int i = threadIdx.x; i < kBins0; i += kSelThreads) sm.hist_t[i] = 0;
-    for (int i = threadIdx.x; i < kBins1; i += kSelThreads) {
-      sm.hist_a[i] = 0;
-      sm.hist_b[i] = 0;
-    }
-    __syncthreads();
-    // top digit: over the candidates, or over all of p
-    bool filled = false;
-    if (fast) {
-      set_up();
-      for_each(
-          [&](uint2 c, bool valid) {
-            warp_hist_add(sm.hist_t, key_bits(c.y) >> 20, valid, kFullMask);
-          },
-          cached);
-      filled = cached;
-    } else {
-      histogram_p();
-    }
-    cluster_sum<kBins0>(cluster, sm.hist_t, sm.pre_t, rank, sm);
-    if (threadIdx.x == 0) {
-      sm.sel[0] = 0;
-      sm.sel[1] = (uint32_t)k;
-    }
-    __syncthreads();
-    block_select<kSelThreads, kBins0>(sm.full, (uint32_t)k, &sm.sel[0], &sm.sel[1], sm.warp_sums);
-    b0 = sm.sel[0];
-    const uint32_t krem0 = sm.sel[1];
-    if (!fast) set_up();  // candidates: every element with top digit >= b0
-    // middle digit
-    for_each(
-        [&](uint2 c, bool valid) {
-          const uint32_t key = key_bits(c.y);
-          if (valid && (key >> 20) == b0) atomicAdd(&sm.hist_a[(key >> 10) & 1023u], 1u);
-        },
-        cached && !filled);
-    cluster_sum<kBins1>(cluster, sm.hist_a, sm.pre_a, rank, sm);
-    if (threadIdx.x == 0) {
-      sm.sel[2] = 0;
-      sm.sel[3] = krem0;
-    }
-    __syncthreads();
-    block_select<kSelThreads, kBins1>(sm.full, krem0, &sm.sel[2], &sm.sel[3], sm.warp_sums);
-    const uint32_t hi21 = (b0 << 10) | sm.sel[2];
-    const uint32_t krem1 = sm.sel[3];
-    // low digit
-    for_each(
-        [&](uint2 c, bool valid) {
-          const uint32_t key = key_bits(c.y);
-          if (valid && (key >> 10) == hi21) atomicAdd(&sm.hist_b[key & 1023u], 1u);
-        },
-        false);
-    cluster_sum<kBins1>(cluster, sm.hist_b, sm.pre_b, rank, sm);
-    if (threadIdx.x == 0) {
-      sm.sel[4] = 0;
-      sm.sel[5] = krem1;
-    }
-    __syncthreads();
-    block_select<kSelThreads, kBins1>(sm.full, krem1, &sm.sel[4], &sm.sel[5], sm.warp_sums);
-    T = (hi21 << 10) | sm.sel[4];
-    need = sm.sel[5];
-    // T is exact when every key >= T was a candidate, i.e. T >= tau (the
-    // same decision in every CTA of the cluster).
-    if (!fast || T >= tau) break;
-    fast = false;
-  }
-
-  // Every read of another CTA's shared memory is done: arrive at the
-  // cluster barrier now, wait for the others only before leaving (no CTA
-  // leaves while another may still read its shared memory).
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-
-  // Keys above and equal to T in the shares of the CTAs before this one, from
-  // the histogram sums over them: top digit above b0, or middle digit above
-  // T's, or low digit above T's; and keys equal to T.
-  uint32_t gt_before = 0, tie_before = 0;
-  {
-    const uint32_t b1 = (T >> 10) & 1023u, b2 = T & 1023u;
-    uint32_t part = 0;
-    for (int i = threadIdx.x; i < kBins0; i += kSelThreads)
-      if ((uint32_t)i > b0) part += sm.pre_t[i];
-    for (int i = threadIdx.x; i < kBins1; i += kSelThreads) {
-      if ((uint32_t)i > b1) part += sm.pre_a[i];
-      if ((uint32_t)i > b2) part += sm.pre_b[i];
-    }
-    gt_before = block_sum<kSelThreads>(part, sm.warp_sums);
-    tie_before = sm.pre_b[b2];
-  }
-
-  // Kept records: position = (keys > T before) + min(keys == T before, need).
-  auto keep = [&](uint2 c) {
-    const uint32_t j = c.x;
-    const float p = __uint_as_float(c.y);
-    const float ej = __fsub_rn(p, p);
-    e[j] = ej;
-    if constexpr (KEEP_H) h[j] = __fadd_rn(__fmul_rn(a.lr, g[j]), ej);
-  };
-  if (cached) {
-    // Each warp takes kEmitRows rows of 32 consecutive candidates; ballots
-    // rank the lanes, one exchange of the warps' counts ranks the warps.
-    constexpr int kEmitRows = 8;
-    constexpr int kWarps = kSelThreads / 32;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint32_t lt = (1u << lane) - 1u;
-    for (uint32_t base = lo1; base < hi1; base += kWarps * kEmitRows * 32) {
-      const uint32_t seg = base + (uint32_t)warp * kEmitRows * 32;
-      uint2 c[kEmitRows];
-      uint32_t gtb[kEmitRows], tieb[kEmitRows];
-      uint32_t wg = 0, wt = 0;
-#pragma unroll
-      for (int u = 0; u < kEmitRows; ++u) {
-        const uint32_t f = seg + 32u * u + lane;
-        const bool valid = f < hi1;
-        c[u] = valid ? sm.cache[f - lo1] : make_uint2(0u, 0u);
-        const uint32_t key = key_bits(c[u].y);
-        gtb[u] = __ballot_sync(kFullMask, valid && key > T);
-        tieb[u] = __ballot_sync(kFullMask, valid && key == T);
-        wg += __popc(gtb[u]);
-        wt += __popc(tieb[u]);
-      }
-      if (lane == 0) sm.warp_sums[warp] = wg | (wt << 16);
-      __syncthreads();
-      uint32_t before = 0, total = 0;
-#pragma unroll
-      for (int w = 0; w < kWarps; ++w) {
-        const uint32_t v = sm.warp_sums[w];
-        if (w < warp) before += v;
-        total += v;
-      }
-      __syncthreads();
-      uint32_t rg = gt_before + (before & 0xFFFFu), rt = tie_before + (before >> 16);
-#pragma unroll
-      for (int u = 0; u < kEmitRows; ++u) {
-        const uint32_t my_g = rg + __popc(gtb[u] & lt), my_t = rt + __popc(tieb[u] & lt);
-        const bool is_gt = (gtb[u] >> lane) & 1u, is_tie = (tieb[u] >> lane) & 1u;
-        if (is_gt || (is_tie && my_t < need)) {
-          const uint32_t pos = my_g + min(my_t, need);
-          if (dq_in_bounds(pos < (uint64_t)k, a.err)) {  // always true; keeps the write inside the message
-            rec[pos] = c[u];
-            keep(c[u]);
-          }
-        }
-        rg += __popc(gtb[u]);
-        rt += __popc(tieb[u]);
-      }
-      gt_before += total & 0xFFFFu;
-      tie_before += total >> 16;
-    }
-  } else {
-    auto emit = [&](uint2 c, bool valid) {
-      const uint32_t key = key_bits(c.y);
-      const bool is_gt = valid && key > T;
-      const bool is_tie = valid && key == T;
-      uint32_t total;
-      const uint32_t ex = block_exclusive_scan<kSelThreads>((uint32_t)is_gt | ((uint32_t)is_tie << 16), &total,
-                                                            sm.warp_sums);
-      const uint32_t ties = tie_before + (ex >> 16);
-      if (is_gt || (is_tie && ties < need)) {
-        const uint32_t pos = gt_before + (ex & 0xFFFFu) + min(ties, need);
-        if (dq_in_bounds(pos < (uint64_t)k, a.err)) {  // always true; keeps the write inside the message
-          rec[pos] = c;
-          keep(c);
-        }
-      }
-      gt_before += total & 0xFFFFu;
-      tie_before += total >> 16;
-    };
-    for (int64_t tc0 = ta; tc0 < tb; tc0 += kChunkTiles) {
-      const int n = (int)min64(kChunkTiles, tb - tc0);
-      if (!one_chunk) load_chunk(tc0, n);
-      const uint32_t lo = max(F0, sm.tpre[0]), hi = min(F1, sm.tpre[n]);
-      for (uint32_t base = lo; base < hi; base += kSelThreads * kBatch) {
-        uint2 c[kBatch];
-#pragma unroll
-        for (int u = 0; u < kBatch; ++u) {
-          const uint32_t f = base + u * kSelThreads + threadIdx.x;
-          c[u] = (f < hi) ? chunk_candidate(rs.cand, sm.tpre, n, tc0, f) : make_uint2(0u, 0u);
-        }
-#pragma unroll
-        for (int u = 0; u < kBatch; ++u) emit(c[u], base + u * kSelThreads + threadIdx.x < hi);
-      }
-      __syncthreads();
+      for (int q = 0; q < 4; ++q)
+        if (j + q < d) atomicAdd(&sm.hist[key_of(v[q]) >> 20], 1u);
     }
   }
-
-  // For the next call: the candidate threshold, 15/16 of T.
-  if (rank == 0 && threadIdx.x == 0) {
-    const float t_next = __fmul_rn(__uint_as_float(T), 0.9375f);
-    rs.state[ST_TAU] = kTauValid | key_of(t_next);
+  uint32_t T = 0, need = (uint32_t)k;
+  uint32_t gt_before = 0, eq_before = 0;  // keys above and equal to T in the parts before this one
+#pragma unroll
+  for (int round = 0; round < 3; ++round) {
+    uint32_t* hist = sm.hist + (round == 0 ? 0 : round == 1 ? 2048 : 3072);
+    uint32_t* coarse = sm.coarse + (round == 0 ? 0 : round == 1 ? 2048 : 3072) / kGroup;
+    const int low = 20 - 10 * round;  // key bits below this round's digit
+    if (round > 0)
+      for (int j = threadIdx.x; j < d; j += kChipThreads) {
+        const uint32_t key = key_of(p[j]);
+        if ((key >> (low + 10)) == T) atomicAdd(&hist[(key >> low) & 1023u], 1u);
+      }
+    __syncthreads();
+    for (int group = warp; group < (round == 0 ? 2048 : 1024) / kGroup; group += kWarps) {
+      const uint32_t n = __reduce_add_sync(kFullMask, hist[group * kGroup + lane] + hist[group * kGroup + 32 + lane]);
+      if (lane == 0) coarse[group] = n;
+    }
+    if constexpr (C > 1) cg::this_cluster().sync();
+    else __syncthreads();
+    if (warp == 0) {
+      if (round == 0) cluster_find<C, 2048>(hist, coarse, need, rank, sm.found[round]);
+      else cluster_find<C, 1024>(hist, coarse, need, rank, sm.found[round]);
+    }
+    __syncthreads();
+    T = round == 0 ? sm.found[0][0] : T << 10 | sm.found[round][0];
+    need = sm.found[round][1];
+    gt_before += sm.found[round][2];
+    eq_before = sm.found[round][3];
   }
-  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  // every read of another CTA's shared memory is done: no CTA leaves before
+  // all have said so
+  if constexpr (C > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  // warp w takes the elements [w, w + 1) * stretch, 32 at a time
+  const int stretch = (d + 32 * kWarps - 1) / (32 * kWarps) * 32;
+  const int j0 = min(warp * stretch, d), j1 = min(j0 + stretch, d);
+  uint32_t gt = 0, eq = 0;
+  for (int j = j0 + lane; j < j1; j += 32) {
+    const uint32_t key = key_of(p[j]);
+    gt += key > T ? 1u : 0u;
+    eq += key == T ? 1u : 0u;
+  }
+  gt = __reduce_add_sync(kFullMask, gt);
+  eq = __reduce_add_sync(kFullMask, eq);
+  if (lane == 0) {
+    sm.warp_gt[warp] = gt;
+    sm.warp_eq[warp] = eq;
+  }
+  __syncthreads();
+  gt = gt_before + __reduce_add_sync(kFullMask, lane < warp ? sm.warp_gt[lane] : 0u);
+  eq = eq_before + __reduce_add_sync(kFullMask, lane < warp ? sm.warp_eq[lane] : 0u);
+  const uint32_t lt = (1u << lane) - 1u;
+  for (int base = j0; base < j1; base += 32) {
+    const int j = base + lane;
+    const bool valid = j < j1;
+    const float v = valid ? p[j] : 0.f;
+    const uint32_t key = key_of(v);
+    const uint32_t gts = __ballot_sync(kFullMask, valid && key > T);
+    const uint32_t eqs = __ballot_sync(kFullMask, valid && key == T);
+    const uint32_t tie = eq + __popc(eqs & lt);
+    if (valid) {
+      const bool kept = key > T || (key == T && tie < need);
+      if (kept) {
+        const uint32_t pos = gt + __popc(gts & lt) + min(tie, need);
+        if (dq_in_bounds(pos < (uint64_t)k, a.err))  // always true; keeps the write inside the message
+          rec[pos] = make_uint2((uint32_t)(first + j), __float_as_uint(v));
+      }
+      const float en = kept ? __fsub_rn(v, v) : v;
+      e[j] = en;
+      if constexpr (KEEP_H) h[j] = __fadd_rn(__fmul_rn(a.lr, g[j]), en);
+    }
+    gt += __popc(gts);
+    eq += __popc(eqs);
+  }
+  if constexpr (C > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
 // ---------------------------------------------------------------------------
@@ -1156,50 +1372,115 @@ size_t topk_scratch_bytes(int64_t d, int32_t rows, int32_t nworkers) {
   return (size_t)(row_words(d) * rows + server_words) * 4u;
 }
 
-// Raises a kernel's dynamic shared memory limit when its static plus dynamic
-// shared memory exceeds the default 48 KB.  The attribute belongs to the
-// function on the current device, so what has been set is remembered per
-// device ordinal (`done` has kSmemDevices slots; the value only grows).
-// Several host threads may race to set it; setting it twice is harmless.
+// Rank in a sample block that its estimate of tau has to reach, or 0 where
+// every element is a candidate instead: k is so near d that a sample rules
+// nothing out.
+static uint32_t sample_rank(int64_t d, int64_t k) {
+  const double expected = (double)k * kSamples / (double)d;
+  const double rank = std::ceil((expected + 7.0 * std::sqrt(expected) + 12.0) / kSampBlocks);
+  return rank < (double)(kSamples / kSampBlocks) ? (uint32_t)rank : 0u;
+}
+
+// CTAs per worker of steps 3 to 5: a warp per group of tiles, but no more
+// than two CTAs per SM in all, which fit at once, so that each reads the
+// row's counts and clears its own once.
+static unsigned select_blocks(int64_t d, int nworkers) {
+  const int64_t need = (groups_of(d) + kSelWarps - 1) / kSelWarps;
+  const int64_t most = (2 * 152 + nworkers - 1) / nworkers;
+  return (unsigned)(need < most ? need : most);
+}
+
+// Allows `kernel` its dynamic shared memory beyond 48 KB (and, for clusters of
+// more than 8 CTAs, their size).  The attributes belong to the function on the
+// current device, so that they were set is remembered per device ordinal.
+// Several host threads may race to set them; setting them twice is harmless.
 constexpr int kSmemDevices = 64;
 
 template <typename K>
-cudaError_t ensure_smem(K kernel, size_t bytes, size_t static_bytes, std::atomic<size_t> (&done)[kSmemDevices]) {
-  if (bytes + static_bytes <= 48u * 1024u) return cudaSuccess;
+static cudaError_t allow_smem(K kernel, size_t bytes, int cluster, std::atomic<bool> (&done)[kSmemDevices]) {
   int dev = 0;
   cudaError_t st = cudaGetDevice(&dev);
   if (st != cudaSuccess) return st;
-  const bool cached = dev >= 0 && dev < kSmemDevices;
-  if (cached && done[dev].load(std::memory_order_acquire) >= bytes) return cudaSuccess;
+  const bool known = dev >= 0 && dev < kSmemDevices;
+  if (known && done[dev].load(std::memory_order_acquire)) return cudaSuccess;
   st = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  if (st == cudaSuccess && cached) {
-    size_t cur = done[dev].load(std::memory_order_relaxed);
-    while (cur < bytes && !done[dev].compare_exchange_weak(cur, bytes, std::memory_order_release)) {
-    }
-  }
+  if (st == cudaSuccess && cluster > 8)
+    st = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (st == cudaSuccess && known) done[dev].store(true, std::memory_order_release);
   return st;
+}
+
+// CTAs per worker of the kernel that keeps p on chip, or 0 where the five
+// kernels are taken: the least of the times that fit what was measured (us,
+// k = d / 100, d from 4096 to 786,432, 1 to 64 workers).  On chip, a wave of
+// as many workers as are resident (152 SMs; 15 clusters of 8; 7 of 16) costs a
+// fixed latency and 0.45 per 1024 elements of a part; the five kernels cost
+// 20, their memory traffic, and a little for every worker's sample.  E.g. one
+// worker, d = 65,536: 9.1 with 16 CTAs (9.9 with 8, 21 with the five kernels);
+// 16 workers of 65,536: 24 with 8 CTAs, 31 with 16, 30 with the five; 64
+// workers of 32,768: 26 with 1, 50 with 8.  (Each with its server step.)
+// Below kSamples the five kernels have no sample, and 70 to 135.
+static int chip_ctas(int64_t d, int nworkers) {
+  double best = d < kSamples ? INFINITY : 20.0 + 2.2e-6 * (double)d * nworkers + 0.15 * nworkers;
+  int ctas = 0;
+  auto consider = [&](int n, int resident, double latency) {
+    const int64_t part = chip_part(d, n);
+    if (part > kChipMax) return;
+    const double t = ((nworkers + resident - 1) / resident) * (latency + 0.45 * (double)part / 1024.0);
+    if (t < best) {
+      best = t;
+      ctas = n;
+    }
+  };
+  consider(1, 152, 4.0);
+  consider(8, 15, 6.8);
+  consider(16, 7, 7.5);
+  return ctas;
+}
+
+static cudaError_t launch_chip(int ctas, bool keep_h, const CompressArgs& a, int64_t k, cudaStream_t stream) {
+  static std::atomic<bool> done[3][2][kSmemDevices];
+  auto go = [&](auto kernel, int n, std::atomic<bool> (&set)[kSmemDevices]) -> cudaError_t {
+    const cudaError_t st = allow_smem(kernel, kChipMax * sizeof(float), n, set);
+    if (st != cudaSuccess) return st;
+    const size_t need = (size_t)chip_part(a.d, n) * sizeof(float);
+    return launch_pdl_cluster(kernel, n, dim3((unsigned)n, (unsigned)a.nworkers), dim3(kChipThreads), need, stream, a, k);
+  };
+  const int h = keep_h ? 1 : 0;
+  switch (ctas) {
+    case 1: return go(keep_h ? topk_chip_kernel<1, true> : topk_chip_kernel<1, false>, 1, done[0][h]);
+    case 8: return go(keep_h ? topk_chip_kernel<8, true> : topk_chip_kernel<8, false>, 8, done[1][h]);
+    default: return go(keep_h ? topk_chip_kernel<16, true> : topk_chip_kernel<16, false>, 16, done[2][h]);
+  }
 }
 
 cudaError_t launch_topk_compress(const CompressArgs& a, int64_t k, bool keep_h, void* scratch,
                                  cudaStream_t stream, uint64_t* launches) {
-  static std::atomic<size_t> smem_done[2][kSmemDevices];
+  static std::atomic<bool> emit_done[kSmemDevices];
   const unsigned rows = (unsigned)a.nworkers;
-  const dim3 tiles((unsigned)tiles_of(a.d), rows);
-  const dim3 clusters(kCluster, rows);
-  const size_t smem = sizeof(SelectSmem);
-  cudaError_t st;
-  if (keep_h) {
-    if ((st = ensure_smem(topk_select_kernel<true>, smem, 0, smem_done[1])) != cudaSuccess) return st;
-    launch_pdl(topk_form_kernel<true>, tiles, dim3(kFormThreads), 0, stream, a, scratch);
-    if ((st = cudaGetLastError()) != cudaSuccess) return st;
-    st = launch_pdl(topk_select_kernel<true>, clusters, dim3(kSelThreads), smem, stream, a, k, scratch);
-  } else {
-    if ((st = ensure_smem(topk_select_kernel<false>, smem, 0, smem_done[0])) != cudaSuccess) return st;
-    launch_pdl(topk_form_kernel<false>, tiles, dim3(kFormThreads), 0, stream, a, scratch);
-    if ((st = cudaGetLastError()) != cudaSuccess) return st;
-    st = launch_pdl(topk_select_kernel<false>, clusters, dim3(kSelThreads), smem, stream, a, k, scratch);
+  cudaError_t st = cudaSuccess;
+  auto launched = [&](cudaError_t r) {
+    st = r;
+    if (st == cudaSuccess) *launches += 1;
+    return st == cudaSuccess;
+  };
+  if (const int ctas = chip_ctas(a.d, a.nworkers)) {
+    launched(launch_chip(ctas, keep_h, a, k, stream));
+    return st;
   }
-  *launches += st == cudaSuccess ? 2 : 1;
+  const dim3 tiles((unsigned)tiles_of(a.d), rows), select(select_blocks(a.d, a.nworkers), rows);
+  // the rows that a tile with its share of 1.3 k candidates has
+  const int64_t mean = 1 + 13 * k / (320 * tiles_of(a.d));
+  const int ahead = (int)(mean < kFirst ? mean : kFirst);
+  const size_t places = groups_of(a.d) * 2 * sizeof(uint32_t);
+  if ((st = allow_smem(topk_emit_kernel, kMaxGroups * 2 * sizeof(uint32_t), 1, emit_done)) != cudaSuccess) return st;
+  (void)(launched(launch_pdl(topk_sample_kernel, dim3(kSampBlocks, rows), dim3(kSampThreads), 0, stream, a,
+                             sample_rank(a.d, k), scratch)) &&
+         launched(launch_pdl(keep_h ? topk_form_kernel<true> : topk_form_kernel<false>, tiles, dim3(kFormThreads), 0,
+                             stream, a, scratch)) &&
+         launched(launch_pdl(topk_count_kernel, select, dim3(kSelThreads), 0, stream, a, ahead, scratch)) &&
+         launched(launch_pdl(topk_resolve_kernel, select, dim3(kSelThreads), 0, stream, a, k, ahead, scratch)) &&
+         launched(launch_pdl(topk_emit_kernel, select, dim3(kSelThreads), places, stream, a, k, ahead, scratch)));
   return st;
 }
 

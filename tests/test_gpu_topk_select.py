@@ -1,0 +1,108 @@
+"""The top-k worker step where its sampled threshold, its candidate lists and
+its counting rounds change course, against the selection's definition.
+
+The k records are fixed by the definition alone (the k largest |p_j|, equal
+ones lowest index first, in index order), so they, e and h are compared bit
+for bit with numpy on the same fp32 p:
+
+* few parameters (one CTA keeps them on chip), more (clusters of 8 and of 16
+  CTAs do), parts that end in the last CTA, and d on both sides of the sizes
+  from which the sampled kernels run;
+* a gradient that is large exactly at the sampled runs, so that too few
+  elements reach the threshold and the candidates are taken again;
+* a few dense tiles among thousands with one candidate each;
+* a k-th key far above the threshold, so many equal keys that their list
+  overflows, k = 1 and k = d.
+"""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def P():
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_2010_13359_gb300 as P
+    return P
+
+
+def sampled(d):
+    """The elements the threshold's sample reads: one run of 8 in each of 8192 strata."""
+    runs, s = d >> 3, np.arange(8192, dtype=np.uint64)
+    lo, hi = runs * s // 8192, runs * (s + 1) // 8192
+    at = lo + (((s * 0x9E3779B1) & 0xFFFFFFFF) * (hi - lo) >> np.uint64(32))
+    return (at[:, None] * 8 + np.arange(8, dtype=np.uint64)).ravel().astype(np.int64)
+
+
+def gradient(kind, d, rng):
+    g = rng.standard_normal(d).astype(np.float32)
+    if kind == "trap":
+        g *= np.float32(1e-3)
+        g[sampled(d)] = 10
+    elif kind == "sparse tiles":  # one large value in each of the first tiles, the rest in the last ones
+        nt = -(-d // 4096)
+        g *= np.float32(1e-6)
+        g[np.arange(nt - 90) * 4096 + 17] = 3
+        tail = np.arange((nt - 90) * 4096, d)
+        g[rng.choice(tail, 20_000, replace=False)] = 5
+    elif kind == "outliers":
+        g[rng.choice(d, 3, replace=False)] *= np.float32(1e25)
+    elif kind == "ties":
+        g = np.sign(g) * (rng.integers(1, 4, d) * 0.5).astype(np.float32)
+    return g
+
+
+CASES = [(1, 1, 2, "gauss"), (3, 2, 2, "gauss"), (2_049, 2_049, 2, "ties"), (20_001, 333, 40, "ties"),
+         (49_152, 10, 20, "gauss"), (9_999, 1, 2, "gauss"), (32_767, 400, 2, "outliers"), (40_000, 30_000, 9, "ties"),
+         (393_215, 4_000, 9, "gauss"), (65_535, 65_535, 20, "gauss"), (65_536, 300, 20, "gauss"),
+         (200_003, 200_003, 9, "gauss"), (786_431, 9_000, 4, "ties"), (300_005, 2, 20, "outliers"),
+         (300_005, 150_000, 20, "ties"), (1_000_003, 1, 2, "gauss"), (1_000_003, 990_000, 2, "gauss"),
+         (1_000_003, 200_000, 2, "trap"), (9_000_001, 400_000, 2, "ties"), (9_000_001, 21_000, 2, "sparse tiles")]
+
+
+@pytest.mark.parametrize("keep", [False, True])
+@pytest.mark.parametrize("d,k,M,kind", CASES)
+def test_records_residual_and_offsets(P, d, k, M, kind, keep):
+    stream = torch.cuda.current_stream()
+    rng = np.random.default_rng(d + k)
+    lr = np.float32(0.25)
+    h = P.create(P.make_config(d=d, M=M, compressor=P.TOPK, lr=float(lr), k=k,
+                               flags=P.KEEP_LOOKAHEAD if keep else 0, cuda_stream=stream.cuda_stream))
+    ld = (d + 3) // 4 * 4
+    i = M - 1  # the worker looked at; the others get zeros
+    e = np.zeros(d, np.float32)
+    g_dev = torch.zeros((M, ld), device="cuda")
+    msgs = torch.zeros((M, h.message_bytes()), dtype=torch.uint8, device="cuda")
+    for step in range(2):
+        g = gradient(kind, d, rng)
+        g_dev[i, :d] = torch.from_numpy(g)
+        h.workers_compress_all(g_dev, ld, msgs)
+        h.synchronize()
+        s = lr * g
+        p = s + e
+        key = p.view(np.uint32) & np.uint32(0x7FFFFFFF)
+        T = np.partition(key, d - k)[d - k]
+        kept = key > T
+        ties = np.flatnonzero(key == T)[:k - int(kept.sum())]
+        kept[ties] = True
+        idx = np.flatnonzero(kept)
+        rec = msgs[i, :8 * k].cpu().numpy().view(np.uint32).reshape(k, 2)
+        assert np.array_equal(rec[:, 0], idx.astype(np.uint32)), step
+        assert np.array_equal(rec[:, 1], p[idx].view(np.uint32)), step
+        if M > 1:  # all zero: the first k indices
+            rec = msgs[0, :8 * k].cpu().numpy().view(np.uint32).reshape(k, 2)
+            assert np.array_equal(rec[:, 0], np.arange(k, dtype=np.uint32)) and not rec[:, 1].any(), step
+        e = np.where(kept, p - p, p)
+        got = np.empty(d, np.float32)
+        h.get_residual(i, got)
+        assert np.array_equal(got.view(np.uint32), e.view(np.uint32)), step
+        if keep:
+            h.get_lookahead(i, got)
+            assert np.array_equal(got.view(np.uint32), (s + e).view(np.uint32)), step
+    h.destroy()
