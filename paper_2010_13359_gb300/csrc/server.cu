@@ -9,15 +9,15 @@
 // The parameters therefore come out the same bit for bit whichever kernel
 // runs.
 //
-// Sign with buckets >= 512: bit-transposed table decode (the column and
-// warp-transpose kernels for M <= 32, words staged by TMA; flat buckets or a
-// per-bucket slice table with layer segments).  Stochastic quantiser with
-// M <= 32: code words staged by TMA, per-worker or pair-table decode (and,
-// for 8-bit codes with layer segments and 16 workers, slices from a
-// per-bucket table).  The rest -- identity, sign with buckets < 512, more
-// than 32 workers -- one thread per 4-element chunk of w walks the M
-// messages in groups of four workers.  w is read and written once; every
-// kernel waits for the grid before it (programmatic dependent launch).
+// Sign: bit-transposed table decode (large problems with buckets >= 1024 and
+// M <= 32: the column and warp-transpose kernels, words staged by TMA, flat
+// buckets or a per-bucket slice table with layer segments; the rest: a warp
+// per chunk of 256 elements).  Stochastic quantiser with M <= 32: code words
+// staged by TMA, per-worker or pair-table decode (and, for 8-bit codes with
+// layer segments and 16 workers, slices from a per-bucket table).  The rest --
+// identity, small buckets of the quantiser, more than 32 workers -- one thread
+// per 4-element chunk of w walks the M messages.  w is read and written once;
+// every kernel waits for the grid before it (programmatic dependent launch).
 #include "device_common.cuh"
 
 namespace dq {
@@ -48,53 +48,7 @@ __device__ __forceinline__ void apply_chunk(const ServerArgs& s, int64_t j, cons
   }
 }
 
-// Scaled sign, any bucket: Q_m(p)_j = bit ? -s_m : s_m, message words and
-// scales fetched 8 workers at a time, summed as two groups of four.
 constexpr int kSumLevels = 11;  // group counts up to 1024 (M <= 4096)
-
-__global__ void __launch_bounds__(256) sign_server_kernel(const ServerArgs s) {
-  dq_pdl_enter();
-  const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t j = 4 * c;
-  if (j >= s.d) return;
-  const int64_t bkt = s.word_bucket ? (int64_t)s.word_bucket[j >> 5] : j / s.bucket;
-  const int64_t word = j >> 5;
-  const int shift = (int)(j & 31);
-  PairwiseAcc<kSumLevels> acc[4];
-  for (int m0 = 0; m0 < s.M; m0 += 8) {
-    float sc[8];
-    uint32_t bits[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      sc[u] = 0.f;
-      bits[u] = 0;
-      if (m0 + u < s.M) {
-        const uint8_t* msg = s.msgs + (int64_t)(m0 + u) * s.msg_stride;
-        sc[u] = __ldg(reinterpret_cast<const float*>(msg) + bkt);
-        bits[u] = __ldg(reinterpret_cast<const uint32_t*>(msg + s.off_payload) + word) >> shift;
-      }
-    }
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      if (m0 + 4 * h < s.M) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          float v[4];
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const int x = 4 * h + u;
-            v[u] = (m0 + x < s.M) ? (((bits[x] >> q) & 1u) ? -sc[x] : sc[x]) : 0.f;  // +0 past M
-          }
-          acc[q].push(group4(v[0], v[1], v[2], v[3], s.M));
-        }
-      }
-    }
-  }
-  float sum[4];
-#pragma unroll
-  for (int q = 0; q < 4; ++q) sum[q] = acc[q].result();
-  apply_chunk(s, j, sum);
-}
 
 // 32x32 bit transpose across a warp: on entry lane m holds row m; on exit
 // lane l holds column l (bit m = bit l of row m).  Five block-swap stages;
@@ -125,19 +79,16 @@ __device__ __forceinline__ uint32_t warp_transpose32(uint32_t x, const Transpose
   return x;
 }
 
-// Scaled sign, buckets of 512..4096.  One warp per (bucket, slice of up to 32
-// message words = 1024 elements), no shared memory and no block barriers.
-// Lane m loads worker m's words of the slice (32 contiguous bytes at a time)
-// and a warp transpose gives lane l the M sign bits of one element.  The sum
-// over workers comes from per-bucket tables of four-worker group values:
-// T_g[v] = the group's subtree (a + b) + (c + d) over the leaves
-// bit r of v ? -s_{4g+r} : s_{4g+r} (+0 past M), held in registers two
-// groups per register -- lane l of register a keeps T_{2a + l/16}[l mod 16]
+// The sum over workers of the scaled signs, 32 elements (one message word) at a
+// time.  Lane m holds worker m's word, and a warp transpose gives lane l the
+// M sign bits of one element.  The sum comes from per-bucket tables of
+// four-worker group values: T_g[v] = the group's subtree (a + b) + (c + d) over
+// the leaves bit r of v ? -s_{4g+r} : s_{4g+r} (+0 past M), held in registers
+// two groups per register -- lane l of register a keeps T_{2a + l/16}[l mod 16]
 // -- so that a lookup is one shuffle whose source lane is the group's 4-bit
 // field, plus 16 for an odd group (shuffles take the lane index mod 32).
-// The NG = ceil(M/4) group values are then summed pairwise, padded with +0
-// groups to a power of two: the library's fixed order of the sum.
-constexpr int kSliceWords = 32;
+// The group values are then summed pairwise, padded with +0 groups to a power
+// of two: the library's fixed order of the sum.
 
 // T[a] of groups 2a (lanes 0..15) and 2a + 1 (lanes 16..31) for the
 // workers of one 32-worker slab: in_slab of them present, M in all.
@@ -197,64 +148,93 @@ __device__ __forceinline__ void sums8(const uint32_t (&wd)[8], const float (&T)[
   for (int k = 0; k < 8; ++k) out[k] = group_sum<NG>(warp_transpose32(wd[k], tl), T);
 }
 
-// M <= 32 workers in NG = ceil(M / 4) groups; w updated after every 8 words.
-// The next 8 words and parameters are fetched before the current ones are
-// decoded.
-template <int NG, bool POW2>
-__global__ void __launch_bounds__(256) sign_server_shfl_kernel(const ServerArgs s) {
+// Any bucket, any number of workers, flat or layer buckets: one warp per
+// chunk of 8 message words (256 elements), no shared memory, no barriers.
+// Lane m loads worker m's 8 words (32 contiguous bytes) of a slab of 32
+// workers and its scales of the chunk's buckets; the tables are rebuilt where
+// the bucket changes, every WPB words (flat; 8: no more than one bucket per
+// chunk) or where the table of word buckets says so (WPB = 0: layer buckets).
+// SLABS = 1: M <= 32 in NG groups, a power of two (groups past M are +0); 2:
+// M <= 64; 0: any M.  With more than 32 workers the padded tree has at least
+// 64 leaves, so a slab is a subtree.
+// Bound by the shuffles (17 per word and slab with 128 elements per scale) and
+// by the loads' one line per lane.  A thread per 4 elements that walked the
+// messages, which this replaces for buckets below 512, spent its time on the
+// sum's bookkeeping: 96 us for d = 1.23M, M = 64, 128 per scale, against
+// 12 here.
+constexpr int kSlabLevels = 8;  // up to 128 slabs (M <= 4096)
+constexpr int kChunkWords = 8;
+
+template <int NG, int SLABS, int WPB>
+__global__ void __launch_bounds__(256) sign_server_words_kernel(const ServerArgs s) {
   dq_pdl_enter();
+  constexpr int NR = (NG + 1) / 2;
+  constexpr int NSC = WPB == 0 ? kChunkWords : kChunkWords / WPB;  // scales of a chunk per worker
   const int lane = threadIdx.x & 31;
-  const int64_t gw = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
-  const int words_per_bucket = s.bucket >> 5;
-  const int sw = words_per_bucket < kSliceWords ? words_per_bucket : kSliceWords;  // 16 or 32
-  const int spb = words_per_bucket / sw;  // slices per bucket
-  const int64_t nb = (s.d + s.bucket - 1) / s.bucket;
-  const int64_t b = gw / spb;
-  if (b >= nb) return;
-  const int64_t wbase = b * words_per_bucket + (gw % spb) * sw;
+  const int64_t w0 = ((int64_t)blockIdx.x * 8 + (threadIdx.x >> 5)) * kChunkWords;
   const int64_t nwords = (s.d + 31) >> 5;
+  if (w0 >= nwords) return;
   const TransposeLane tl(lane);
-  const uint8_t* my_msg = s.msgs + (int64_t)lane * s.msg_stride;
-  const bool active = lane < s.M;
-  const float my_scale = active ? __ldg(reinterpret_cast<const float*>(my_msg) + b) : 0.f;
-  float T[(NG + 1) / 2];
-  build_group_tables(my_scale, s.M, s.M, lane, T);
-  const uint32_t* wp = reinterpret_cast<const uint32_t*>(my_msg + s.off_payload) + wbase;
-  float* wl = s.w + 32 * wbase + lane;
-  const int64_t jmax = s.d - 32 * wbase - lane;  // wl[32 i] is a parameter iff 32 i < jmax
-  const int iters = sw / 8;
-  uint32_t wd[8];
-  float wv[8];
-  load_words8(wp, wbase, nwords, active, wd);
+  float* wl = s.w + 32 * w0 + lane;
+  const int64_t jmax = s.d - 32 * w0 - lane;  // wl[32 i] is a parameter iff 32 i < jmax
+  float wv[kChunkWords];
 #pragma unroll
-  for (int k = 0; k < 8; ++k) wv[k] = (32 * k < jmax) ? __ldcs(wl + 32 * k) : 0.f;
-#pragma unroll 1
-  for (int it = 0; it < iters; ++it) {
-    uint32_t wd_next[8];
-    float wv_next[8];
-    const bool more = it + 1 < iters;
-    if (more) {
-      load_words8(wp + 8 * (it + 1), wbase + 8 * (it + 1), nwords, active, wd_next);
+  for (int k = 0; k < kChunkWords; ++k) wv[k] = (32 * k < jmax) ? __ldcs(wl + 32 * k) : 0.f;
+  uint32_t bkt[WPB == 0 ? kChunkWords : 1];  // layer buckets: of each word (past the end: the last word's)
+  if constexpr (WPB == 0) {
 #pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        const int64_t off = 32 * (8 * (it + 1) + k);
-        wv_next[k] = (off < jmax) ? __ldcs(wl + off) : 0.f;
+    for (int k = 0; k < kChunkWords; ++k) bkt[k] = __ldg(s.word_bucket + min64(w0 + k, nwords - 1));
+  } else {
+    bkt[0] = (uint32_t)(w0 / (s.bucket >> 5));
+  }
+  const int slabs = SLABS ? SLABS : (s.M + 31) / 32;
+  float sum[kChunkWords] = {};
+  PairwiseAcc<SLABS == 0 ? kSlabLevels : 1> acc[SLABS == 0 ? kChunkWords : 1];
+#pragma unroll(SLABS ? SLABS : 1)
+  for (int slab = 0; slab < slabs; ++slab) {
+    const int in_slab = min(32, s.M - 32 * slab);
+    const bool active = lane < in_slab;
+    const uint8_t* msg = s.msgs + (int64_t)(32 * slab + (active ? lane : 0)) * s.msg_stride;
+    uint32_t wd[kChunkWords];
+    load_words8(reinterpret_cast<const uint32_t*>(msg + s.off_payload) + w0, w0, nwords, active, wd);
+    // (flat: a chunk's scales end within the message's scale section, which
+    // is padded to 256 bytes)
+    float sc[NSC];
+    const float* scales = reinterpret_cast<const float*>(msg) + bkt[0];
+    if constexpr (WPB == 0) {
+#pragma unroll
+      for (int k = 0; k < kChunkWords; ++k)
+        if (k == 0 || bkt[k] != bkt[k - 1]) sc[k] = __ldg(reinterpret_cast<const float*>(msg) + bkt[k]);
+    } else if constexpr (NSC >= 4) {
+#pragma unroll
+      for (int k = 0; k < NSC; k += 4) {
+        const float4 x = __ldg(reinterpret_cast<const float4*>(scales + k));
+        sc[k] = x.x;
+        sc[k + 1] = x.y;
+        sc[k + 2] = x.z;
+        sc[k + 3] = x.w;
       }
+    } else if constexpr (NSC == 2) {
+      const float2 x = __ldg(reinterpret_cast<const float2*>(scales));
+      sc[0] = x.x;
+      sc[1] = x.y;
+    } else {
+      sc[0] = __ldg(scales);
     }
-    float sum[8];
-    sums8<NG>(wd, T, tl, sum);
+    float T[NR];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const int64_t off = 32 * (8 * it + k);
-      if (off < jmax) __stcs(wl + off, server_out(s, wv[k], average_t<POW2>(sum[k], s)));
+    for (int k = 0; k < kChunkWords; ++k) {
+      const bool fresh = WPB == 0 ? (k == 0 || bkt[k] != bkt[k - 1]) : k % (WPB ? WPB : 1) == 0;  // warp-uniform
+      if (fresh) build_group_tables(active ? sc[WPB == 0 ? k : k / (WPB ? WPB : 1)] : 0.f, in_slab, s.M, lane, T);
+      const float v = group_sum<NG>(warp_transpose32(wd[k], tl), T);
+      if constexpr (SLABS == 0) acc[k].push(v);
+      else sum[k] = slab == 0 ? v : __fadd_rn(sum[k], v);
     }
-    if (more) {
+  }
 #pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        wd[k] = wd_next[k];
-        wv[k] = wv_next[k];
-      }
-    }
+  for (int k = 0; k < kChunkWords; ++k) {
+    if constexpr (SLABS == 0) sum[k] = acc[k].result();
+    if (32 * k < jmax) __stcs(wl + 32 * k, server_out(s, wv[k], average(sum[k], s)));
   }
 }
 
@@ -656,51 +636,6 @@ sign_server_col_kernel(const ServerArgs s, const SegSlices seg, const __grid_con
       if (w_issued1 > w_done1) mbar_wait_bounded(&wbar[1], w_done1 & 1u, s.err);
       if (p_issued0 > p_done0) mbar_wait_bounded(&pbar[0], p_done0 & 1u, s.err);
       if (p_issued1 > p_done1) mbar_wait_bounded(&pbar[1], p_done1 & 1u, s.err);
-    }
-  }
-}
-
-// M above 32: workers taken 32 at a time.  With M > 32 the padded tree has
-// at least 64 leaves, so each 32-worker slab (the last one padded with +0
-// groups) is a subtree: per 8-word chunk of the slice, every slab's sum of
-// the chunk's elements goes into a per-element pairwise accumulator over
-// slabs, and w is updated once all slabs are in.
-constexpr int kSlabLevels = 8;  // up to 128 slabs (M <= 4096)
-
-__global__ void __launch_bounds__(256) sign_server_slabs_kernel(const ServerArgs s) {
-  dq_pdl_enter();
-  const int lane = threadIdx.x & 31;
-  const int64_t gw = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
-  const int words_per_bucket = s.bucket >> 5;
-  const int sw = words_per_bucket < kSliceWords ? words_per_bucket : kSliceWords;
-  const int spb = words_per_bucket / sw;
-  const int64_t nb = (s.d + s.bucket - 1) / s.bucket;
-  const int64_t b = gw / spb;
-  if (b >= nb) return;
-  const int64_t wbase = b * words_per_bucket + (gw % spb) * sw;
-  const int64_t nwords = (s.d + 31) >> 5;
-  const TransposeLane tl(lane);
-  const int nslabs = (s.M + 31) / 32;
-  for (int it = 0; it * 8 < sw; ++it) {
-    PairwiseAcc<kSlabLevels> acc[8];
-    for (int slab = 0; slab < nslabs; ++slab) {
-      const int in_slab = min(32, s.M - slab * 32);
-      const uint8_t* my_msg = s.msgs + (int64_t)(slab * 32 + lane) * s.msg_stride;
-      const float my_scale = (lane < in_slab) ? __ldg(reinterpret_cast<const float*>(my_msg) + b) : 0.f;
-      float T[4];
-      build_group_tables(my_scale, in_slab, s.M, lane, T);
-      const int64_t w0 = wbase + 8 * it;
-      uint32_t wd[8];
-      load_words8(reinterpret_cast<const uint32_t*>(my_msg + s.off_payload) + w0, w0, nwords, lane < in_slab, wd);
-      float v[8];
-      sums8<8>(wd, T, tl, v);
-#pragma unroll
-      for (int k = 0; k < 8; ++k) acc[k].push(v[k]);
-    }
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const int64_t j = 32 * (wbase + 8 * it + k) + lane;
-      if (j < s.d) __stcs(s.w + j, server_out(s, __ldcs(s.w + j), average(acc[k].result(), s)));
     }
   }
 }
@@ -1692,88 +1627,67 @@ unsigned chunk_blocks(int64_t d, int threads) {
 
 }  // namespace
 
+// The warp-per-chunk sign server, by workers and words per bucket.
+static cudaError_t launch_sign_words(const ServerArgs& s, cudaStream_t stream) {
+  const unsigned blocks = (unsigned)((((s.d + 31) >> 5) + 8 * kChunkWords - 1) / (8 * kChunkWords));
+  auto go = [&](auto kernel) { return launch_pdl(kernel, dim3(blocks), dim3(256), 0, stream, s); };
+#define DQ_SIGN_WORDS(NG, SLABS)                                  \
+  (wpb == 0   ? go(sign_server_words_kernel<NG, SLABS, 0>)        \
+   : wpb == 1 ? go(sign_server_words_kernel<NG, SLABS, 1>)        \
+   : wpb == 2 ? go(sign_server_words_kernel<NG, SLABS, 2>)        \
+   : wpb == 4 ? go(sign_server_words_kernel<NG, SLABS, 4>)        \
+              : go(sign_server_words_kernel<NG, SLABS, 8>))
+  const int wpb = s.word_bucket ? 0 : s.bucket >> 5;
+  cudaError_t st;
+  if (s.M <= 4) st = DQ_SIGN_WORDS(1, 1);
+  else if (s.M <= 8) st = DQ_SIGN_WORDS(2, 1);
+  else if (s.M <= 16) st = DQ_SIGN_WORDS(4, 1);
+  else if (s.M <= 32) st = DQ_SIGN_WORDS(8, 1);
+  else if (s.M <= 64) st = DQ_SIGN_WORDS(8, 2);
+  else st = DQ_SIGN_WORDS(8, 0);
+#undef DQ_SIGN_WORDS
+  return st;
+}
+
 cudaError_t launch_sign_server(const ServerArgs& s, const SignServerExtras& x, cudaStream_t stream,
                                uint64_t* launches) {
-  if (s.word_bucket) {  // buckets restart at layer segments
-    if (x.seg_slices && s.sign_words_map && s.bucket >= 1024 && s.M <= 32) {
-      const bool p2 = s.M_pow2 != 0;
-      // the column kernel where it pays (as for flat buckets), else the
-      // warp-transpose kernel; DQGAN_SIGN_SERVER fixes the choice
-      const bool col = x.params_map != nullptr && (x.path == 1 || (x.path == 0 && sign_col_pays(x.seg_nslices)));
-      cudaError_t st;
-#define DQ_SIGN_SEG(NG)                                                                                     \
-  st = col ? (p2 ? launch_sign_col<NG, true, true>(s, x, stream) : launch_sign_col<NG, false, true>(s, x, stream)) \
-           : (p2 ? launch_sign_tma<NG, true, true>(s, x, stream) : launch_sign_tma<NG, false, true>(s, x, stream))
-      switch ((s.M + 3) / 4) {
-        case 1: DQ_SIGN_SEG(1); break;
-        case 2: DQ_SIGN_SEG(2); break;
-        case 3: DQ_SIGN_SEG(3); break;
-        case 4: DQ_SIGN_SEG(4); break;
-        case 5: DQ_SIGN_SEG(5); break;
-        case 6: DQ_SIGN_SEG(6); break;
-        case 7: DQ_SIGN_SEG(7); break;
-        default: DQ_SIGN_SEG(8); break;
-      }
-#undef DQ_SIGN_SEG
-      *launches += 1;
-      return st;
-    }
-    launch_pdl(sign_server_kernel, dim3(chunk_blocks(s.d, 256)), dim3(256), 0, stream, s);  // per-element scale lookup
-    *launches += 1;
-    return cudaGetLastError();
-  }
-  if (s.bucket >= 1024 && s.M <= 32 && s.sign_words_map != nullptr) {
+  cudaError_t st;
+  const bool seg = s.word_bucket != nullptr;  // buckets restart at layer segments
+  const int64_t nslices = seg ? x.seg_nslices : ((s.d + s.bucket - 1) / s.bucket) * (s.bucket / 1024);
+  // Below some 600 slices of 1024 elements most SMs have a warp or two of the
+  // TMA kernels, and the warp-per-chunk kernel, with four times the warps and
+  // no copy to wait for, is faster (8 workers, d = 65,536: 2.9 us against 3.8;
+  // 524,288: 3.0 / 3.9; 1,000,000: 3.8 / 3.9; 2,000,000: 5.6 / 5.1).
+  const bool few = x.path == 0 && nslices <= 600;
+  if (s.bucket >= 1024 && s.M <= 32 && !few && s.sign_words_map != nullptr && (!seg || x.seg_slices)) {
     const bool p2 = s.M_pow2 != 0;
-    const bool col = x.params_map != nullptr &&
-                     (x.path == 1 || (x.path == 0 && sign_col_pays(((s.d + s.bucket - 1) / s.bucket) * (s.bucket / 1024))));
-    cudaError_t st;
-#define DQ_SIGN_TMA(NG)                                                                           \
-  st = col ? (p2 ? launch_sign_col<NG, true, false>(s, x, stream) : launch_sign_col<NG, false, false>(s, x, stream)) \
-           : (p2 ? launch_sign_tma<NG, true, false>(s, x, stream) : launch_sign_tma<NG, false, false>(s, x, stream))
+    // the column kernel where it pays, else the warp-transpose kernel;
+    // DQGAN_SIGN_SERVER fixes the choice
+    const bool col = x.params_map != nullptr && (x.path == 1 || (x.path == 0 && sign_col_pays(nslices)));
+#define DQ_SIGN_TMA(NG, SEG)                                                                                     \
+  st = col ? (p2 ? launch_sign_col<NG, true, SEG>(s, x, stream) : launch_sign_col<NG, false, SEG>(s, x, stream)) \
+           : (p2 ? launch_sign_tma<NG, true, SEG>(s, x, stream) : launch_sign_tma<NG, false, SEG>(s, x, stream))
+#define DQ_SIGN_CASE(NG)          \
+  if (seg) DQ_SIGN_TMA(NG, true); \
+  else DQ_SIGN_TMA(NG, false);    \
+  break
     switch ((s.M + 3) / 4) {
-      case 1: DQ_SIGN_TMA(1); break;
-      case 2: DQ_SIGN_TMA(2); break;
-      case 3: DQ_SIGN_TMA(3); break;
-      case 4: DQ_SIGN_TMA(4); break;
-      case 5: DQ_SIGN_TMA(5); break;
-      case 6: DQ_SIGN_TMA(6); break;
-      case 7: DQ_SIGN_TMA(7); break;
-      default: DQ_SIGN_TMA(8); break;
+      case 1: DQ_SIGN_CASE(1);
+      case 2: DQ_SIGN_CASE(2);
+      case 3: DQ_SIGN_CASE(3);
+      case 4: DQ_SIGN_CASE(4);
+      case 5: DQ_SIGN_CASE(5);
+      case 6: DQ_SIGN_CASE(6);
+      case 7: DQ_SIGN_CASE(7);
+      default: DQ_SIGN_CASE(8);
     }
+#undef DQ_SIGN_CASE
 #undef DQ_SIGN_TMA
-    *launches += 1;
-    return st;
-  }
-  if (s.bucket >= 512) {
-    const int64_t nb = (s.d + s.bucket - 1) / s.bucket;
-    const int64_t wpb = s.bucket >= 1024 ? s.bucket / 1024 : 1;  // warps per bucket
-    const int64_t warps = nb * wpb;
-    const unsigned blocks = (unsigned)((warps + 7) / 8);
-    if (s.M > 32) {
-      launch_pdl(sign_server_slabs_kernel, dim3(blocks), dim3(256), 0, stream, s);
-    } else {
-      const int ng = (s.M + 3) / 4;
-      const bool p2 = s.M_pow2 != 0;
-#define DQ_SIGN_SERVER(NG) \
-      (p2 ? launch_pdl(sign_server_shfl_kernel<NG, true>, dim3(blocks), dim3(256), 0, stream, s) \
-          : launch_pdl(sign_server_shfl_kernel<NG, false>, dim3(blocks), dim3(256), 0, stream, s))
-      switch (ng) {
-        case 1: DQ_SIGN_SERVER(1); break;
-        case 2: DQ_SIGN_SERVER(2); break;
-        case 3: DQ_SIGN_SERVER(3); break;
-        case 4: DQ_SIGN_SERVER(4); break;
-        case 5: DQ_SIGN_SERVER(5); break;
-        case 6: DQ_SIGN_SERVER(6); break;
-        case 7: DQ_SIGN_SERVER(7); break;
-        default: DQ_SIGN_SERVER(8); break;
-      }
-#undef DQ_SIGN_SERVER
-    }
   } else {
-    launch_pdl(sign_server_kernel, dim3(chunk_blocks(s.d, 256)), dim3(256), 0, stream, s);
+    st = launch_sign_words(s, stream);
   }
   *launches += 1;
-  return cudaGetLastError();
+  return st;
 }
 
 cudaError_t launch_squant_server(const ServerArgs& s, const SignServerExtras& x, cudaStream_t stream,

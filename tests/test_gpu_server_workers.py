@@ -1,0 +1,62 @@
+"""The server kernels' worker sums at the edges of their groups: 1 worker to
+more than two slabs of 32, every bucket size that has a form of its own, flat
+and layer buckets, a vector that ends inside a word and a chunk; w against
+the oracle bit for bit."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+import oracle
+from parity_helpers import assert_params_equal, oracle_config
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+D = 8 * 256 + 5 * 32 + 7
+SEGMENTS = (0, 32, 96, 1056, 1088, 2112, D)
+
+
+@pytest.fixture(scope="module")
+def P():
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_2010_13359_gb300 as P
+    return P
+
+
+def run(P, comp, M, segments=None, d=D, **kw):
+    ocfg = oracle_config(d, M, comp, lr=0.03, seed=M, segments=segments, **kw)
+    h = P.create(P.make_config(d=d, M=M, compressor=comp, lr=0.03, seed=M,
+                               cuda_stream=torch.cuda.current_stream().cuda_stream, **kw))
+    if segments:
+        h.set_segments(segments)
+    rng = np.random.default_rng(M)
+    g = (rng.standard_normal((M, d)) * np.exp(rng.uniform(-3, 1, (M, d)))).astype(np.float32)
+    ld = (d + 3) // 4 * 4
+    g_dev = torch.zeros((M, ld), device="cuda")
+    g_dev[:, :d] = torch.from_numpy(g)
+    msgs = torch.zeros((M, h.message_bytes()), dtype=torch.uint8, device="cuda")
+    w = (rng.standard_normal(d) * 0.02).astype(np.float32)
+    w_gpu = torch.full((d + 64,), 12345.0, device="cuda")
+    w_gpu[:d] = torch.from_numpy(w)
+    h.workers_compress_all(g_dev, ld, msgs)
+    h.server_aggregate_update(msgs, w_gpu[:d])
+    st = oracle.State(ocfg)
+    st.server(st.compress_all(g), w)
+    h.synchronize()
+    got = w_gpu.cpu().numpy()
+    assert_params_equal(got[:d], w)
+    assert np.all(got[d:] == 12345.0)
+    h.destroy()
+
+
+WORKERS = [1, 2, 3, 4, 5, 8, 9, 16, 17, 32, 33, 64, 65, 100]
+
+
+@pytest.mark.parametrize("segments", [None, SEGMENTS], ids=["flat", "layers"])
+@pytest.mark.parametrize("bucket", [32, 64, 128, 256, 2048])
+@pytest.mark.parametrize("M", WORKERS)
+def test_sign(P, M, bucket, segments):
+    run(P, oracle.SIGN, M, segments, bucket=bucket)
