@@ -48,7 +48,56 @@ __device__ __forceinline__ void apply_chunk(const ServerArgs& s, int64_t j, cons
   }
 }
 
-constexpr int kSumLevels = 11;  // group counts up to 1024 (M <= 4096)
+constexpr int kSumLevels = 7;  // blocks of 64 workers (M <= 4096)
+
+// The sum over workers of the four elements of a chunk, from the values of
+// 8 consecutive workers at a time: eight(m, v) gives v[u][q] of worker m + u,
+// element q, +0 past M.  P8 blocks of 8 workers, a power of two, P8 * 8 >= M;
+// P8 = 0: any M, by subtrees of 64 workers.  (The tree is laid out at compile
+// time: kept as a binary counter over groups of four workers, its bookkeeping
+// took more instructions than the sum.  d = 3.6M, M = 8, identity: 44 -> 23
+// us; d = 2.4M, M = 48, b = 4: 119 -> 40, b = 2: 198 -> 36.)
+template <int FIRST, int N, typename Eight>
+__device__ __forceinline__ void tree_of_eights(int M, Eight&& eight, float (&out)[4]) {
+  if constexpr (N == 1) {
+    float v[8][4];
+    eight(8 * FIRST, v);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const float lo = group4(v[0][q], v[1][q], v[2][q], v[3][q], M);
+      out[q] = M > 4 ? __fadd_rn(lo, tree4(v[4][q], v[5][q], v[6][q], v[7][q])) : lo;
+    }
+  } else {
+    float a[4], b[4] = {0.f, 0.f, 0.f, 0.f};
+    tree_of_eights<FIRST, N / 2>(M, eight, a);
+    if (8 * (FIRST + N / 2) < M) tree_of_eights<FIRST + N / 2, N / 2>(M, eight, b);  // else all +0
+#pragma unroll
+    for (int q = 0; q < 4; ++q) out[q] = __fadd_rn(a[q], b[q]);
+  }
+}
+
+template <int P8, typename Eight>
+__device__ __forceinline__ void worker_sum(int M, Eight&& eight, float (&out)[4]) {
+  if constexpr (P8 > 0) {
+    tree_of_eights<0, P8>(M, eight, out);
+  } else {
+    PairwiseAcc<kSumLevels> acc[4];
+#pragma unroll 1
+    for (int m0 = 0; m0 < M; m0 += 64) {
+      float block[4];
+      // (a block's own group rule is that of 64 workers, also for the last
+      // one's few; the tree has more than 64 leaves)
+      tree_of_eights<0, 8>(64, [&](int m, float (&v)[8][4]) { eight(m0 + m, v); }, block);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc[q].push(block[q]);
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) out[q] = acc[q].result();
+  }
+}
+
+// The P8 of worker_sum for M workers.
+int eights_of(int M) { return M <= 64 ? next_pow2((M + 7) / 8) : 0; }
 
 // 32x32 bit transpose across a warp: on entry lane m holds row m; on exit
 // lane l holds column l (bit m = bit l of row m).  Five block-swap stages;
@@ -641,19 +690,19 @@ sign_server_col_kernel(const ServerArgs s, const SegSlices seg, const __grid_con
 }
 
 // b-bit stochastic quantiser: Q_m(p)_j = fl(s_m * V[code]) with
-// V[code] = sign(code - K) * fl(|code - K| / K) (so V[K] = +0), summed as
-// groups of four workers in the library's pairwise order.  One thread per
-// 4-element chunk (a fixed grid strides over the chunks), code words of 8
-// workers fetched before they are decoded.  For
-// b = 4, 8 V lives in shared memory replicated once per bank (entry c of lane
-// l at [c][l]), so the random code lookups of a warp never conflict; for
-// b = 2 (V in {-1, 0, +1}) the value is a select.
-template <int BITS, bool POW2>
-__global__ void __launch_bounds__(256) squant_server_kernel(const ServerArgs s) {
+// V[code] = sign(code - K) * fl(|code - K| / K) (so V[K] = +0), any bucket and
+// number of workers.  One thread per 4-element chunk (a fixed grid strides
+// over the chunks), code words and scales of 8 workers fetched before they
+// are decoded.  For b = 4, 8 V lives in shared memory replicated once per bank
+// (entry c of lane l at [c][l]), so the random code lookups of a warp never
+// conflict; for b = 2 (V in {-1, 0, +1}) the value is a select.
+template <int BITS, int P8>
+__global__ void __launch_bounds__(256, 4) squant_server_kernel(const ServerArgs s) {
   dq_pdl_enter();
   constexpr int K = (1 << (BITS - 1)) - 1;
   constexpr uint32_t MASK = (1u << BITS) - 1u;
   constexpr int CODES = (BITS == 2) ? 1 : (1 << BITS);
+  constexpr uint32_t kLevel0 = (BITS == 8 ? 0x01010101u : BITS == 4 ? 0x1111u : 0x55u) * K;  // four codes K
   __shared__ float V[CODES * 32];
   if constexpr (BITS != 2) {
     for (int t = threadIdx.x; t < CODES * 32; t += blockDim.x) {
@@ -679,55 +728,41 @@ __global__ void __launch_bounds__(256) squant_server_kernel(const ServerArgs s) 
     const int shift = (int)(bitpos & 31);
     const uint8_t* m_scale = s.msgs + 4 * bkt;
     const uint8_t* m_word = s.msgs + s.off_payload + 4 * word;
-    PairwiseAcc<kSumLevels> sum[4];
-    for (int m0 = 0; m0 < s.M; m0 += 8) {
-      uint32_t bits[8];
-      float sc[8];
+    float sum[4];
+    worker_sum<P8>(
+        s.M,
+        [&](int m, float (&v)[8][4]) {
+          uint32_t bits[8];
+          float sc[8];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const bool ok = m0 + u < s.M;
-        const int64_t off = (int64_t)(m0 + u) * s.msg_stride;
-        bits[u] = ok ? __ldcs(reinterpret_cast<const uint32_t*>(m_word + off)) >> shift : 0u;
-        sc[u] = ok ? __ldg(reinterpret_cast<const float*>(m_scale + off)) : 0.f;
-      }
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        if (m0 + 4 * h < s.M) {
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            float v[4];
-#pragma unroll
-            for (int x = 0; x < 4; ++x) {
-              const int u = 4 * h + x;
-              if constexpr (BITS == 2) {
-                const uint32_t code = (bits[u] >> (2 * q)) & 3u;
-                v[x] = (code == 0) ? -sc[u] : (code == 2 ? sc[u] : 0.f);  // fl(s * 1) = s
-              } else if constexpr (BITS == 8) {
-                v[x] = __fmul_rn(sc[u], Vl[__byte_perm(bits[u], 0, 0x4440 | q) << 5]);
-              } else {
-                v[x] = __fmul_rn(sc[u], Vl[((bits[u] >> (q * BITS)) & MASK) << 5]);
-              }
-              if (m0 + u >= s.M) v[x] = 0.f;  // padding leaves
+          for (int u = 0; u < 8; ++u) {
+            // padding leaves: level-0 codes and scale 0, which decode to +0
+            bits[u] = kLevel0;
+            sc[u] = 0.f;
+            if (m + u < s.M) {
+              const int64_t off = (int64_t)(m + u) * s.msg_stride;
+              bits[u] = __ldcs(reinterpret_cast<const uint32_t*>(m_word + off)) >> shift;
+              sc[u] = __ldg(reinterpret_cast<const float*>(m_scale + off));
             }
-            sum[q].push(group4(v[0], v[1], v[2], v[3], s.M));
           }
-        }
-      }
-    }
-    float acc[4];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) acc[q] = sum[q].result();
-    if (j + 3 < s.d) {
-      float4 wv = __ldcs(reinterpret_cast<const float4*>(s.w + j));
-      wv.x = server_out(s, wv.x, average_t<POW2>(acc[0], s));
-      wv.y = server_out(s, wv.y, average_t<POW2>(acc[1], s));
-      wv.z = server_out(s, wv.z, average_t<POW2>(acc[2], s));
-      wv.w = server_out(s, wv.w, average_t<POW2>(acc[3], s));
-      __stcs(reinterpret_cast<float4*>(s.w + j), wv);
-    } else {
-      for (int q = 0; q < 4 && j + q < s.d; ++q)
-        s.w[j + q] = server_out(s, s.w[j + q], average_t<POW2>(acc[q], s));
-    }
+          for (int u = 0; u < 8; ++u)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              if constexpr (BITS == 2) {
+                // code 0: -s, 1: +0, 2: +s (fl(s * 1) = s): the high bit clears
+                // the sign, the low one the value
+                const uint32_t signed_s = __float_as_uint(sc[u]) ^ (~(bits[u] << (30 - 2 * q)) & 0x80000000u);
+                v[u][q] = (bits[u] >> (2 * q)) & 1u ? 0.f : __uint_as_float(signed_s);
+              } else if constexpr (BITS == 8) {
+                v[u][q] = __fmul_rn(sc[u], Vl[__byte_perm(bits[u], 0, 0x4440 | q) << 5]);
+              } else {
+                v[u][q] = __fmul_rn(sc[u], Vl[((bits[u] >> (q * BITS)) & MASK) << 5]);
+              }
+            }
+        },
+        sum);
+    apply_chunk(s, j, sum);
   }
 }
 
@@ -1412,40 +1447,39 @@ squant8_server_table_kernel(const ServerArgs s, const SegSlices seg, const __gri
     mbar_wait_bounded(&bar[(it & 1u) ^ 1u], ((it + 1) >> 1) & 1u, s.err);
 }
 
-// Identity: the messages are the p vectors themselves, summed in groups of
-// four workers in the library's pairwise order.
-__global__ void __launch_bounds__(256) identity_server_kernel(const ServerArgs s) {
+// Identity: the messages are the p vectors themselves.
+template <int P8>
+__global__ void __launch_bounds__(256, 4) identity_server_kernel(const ServerArgs s) {
   dq_pdl_enter();
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t j = 4 * c;
   if (j >= s.d) return;
-  PairwiseAcc<kSumLevels> sum[4];
   const bool vec = j + 3 < s.d;
-  for (int m0 = 0; m0 < s.M; m0 += 4) {
-    float4 v[4];
+  float sum[4];
+  worker_sum<P8>(
+      s.M,
+      [&](int m, float (&v)[8][4]) {
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      v[u] = make_float4(0.f, 0.f, 0.f, 0.f);  // +0 leaves past M and past d
-      if (m0 + u < s.M) {
-        const float* vals = reinterpret_cast<const float*>(s.msgs + (int64_t)(m0 + u) * s.msg_stride);
-        if (vec) {
-          v[u] = __ldcs(reinterpret_cast<const float4*>(vals + j));
-        } else {
-          v[u].x = vals[j];
-          if (j + 1 < s.d) v[u].y = vals[j + 1];
-          if (j + 2 < s.d) v[u].z = vals[j + 2];
+        for (int u = 0; u < 8; ++u) {
+          float4 x = make_float4(0.f, 0.f, 0.f, 0.f);  // +0 leaves past M and past d
+          if (m + u < s.M) {
+            const float* vals = reinterpret_cast<const float*>(s.msgs + (int64_t)(m + u) * s.msg_stride);
+            if (vec) {
+              x = __ldcs(reinterpret_cast<const float4*>(vals + j));
+            } else {
+              x.x = vals[j];
+              if (j + 1 < s.d) x.y = vals[j + 1];
+              if (j + 2 < s.d) x.z = vals[j + 2];
+            }
+          }
+          v[u][0] = x.x;
+          v[u][1] = x.y;
+          v[u][2] = x.z;
+          v[u][3] = x.w;
         }
-      }
-    }
-    sum[0].push(group4(v[0].x, v[1].x, v[2].x, v[3].x, s.M));
-    sum[1].push(group4(v[0].y, v[1].y, v[2].y, v[3].y, s.M));
-    sum[2].push(group4(v[0].z, v[1].z, v[2].z, v[3].z, s.M));
-    sum[3].push(group4(v[0].w, v[1].w, v[2].w, v[3].w, s.M));
-  }
-  float acc[4];
-#pragma unroll
-  for (int q = 0; q < 4; ++q) acc[q] = sum[q].result();
-  apply_chunk(s, j, acc);
+      },
+      sum);
+  apply_chunk(s, j, sum);
 }
 
 __global__ void __launch_bounds__(256)
@@ -1731,26 +1765,37 @@ cudaError_t launch_squant_server(const ServerArgs& s, const SignServerExtras& x,
   }
   const unsigned chunk_grid = chunk_blocks(s.d, 256);
   const unsigned blocks = chunk_grid < 152u * 6u ? chunk_grid : 152u * 6u;  // V is built once per block
-  const bool p2 = s.M_pow2 != 0;
-  switch (s.bits) {
-    case 2: p2 ? launch_pdl(squant_server_kernel<2, true>, dim3(blocks), dim3(256), 0, stream, s)
-               : launch_pdl(squant_server_kernel<2, false>, dim3(blocks), dim3(256), 0, stream, s); break;
-    case 4: p2 ? launch_pdl(squant_server_kernel<4, true>, dim3(blocks), dim3(256), 0, stream, s)
-               : launch_pdl(squant_server_kernel<4, false>, dim3(blocks), dim3(256), 0, stream, s); break;
-    case 8: p2 ? launch_pdl(squant_server_kernel<8, true>, dim3(blocks), dim3(256), 0, stream, s)
-               : launch_pdl(squant_server_kernel<8, false>, dim3(blocks), dim3(256), 0, stream, s); break;
-    default: return cudaErrorInvalidValue;
+  auto go = [&](auto kernel) { return launch_pdl(kernel, dim3(blocks), dim3(256), 0, stream, s); };
+#define DQ_SQUANT(P8)                                 \
+  (s.bits == 2   ? go(squant_server_kernel<2, P8>)    \
+   : s.bits == 4 ? go(squant_server_kernel<4, P8>)    \
+   : s.bits == 8 ? go(squant_server_kernel<8, P8>) : cudaErrorInvalidValue)
+  cudaError_t st;
+  switch (eights_of(s.M)) {
+    case 1: st = DQ_SQUANT(1); break;
+    case 2: st = DQ_SQUANT(2); break;
+    case 4: st = DQ_SQUANT(4); break;
+    case 8: st = DQ_SQUANT(8); break;
+    default: st = DQ_SQUANT(0); break;
   }
+#undef DQ_SQUANT
   *launches += 1;
-  return cudaGetLastError();
+  return st;
 }
 
 cudaError_t launch_identity_server(const ServerArgs& s, cudaStream_t stream, uint64_t* launches) {
-  launch_pdl(identity_server_kernel, dim3(chunk_blocks(s.d, 256)), dim3(256), 0, stream, s);
+  auto go = [&](auto kernel) { return launch_pdl(kernel, dim3(chunk_blocks(s.d, 256)), dim3(256), 0, stream, s); };
+  cudaError_t st;
+  switch (eights_of(s.M)) {
+    case 1: st = go(identity_server_kernel<1>); break;
+    case 2: st = go(identity_server_kernel<2>); break;
+    case 4: st = go(identity_server_kernel<4>); break;
+    case 8: st = go(identity_server_kernel<8>); break;
+    default: st = go(identity_server_kernel<0>); break;
+  }
   *launches += 1;
-  return cudaGetLastError();
+  return st;
 }
-
 
 cudaError_t launch_oadam_update(const OAdamArgs& a, cudaStream_t stream, uint64_t* launches) {
   launch_pdl(oadam_update_kernel, dim3(chunk_blocks(a.d, 256)), dim3(256), 0, stream, a);

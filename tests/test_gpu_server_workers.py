@@ -60,3 +60,15 @@ WORKERS = [1, 2, 3, 4, 5, 8, 9, 16, 17, 32, 33, 64, 65, 100]
 @pytest.mark.parametrize("M", WORKERS)
 def test_sign(P, M, bucket, segments):
     run(P, oracle.SIGN, M, segments, bucket=bucket)
+
+
+@pytest.mark.parametrize("M", [*WORKERS, 129])
+def test_identity(P, M):
+    run(P, oracle.IDENTITY, M)
+
+
+@pytest.mark.parametrize("segments", [None, SEGMENTS], ids=["flat", "layers"])
+@pytest.mark.parametrize("bits", [2, 4, 8])
+@pytest.mark.parametrize("M", [*WORKERS, 129])
+def test_quantiser_small_buckets(P, M, bits, segments):
+    run(P, oracle.SQUANT, M, segments, bucket=64, bits=bits)
