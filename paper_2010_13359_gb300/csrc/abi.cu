@@ -29,7 +29,7 @@ struct dqgan_handle {
   uint32_t* err_word = nullptr;  // device error word written by bounded waits
   int64_t* seg_bstart = nullptr;     // layer segments: nb + 1 bucket starts (device)
   uint32_t* seg_wbucket = nullptr;   // layer segments: bucket of every 32-element word (device)
-  uint32_t* seg_slices = nullptr;    // layer segments, sign and 8-bit codes: {first word, bucket | (rows - 1) << 27} per slice
+  uint32_t* seg_slices = nullptr;    // layer segments, sign, 4- and 8-bit codes: {first word, bucket | (rows - 1) << 27} per slice
   int64_t seg_nslices = 0;
   CUtensorMap words_map;         // TMA map of the last message buffer the server saw
   const void* words_map_msgs = nullptr;
@@ -516,13 +516,16 @@ int dqgan_set_segments(dqgan_handle* h, const int64_t* offsets, int32_t nseg) {
         slices.push_back((uint32_t)b | (uint32_t)(rows - 1) << 27);
       }
     }
-  // 8-bit codes with 16 workers (four codes per word; buckets start on
-  // multiples of 32 elements): the quantiser server's slices, each bucket's
-  // code words in runs of up to 32, so that no slice spans two buckets
-  if ((c.compressor == DQGAN_SQUANT || c.compressor == DQGAN_QSGD) && c.bits == 8 && c.M == 16)
+  // 4- and 8-bit codes, up to 32 workers, buckets of at least 32 code words
+  // (a word holds 32 / bits elements; buckets start on multiples of 32): the
+  // quantiser server's slices, each bucket's code words in runs of up to 32,
+  // so that no slice spans two buckets
+  const int64_t per_word = c.bits > 0 ? 32 / c.bits : 0;
+  if ((c.compressor == DQGAN_SQUANT || c.compressor == DQGAN_QSGD) && c.bits != 2 && c.M <= 32 &&
+      c.bucket >= 32 * per_word)
     for (int64_t b = 0; b < nb; ++b) {
-      const int64_t we = (starts[b + 1] + 3) / 4;
-      for (int64_t w = starts[b] / 4; w < we; w += 32) {
+      const int64_t we = (starts[b + 1] + per_word - 1) / per_word;
+      for (int64_t w = starts[b] / per_word; w < we; w += 32) {
         const int64_t rows = we - w < 32 ? we - w : 32;
         slices.push_back((uint32_t)w);
         slices.push_back((uint32_t)b | (uint32_t)(rows - 1) << 27);

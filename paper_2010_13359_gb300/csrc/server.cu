@@ -13,11 +13,13 @@
 // M <= 32: the column and warp-transpose kernels, words staged by TMA, flat
 // buckets or a per-bucket slice table with layer segments; the rest: a warp
 // per chunk of 256 elements).  Stochastic quantiser with M <= 32: code words
-// staged by TMA, per-worker or pair-table decode (and, for 8-bit codes with
-// layer segments and 16 workers, slices from a per-bucket table).  The rest --
+// staged by TMA, per-worker or pair-table decode (and, for 4- and 8-bit codes
+// with layer segments, slices from a per-bucket table).  The rest --
 // identity, small buckets of the quantiser, more than 32 workers -- one thread
 // per 4-element chunk of w walks the M messages.  w is read and written once;
 // every kernel waits for the grid before it (programmatic dependent launch).
+#include <atomic>
+
 #include "device_common.cuh"
 
 namespace dq {
@@ -93,6 +95,21 @@ __device__ __forceinline__ void worker_sum(int M, Eight&& eight, float (&out)[4]
     }
 #pragma unroll
     for (int q = 0; q < 4; ++q) out[q] = acc[q].result();
+  }
+}
+
+// Pairwise sum of the values of groups FIRST .. FIRST + N - 1 (N a power of
+// two; groups from NG on are +0), element by element.
+template <int FIRST, int N, int NG, typename Group, int E>
+__device__ __forceinline__ void tree_of_groups(Group&& group, float (&out)[E]) {
+  if constexpr (N == 1) {
+    group(4 * FIRST, out);
+  } else {
+    float b[E] = {};
+    tree_of_groups<FIRST, N / 2, NG>(group, out);
+    if constexpr (FIRST + N / 2 < NG) tree_of_groups<FIRST + N / 2, N / 2, NG>(group, b);
+#pragma unroll
+    for (int e = 0; e < E; ++e) out[e] = __fadd_rn(out[e], b[e]);
   }
 }
 
@@ -891,9 +908,9 @@ constexpr bool sq_params_boxed(int bits) { return bits != 8; }
 // summed pairwise: the library's fixed order.  b = 2 sums by pair tables
 // instead (b2_pair_table_update, NSET sets of 16 workers; tables rebuilt only
 // when the bucket changes), which reach the same tree from pairs of workers.
-// With layer segments (SEG) a slice may hold words of several buckets: each
-// lane then reads the workers' scales of its own word's bucket (b = 2: two
-// bit tests per worker and element, then the groups of four).
+// With layer segments (SEG, b = 2 only) a slice may hold words of several
+// buckets: each lane then reads the workers' scales of its own word's bucket
+// and decodes by two bit tests per worker and element, in groups of four.
 // For b = 2 and 4 (a lane owns 64 or 32 contiguous bytes of w, which plain
 // loads would fetch at a 64- or 32-byte lane stride) the slice's parameters
 // come by TMA as well: w viewed as rows of 32 floats (pmap), a box of
@@ -910,6 +927,7 @@ __global__ void __launch_bounds__(32 * kTmaWarps)
 squant_server_tma_kernel(const ServerArgs s, const __grid_constant__ CUtensorMap tmap,
                          const __grid_constant__ CUtensorMap pmap) {
   dq_pdl_enter();
+  static_assert(!SEG || BITS == 2, "4- and 8-bit codes with layer segments take the table kernel");
   constexpr int K = (1 << (BITS - 1)) - 1;
   constexpr int EPL = 32 / BITS;  // elements per lane (one code word)
   constexpr int SLICE = 32 * EPL; // elements per slice
@@ -984,11 +1002,8 @@ squant_server_tma_kernel(const ServerArgs s, const __grid_constant__ CUtensorMap
     return (sl_ < nslices && j < s.d) ? (int64_t)__ldg(s.word_bucket + (j >> 5)) : -1;
   };
   int64_t wb_next = SEG ? word_bucket_of(sl) : 0;
-  // (b = 4, 8: two slices ahead, so that the scale can be loaded one ahead)
-  int64_t wb_next2 = (SEG && kSqPrefetch) ? word_bucket_of(sl + stride) : 0;
-  // b = 4, 8: this lane's worker's scale of the slice's bucket (the bucket
-  // of lane 0's word), and (b = 8) the lane's four parameters, loaded one
-  // slice ahead
+  // b = 4, 8: this lane's worker's scale of the slice's bucket, and (b = 8)
+  // the lane's four parameters, loaded one slice ahead
   const float* const lane_scales =
       reinterpret_cast<const float*>(s.msgs + (int64_t)(active ? lane : 0) * s.msg_stride);
   auto load_w4 = [&](int64_t sl_) -> float4 {
@@ -1002,10 +1017,7 @@ squant_server_tma_kernel(const ServerArgs s, const __grid_constant__ CUtensorMap
     return x;
   };
   float scale_nx = 0.f;
-  if constexpr (kSqPrefetch) {
-    const int64_t b0 = SEG ? (int64_t)__shfl_sync(kFullMask, wb_next, 0) : sl / spb;
-    scale_nx = (active && sl < nslices && b0 >= 0) ? __ldg(lane_scales + b0) : 0.f;
-  }
+  if constexpr (kSqPrefetch) scale_nx = (active && sl < nslices) ? __ldg(lane_scales + sl / spb) : 0.f;
   float4 w_nx = (kSqPrefetch && !WB) ? load_w4(sl) : make_float4(0.f, 0.f, 0.f, 0.f);
   uint32_t it = 0;
   bool ok = true;
@@ -1020,12 +1032,7 @@ squant_server_tma_kernel(const ServerArgs s, const __grid_constant__ CUtensorMap
       issue(nxt, cur ^ 1);
     }
     const int64_t wb_cur = wb_next;
-    if constexpr (SEG && kSqPrefetch) {
-      wb_next = wb_next2;
-      wb_next2 = word_bucket_of(nxt + stride);
-    } else if constexpr (SEG) {
-      wb_next = word_bucket_of(nxt);
-    }
+    if constexpr (SEG) wb_next = word_bucket_of(nxt);
     const int64_t b = sl / spb;
     const int64_t j0 = SLICE * sl + EPL * lane;  // this lane's first element
     // the lane's parameters: row pr of the box, 16-byte chunks pc0 ..
@@ -1064,8 +1071,7 @@ squant_server_tma_kernel(const ServerArgs s, const __grid_constant__ CUtensorMap
     float my_scale;
     if constexpr (kSqPrefetch) {
       my_scale = scale_nx;
-      const int64_t bn = SEG ? (int64_t)__shfl_sync(kFullMask, wb_next, 0) : nxt / spb;
-      scale_nx = (active && nxt < nslices && bn >= 0) ? __ldg(lane_scales + bn) : 0.f;
+      scale_nx = (active && nxt < nslices) ? __ldg(lane_scales + nxt / spb) : 0.f;
     } else {
       my_scale = active ? __ldg(reinterpret_cast<const float*>(s.msgs + (int64_t)lane * s.msg_stride) + bkt) : 0.f;
     }
@@ -1127,7 +1133,7 @@ squant_server_tma_kernel(const ServerArgs s, const __grid_constant__ CUtensorMap
     constexpr int kParts = BITS == 4 ? kSquant4Parts : 1;
     constexpr int NE = EPL / kParts;
     // one worker's decoded values of this lane's elements e0 .. e0 + NE - 1
-    auto decode_part = [&](bool MX, uint32_t word, float sc, int e0, float (&v)[NE]) {
+    auto decode_part = [&](uint32_t word, float sc, int e0, float (&v)[NE]) {
       if constexpr (BITS == 2) {
         // code 0: -s, 1: +0, 2: +s (fl(s * 1) = s): one bit test picks +0,
         // one the sign
@@ -1142,15 +1148,12 @@ squant_server_tma_kernel(const ServerArgs s, const __grid_constant__ CUtensorMap
       // b = 4: lane c first forms this worker's decoded value of code c mod 16,
       // fl(s * V[c mod 16]); each element then fetches its value with one
       // shuffle (the lane index is taken mod 32 and the values repeat in lanes
-      // 16..31, so the bits above the element's code need no mask).  (With
-      // layer segments the lanes' scales may differ: look up V[c] and multiply
-      // by the lane's own scale instead.)
-      const float T4 = (BITS == 4) ? __fmul_rn(MX ? 1.0f : sc, V4) : 0.f;
+      // 16..31, so the bits above the element's code need no mask).
+      const float T4 = (BITS == 4) ? __fmul_rn(sc, V4) : 0.f;
 #pragma unroll
       for (int e = 0; e < NE; ++e) {
         if constexpr (BITS == 4) {
           v[e] = __shfl_sync(kFullMask, T4, (int)(word >> (4 * (e0 + e))));
-          if (MX) v[e] = __fmul_rn(sc, v[e]);
         } else {
           v[e] = __fmul_rn(sc, V8l[__byte_perm(word, 0u, 0x4440u | (uint32_t)(e0 + e)) * 32u]);
         }
@@ -1189,14 +1192,14 @@ squant_server_tma_kernel(const ServerArgs s, const __grid_constant__ CUtensorMap
             sc[u] = here ? scale_of(mx, m + u) : 0.f;
           }
           float va[NE], vb[NE];
-          decode_part(mx, wd[0], sc[0], e0, va);
-          decode_part(mx, wd[1], sc[1], e0, vb);
+          decode_part(wd[0], sc[0], e0, va);
+          decode_part(wd[1], sc[1], e0, vb);
           const bool h1 = m + 1 < M;
 #pragma unroll
           for (int e = 0; e < NE; ++e) g[e] = M == 1 ? va[e] : __fadd_rn(va[e], h1 ? vb[e] : 0.f);
           if (M <= 2) return;
-          decode_part(mx, wd[2], sc[2], e0, va);
-          decode_part(mx, wd[3], sc[3], e0, vb);
+          decode_part(wd[2], sc[2], e0, va);
+          decode_part(wd[3], sc[3], e0, vb);
           const bool h2 = m + 2 < M, h3 = m + 3 < M;
 #pragma unroll
           for (int e = 0; e < NE; ++e) g[e] = __fadd_rn(g[e], __fadd_rn(h2 ? va[e] : 0.f, h3 ? vb[e] : 0.f));
@@ -1299,42 +1302,48 @@ squant_server_tma_kernel(const ServerArgs s, const __grid_constant__ CUtensorMap
   }
 }
 
-// 8-bit codes with layer segments and 16 workers: the slices come from a
+// 4- and 8-bit codes with layer segments, M <= 32: the slices come from a
 // host-built table of each bucket's code words in runs of up to 32, so no
-// slice spans two buckets (the per-lane bucket lookups and the mixed-slice
-// decode of the kernel above are not needed).  The word box starts at the
-// 16-byte boundary at or before the slice (36 words wide, no swizzle); lane l
-// takes word first + l of every worker when l < rows.  The decode and the
-// sum over workers are the b = 8 ones above: level table replicated per
-// shared-memory bank, groups of four workers (a + b) + (c + d), the four
-// group values added pairwise.  The slice's scale, the next slice's table
-// entry and the lane's four parameters are loaded one slice ahead.
-template <bool POW2>
+// slice spans two buckets.  The word box starts at the 16-byte boundary at or
+// before the slice (36 words wide, no swizzle); lane l takes word first + l of
+// every worker when l < rows.  The decode is that of the flat kernel above
+// (b = 8: level table replicated per shared-memory bank; b = 4: the worker's
+// products fl(s * V[c]), one per lane, looked up by shuffle), and the NG =
+// ceil(M / 4) groups of four workers are added pairwise, the tree laid out at
+// compile time; workers past M read as level-0 codes with scale 0, which
+// decode to +0 (FULL: M = 4 NG, a power of two, and there are none: 16 workers,
+// b = 8, d = 25M 115 us, 129 with the tests).  The slice's scale, the next slice's table entry and the
+// lane's parameters are loaded one slice ahead.  (Slices of 32 words whatever
+// the buckets, each lane looking up its own word's bucket, took 140 us for 16
+// workers, b = 4, d = 25M, 512 per scale, against 89 here, and 157 for 12
+// workers, b = 8, against 116.)
+template <int BITS, int NG, bool FULL>
 __global__ void __launch_bounds__(32 * kTmaWarps)
-squant8_server_table_kernel(const ServerArgs s, const SegSlices seg, const __grid_constant__ CUtensorMap tmap) {
+squant_server_table_kernel(const ServerArgs s, const SegSlices seg, const __grid_constant__ CUtensorMap tmap) {
   dq_pdl_enter();
-  constexpr int K = 127;
-  constexpr int M = 16;
-  constexpr int RW = kSignSegBoxWords;                       // words per box row
-  constexpr uint32_t kBoxBytes = (uint32_t)M * RW * 4u;      // 2304: a multiple of 128
+  constexpr int K = (1 << (BITS - 1)) - 1;
+  constexpr int EPL = 32 / BITS;         // elements per lane (one code word)
+  constexpr int RW = kSignSegBoxWords;   // words per box row
+  constexpr uint32_t kBoxBytes = 4u * NG * RW * 4u;  // room for whole groups: a multiple of 128 + 64
+  constexpr uint32_t kBoxPitch = (kBoxBytes + 127u) / 128u * 128u;
+  constexpr uint32_t kLevel0 = (BITS == 8 ? 0x01010101u : 0x11111111u) * K;
   extern __shared__ uint8_t smem_raw[];
   __shared__ uint64_t bars[kTmaWarps][2];
-  __shared__ float V8[256 * 32];
+  __shared__ float V8[BITS == 8 ? 256 * 32 : 1];
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
   const uint32_t raw = smem_addr(smem_raw);
-  uint8_t* const buf0 = smem_raw + ((128u - (raw & 127u)) & 127u) + warp * 2 * kBoxBytes;  // + i * kBoxBytes
+  uint8_t* const buf0 = smem_raw + ((128u - (raw & 127u)) & 127u) + warp * 2 * kBoxPitch;  // + i * kBoxPitch
   uint64_t* bar = bars[warp];
-  for (int t = threadIdx.x; t < 256 * 32; t += blockDim.x) {
-    const int code = t >> 5;
+  auto level_value = [](int code) -> float {
     const int level = code - K;
-    float v = 0.f;
-    if (code <= 2 * K && level != 0) {
-      const float mag = __fdiv_rn((float)(level < 0 ? -level : level), (float)K);
-      v = level < 0 ? -mag : mag;
-    }
-    V8[t] = v;
-  }
+    if (code > 2 * K || level == 0) return 0.f;
+    const float mag = __fdiv_rn((float)(level < 0 ? -level : level), (float)K);
+    return level < 0 ? -mag : mag;
+  };
+  if constexpr (BITS == 8)
+    for (int t = threadIdx.x; t < 256 * 32; t += blockDim.x) V8[t] = level_value(t >> 5);
+  const float V4 = BITS == 4 ? level_value(lane & 15) : 0.f;  // b = 4: lane l holds V[l mod 16]
   if (lane == 0) {
     mbar_init(&bar[0], 1);
     mbar_init(&bar[1], 1);
@@ -1345,7 +1354,8 @@ squant8_server_table_kernel(const ServerArgs s, const SegSlices seg, const __gri
   const int64_t nslices = seg.n;
   const int64_t stride = (int64_t)gridDim.x * kTmaWarps;
   const int32_t x0 = (int32_t)(s.off_payload >> 2);  // a multiple of 64 words
-  const bool active = lane < M;
+  const uint32_t box_bytes = (uint32_t)s.M * RW * 4u;
+  const bool active = lane < s.M;
   struct Slice {
     int64_t word;    // first code word
     int64_t bucket;
@@ -1357,28 +1367,36 @@ squant8_server_table_kernel(const ServerArgs s, const SegSlices seg, const __gri
     return Slice{(int64_t)e.x, (int64_t)(e.y & 0x7FFFFFFu), (int)(e.y >> 27) + 1};
   };
   auto issue = [&](const Slice& c, int i) {
-    mbar_arrive_expect_tx(&bar[i], kBoxBytes);
-    tma_load_2d(buf0 + i * kBoxBytes, &tmap, (x0 + (int32_t)c.word) & ~3, 0, &bar[i]);
+    mbar_arrive_expect_tx(&bar[i], box_bytes);
+    tma_load_2d(buf0 + i * kBoxPitch, &tmap, (x0 + (int32_t)c.word) & ~3, 0, &bar[i]);
   };
   const float* const lane_scales =
       reinterpret_cast<const float*>(s.msgs + (int64_t)(active ? lane : 0) * s.msg_stride);
-  // the lane's four parameters of slice c (none past its rows or past d)
-  auto load_w4 = [&](const Slice& c) -> float4 {
-    float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (lane >= c.rows) return x;
-    const int64_t j = 4 * (c.word + lane);
-    if (j + 3 < s.d) return __ldcs(reinterpret_cast<const float4*>(s.w + j));
-    if (j < s.d) x.x = s.w[j];
-    if (j + 1 < s.d) x.y = s.w[j + 1];
-    if (j + 2 < s.d) x.z = s.w[j + 2];
-    return x;
+  // the lane's parameters of slice c (none past its rows or past d)
+  auto load_w = [&](const Slice& c, float (&x)[EPL]) {
+#pragma unroll
+    for (int q = 0; q < EPL; ++q) x[q] = 0.f;
+    if (lane >= c.rows) return;
+    const int64_t j = EPL * (c.word + lane);
+#pragma unroll
+    for (int q = 0; q < EPL; q += 4) {
+      if (j + q + 3 < s.d) {
+        const float4 v = __ldcs(reinterpret_cast<const float4*>(s.w + j + q));
+        x[q] = v.x; x[q + 1] = v.y; x[q + 2] = v.z; x[q + 3] = v.w;
+      } else {
+#pragma unroll
+        for (int r = 0; r < 3; ++r)
+          if (j + q + r < s.d) x[q + r] = s.w[j + q + r];
+      }
+    }
   };
   int64_t sl = (int64_t)blockIdx.x * kTmaWarps + warp;
   Slice c = slice_of(sl);
   Slice cn = slice_of(sl + stride);
   if (sl < nslices && lane == 0) issue(c, 0);
   float scale_nx = (active && sl < nslices) ? __ldg(lane_scales + c.bucket) : 0.f;
-  float4 w_nx = load_w4(c);
+  float w_nx[EPL];
+  load_w(c, w_nx);
   uint32_t it = 0;
   bool ok = true;
   for (; sl < nslices; sl += stride, ++it) {
@@ -1389,53 +1407,56 @@ squant8_server_table_kernel(const ServerArgs s, const SegSlices seg, const __gri
       fence_proxy_async_shared();  // this warp's reads of that buffer came before
       issue(cn, cur ^ 1);
     }
-    const float my_scale = scale_nx;
+    const float my_scale = scale_nx;  // 0 past M
     scale_nx = (active && nxt < nslices) ? __ldg(lane_scales + cn.bucket) : 0.f;
-    const float wv[4] = {w_nx.x, w_nx.y, w_nx.z, w_nx.w};
-    w_nx = load_w4(cn);
+    float wv[EPL];
+#pragma unroll
+    for (int q = 0; q < EPL; ++q) wv[q] = w_nx[q];
+    load_w(cn, w_nx);
     ok = mbar_wait_bounded(&bar[cur], (it >> 1) & 1u, s.err);
     ok = __all_sync(kFullMask, ok);
     if (!ok) break;
-    const uint32_t* words = reinterpret_cast<const uint32_t*>(buf0 + cur * kBoxBytes) + (int)((x0 + c.word) & 3) + lane;
+    const uint32_t* words = reinterpret_cast<const uint32_t*>(buf0 + cur * kBoxPitch) + (int)((x0 + c.word) & 3) + lane;
     const float* V8l = V8 + lane;
-    // group value of workers m .. m + 3: (a + b) + (c + d)
-    auto group = [&](int m, float (&g)[4]) {
+    // group value of workers m .. m + 3
+    auto group = [&](int m, float (&g)[EPL]) {
       uint32_t wd[4];
       float sc[4];
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
-        wd[u] = words[RW * (m + u)];
+        wd[u] = FULL || m + u < s.M ? words[RW * (m + u)] : kLevel0;  // warp-uniform
         sc[u] = __shfl_sync(kFullMask, my_scale, m + u);
       }
-      float v[4][4];
+      float v[4][EPL];
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
+      for (int u = 0; u < 4; ++u) {
+        const float T4 = BITS == 4 ? __fmul_rn(sc[u], V4) : 0.f;
 #pragma unroll
-        for (int e = 0; e < 4; ++e)
-          v[u][e] = __fmul_rn(sc[u], V8l[__byte_perm(wd[u], 0u, 0x4440u | (uint32_t)e) * 32u]);
+        for (int e = 0; e < EPL; ++e) {
+          if constexpr (BITS == 4) v[u][e] = __shfl_sync(kFullMask, T4, (int)(wd[u] >> (4 * e)));
+          else v[u][e] = __fmul_rn(sc[u], V8l[__byte_perm(wd[u], 0u, 0x4440u | (uint32_t)e) * 32u]);
+        }
+      }
 #pragma unroll
-      for (int e = 0; e < 4; ++e) g[e] = __fadd_rn(__fadd_rn(v[0][e], v[1][e]), __fadd_rn(v[2][e], v[3][e]));
+      for (int e = 0; e < EPL; ++e) g[e] = group4(v[0][e], v[1][e], v[2][e], v[3][e], FULL ? 4 * NG : s.M);
     };
-    float g0[4], g1[4], r[4];
-    group(0, g0);
-    group(4, g1);
-#pragma unroll
-    for (int e = 0; e < 4; ++e) r[e] = __fadd_rn(g0[e], g1[e]);
-    group(8, g0);
-    group(12, g1);
-#pragma unroll
-    for (int e = 0; e < 4; ++e) r[e] = __fadd_rn(r[e], __fadd_rn(g0[e], g1[e]));
+    float r[EPL];
+    tree_of_groups<0, next_pow2(NG), NG>(group, r);
     if (lane < c.rows) {
-      const int64_t j = 4 * (c.word + lane);
-      float o[4];
+      const int64_t j = EPL * (c.word + lane);
 #pragma unroll
-      for (int e = 0; e < 4; ++e) o[e] = server_out(s, wv[e], average_t<POW2>(r[e], s));
-      if (j + 3 < s.d) {
-        __stcs(reinterpret_cast<float4*>(s.w + j), make_float4(o[0], o[1], o[2], o[3]));
-      } else {
+      for (int q = 0; q < EPL; q += 4) {
+        float o[4];
 #pragma unroll
         for (int e = 0; e < 4; ++e)
-          if (j + e < s.d) s.w[j + e] = o[e];
+          o[e] = server_out(s, wv[q + e], FULL ? average_t<true>(r[q + e], s) : average(r[q + e], s));
+        if (j + q + 3 < s.d) {
+          __stcs(reinterpret_cast<float4*>(s.w + j + q), make_float4(o[0], o[1], o[2], o[3]));
+        } else {
+#pragma unroll
+          for (int e = 0; e < 4; ++e)
+            if (j + q + e < s.d) s.w[j + q + e] = o[e];
+        }
       }
     }
     __syncwarp();
@@ -1614,24 +1635,36 @@ cudaError_t launch_squant_tma(const ServerArgs& s, const CUtensorMap* params_map
   int dev = 0;
   cudaError_t st = cudaGetDevice(&dev);
   if (st != cudaSuccess) return st;
-  if ((st = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess) return st;
-  int sms = 0, per_sm = 0;
-  if ((st = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return st;
-  if ((st = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * kTmaWarps, smem)) != cudaSuccess)
-    return st;
+  // resident CTAs on the device by worker count (asking on every call took a
+  // quarter of a small call's time)
+  static std::atomic<int> blocks_for[64][33];
+  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  int cap = blocks_for[dev][s.M].load(std::memory_order_acquire);
+  if (cap == 0) {
+    constexpr int most = kTmaWarps * 2 * (pbox + 32 * 128) + 1024;  // of any worker count
+    if ((st = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most)) != cudaSuccess)
+      return st;
+    int sms = 0, per_sm = 0;
+    if ((st = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return st;
+    if ((st = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * kTmaWarps, smem)) != cudaSuccess)
+      return st;
+    cap = sms * (per_sm > 0 ? per_sm : 1);
+    blocks_for[dev][s.M].store(cap, std::memory_order_release);
+  }
   const int64_t nslices = SEG ? (s.d + 32 * (32 / BITS) - 1) / (32 * (32 / BITS))
                               : ((s.d + s.bucket - 1) / s.bucket) * (s.bucket / (32 * (32 / BITS)));
   const int64_t need = (nslices + kTmaWarps - 1) / kTmaWarps;
-  const int64_t cap = (int64_t)sms * (per_sm > 0 ? per_sm : 1);
   // (b = 8 takes no parameter map: the word map stands in for the unused argument)
   launch_pdl(kern, dim3((unsigned)(need < cap ? need : cap)), dim3(32 * kTmaWarps), smem, stream,
       s, *s.squant_words_map, sq_params_boxed(BITS) ? *params_map : *s.squant_words_map);
   return cudaGetLastError();
 }
 
-cudaError_t launch_squant8_table(const ServerArgs& s, const SignServerExtras& x, cudaStream_t stream) {
-  auto kern = squant8_server_table_kernel<true>;
-  constexpr int smem = kTmaWarps * 2 * 16 * kSignSegBoxWords * 4 + 128;  // + alignment slack
+template <int BITS, int NG, bool FULL = false>
+cudaError_t launch_squant_table(const ServerArgs& s, const SignServerExtras& x, cudaStream_t stream) {
+  auto kern = squant_server_table_kernel<BITS, NG, FULL>;
+  constexpr int box = (4 * NG * kSignSegBoxWords * 4 + 127) / 128 * 128;
+  constexpr int smem = kTmaWarps * 2 * box + 128;  // + alignment slack
   int dev = 0;
   cudaError_t st = cudaGetDevice(&dev);
   if (st != cudaSuccess) return st;
@@ -1648,10 +1681,28 @@ cudaError_t launch_squant8_table(const ServerArgs& s, const SignServerExtras& x,
   }
   const int64_t need = (x.seg_nslices + kTmaWarps - 1) / kTmaWarps;
   const unsigned blocks = (unsigned)(need < blocks_for[dev] ? need : blocks_for[dev]);
-  if (blocks == 0) return cudaSuccess;
-  launch_pdl(kern, dim3(blocks), dim3(32 * kTmaWarps), smem, stream, s, SegSlices{x.seg_slices, x.seg_nslices},
-             *s.squant_words_map);
-  return cudaGetLastError();
+  return launch_pdl(kern, dim3(blocks), dim3(32 * kTmaWarps), smem, stream, s, SegSlices{x.seg_slices, x.seg_nslices},
+                    *s.squant_words_map);
+}
+
+template <int BITS>
+cudaError_t launch_squant_table(const ServerArgs& s, const SignServerExtras& x, cudaStream_t stream) {
+  switch (s.M) {
+    case 4: return launch_squant_table<BITS, 1, true>(s, x, stream);
+    case 8: return launch_squant_table<BITS, 2, true>(s, x, stream);
+    case 16: return launch_squant_table<BITS, 4, true>(s, x, stream);
+    case 32: return launch_squant_table<BITS, 8, true>(s, x, stream);
+  }
+  switch ((s.M + 3) / 4) {
+    case 1: return launch_squant_table<BITS, 1>(s, x, stream);
+    case 2: return launch_squant_table<BITS, 2>(s, x, stream);
+    case 3: return launch_squant_table<BITS, 3>(s, x, stream);
+    case 4: return launch_squant_table<BITS, 4>(s, x, stream);
+    case 5: return launch_squant_table<BITS, 5>(s, x, stream);
+    case 6: return launch_squant_table<BITS, 6>(s, x, stream);
+    case 7: return launch_squant_table<BITS, 7>(s, x, stream);
+    default: return launch_squant_table<BITS, 8>(s, x, stream);
+  }
 }
 
 unsigned chunk_blocks(int64_t d, int threads) {
@@ -1727,36 +1778,44 @@ cudaError_t launch_sign_server(const ServerArgs& s, const SignServerExtras& x, c
 cudaError_t launch_squant_server(const ServerArgs& s, const SignServerExtras& x, cudaStream_t stream,
                                  uint64_t* launches) {
   const CUtensorMap* params_map = x.params_map;
-  if (s.word_bucket && x.seg_slices && s.squant_words_map != nullptr && s.bits == 8 && s.M == 16) {
-    // 8-bit codes, layer segments, 16 workers: slices from the per-bucket table
-    const cudaError_t st = launch_squant8_table(s, x, stream);
+  // The TMA kernels for 2-bit codes work on slices of 512 elements and wait
+  // for their copies; while there are few, a thread per 4 elements is faster
+  // (16 workers, flat, d = 131,072 / 524,288: 2.8 / 4.4 us against 3.4 / 3.5;
+  // layer segments, 524,288: 4.3 against 6.7).
+  const bool few = s.bits == 2 && s.d <= (s.word_bucket ? 524288 : 262144);
+  if (s.word_bucket && x.seg_slices && s.squant_words_map != nullptr) {
+    // 4- and 8-bit codes, layer segments: slices from the per-bucket table
+    const cudaError_t st = s.bits == 8 ? launch_squant_table<8>(s, x, stream) : launch_squant_table<4>(s, x, stream);
     *launches += 1;
     return st;
   }
-  if (s.squant_words_map != nullptr && s.M <= 32 && s.bucket >= 32 * (32 / s.bits) &&
+  if (s.squant_words_map != nullptr && s.M <= 32 && s.bucket >= 32 * (32 / s.bits) && !few &&
       (params_map != nullptr || !sq_params_boxed(s.bits))) {
     const bool p2 = s.M_pow2 != 0;
     cudaError_t st = cudaErrorInvalidValue;
-#define DQ_SQ_TMA(B, NSET)                                                                              \
-  st = s.word_bucket ? (p2 ? launch_squant_tma<B, true, true, NSET>(s, params_map, stream)              \
-                           : launch_squant_tma<B, false, true, NSET>(s, params_map, stream))            \
-                     : (p2 ? launch_squant_tma<B, true, false, NSET>(s, params_map, stream)             \
-                           : launch_squant_tma<B, false, false, NSET>(s, params_map, stream))
+#define DQ_SQ_TMA(B, SEG, NSET)                                               \
+  st = p2 ? launch_squant_tma<B, true, SEG, NSET>(s, params_map, stream)       \
+          : launch_squant_tma<B, false, SEG, NSET>(s, params_map, stream)
     switch (s.bits) {
       case 2:
-        if (s.M == 16 && !s.word_bucket) st = launch_squant_tma<2, true, false, 1, 16>(s, params_map, stream);
-        else if (s.M <= 16) DQ_SQ_TMA(2, 1);
-        else DQ_SQ_TMA(2, 2);
+        if (s.word_bucket) {
+          if (s.M <= 16) DQ_SQ_TMA(2, true, 1);
+          else DQ_SQ_TMA(2, true, 2);
+        } else if (s.M == 16) {
+          st = launch_squant_tma<2, true, false, 1, 16>(s, params_map, stream);
+        } else if (s.M <= 16) {
+          DQ_SQ_TMA(2, false, 1);
+        } else {
+          DQ_SQ_TMA(2, false, 2);
+        }
         break;
       case 4:
-        if (s.M == 16 && !s.word_bucket) st = launch_squant_tma<4, true, false, 1, 16>(s, params_map, stream);
-        else DQ_SQ_TMA(4, 1);
+        if (s.M == 16) st = launch_squant_tma<4, true, false, 1, 16>(s, params_map, stream);
+        else DQ_SQ_TMA(4, false, 1);
         break;
       case 8:
-        if (s.M == 16)
-          st = s.word_bucket ? launch_squant_tma<8, true, true, 1, 16>(s, params_map, stream)
-                             : launch_squant_tma<8, true, false, 1, 16>(s, params_map, stream);
-        else DQ_SQ_TMA(8, 1);
+        if (s.M == 16) st = launch_squant_tma<8, true, false, 1, 16>(s, params_map, stream);
+        else DQ_SQ_TMA(8, false, 1);
         break;
     }
 #undef DQ_SQ_TMA

@@ -72,3 +72,17 @@ def test_identity(P, M):
 @pytest.mark.parametrize("M", [*WORKERS, 129])
 def test_quantiser_small_buckets(P, M, bits, segments):
     run(P, oracle.SQUANT, M, segments, bucket=64, bits=bits)
+
+
+@pytest.mark.parametrize("bits", [4, 8])
+@pytest.mark.parametrize("M", WORKERS)
+def test_quantiser_layer_buckets(P, M, bits):
+    run(P, oracle.SQUANT, M, SEGMENTS, bucket=256, bits=bits)
+
+
+@pytest.mark.parametrize("M", [1, 3, 8, 16, 17, 32])
+def test_two_bits_beyond_the_small_sizes(P, M):
+    run(P, oracle.SQUANT, M, d=262_144 + 519, bucket=512, bits=2)
+    d = 524_288 + 519
+    cuts = tuple(32 * c for c in np.sort(np.random.default_rng(M).choice(d // 32, 20, replace=False)) if c)
+    run(P, oracle.SQUANT, M, (0, *cuts, d), d=d, bucket=512, bits=2)
