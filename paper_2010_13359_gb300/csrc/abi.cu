@@ -427,7 +427,7 @@ int dqgan_create(const dqgan_config* cfg, dqgan_handle** out) {
   if (cfg->flags & DQGAN_KEEP_LOOKAHEAD)
     if ((st = dq_malloc(&h->h, rows_bytes)) != cudaSuccess) return fail_oom("allocating h", st);
   if (cfg->compressor == DQGAN_TOPK) {
-    h->scratch_bytes = dq::topk_scratch_bytes(cfg->d, cfg->M, cfg->M);
+    h->scratch_bytes = dq::topk_scratch_bytes(cfg->d, cfg->k, cfg->M, cfg->M);
     if ((st = scratch_alloc(&h->scratch, h->scratch_bytes)) != cudaSuccess)
       return fail_oom("allocating top-k scratch", st);
   }
@@ -612,7 +612,7 @@ int dqgan_set_local_workers(dqgan_handle* h, int32_t first, int32_t count) {
   if (st != cudaSuccess) return cuda_fail(h, st, "synchronize");
   const size_t rows_bytes = (size_t)count * (size_t)h->ld * sizeof(float);
   const size_t scratch_bytes =
-      h->cfg.compressor == DQGAN_TOPK ? dq::topk_scratch_bytes(h->cfg.d, count, h->cfg.M) : 0;
+      h->cfg.compressor == DQGAN_TOPK ? dq::topk_scratch_bytes(h->cfg.d, h->cfg.k, count, h->cfg.M) : 0;
   float *e = nullptr, *hh = nullptr;
   void* scratch = nullptr;
   auto fail = [&](const char* what, cudaError_t err) {

@@ -171,9 +171,9 @@ cudaError_t launch_identity_compress(const CompressArgs& a, bool keep_h, cudaStr
 // Scratch of the top-k path: `rows` rows (one per local worker) and the
 // server's tables for `nworkers` messages (none for 0).  A row needs no
 // clearing between calls: every call rewrites what it reads of it.  The
-// server's per-index worker masks (up to 64 workers) must be zero when the
-// scratch is created; each server call clears the masks it set.
-size_t topk_scratch_bytes(int64_t d, int32_t rows, int32_t nworkers);
+// server's per-index worker masks (sparse records, up to 64 workers) must be
+// zero when the scratch is created; each server call clears the masks it set.
+size_t topk_scratch_bytes(int64_t d, int64_t k, int32_t rows, int32_t nworkers);
 cudaError_t launch_topk_compress(const CompressArgs& a, int64_t k, bool keep_h, void* scratch,
                                  cudaStream_t stream, uint64_t* launches);
 
@@ -186,7 +186,7 @@ cudaError_t launch_sign_server(const ServerArgs& s, const SignServerExtras& x, c
 cudaError_t launch_squant_server(const ServerArgs& s, const SignServerExtras& x, cudaStream_t stream,
                                  uint64_t* launches);
 cudaError_t launch_identity_server(const ServerArgs& s, cudaStream_t stream, uint64_t* launches);
-// scratch: topk_scratch_bytes(d, rows, M); the server's table follows the rows.
+// scratch: topk_scratch_bytes(d, k, rows, M); the server's table follows the rows.
 cudaError_t launch_topk_server(const ServerArgs& s, void* scratch, int32_t rows, cudaStream_t stream,
                                uint64_t* launches);
 

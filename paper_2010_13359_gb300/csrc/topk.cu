@@ -33,13 +33,15 @@
 //
 // Server: w_j -= (sum over workers of the value recorded for j, absent
 // workers as +0, in the library's pairwise order) / M at the indices some
-// worker sent; elsewhere the sum is +0 and w is unchanged.  Up to 64
-// workers, one thread per record in two launches: the records scatter their
-// values into per-worker rows and set their worker's bit in a per-index
-// mask, then the lowest worker of each index sums the index's values and
-// updates w_j.  Above 64 workers, a first kernel finds where each worker's
-// records of each 256-index tile start, and one thread per record searches
-// the other workers' records of its tile.
+// worker sent; elsewhere the sum is +0 and w is unchanged.  Where the records
+// are dense enough (tile_server), a first kernel finds where each worker's
+// records of each tile of indices start, and a CTA per tile merges the
+// workers' records of it in shared memory.  Sparse records of up to 64
+// workers: one thread per record in two launches, which scatter the values
+// into a table and set the worker's bit in a per-index mask, then let the
+// lowest worker of each index sum the index's values and update w_j.  Above
+// 64 workers one thread per record searches the other workers' records of its
+// tile.
 #include <atomic>
 #include <cmath>
 
@@ -1182,9 +1184,9 @@ __device__ __forceinline__ float srv_average(float acc, const ServerArgs& s) {
 }
 
 // Server for M <= kSrvMaskMaxM: two launches over the M * k records, with
-// two tables in the scratch -- a worker mask per index (u64; all zero
-// between calls) and a value row per worker (d floats, never cleared).
-//   1. scatter: record (m, r) with index j writes its value to row m at j
+// two tables in the scratch -- a worker mask per index (u32, u64 above 32
+// workers; all zero between calls) and M values per index (never cleared).
+//   1. scatter: record (m, r) with index j writes its value to entry (j, m)
 //      and sets bit m of j's mask.
 //   2. reduce: the record of the lowest worker in j's mask owns j.  It sums
 //      the values of the workers in the mask, in worker order with the
@@ -1194,44 +1196,91 @@ __device__ __forceinline__ float srv_average(float acc, const ServerArgs& s) {
 //      its lowest, so they do nothing.
 // Indices nobody sent have the sum +0 and keep w_j; with store_q the q_hat
 // buffer is cleared before the scatter.
+// Bound by the tables' scattered sectors.  Consecutive blocks take the same
+// stretch of records of the M workers in turn: the records are sorted, so the
+// workers' blocks touch the same masks and values about the same time, while
+// those are in L2 (worker after worker each swept the whole table through
+// DRAM: 25M x 16, k = d / 100, 453 us against 282).
 constexpr int kSrvMaskMaxM = 64;
 
-
+template <typename Mask>
 struct SrvTables {
-  unsigned long long* mask;  // d masks
-  float* vals;               // row m at vals + m * ldv
-  int64_t ldv;
+  Mask* mask;   // d masks
+  float* vals;  // worker m's value of index j at vals[j * M + m]
 };
 
+// Words of a mask: one bit per worker.
+__host__ __device__ constexpr int srv_mask_words(int32_t nworkers) { return nworkers <= 32 ? 1 : 2; }
+
 __host__ __device__ constexpr int64_t srv_mask_table_words(int64_t d, int32_t nworkers) {
-  return 2 * round64(d) + (int64_t)nworkers * round64(d);
+  return (srv_mask_words(nworkers) + (int64_t)nworkers) * round64(d);
 }
 
-inline SrvTables srv_tables(void* scratch, int64_t d, int32_t rows) {
+template <typename Mask>
+inline SrvTables<Mask> srv_tables(void* scratch, int64_t d, int32_t rows) {
   uint32_t* base = reinterpret_cast<uint32_t*>(scratch) + row_words(d) * rows;
-  SrvTables t;
-  t.mask = reinterpret_cast<unsigned long long*>(base);
-  t.vals = reinterpret_cast<float*>(base + 2 * round64(d));
-  t.ldv = round64(d);
-  return t;
+  return SrvTables<Mask>{reinterpret_cast<Mask*>(base),
+                         reinterpret_cast<float*>(base + sizeof(Mask) / sizeof(uint32_t) * round64(d))};
 }
 
-__global__ void __launch_bounds__(kSrvThreads) topk_server_scatter_kernel(const ServerArgs s, SrvTables t) {
+// This thread's record: worker m's r-th.
+struct SrvRecord {
+  int m;
+  int64_t r;
+};
+__device__ __forceinline__ SrvRecord srv_record(const ServerArgs& s) {
+  return SrvRecord{(int)(blockIdx.x % (unsigned)s.M),
+                   (int64_t)(blockIdx.x / (unsigned)s.M) * kSrvThreads + threadIdx.x};
+}
+
+template <typename Mask>
+__global__ void __launch_bounds__(kSrvThreads) topk_server_scatter_kernel(const ServerArgs s, SrvTables<Mask> t) {
   dq_pdl_enter();
-  const int m = blockIdx.y;
-  const int64_t r = (int64_t)blockIdx.x * kSrvThreads + threadIdx.x;
+  const auto [m, r] = srv_record(s);
   if (r >= s.k) return;
   const uint2 rec = reinterpret_cast<const uint2*>(s.msgs + (int64_t)m * s.msg_stride)[r];
   // records come from the compressor and are below d
   if (!dq_in_bounds((int64_t)rec.x < s.d, s.err)) return;
-  t.vals[(int64_t)m * t.ldv + rec.x] = __uint_as_float(rec.y);
-  atomicOr(t.mask + rec.x, 1ull << m);
+  t.vals[(int64_t)rec.x * s.M + m] = __uint_as_float(rec.y);
+  atomicOr(t.mask + rec.x, (Mask)1 << m);
 }
 
-template <bool POW2, int P>
-__global__ void __launch_bounds__(kSrvThreads) topk_server_reduce_kernel(const ServerArgs s, SrvTables t) {
-  const int m = blockIdx.y;
-  const int64_t r = (int64_t)blockIdx.x * kSrvThreads + threadIdx.x;
+// The sum at an index whose mask of workers is `mask`, by the owner m with its
+// value v; value(who): another worker's.
+template <int P, typename Mask, typename Value>
+__device__ __forceinline__ float owner_sum(Mask mask, int m, float v, Value&& value) {
+  if ((mask & (mask - 1u)) == 0u) return P == 1 ? v : __fadd_rn(v, 0.f);  // one value among +0 leaves
+  // the padded tree itself: chunks of C leaves (workers), each summed
+  // pairwise from its values (+0 where a worker is absent), then the
+  // P / C chunk sums pairwise -- the chunks are the tree's subtrees
+  constexpr int C = P < 16 ? P : 16;
+  float part[P / C];
+#pragma unroll
+  for (int c = 0; c < P / C; ++c) {
+    const uint32_t bits = (uint32_t)(mask >> (C * c)) & (uint32_t)((1ull << C) - 1ull);
+    float x[C];
+#pragma unroll
+    for (int u = 0; u < C; ++u) {
+      const int who = C * c + u;
+      x[u] = 0.f;
+      if ((bits >> u) & 1u) x[u] = who == m ? v : value(who);
+    }
+#pragma unroll
+    for (int width = C / 2; width >= 1; width /= 2)
+#pragma unroll
+      for (int i = 0; i < width; ++i) x[i] = __fadd_rn(x[2 * i], x[2 * i + 1]);
+    part[c] = x[0];
+  }
+#pragma unroll
+  for (int width = P / C / 2; width >= 1; width /= 2)
+#pragma unroll
+    for (int i = 0; i < width; ++i) part[i] = __fadd_rn(part[2 * i], part[2 * i + 1]);
+  return part[0];
+}
+
+template <typename Mask, bool POW2, int P>
+__global__ void __launch_bounds__(kSrvThreads) topk_server_reduce_kernel(const ServerArgs s, SrvTables<Mask> t) {
+  const auto [m, r] = srv_record(s);
   if (r >= s.k) return;
   const uint2 rec = reinterpret_cast<const uint2*>(s.msgs + (int64_t)m * s.msg_stride)[r];
   const int64_t j = rec.x;
@@ -1239,43 +1288,189 @@ __global__ void __launch_bounds__(kSrvThreads) topk_server_reduce_kernel(const S
   // the scatter grid has completed and its writes are visible (the record
   // was complete before the scatter ran)
   dq_pdl_enter();
-  const unsigned long long mask = t.mask[j];
+  const Mask mask = t.mask[j];
   // the owner: bit m set and no bit below it
-  if (!((mask >> m) & 1ull) || (mask & ((1ull << m) - 1ull))) return;
-  const float v = __uint_as_float(rec.y);
-  float sum;
-  if ((mask & (mask - 1ull)) == 0ull) {
-    sum = P == 1 ? v : __fadd_rn(v, 0.f);  // one value among +0 leaves
-  } else {
-    // the padded tree itself: chunks of C leaves (workers), each summed
-    // pairwise from its values (+0 where a worker is absent), then the
-    // P / C chunk sums pairwise -- the chunks are the tree's subtrees
-    constexpr int C = P < 16 ? P : 16;
-    float part[P / C];
-#pragma unroll
-    for (int c = 0; c < P / C; ++c) {
-      const uint32_t bits = (uint32_t)(mask >> (C * c)) & (uint32_t)((1ull << C) - 1ull);
-      float x[C];
-#pragma unroll
-      for (int u = 0; u < C; ++u) {
-        const int who = C * c + u;
-        x[u] = 0.f;
-        if ((bits >> u) & 1u) x[u] = who == m ? v : t.vals[(int64_t)who * t.ldv + j];
-      }
-#pragma unroll
-      for (int width = C / 2; width >= 1; width /= 2)
-#pragma unroll
-        for (int i = 0; i < width; ++i) x[i] = __fadd_rn(x[2 * i], x[2 * i + 1]);
-      part[c] = x[0];
-    }
-#pragma unroll
-    for (int width = P / C / 2; width >= 1; width /= 2)
-#pragma unroll
-      for (int i = 0; i < width; ++i) part[i] = __fadd_rn(part[2 * i], part[2 * i + 1]);
-    sum = part[0];
-  }
+  if (!((mask >> m) & 1u) || (mask & (((Mask)1 << m) - 1u))) return;
+  const float sum = owner_sum<P>(mask, m, __uint_as_float(rec.y), [&](int who) { return t.vals[j * s.M + who]; });
   s.w[j] = server_out(s, s.w[j], srv_average<POW2>(sum, s));
-  t.mask[j] = 0ull;
+  t.mask[j] = 0;
+}
+
+// Server for dense records (tile_server), M <= kSrvMaskMaxM: one CTA per
+// kMergeTile indices.  starts[m][t] tells where worker m's records of each run
+// of kSrvTile indices are.  Two ways to merge, by the tile's number of records:
+//   list (up to half a record per index): the records go to shared memory,
+//     worker after worker, and set their worker's bit in their index's mask;
+//     the record of the lowest worker of an index owns it.  A sole worker's
+//     record updates w; the indices of several workers get rows of M values in
+//     what the list leaves free, as many at a time as fit, which their records
+//     fill and their owners sum.
+//   table: a zeroed value per worker and index, as many runs of indices at a
+//     time as fit; the records set theirs and every index sums its column (+0
+//     where nobody sent it, which leaves w as it is).
+// Records and touched parameters are all it moves: against the tables of the
+// two kernels above, whose scattered sectors go through DRAM twice, 25M x 16,
+// k = d / 100: 453 -> 143 us (k = d / 20: 1611 -> 348), the starts included.
+constexpr int kMergeThreads = 256;
+constexpr int kMergeRuns = 16;
+constexpr int kMergeTile = kMergeRuns * kSrvTile;  // indices per CTA
+constexpr int kMergeCap = 2048;                    // records in the list
+constexpr int kMergeRow = 2048;                    // words for the rows of shared indices
+
+// Shared memory: the list, the rows, the masks and the rows' numbers, or the
+// table (at least one run).
+constexpr size_t merge_smem(size_t mask_bytes) {
+  return kMergeCap * sizeof(uint2) + kMergeRow * sizeof(float) + kMergeTile * (mask_bytes + sizeof(uint16_t));
+}
+static_assert(kSrvMaskMaxM * kSrvTile * sizeof(float) <= merge_smem(8) && 32 * kSrvTile * sizeof(float) <= merge_smem(4),
+              "a run of every worker fits");
+
+// Whether the merge kernel runs: it wants some records in each tile, and so
+// many in all that the other kernels' tables do not stay in L2 (us, tables in
+// worker order / merged: 3.6M x 8, 1 %, 288,000 records, the layers' scales
+// such that most share a few tiles, 15 / 20; 3.6M x 16, 1 %, 48 / 32; 25M x 16,
+// 1 %, 453 / 143; 25M x 32, 0.1 %, 107 / 61; 25M x 4, 0.1 %, 19 / 22).
+bool tile_server(int64_t d, int64_t k, int nworkers) {
+  const double records = (double)k * nworkers;
+  return nworkers <= kSrvMaskMaxM && d >= 500'000 && records >= 500e3 && records >= 0.03 * (double)d;
+}
+
+template <typename Mask, bool POW2, int P>
+__global__ void __launch_bounds__(kMergeThreads, 4) topk_server_tile_kernel(const ServerArgs s, const uint32_t* starts) {
+  dq_pdl_enter();
+  extern __shared__ __align__(16) unsigned char tile_smem[];
+  uint2* list = reinterpret_cast<uint2*>(tile_smem);             // {index in the tile | worker << 16, value}
+  float* rows = reinterpret_cast<float*>(list + kMergeCap);      // M values per row
+  Mask* mask = reinterpret_cast<Mask*>(rows + kMergeRow);
+  uint16_t* row_of = reinterpret_cast<uint16_t*>(mask + kMergeTile);  // of a shared index
+  __shared__ uint32_t nshared;
+  float* table = reinterpret_cast<float*>(tile_smem);
+  __shared__ uint32_t st[kMergeRuns + 1][P];                     // each worker's first record of each run
+  __shared__ uint32_t off[P + 1];                                // the workers' parts of the records at hand
+  const int64_t nts = srv_tiles(s.d);
+  const int64_t run0 = (int64_t)blockIdx.x * kMergeRuns;
+  const int64_t t0 = run0 * kSrvTile;
+  const int lane = threadIdx.x & 31;
+  for (int i = threadIdx.x; i < (kMergeRuns + 1) * s.M; i += kMergeThreads) {
+    const int m = i / (kMergeRuns + 1), r = i - m * (kMergeRuns + 1);
+    st[r][m] = (uint32_t)min64(starts[(int64_t)m * (nts + 1) + min64(run0 + r, nts)], s.k);
+  }
+  // the tile's parameters on their way while the records come
+  if (threadIdx.x < kMergeTile / 32 && t0 + 32 * (int)threadIdx.x < s.d)
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(s.w + t0 + 32 * threadIdx.x));
+  for (int i = threadIdx.x; i < kMergeTile; i += kMergeThreads) mask[i] = 0;
+  if (threadIdx.x == 0) nshared = 0;
+  __syncthreads();
+  // off[] for the records of the runs [a, b), by one warp
+  auto place = [&](int a, int b) {
+    if (threadIdx.x < 32) {
+      uint32_t run = 0;
+      for (int m0 = 0; m0 < s.M; m0 += 32) {
+        const uint32_t n = m0 + lane < s.M ? max(st[b][m0 + lane], st[a][m0 + lane]) - st[a][m0 + lane] : 0u;
+        uint32_t x = n;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const uint32_t y = __shfl_up_sync(kFullMask, x, o);
+          if (lane >= o) x += y;
+        }
+        if (m0 + lane < s.M) off[m0 + lane] = run + x - n;
+        run += __shfl_sync(kFullMask, x, 31);
+      }
+      if (lane == 0) off[s.M] = run;
+    }
+    __syncthreads();
+  };
+  // body(place, worker, index in the tile, value bits) over those records
+  // (they come from the compressor: sorted, and below d)
+  auto for_records = [&](int a, auto&& body) {
+    for (uint32_t f = threadIdx.x; f < off[s.M]; f += kMergeThreads) {
+      int m = 0;  // the worker: off[m] <= f < off[m + 1]
+#pragma unroll
+      for (int step = P / 2; step >= 1; step >>= 1)
+        if (m + step < s.M && off[m + step] <= f) m += step;
+      const uint2 rec = reinterpret_cast<const uint2*>(s.msgs + (int64_t)m * s.msg_stride)[st[a][m] + (f - off[m])];
+      const int64_t i = (int64_t)rec.x - t0;
+      body(f, m, dq_in_bounds(i >= 0 && i < kMergeTile && (int64_t)rec.x < s.d, s.err) ? (int)i : -1, rec.y);
+    }
+    __syncthreads();
+  };
+  place(0, kMergeRuns);
+  const uint32_t n = off[s.M];
+  if (n <= (uint32_t)kMergeCap) {
+    for_records(0, [&](uint32_t f, int m, int i, uint32_t v) {
+      list[f] = make_uint2(i < 0 ? 0xFFFFFFFFu : (uint32_t)i | (uint32_t)m << 16, v);
+      if (i >= 0) atomicOr(mask + i, (Mask)1 << m);
+    });
+    for (uint32_t f = threadIdx.x; f < n; f += kMergeThreads) {
+      const uint2 e = list[f];
+      if (e.x == 0xFFFFFFFFu) continue;
+      const uint32_t i = e.x & 0xFFFFu;
+      const int m = (int)(e.x >> 16);
+      const Mask bits = mask[i];
+      if (bits & (((Mask)1 << m) - 1u)) continue;  // a lower worker owns the index
+      if (bits != (Mask)1 << m) {
+        row_of[i] = (uint16_t)atomicAdd(&nshared, 1u);
+        continue;
+      }
+      const float sum = owner_sum<P>(bits, m, __uint_as_float(e.y), [](int) { return 0.f; });
+      s.w[t0 + i] = server_out(s, s.w[t0 + i], srv_average<POW2>(sum, s));
+    }
+    __syncthreads();
+    const uint32_t at_once = kMergeRow / (uint32_t)s.M, shared = nshared;
+    for (uint32_t row0 = 0; row0 < shared; row0 += at_once) {
+      // body(row, record, index, worker, mask) for the records of these rows
+      auto for_shared = [&](auto&& body) {
+        for (uint32_t f = threadIdx.x; f < n; f += kMergeThreads) {
+          const uint2 e = list[f];
+          if (e.x == 0xFFFFFFFFu) continue;
+          const uint32_t i = e.x & 0xFFFFu;
+          const int m = (int)(e.x >> 16);
+          const Mask bits = mask[i];
+          if (bits == (Mask)1 << m) continue;
+          const uint32_t row = row_of[i] - row0;
+          if (row < at_once) body(row, e.y, i, m, bits);
+        }
+        __syncthreads();
+      };
+      for_shared([&](uint32_t row, uint32_t v, uint32_t, int m, Mask) { rows[row * s.M + m] = __uint_as_float(v); });
+      for_shared([&](uint32_t row, uint32_t v, uint32_t i, int m, Mask bits) {
+        if (bits & (((Mask)1 << m) - 1u)) return;
+        const float sum = owner_sum<P>(bits, m, __uint_as_float(v), [&](int who) { return rows[row * s.M + who]; });
+        s.w[t0 + i] = server_out(s, s.w[t0 + i], srv_average<POW2>(sum, s));
+      });
+    }
+    return;
+  }
+  constexpr int kTableRuns = (int)(merge_smem(sizeof(Mask)) / (P * kSrvTile * sizeof(float)));
+  constexpr int kRuns = kTableRuns < kMergeRuns ? kTableRuns : kMergeRuns;
+  constexpr int kWidth = kRuns * kSrvTile;
+  for (int a = 0; a < kMergeRuns && t0 + a * kSrvTile < s.d; a += kRuns) {
+    const int b = min(a + kRuns, kMergeRuns);
+    __syncthreads();
+    for (int i = threadIdx.x; i < s.M * (kWidth / 4); i += kMergeThreads)
+      reinterpret_cast<float4*>(table)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    place(a, b);
+    for_records(a, [&](uint32_t, int m, int i, uint32_t v) {
+      const int x = i - a * kSrvTile;
+      if (i >= 0 && x >= 0 && x < kWidth) table[m * kWidth + x] = __uint_as_float(v);
+    });
+    const int width = (int)min64((int64_t)(b - a) * kSrvTile, s.d - t0 - a * kSrvTile);
+    for (int i = threadIdx.x; i < width; i += kMergeThreads) {
+      // the padded tree, in chunks of up to 16 workers
+      constexpr int C = P < 16 ? P : 16;
+      float part[P / C];
+#pragma unroll
+      for (int c = 0; c < P / C; ++c) {
+        float x[C];
+#pragma unroll
+        for (int u = 0; u < C; ++u) x[u] = C * c + u < s.M ? table[(C * c + u) * kWidth + i] : 0.f;
+        part[c] = pairwise_n<C>(x);
+      }
+      const float sum = pairwise_n<P / C>(part);
+      const int64_t j = t0 + a * kSrvTile + i;
+      s.w[j] = server_out(s, s.w[j], srv_average<POW2>(sum, s));
+    }
+  }
 }
 
 // One thread per record of every worker.  The record of the lowest worker
@@ -1363,12 +1558,14 @@ __global__ void __launch_bounds__(kSrvThreads) topk_server_owner_kernel(const Se
 
 }  // namespace
 
-size_t topk_scratch_bytes(int64_t d, int32_t rows, int32_t nworkers) {
-  // the server's tables: masks and value rows (M <= kSrvMaskMaxM), or the
-  // record-range table of the owner kernel (more workers); none for 0
+size_t topk_scratch_bytes(int64_t d, int64_t k, int32_t rows, int32_t nworkers) {
+  // the server's tables: masks and values, or the record starts of every
+  // run of kSrvTile indices (dense records; more than kSrvMaskMaxM workers);
+  // none for 0
   const int64_t server_words = nworkers <= 0 ? 0
-                               : nworkers <= kSrvMaskMaxM ? srv_mask_table_words(d, nworkers)
-                                                          : round64((int64_t)nworkers * (srv_tiles(d) + 1));
+                               : nworkers <= kSrvMaskMaxM && !tile_server(d, k, nworkers)
+                                   ? srv_mask_table_words(d, nworkers)
+                                   : round64((int64_t)nworkers * (srv_tiles(d) + 1));
   return (size_t)(row_words(d) * rows + server_words) * 4u;
 }
 
@@ -1484,40 +1681,78 @@ cudaError_t launch_topk_compress(const CompressArgs& a, int64_t k, bool keep_h, 
   return st;
 }
 
+static cudaError_t launch_tile_server(const ServerArgs& s, const uint32_t* starts, cudaStream_t stream) {
+  const dim3 grid((unsigned)((s.d + kMergeTile - 1) / kMergeTile));
+  auto go = [&](auto kernel, size_t mask_bytes, std::atomic<bool> (&done)[kSmemDevices]) -> cudaError_t {
+    const cudaError_t st = allow_smem(kernel, merge_smem(mask_bytes), 1, done);
+    if (st != cudaSuccess) return st;
+    return launch_pdl(kernel, grid, dim3(kMergeThreads), merge_smem(mask_bytes), stream, s, starts);
+  };
+  switch (next_pow2(s.M)) {
+#define DQ_TILE(P, MASK)                                                                  \
+  case P: {                                                                               \
+    static std::atomic<bool> done[2][kSmemDevices];                                       \
+    return s.M_pow2 ? go(topk_server_tile_kernel<MASK, true, P>, sizeof(MASK), done[0])   \
+                    : go(topk_server_tile_kernel<MASK, false, P>, sizeof(MASK), done[1]); \
+  }
+    DQ_TILE(1, uint32_t) DQ_TILE(2, uint32_t) DQ_TILE(4, uint32_t) DQ_TILE(8, uint32_t) DQ_TILE(16, uint32_t)
+    DQ_TILE(32, uint32_t) DQ_TILE(64, unsigned long long)
+#undef DQ_TILE
+  }
+  return cudaErrorInvalidValue;
+}
+
 cudaError_t launch_topk_server(const ServerArgs& s, void* scratch, int32_t rows, cudaStream_t stream,
                                 uint64_t* launches) {
+  if (s.store_q) {  // the dense q_hat buffer: +0 wherever nobody sent an index
+    if (s.M > kSrvMaskMaxM) return cudaErrorNotSupported;  // the owner kernel is sparse
+    const cudaError_t st = cudaMemsetAsync(s.w, 0, (size_t)s.d * sizeof(float), stream);
+    if (st != cudaSuccess) return st;
+  }
+  uint32_t* starts = reinterpret_cast<uint32_t*>(scratch) + row_words(s.d) * rows;
+  const dim3 starts_grid((unsigned)((s.k + 255) / 256), (unsigned)s.M);
+  if (tile_server(s.d, s.k, s.M)) {
+    cudaError_t st = launch_pdl(topk_server_starts_kernel, starts_grid, dim3(256), 0, stream, s, starts);
+    if (st != cudaSuccess) return st;
+    *launches += 1;
+    st = launch_tile_server(s, starts, stream);
+    *launches += st == cudaSuccess ? 1 : 0;
+    return st;
+  }
   if (s.M <= kSrvMaskMaxM) {
-    const SrvTables t = srv_tables(scratch, s.d, rows);
-    const dim3 grid((unsigned)((s.k + kSrvThreads - 1) / kSrvThreads), (unsigned)s.M);
-    if (s.store_q) {  // the dense q_hat buffer: +0 wherever nobody sent an index
-      const cudaError_t st = cudaMemsetAsync(s.w, 0, (size_t)s.d * sizeof(float), stream);
-      if (st != cudaSuccess) return st;
-    }
-    launch_pdl(topk_server_scatter_kernel, grid, dim3(kSrvThreads), 0, stream, s, t);
-    cudaError_t st = cudaGetLastError();
+    const dim3 grid((unsigned)((s.k + kSrvThreads - 1) / kSrvThreads * s.M));
+    const auto t32 = srv_tables<uint32_t>(scratch, s.d, rows);
+    const auto t64 = srv_tables<unsigned long long>(scratch, s.d, rows);
+    const bool narrow = srv_mask_words(s.M) == 1;
+    cudaError_t st =
+        narrow ? launch_pdl(topk_server_scatter_kernel<uint32_t>, grid, dim3(kSrvThreads), 0, stream, s, t32)
+               : launch_pdl(topk_server_scatter_kernel<unsigned long long>, grid, dim3(kSrvThreads), 0, stream, s, t64);
     if (st != cudaSuccess) return st;
     // the reduce kernel's blocks read their records while the scatter's last
     // blocks finish, then wait for the scatter grid
+    auto go = [&](auto kernel, auto t) { return launch_pdl(kernel, grid, dim3(kSrvThreads), 0, stream, s, t); };
     st = cudaErrorInvalidValue;
     switch (next_pow2(s.M)) {
-#define DQ_TOPK_REDUCE(P)                                                                             \
-  case P:                                                                                             \
-    st = s.M_pow2 ? launch_pdl(topk_server_reduce_kernel<true, P>, grid, dim3(kSrvThreads), 0, stream, s, t) \
-                  : launch_pdl(topk_server_reduce_kernel<false, P>, grid, dim3(kSrvThreads), 0, stream, s, t); \
+#define DQ_TOPK_REDUCE(P)                                                 \
+  case P:                                                                 \
+    st = s.M_pow2 ? go(topk_server_reduce_kernel<uint32_t, true, P>, t32) \
+                  : go(topk_server_reduce_kernel<uint32_t, false, P>, t32); \
     break;
       DQ_TOPK_REDUCE(1) DQ_TOPK_REDUCE(2) DQ_TOPK_REDUCE(4) DQ_TOPK_REDUCE(8) DQ_TOPK_REDUCE(16)
-      DQ_TOPK_REDUCE(32) DQ_TOPK_REDUCE(64)
+      DQ_TOPK_REDUCE(32)
 #undef DQ_TOPK_REDUCE
+      case 64:
+        st = s.M_pow2 ? go(topk_server_reduce_kernel<unsigned long long, true, 64>, t64)
+                      : go(topk_server_reduce_kernel<unsigned long long, false, 64>, t64);
+        break;
     }
     // (a failure here would leave the scatter's mask bits set; the launch has
     // the scatter's grid and block, which were just accepted)
     *launches += st == cudaSuccess ? 2 : 1;
     return st;
   }
-  if (s.store_q) return cudaErrorNotSupported;  // the owner kernel is sparse
-  uint32_t* starts = reinterpret_cast<uint32_t*>(scratch) + row_words(s.d) * rows;
   const int64_t n = (int64_t)s.M * s.k;
-  launch_pdl(topk_server_starts_kernel, dim3((unsigned)((s.k + 255) / 256), (unsigned)s.M), dim3(256), 0, stream, s, starts);
+  launch_pdl(topk_server_starts_kernel, starts_grid, dim3(256), 0, stream, s, starts);
   const unsigned blocks = (unsigned)((n + kSrvThreads - 1) / kSrvThreads);
   if (s.M_pow2) launch_pdl(topk_server_owner_kernel<true>, dim3(blocks), dim3(kSrvThreads), 0, stream, s, starts);
   else launch_pdl(topk_server_owner_kernel<false>, dim3(blocks), dim3(kSrvThreads), 0, stream, s, starts);

@@ -26,7 +26,7 @@ def P():
     return P
 
 
-def run(P, comp, M, segments=None, d=D, **kw):
+def run(P, comp, M, segments=None, d=D, hot=0, **kw):
     ocfg = oracle_config(d, M, comp, lr=0.03, seed=M, segments=segments, **kw)
     h = P.create(P.make_config(d=d, M=M, compressor=comp, lr=0.03, seed=M,
                                cuda_stream=torch.cuda.current_stream().cuda_stream, **kw))
@@ -34,6 +34,7 @@ def run(P, comp, M, segments=None, d=D, **kw):
         h.set_segments(segments)
     rng = np.random.default_rng(M)
     g = (rng.standard_normal((M, d)) * np.exp(rng.uniform(-3, 1, (M, d)))).astype(np.float32)
+    g[:, :hot] *= 1e3
     ld = (d + 3) // 4 * 4
     g_dev = torch.zeros((M, ld), device="cuda")
     g_dev[:, :d] = torch.from_numpy(g)
@@ -86,3 +87,36 @@ def test_two_bits_beyond_the_small_sizes(P, M):
     d = 524_288 + 519
     cuts = tuple(32 * c for c in np.sort(np.random.default_rng(M).choice(d // 32, 20, replace=False)) if c)
     run(P, oracle.SQUANT, M, (0, *cuts, d), d=d, bucket=512, bits=2)
+
+
+@pytest.mark.parametrize("kind", ["spread", "shared", "dense"])
+@pytest.mark.parametrize("M", [1, 2, 3, 8, 16, 17, 32, 33, 64])
+def test_top_k_merged_by_tiles(P, M, kind):
+    """Half a million records: spread over the vector; two in three of them at
+    indices every worker sends; and all of them in a few tiles, more than a
+    list holds."""
+    d, k = 4_100_007, -(-510_000 // M)
+    rng = np.random.default_rng(M)
+    ocfg = oracle_config(d, M, oracle.TOPK, lr=0.03, k=k)
+    h = P.create(P.make_config(d=d, M=M, compressor=P.TOPK, lr=0.03, k=k,
+                               cuda_stream=torch.cuda.current_stream().cuda_stream))
+    common = rng.choice(d, 2 * k // 3, replace=False)
+    msgs = np.zeros((M, h.message_bytes() // 8, 2), np.uint32)
+    for m in range(M):
+        if kind == "spread":
+            idx = rng.choice(d, k, replace=False)
+        elif kind == "shared":
+            own = rng.permutation(np.setdiff1d(rng.choice(d, 2 * k, replace=False), common))
+            idx = np.concatenate([common, own[:k - len(common)]])
+        else:
+            idx = d - 1 - rng.choice(k + k // 3, k, replace=False)
+        msgs[m, :k, 0] = np.sort(idx)
+        msgs[m, :k, 1] = rng.standard_normal(k).astype(np.float32).view(np.uint32)
+    msgs = msgs.view(np.uint8).reshape(M, -1)
+    w = (rng.standard_normal(d) * 0.02).astype(np.float32)
+    w_gpu = torch.from_numpy(w.copy()).to("cuda")
+    h.server_aggregate_update(torch.from_numpy(msgs).to("cuda"), w_gpu)
+    oracle.server_step(ocfg, msgs, w)
+    h.synchronize()
+    assert_params_equal(w_gpu.cpu().numpy(), w)
+    h.destroy()
