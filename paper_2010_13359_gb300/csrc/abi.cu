@@ -732,7 +732,7 @@ int dqgan_worker_lookahead(dqgan_handle* h, int32_t i, const float* params, floa
   if (!aligned16(params) || !aligned16(out_w_half))
     return set_error(h, DQGAN_ERR_INVALID_ARG, "pointers must be 16-byte aligned");
   NvtxRange range("dqgan worker lookahead");
-  const cudaError_t st = dq::launch_lookahead(params, h->h + (int64_t)i * h->ld, out_w_half, h->cfg.d,
+  const cudaError_t st = dq::launch_lookahead(params, h->h + (int64_t)(i - h->row0) * h->ld, out_w_half, h->cfg.d,
                                               h->stream, &h->launches);
   if (st != cudaSuccess) return cuda_fail(h, st, "lookahead launch");
   return DQGAN_OK;
