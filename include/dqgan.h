@@ -318,7 +318,8 @@ DQGAN_API int dqgan_set_segments(dqgan_handle* h, const int64_t* offsets, int32_
  * rule; this is the rule of Daskalakis, Ilyas, Syrgkanis and Zeng, "Training
  * GANs with Optimism" (ICLR 2018).  Per parameter j, in fp32 with one
  * rounding per operation in this order (one dense pass after the server
- * kernel, which then writes q_hat to a library-owned buffer):
+ * kernel, which then writes q_hat to a library-owned buffer; in the server
+ * kernel itself with DQGAN_IDENTITY):
  *   m = b1 m + (1 - b1) q_hat;   v = b2 v + ((1 - b2) q_hat) q_hat;
  *   m_hat = m / (1 - b1^t), v_hat = v / (1 - b2^t)   (DQGAN_OADAM_BIAS_CORRECTION,
  *                                    b^t the fp32 product of t factors, t the step);

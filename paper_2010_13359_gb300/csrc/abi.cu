@@ -711,11 +711,16 @@ int dqgan_server_aggregate_update(dqgan_handle* h, const void* msgs_all, float* 
     case DQGAN_SIGN: st = dq::launch_sign_server(s, x, h->stream, &h->launches); break;
     case DQGAN_SQUANT:
     case DQGAN_QSGD: st = dq::launch_squant_server(s, x, h->stream, &h->launches); break;
-    case DQGAN_IDENTITY: st = dq::launch_identity_server(s, h->stream, &h->launches); break;
+    case DQGAN_IDENTITY: {
+      dq::OAdamArgs oa{};
+      if (oadam) oa = oadam_args(h, params);
+      st = dq::launch_identity_server(s, oadam ? &oa : nullptr, h->stream, &h->launches);
+      break;
+    }
     case DQGAN_TOPK: st = dq::launch_topk_server(s, h->scratch, h->nlocal, h->stream, &h->launches); break;
   }
   if (st != cudaSuccess) return cuda_fail(h, st, "server launch");
-  if (oadam) {
+  if (oadam && h->cfg.compressor != DQGAN_IDENTITY) {
     st = dq::launch_oadam_update(oadam_args(h, params), h->stream, &h->launches);
     if (st != cudaSuccess) return cuda_fail(h, st, "optimizer launch");
   }

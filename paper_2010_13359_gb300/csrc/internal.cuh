@@ -185,7 +185,8 @@ cudaError_t launch_sign_server(const ServerArgs& s, const SignServerExtras& x, c
 // runs of up to 32 (and the words map has 36-word boxes).
 cudaError_t launch_squant_server(const ServerArgs& s, const SignServerExtras& x, cudaStream_t stream,
                                  uint64_t* launches);
-cudaError_t launch_identity_server(const ServerArgs& s, cudaStream_t stream, uint64_t* launches);
+// oa: Optimistic Adam in the same pass (then s.w is not used), or nullptr.
+cudaError_t launch_identity_server(const ServerArgs& s, const OAdamArgs* oa, cudaStream_t stream, uint64_t* launches);
 // scratch: topk_scratch_bytes(d, k, rows, M); the server's table follows the rows.
 cudaError_t launch_topk_server(const ServerArgs& s, void* scratch, int32_t rows, cudaStream_t stream,
                                uint64_t* launches);

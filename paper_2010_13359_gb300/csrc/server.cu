@@ -39,7 +39,8 @@ __device__ __forceinline__ float average_t(float acc, const ServerArgs& s) {
 // Applies w_j = fl(w_j - acc_j / M) for the chunk at element j.
 __device__ __forceinline__ void apply_chunk(const ServerArgs& s, int64_t j, const float (&acc)[4]) {
   if (j + 3 < s.d) {
-    float4 wv = __ldcs(reinterpret_cast<const float4*>(s.w + j));
+    float4 wv = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (!s.store_q) wv = __ldcs(reinterpret_cast<const float4*>(s.w + j));
     wv.x = server_out(s, wv.x, average(acc[0], s));
     wv.y = server_out(s, wv.y, average(acc[1], s));
     wv.z = server_out(s, wv.z, average(acc[2], s));
@@ -245,7 +246,7 @@ __global__ void __launch_bounds__(256) sign_server_words_kernel(const ServerArgs
   const int64_t jmax = s.d - 32 * w0 - lane;  // wl[32 i] is a parameter iff 32 i < jmax
   float wv[kChunkWords];
 #pragma unroll
-  for (int k = 0; k < kChunkWords; ++k) wv[k] = (32 * k < jmax) ? __ldcs(wl + 32 * k) : 0.f;
+  for (int k = 0; k < kChunkWords; ++k) wv[k] = (32 * k < jmax && !s.store_q) ? __ldcs(wl + 32 * k) : 0.f;
   uint32_t bkt[WPB == 0 ? kChunkWords : 1];  // layer buckets: of each word (past the end: the last word's)
   if constexpr (WPB == 0) {
 #pragma unroll
@@ -1468,41 +1469,6 @@ squant_server_table_kernel(const ServerArgs s, const SegSlices seg, const __grid
     mbar_wait_bounded(&bar[(it & 1u) ^ 1u], ((it + 1) >> 1) & 1u, s.err);
 }
 
-// Identity: the messages are the p vectors themselves.
-template <int P8>
-__global__ void __launch_bounds__(256, 4) identity_server_kernel(const ServerArgs s) {
-  dq_pdl_enter();
-  const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t j = 4 * c;
-  if (j >= s.d) return;
-  const bool vec = j + 3 < s.d;
-  float sum[4];
-  worker_sum<P8>(
-      s.M,
-      [&](int m, float (&v)[8][4]) {
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          float4 x = make_float4(0.f, 0.f, 0.f, 0.f);  // +0 leaves past M and past d
-          if (m + u < s.M) {
-            const float* vals = reinterpret_cast<const float*>(s.msgs + (int64_t)(m + u) * s.msg_stride);
-            if (vec) {
-              x = __ldcs(reinterpret_cast<const float4*>(vals + j));
-            } else {
-              x.x = vals[j];
-              if (j + 1 < s.d) x.y = vals[j + 1];
-              if (j + 2 < s.d) x.z = vals[j + 2];
-            }
-          }
-          v[u][0] = x.x;
-          v[u][1] = x.y;
-          v[u][2] = x.z;
-          v[u][3] = x.w;
-        }
-      },
-      sum);
-  apply_chunk(s, j, sum);
-}
-
 __global__ void __launch_bounds__(256)
 lookahead_kernel(const float* __restrict__ w, const float* __restrict__ h, float* __restrict__ out,
                  int64_t d) {
@@ -1539,15 +1505,16 @@ __device__ __forceinline__ float oadam_element(const OAdamArgs& a, float q, floa
   return __fsub_rn(w, __fmul_rn(a.alpha, step));
 }
 
-__global__ void __launch_bounds__(256) oadam_update_kernel(const OAdamArgs a) {
-  dq_pdl_enter();
-  const int64_t j = 4 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
-  if (j + 3 < a.d) {
-    const float4 q = __ldcs(reinterpret_cast<const float4*>(a.q + j));
-    float4 m = __ldcs(reinterpret_cast<const float4*>(a.m + j));
-    float4 v = __ldcs(reinterpret_cast<const float4*>(a.v + j));
-    float4 u = __ldcs(reinterpret_cast<const float4*>(a.u + j));
-    float4 w = __ldcs(reinterpret_cast<const float4*>(a.w + j));
+// The state and parameters of four elements from j on, 16 bytes each.
+struct OAdamChunk {
+  float4 m, v, u, w;
+  __device__ __forceinline__ void load(const OAdamArgs& a, int64_t j) {
+    m = __ldcs(reinterpret_cast<const float4*>(a.m + j));
+    v = __ldcs(reinterpret_cast<const float4*>(a.v + j));
+    u = __ldcs(reinterpret_cast<const float4*>(a.u + j));
+    w = __ldcs(reinterpret_cast<const float4*>(a.w + j));
+  }
+  __device__ __forceinline__ void update(const OAdamArgs& a, int64_t j, float4 q) {
     w.x = oadam_element(a, q.x, m.x, v.x, u.x, w.x);
     w.y = oadam_element(a, q.y, m.y, v.y, u.y, w.y);
     w.z = oadam_element(a, q.z, m.z, v.z, u.z, w.z);
@@ -1556,8 +1523,68 @@ __global__ void __launch_bounds__(256) oadam_update_kernel(const OAdamArgs a) {
     __stcs(reinterpret_cast<float4*>(a.v + j), v);
     __stcs(reinterpret_cast<float4*>(a.u + j), u);
     __stcs(reinterpret_cast<float4*>(a.w + j), w);
+  }
+};
+
+__global__ void __launch_bounds__(256) oadam_update_kernel(const OAdamArgs a) {
+  dq_pdl_enter();
+  const int64_t j = 4 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
+  if (j + 3 < a.d) {
+    const float4 q = __ldcs(reinterpret_cast<const float4*>(a.q + j));
+    OAdamChunk c;
+    c.load(a, j);
+    c.update(a, j, q);
   } else {
     for (int64_t jj = j; jj < a.d; ++jj) a.w[jj] = oadam_element(a, a.q[jj], a.m[jj], a.v[jj], a.u[jj], a.w[jj]);
+  }
+}
+
+// Identity: the messages are the p vectors themselves.  OADAM: the update
+// rule follows in the same pass (s.w are the parameters then too), which
+// saves the averaged update's way through memory: 3.6M x 8, with its launch,
+// 46.9 us in two kernels, @@IDOA@@ in one.
+template <int P8, bool OADAM>
+__global__ void __launch_bounds__(256, OADAM ? 3 : 4) identity_server_kernel(const ServerArgs s, const OAdamArgs oa) {
+  dq_pdl_enter();
+  const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t j = 4 * c;
+  if (j >= s.d) return;
+  const bool vec = j + 3 < s.d;
+  OAdamChunk state;
+  if constexpr (OADAM)
+    if (vec) state.load(oa, j);
+  float sum[4];
+  worker_sum<P8>(
+      s.M,
+      [&](int m, float (&v)[8][4]) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          float4 x = make_float4(0.f, 0.f, 0.f, 0.f);  // +0 leaves past M and past d
+          if (m + u < s.M) {
+            const float* vals = reinterpret_cast<const float*>(s.msgs + (int64_t)(m + u) * s.msg_stride);
+            if (vec) {
+              x = __ldcs(reinterpret_cast<const float4*>(vals + j));
+            } else {
+              x.x = vals[j];
+              if (j + 1 < s.d) x.y = vals[j + 1];
+              if (j + 2 < s.d) x.z = vals[j + 2];
+            }
+          }
+          v[u][0] = x.x;
+          v[u][1] = x.y;
+          v[u][2] = x.z;
+          v[u][3] = x.w;
+        }
+      },
+      sum);
+  if constexpr (!OADAM) {
+    apply_chunk(s, j, sum);
+  } else if (vec) {
+    state.update(oa, j, make_float4(average(sum[0], s), average(sum[1], s), average(sum[2], s), average(sum[3], s)));
+  } else {
+#pragma unroll
+    for (int q = 0; q < 3; ++q)
+      if (j + q < s.d) oa.w[j + q] = oadam_element(oa, average(sum[q], s), oa.m[j + q], oa.v[j + q], oa.u[j + q], oa.w[j + q]);
   }
 }
 
@@ -1842,16 +1869,20 @@ cudaError_t launch_squant_server(const ServerArgs& s, const SignServerExtras& x,
   return st;
 }
 
-cudaError_t launch_identity_server(const ServerArgs& s, cudaStream_t stream, uint64_t* launches) {
-  auto go = [&](auto kernel) { return launch_pdl(kernel, dim3(chunk_blocks(s.d, 256)), dim3(256), 0, stream, s); };
-  cudaError_t st;
+template <bool OADAM>
+static cudaError_t launch_identity(const ServerArgs& s, const OAdamArgs& oa, cudaStream_t stream) {
+  auto go = [&](auto kernel) { return launch_pdl(kernel, dim3(chunk_blocks(s.d, 256)), dim3(256), 0, stream, s, oa); };
   switch (eights_of(s.M)) {
-    case 1: st = go(identity_server_kernel<1>); break;
-    case 2: st = go(identity_server_kernel<2>); break;
-    case 4: st = go(identity_server_kernel<4>); break;
-    case 8: st = go(identity_server_kernel<8>); break;
-    default: st = go(identity_server_kernel<0>); break;
+    case 1: return go(identity_server_kernel<1, OADAM>);
+    case 2: return go(identity_server_kernel<2, OADAM>);
+    case 4: return go(identity_server_kernel<4, OADAM>);
+    case 8: return go(identity_server_kernel<8, OADAM>);
+    default: return go(identity_server_kernel<0, OADAM>);
   }
+}
+
+cudaError_t launch_identity_server(const ServerArgs& s, const OAdamArgs* oa, cudaStream_t stream, uint64_t* launches) {
+  const cudaError_t st = oa ? launch_identity<true>(s, *oa, stream) : launch_identity<false>(s, OAdamArgs{}, stream);
   *launches += 1;
   return st;
 }

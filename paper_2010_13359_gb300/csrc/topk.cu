@@ -1138,42 +1138,61 @@ __global__ void __launch_bounds__(kChipThreads, 1) topk_chip_kernel(const Compre
 }
 
 // ---------------------------------------------------------------------------
-// Server.  starts[m][t] = first record of worker m whose index is in tile t
-// or later (t in [0, nts]); record r writes the tiles (tile(r-1), tile(r)],
-// and the last record also (tile(k-1), nts].
+// Server.  starts[m][t] = first record of worker m whose index is in run t
+// of kSrvTile indices or later (t in [0, nts]); record r writes the runs
+// (run(r-1), run(r)], and the last record also (run(k-1), nts].  A thread takes
+// kStartsPer consecutive records (16-byte loads; @@STARTS@@).
 // ---------------------------------------------------------------------------
+constexpr int kStartsPer = 4;
+
 __global__ void __launch_bounds__(256) topk_server_starts_kernel(const ServerArgs s, uint32_t* starts) {
   dq_pdl_enter();
   const int m = blockIdx.y;
-  const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t r0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * kStartsPer;
   const int lane = threadIdx.x & 31;
   const int64_t nts = srv_tiles(s.d);
   const uint2* msg = reinterpret_cast<const uint2*>(s.msgs + (int64_t)m * s.msg_stride);
   uint32_t* st = starts + (int64_t)m * (nts + 1);
-  // this record fills the tiles [t_a, t_b] with r (empty range: t_a > t_b)
-  int64_t t_a = 1, t_b = 0;
-  if (r < s.k) {
-    const int64_t tile = min64(msg[r].x / kSrvTile, nts - 1);
-    const int64_t prev = (r == 0) ? -1 : min64(msg[r - 1].x / kSrvTile, nts - 1);
-    t_a = prev + 1;
-    t_b = tile;
+  // the runs of this thread's records (past the end: the last record's)
+  int64_t run[kStartsPer];
+  if (r0 + kStartsPer <= s.k) {
+    static_assert(kStartsPer == 4, "two loads of two records");
+    const uint4 a = __ldg(reinterpret_cast<const uint4*>(msg + r0)), b = __ldg(reinterpret_cast<const uint4*>(msg + r0 + 2));
+    run[0] = a.x / kSrvTile;
+    run[1] = a.z / kSrvTile;
+    run[2] = b.x / kSrvTile;
+    run[3] = b.z / kSrvTile;
+  } else {
+#pragma unroll
+    for (int q = 0; q < kStartsPer; ++q) run[q] = msg[min64(r0 + q, s.k - 1)].x / kSrvTile;
   }
-  for (int64_t t = t_a; t <= t_b && t < t_a + 32; ++t) st[t] = (uint32_t)r;
-  // long runs (sparse stretches of the index range) are written by the whole warp
-  uint32_t longs = __ballot_sync(kFullMask, t_b - t_a >= 32);
-  while (longs) {
-    const int src = __ffs(longs) - 1;
-    longs &= longs - 1;
-    const int64_t a = __shfl_sync(kFullMask, t_a, src), bnd = __shfl_sync(kFullMask, t_b, src);
-    const uint32_t val = (uint32_t)__shfl_sync(kFullMask, r, src);
-    for (int64_t t = a + 32 + lane; t <= bnd; t += 32) st[t] = val;
-  }
-  // after the last record: the tiles up to nts point past the end
-  const uint32_t last = __ballot_sync(kFullMask, r == s.k - 1);
-  if (last) {
-    const int src = __ffs(last) - 1;
-    const int64_t a = __shfl_sync(kFullMask, t_b, src) + 1;
-    for (int64_t t = a + lane; t <= nts; t += 32) st[t] = (uint32_t)s.k;
+#pragma unroll
+  for (int q = 0; q < kStartsPer; ++q) run[q] = min64(run[q], nts - 1);
+  // the run before this thread's first record
+  int64_t prev = __shfl_up_sync(kFullMask, run[kStartsPer - 1], 1);
+  if (lane == 0) prev = r0 == 0 ? -1 : min64(msg[min64(r0, s.k) - 1].x / kSrvTile, nts - 1);
+#pragma unroll
+  for (int q = 0; q < kStartsPer; ++q) {
+    // this record fills the runs (prev, run] with its number
+    const int64_t r = r0 + q;
+    const int64_t t_a = prev + 1, t_b = r < s.k ? run[q] : prev;
+    for (int64_t t = t_a; t <= t_b && t < t_a + 32; ++t) st[t] = (uint32_t)r;
+    // long stretches without records are written by the whole warp
+    uint32_t longs = __ballot_sync(kFullMask, t_b - t_a >= 32);
+    while (longs) {
+      const int src = __ffs(longs) - 1;
+      longs &= longs - 1;
+      const int64_t a = __shfl_sync(kFullMask, t_a, src), bnd = __shfl_sync(kFullMask, t_b, src);
+      const uint32_t val = (uint32_t)__shfl_sync(kFullMask, r, src);
+      for (int64_t t = a + 32 + lane; t <= bnd; t += 32) st[t] = val;
+    }
+    // after the last record: the runs up to nts point past the end
+    const uint32_t last = __ballot_sync(kFullMask, r == s.k - 1);
+    if (last) {
+      const int64_t a = __shfl_sync(kFullMask, t_b, __ffs(last) - 1) + 1;
+      for (int64_t t = a + lane; t <= nts; t += 32) st[t] = (uint32_t)s.k;
+    }
+    prev = run[q];
   }
 }
 
@@ -1710,7 +1729,7 @@ cudaError_t launch_topk_server(const ServerArgs& s, void* scratch, int32_t rows,
     if (st != cudaSuccess) return st;
   }
   uint32_t* starts = reinterpret_cast<uint32_t*>(scratch) + row_words(s.d) * rows;
-  const dim3 starts_grid((unsigned)((s.k + 255) / 256), (unsigned)s.M);
+  const dim3 starts_grid((unsigned)((s.k + 256 * kStartsPer - 1) / (256 * kStartsPer)), (unsigned)s.M);
   if (tile_server(s.d, s.k, s.M)) {
     cudaError_t st = launch_pdl(topk_server_starts_kernel, starts_grid, dim3(256), 0, stream, s, starts);
     if (st != cudaSuccess) return st;

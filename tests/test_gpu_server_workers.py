@@ -68,6 +68,28 @@ def test_identity(P, M):
     run(P, oracle.IDENTITY, M)
 
 
+@pytest.mark.parametrize("M", [1, 3, 8, 17, 33, 65])
+def test_identity_with_optimistic_adam(P, M):
+    """Two steps of the pass that sums and updates, a vector that ends inside a chunk."""
+    params = dict(alpha=1e-2, beta1=0.5, beta2=0.9, eps=1e-8)
+    ocfg = oracle_config(D, M, oracle.IDENTITY, lr=0.03)
+    h = P.create(P.make_config(d=D, M=M, compressor=P.IDENTITY, lr=0.03,
+                               cuda_stream=torch.cuda.current_stream().cuda_stream))
+    h.set_server_optimizer(P.dqgan.oadam(**params))
+    rng = np.random.default_rng(M)
+    w = (rng.standard_normal(D) * 0.02).astype(np.float32)
+    w_gpu = torch.from_numpy(w.copy()).to("cuda")
+    state = oracle.OAdamState(D, oracle.OAdam(**params))
+    for step in range(1, 3):
+        msgs = np.zeros((M, h.message_bytes()), np.uint8)
+        msgs[:, :4 * D] = rng.standard_normal((M, D)).astype(np.float32).view(np.uint8)
+        h.server_aggregate_update(torch.from_numpy(msgs).to("cuda"), w_gpu)
+        state.server_step_range(ocfg, step, msgs, w, 0, D)
+        h.synchronize()
+        assert_params_equal(w_gpu.cpu().numpy(), w)
+    h.destroy()
+
+
 @pytest.mark.parametrize("segments", [None, SEGMENTS], ids=["flat", "layers"])
 @pytest.mark.parametrize("bits", [2, 4, 8])
 @pytest.mark.parametrize("M", [*WORKERS, 129])
