@@ -1046,15 +1046,24 @@ __global__ void __launch_bounds__(kChipThreads, 1) topk_chip_kernel(const Compre
       const int j = j0 + 4 * i * kChipThreads;
       float v[4];
       if (j + 3 < d) {
-        v[0] = ef_p(a.lr, gv[i].x, ev[i].x);
-        v[1] = ef_p(a.lr, gv[i].y, ev[i].y);
-        v[2] = ef_p(a.lr, gv[i].z, ev[i].z);
-        v[3] = ef_p(a.lr, gv[i].w, ev[i].w);
+        const float sg[4] = {__fmul_rn(a.lr, gv[i].x), __fmul_rn(a.lr, gv[i].y), __fmul_rn(a.lr, gv[i].z),
+                             __fmul_rn(a.lr, gv[i].w)};
+        v[0] = __fadd_rn(sg[0], ev[i].x);
+        v[1] = __fadd_rn(sg[1], ev[i].y);
+        v[2] = __fadd_rn(sg[2], ev[i].z);
+        v[3] = __fadd_rn(sg[3], ev[i].w);
         *reinterpret_cast<float4*>(p + j) = make_float4(v[0], v[1], v[2], v[3]);
+        if constexpr (KEEP_H)  // as if nothing were kept
+          *reinterpret_cast<float4*>(h + j) = make_float4(__fadd_rn(sg[0], v[0]), __fadd_rn(sg[1], v[1]),
+                                                          __fadd_rn(sg[2], v[2]), __fadd_rn(sg[3], v[3]));
       } else {
 #pragma unroll
         for (int q = 0; q < 4; ++q)
-          if (j + q < d) p[j + q] = v[q] = ef_p(a.lr, g[j + q], e[j + q]);
+          if (j + q < d) {
+            const float sg = __fmul_rn(a.lr, g[j + q]);
+            p[j + q] = v[q] = __fadd_rn(sg, e[j + q]);
+            if constexpr (KEEP_H) h[j + q] = __fadd_rn(sg, v[q]);
+          }
       }
 #pragma unroll
       for (int q = 0; q < 4; ++q)
@@ -1129,7 +1138,8 @@ __global__ void __launch_bounds__(kChipThreads, 1) topk_chip_kernel(const Compre
       }
       const float en = kept ? __fsub_rn(v, v) : v;
       e[j] = en;
-      if constexpr (KEEP_H) h[j] = __fadd_rn(__fmul_rn(a.lr, g[j]), en);
+      if constexpr (KEEP_H)
+        if (kept) h[j] = __fadd_rn(__fmul_rn(a.lr, g[j]), en);
     }
     gt += __popc(gts);
     eq += __popc(eqs);
@@ -1141,7 +1151,7 @@ __global__ void __launch_bounds__(kChipThreads, 1) topk_chip_kernel(const Compre
 // Server.  starts[m][t] = first record of worker m whose index is in run t
 // of kSrvTile indices or later (t in [0, nts]); record r writes the runs
 // (run(r-1), run(r)], and the last record also (run(k-1), nts].  A thread takes
-// kStartsPer consecutive records (16-byte loads; @@STARTS@@).
+// kStartsPer consecutive records (25M x 16, k = d / 100: 22 us with one).
 // ---------------------------------------------------------------------------
 constexpr int kStartsPer = 4;
 
