@@ -9,7 +9,7 @@
 //
 // Small problems (chip_ctas): one kernel, 1, 8 or 16 CTAs per worker that keep
 // p on chip.  Large ones: five kernels, one pass over the dense vectors:
-//   1. sample (8 blocks per worker): p at 65,536 elements spread over the
+//   1. sample (16 blocks per worker): p at 65,536 elements spread over the
 //      vector; tau, a key that rather more than k of the d keys reach (1.3 k
 //      for k = d / 100), is read off their ranks.
 //   2. form (tiles of 4096 elements): p, h (optional), and the tile's
@@ -70,8 +70,8 @@ constexpr int kGroup = 64;                                    // bins per coarse
 constexpr int kChipMax = 49152;                               // parameters of a part, at most
 constexpr int kStateWords = 64;
 constexpr int kFirst = 4, kBatch = 8;                         // rows of 32 candidates a warp loads at once
-constexpr int kSampBlocks = 8;                                // sample blocks per worker
-constexpr int kSampThreads = 512;
+constexpr int kSampBlocks = 16;                               // sample blocks per worker
+constexpr int kSampThreads = 256;
 constexpr int kSampRuns = 8192;                               // sampled runs of 8 elements
 constexpr int kSamples = 8 * kSampRuns;
 constexpr int kSampBits = 14;                                 // key bits a block's estimate is resolved to
@@ -145,11 +145,13 @@ __device__ __forceinline__ RowScratch row_scratch(void* base, int64_t d, int row
 }
 
 __device__ __forceinline__ uint32_t key_of(float v) { return __float_as_uint(v) & 0x7FFFFFFFu; }
-// tau of the call under way: the mean of the sample blocks' estimates.
+// tau of the call under way: the mean of the sample blocks' estimates, one to
+// a lane (the form kernel has no registers for all of them in every thread).
+// All lanes of a warp call it together.
 __device__ __forceinline__ uint32_t call_tau(const uint32_t* state) {
-  static_assert(kSampBlocks == 8 && ST_TAU == 0, "two loads of four estimates, an eighth of each");
-  const uint4 a = __ldcg(reinterpret_cast<const uint4*>(state)), b = __ldcg(reinterpret_cast<const uint4*>(state) + 1);
-  return (a.x >> 3) + (a.y >> 3) + (a.z >> 3) + (a.w >> 3) + (b.x >> 3) + (b.y >> 3) + (b.z >> 3) + (b.w >> 3);
+  static_assert(kSampBlocks == 16 && ST_TAU == 0, "a sixteenth of each");
+  const uint32_t lane = threadIdx.x & 31;
+  return __reduce_add_sync(kFullMask, lane < (uint32_t)kSampBlocks ? __ldcg(state + lane) >> 4 : 0u);
 }
 __device__ __forceinline__ uint32_t key_bits(uint32_t bits) { return bits & 0x7FFFFFFFu; }
 
@@ -240,9 +242,9 @@ __device__ __forceinline__ uint32_t first_bin(uint32_t key, uint32_t tau) {
 // 1. tau from a sample.  The vector's whole 8-element runs are cut into
 // kSampRuns equal strata, and one run of each is read, at a place in the
 // stratum that a multiplicative hash picks (so that no period of the vector
-// lines up with the sample).  Block b of a worker takes the strata b, b + 8,
+// lines up with the sample).  Block b of a worker takes the strata b, b + 16,
 // ... and writes the largest key of kSampBits leading bits that at least
-// `rank` of its samples reach.  The caller's rank is an eighth of the expected
+// `rank` of its samples reach.  The caller's rank is a sixteenth of the expected
 // one of the k-th largest key, r = k kSamples / d, plus seven standard
 // deviations sqrt(r) of a binomial count (2.5, when the eight elements of a
 // run are always large together); tau is the mean of the blocks' estimates, which varies
@@ -251,12 +253,15 @@ __device__ __forceinline__ uint32_t first_bin(uint32_t key, uint32_t tau) {
 // that counts here: 8 loads of 16 bytes in flight per thread, then a bisection
 // over samples in registers.  The blocks also clear the row's counts.  They
 // let the form kernel start at once: it loads its first tiles meanwhile.
+// 16 blocks of 256 threads, with the warps' counts in words of their own, take
+// 8.4 us for 8 workers; 8 blocks of 512 with one shared counter took 10.8.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(kSampThreads) topk_sample_kernel(const CompressArgs a, uint32_t rank, void* scratch) {
   dq_pdl_enter();
   dq_pdl_release();
   constexpr int kHalves = 2 * kSampRuns / kSampBlocks / kSampThreads;  // half runs (float4) per thread
-  __shared__ uint32_t count[kSampBits];
+  constexpr int kWarps = kSampThreads / 32;
+  __shared__ __align__(16) uint32_t count[kSampBits][kWarps];
   const int row = blockIdx.y;
   const int worker = a.worker0 + row;
   const float* g = a.g + (int64_t)row * a.g_stride;
@@ -269,7 +274,6 @@ __global__ void __launch_bounds__(kSampThreads) topk_sample_kernel(const Compres
     if (threadIdx.x == 0) rs.state[ST_TAU + blockIdx.x] = 0;
     return;
   }
-  if (threadIdx.x < kSampBits) count[threadIdx.x] = 0;
   const int64_t runs = a.d >> 3;  // >= kSampRuns
   float4 gv[kHalves], ev[kHalves];
 #pragma unroll
@@ -289,7 +293,6 @@ __global__ void __launch_bounds__(kSampThreads) topk_sample_kernel(const Compres
     key[i][2] = key_of(ef_p(a.lr, gv[i].z, ev[i].z));
     key[i][3] = key_of(ef_p(a.lr, gv[i].w, ev[i].w));
   }
-  __syncthreads();
   uint32_t tau = 0;
 #pragma unroll 1
   for (int it = 0; it < kSampBits; ++it) {
@@ -300,9 +303,12 @@ __global__ void __launch_bounds__(kSampThreads) topk_sample_kernel(const Compres
 #pragma unroll
       for (int q = 0; q < 4; ++q) n += key[i][q] >= trial ? 1u : 0u;
     n = __reduce_add_sync(kFullMask, n);
-    if ((threadIdx.x & 31) == 0) atomicAdd(&count[it], n);
+    if ((threadIdx.x & 31) == 0) count[it][threadIdx.x >> 5] = n;
     __syncthreads();
-    if (count[it] >= rank) tau = trial;
+    n = 0;
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) n += count[it][w];
+    if (n >= rank) tau = trial;
   }
   if (threadIdx.x == 0) rs.state[ST_TAU + blockIdx.x] = tau;
 }
