@@ -203,8 +203,8 @@ __device__ __forceinline__ float server_out(const ServerArgs& s, float w, float 
 // programmatic-stream-serialization attribute, so that a kernel is scheduled
 // as the blocks of the kernel before it in the stream exit, instead of after
 // the whole grid has drained.  Each kernel first waits for that grid to
-// complete (its writes visible); it reads and writes nothing before the
-// wait (one exception, which states why: the top-k form kernel).  No kernel
+// complete (its writes visible); it reads and writes no memory before the
+// wait, so that no kernel needs to know which one precedes it.  No kernel
 // that fills the GPU triggers its dependents early: that let the next grid's
 // blocks sit waiting on the SMs, and measured up to a third slower per step
 // (compress and server alternating on the 25M-parameter workload) against
