@@ -25,11 +25,16 @@
 //      the number kept); a candidate that is not kept gets its e_j = p_j (and
 //      h_j) back.
 // With k candidates or more T >= tau, so every key >= T was a candidate and T
-// is exact.  With fewer (the sample sat where p is larger than elsewhere)
-// steps 4 and 5 put e back, take the candidates again from the top digits of
-// all of p, and select among those.  tau only decides how much work the first
-// pass saves; the result is the same bit for bit.  Nothing carries over from
-// call to call.
+// is exact.  With fewer, either p has fewer than k non-zero entries (tau is
+// then 1 and they are the candidates: T is 0, and the first zeros fill the
+// records), or the sample sat where p is larger than elsewhere: then every
+// element becomes a candidate.  tau only decides how much work the first pass
+// saves; the result is the same bit for bit.  Nothing carries over from call
+// to call.
+//   Sparse gradients are ordinary input (frozen layers, rows nobody looked
+// up).  With tau = 0 for them and one CTA per worker for what the list does not
+// hold, 3.6M x 8, k = d / 100, k / 2 non-zero entries took 9.6 ms, 1.1 k 199 us;
+// now 139 and 79 (25M x 16: 64.8 ms and 2.19 ms; now 794 and 776 us).
 //
 // Server: w_j -= (sum over workers of the value recorded for j, absent
 // workers as +0, in the library's pairwise order) / M at the indices some
@@ -63,7 +68,6 @@ constexpr int kSelWarps = kSelThreads / 32;
 constexpr int kFineShift = 12, kFineBins = 1792;              // bins of 4096 keys from tau up (7/8 of a binade)
 constexpr int kBins = kFineBins + 256;                        // first round: then one bin per exponent
 constexpr int kBins2 = 1 << kFineShift;                       // second round
-constexpr int kTopBins = 2048;                                // bins of 2^20 keys
 constexpr int kMaxGroups = 8192;                              // groups of tiles per worker, at most
 constexpr int kChipThreads = 1024;                            // CTAs that keep their part of p on chip
 constexpr int kGroup = 64;                                    // bins per coarse count
@@ -82,15 +86,16 @@ constexpr int kSrvThreads = 256;
 // what one step of a call leaves for the next.
 enum : int {
   ST_TAU = 0,
-  ST_TICKET = kSampBlocks,    // finished CTAs of steps 4 and 5
-  ST_LISTED = ST_TICKET + 2,  // keys of T's bin put into the list so far
-  ST_PLACED,                  // step 4 finds T and the groups' places as well
-  ST_SHORT,                   // too few candidates
+  ST_LISTED = kSampBlocks,    // keys of T's bin put into the list so far
+  ST_ROUTE,                   // how step 5 goes on
   ST_BIN,                     // T's first-round bin
-  ST_REST,                    // k less the keys above it
-  ST_T,
-  ST_NEED,                    // keys equal to T that are kept
-  ST_TAU2                     // tau of a row with too few candidates
+  ST_REST                     // k less the keys above it (ROUTE_ZERO: less the candidates)
+};
+enum : uint32_t {
+  ROUTE_LIST = 0,   // T's bin is listed: every CTA finds T by itself
+  ROUTE_BIN = 1,    // it holds too many keys: a cluster reads the candidates again
+  ROUTE_SHORT = 2,  // there were too few candidates: every element is one now
+  ROUTE_ZERO = 3    // the candidates are all non-zero keys, and fewer than k: T is 0
 };
 
 __host__ __device__ constexpr int64_t tiles_of(int64_t d) { return (d + kTile - 1) / kTile; }
@@ -146,12 +151,15 @@ __device__ __forceinline__ RowScratch row_scratch(void* base, int64_t d, int row
 
 __device__ __forceinline__ uint32_t key_of(float v) { return __float_as_uint(v) & 0x7FFFFFFFu; }
 // tau of the call under way: the mean of the sample blocks' estimates, one to
-// a lane (the form kernel has no registers for all of them in every thread).
+// a lane (the form kernel has no registers for all of them in every thread);
+// 1, every non-zero key, where a block found too few of them for an estimate.
 // All lanes of a warp call it together.
 __device__ __forceinline__ uint32_t call_tau(const uint32_t* state) {
   static_assert(kSampBlocks == 16 && ST_TAU == 0, "a sixteenth of each");
   const uint32_t lane = threadIdx.x & 31;
-  return __reduce_add_sync(kFullMask, lane < (uint32_t)kSampBlocks ? __ldcg(state + lane) >> 4 : 0u);
+  const uint32_t own = lane < (uint32_t)kSampBlocks ? __ldcg(state + lane) : ~0u;
+  const uint32_t mean = __reduce_add_sync(kFullMask, lane < (uint32_t)kSampBlocks ? own >> 4 : 0u);
+  return __any_sync(kFullMask, own == 0u) ? 1u : mean;
 }
 __device__ __forceinline__ uint32_t key_bits(uint32_t bits) { return bits & 0x7FFFFFFFu; }
 
@@ -178,56 +186,6 @@ __device__ __forceinline__ T block_exclusive_scan(T v, T* total, T* warp_sums) {
   __syncthreads();
   *total = sum;
   return before + x - v;
-}
-
-// Writes one tile's flagged elements to its candidate slot in index order.
-// Element order in the tile: thread t, component q is tile offset 4 (i NT + t)
-// + q for row i < R.  Per lane and row at most 4 flags, per warp and row at
-// most 128, so the R <= 4 row counts share one 32-bit warp scan (8 bits
-// each).  `totals` is shared memory of NT/32 words.  Returns the tile's
-// count (in every thread); two barriers.
-template <int NT, int R>
-__device__ __forceinline__ uint32_t write_tile_candidates(const float (&v)[R][4], const uint32_t (&cmask)[R],
-                                                          int64_t tile0, uint2* slot, uint32_t* totals,
-                                                          uint32_t* err) {
-  static_assert(R <= 4, "four 8-bit row counts per word");
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  uint32_t packed = 0;
-#pragma unroll
-  for (int i = 0; i < R; ++i) packed |= (uint32_t)__popc(cmask[i]) << (8 * i);
-  uint32_t incl = packed;
-#pragma unroll
-  for (int off = 1; off < 32; off <<= 1) {
-    const uint32_t y = __shfl_up_sync(kFullMask, incl, off);
-    if (lane >= off) incl += y;
-  }
-  const uint32_t excl = incl - packed;
-  if (lane == 31) totals[warp] = incl;
-  __syncthreads();
-  uint32_t done = 0;
-#pragma unroll
-  for (int i = 0; i < R; ++i) {
-    uint32_t row_before = 0, row_total = 0;
-#pragma unroll
-    for (int w = 0; w < NT / 32; ++w) {
-      const uint32_t f = (totals[w] >> (8 * i)) & 0xFFu;
-      if (w < warp) row_before += f;
-      row_total += f;
-    }
-    uint32_t pos = done + row_before + ((excl >> (8 * i)) & 0xFFu);
-    done += row_total;
-    if (cmask[i]) {
-      const int64_t j = tile0 + 4 * ((int64_t)i * NT + threadIdx.x);
-#pragma unroll
-      for (int q = 0; q < 4; ++q)
-        if ((cmask[i] >> q) & 1u) {
-          if (dq_in_bounds(pos < (uint32_t)kTile, err)) slot[pos] = make_uint2((uint32_t)(j + q), __float_as_uint(v[i][q]));
-          ++pos;
-        }
-    }
-  }
-  __syncthreads();
-  return done;
 }
 
 // First-round bin of a candidate: 1792 bins of 4096 keys from tau up, then
@@ -271,8 +229,7 @@ __global__ void __launch_bounds__(kSampThreads) topk_sample_kernel(const Compres
   const float* e = a.e + (int64_t)(worker - a.row0) * a.ld;
   const RowScratch rs = row_scratch(scratch, a.d, worker - a.row0);
   for (int i = blockIdx.x * kSampThreads + threadIdx.x; i < kHistWords; i += kSampBlocks * kSampThreads) rs.hist[i] = 0;
-  if (blockIdx.x == 0 && threadIdx.x < 3) rs.state[ST_TICKET + threadIdx.x] = 0;
-  static_assert(ST_LISTED == ST_TICKET + 2, "three counters");
+  if (blockIdx.x == 0 && threadIdx.x == 0) rs.state[ST_LISTED] = 0;
   if (rank == 0) {
     if (threadIdx.x == 0) rs.state[ST_TAU + blockIdx.x] = 0;
     return;
@@ -466,14 +423,15 @@ struct SelectTask {
   int rows;           // rows of 32 candidates of a tile worth loading before its count is known
 };
 
-__device__ __forceinline__ SelectTask select_task(const CompressArgs& a, int64_t k, int rows, void* scratch) {
-  const int row = blockIdx.y;
+// The CTA that is the `slot`-th of `ctas` that share row `row`.
+__device__ __forceinline__ SelectTask select_task(const CompressArgs& a, int64_t k, int rows, void* scratch, int row,
+                                                  int slot, int ctas) {
   const int worker = a.worker0 + row;
   const int64_t at = (int64_t)(worker - a.row0) * a.ld;
   return SelectTask{a, row_scratch(scratch, a.d, worker - a.row0), k, tiles_of(a.d), groups_of(a.d), group_shift(a.d),
                     a.e + at, a.h ? a.h + at : nullptr, a.g + (int64_t)row * a.g_stride,
                     reinterpret_cast<uint2*>(a.msg + (int64_t)row * a.msg_stride),
-                    (int)blockIdx.x * kSelWarps + (int)(threadIdx.x >> 5), (int)gridDim.x * kSelWarps, rows};
+                    slot * kSelWarps + (int)(threadIdx.x >> 5), ctas * kSelWarps, rows};
 }
 
 // A tile's count and first rows of 32 candidates, loaded together (a slot has
@@ -543,32 +501,27 @@ struct SelectSmem {
   uint64_t scan[NT / 32];
   uint32_t warp_sums[NT / 32];
   uint32_t found[3];
-  uint32_t ticket;
+  uint32_t list_at;
   uint32_t listed;
   uint2 list[NT == kSelThreads ? kOwnList : 1];
 };
 
 // The bin b of BINS counts with count(> b) < k_rem <= count(>= b), k_rem -
 // count(> b) and count(b), in sm.found (as they were when there are fewer).
-// Returns the sum of all counts.  GLOBAL: counts other CTAs have added to.
-template <int NT, int BINS, bool GLOBAL>
-__device__ __forceinline__ uint32_t find_bin(SelectSmem<NT>& sm, const uint32_t* counts, uint32_t k_rem) {
+// Returns the sum of all counts.  load(i): the counts i .. i + 3.
+template <int NT, int BINS, typename Load>
+__device__ __forceinline__ uint32_t find_bin(SelectSmem<NT>& sm, uint32_t k_rem, Load&& load) {
   constexpr int kPer = BINS / NT;  // bins per thread, from the top down
-  static_assert(kPer * NT == BINS, "whole bins per thread");
+  static_assert(kPer * NT == BINS && kPer % 4 == 0, "whole bins per thread, four at a time");
   const int first = BINS - ((int)threadIdx.x + 1) * kPer;
   uint32_t cnt[kPer], sum = 0;
-  if constexpr (GLOBAL && kPer % 4 == 0) {
 #pragma unroll
-    for (int q = 0; q < kPer; q += 4) {
-      const uint4 x = __ldcg(reinterpret_cast<const uint4*>(counts + first + q));
-      cnt[q] = x.x;
-      cnt[q + 1] = x.y;
-      cnt[q + 2] = x.z;
-      cnt[q + 3] = x.w;
-    }
-  } else {
-#pragma unroll
-    for (int q = 0; q < kPer; ++q) cnt[q] = GLOBAL ? __ldcg(counts + first + q) : counts[first + q];
+  for (int q = 0; q < kPer; q += 4) {
+    const uint4 x = load(first + q);
+    cnt[q] = x.x;
+    cnt[q + 1] = x.y;
+    cnt[q + 2] = x.z;
+    cnt[q + 3] = x.w;
   }
 #pragma unroll
   for (int q = 0; q < kPer; ++q) sum += cnt[q];
@@ -587,22 +540,23 @@ __device__ __forceinline__ uint32_t find_bin(SelectSmem<NT>& sm, const uint32_t*
   return total;
 }
 
+// Counts that other CTAs' finished grid added to.
+struct RowCounts {
+  const uint32_t* counts;
+  __device__ __forceinline__ uint4 operator()(int i) const {
+    return __ldcg(reinterpret_cast<const uint4*>(counts + i));
+  }
+};
+// This CTA's own counts.
+struct OwnCounts {
+  const uint32_t* counts;
+  __device__ __forceinline__ uint4 operator()(int i) const { return *reinterpret_cast<const uint4*>(counts + i); }
+};
+
 template <int NT>
 __device__ __forceinline__ void clear_hist(SelectSmem<NT>& sm, int bins) {
   for (int i = threadIdx.x; i < bins; i += NT) sm.hist[i] = 0;
   __syncthreads();
-}
-
-// Whether every CTA of the row has come here: told to all threads of the one
-// that comes last, which then sees what the others wrote before.
-__device__ __forceinline__ bool last_of_row(SelectSmem<kSelThreads>& sm, uint32_t* ticket) {
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) sm.ticket = atomicAdd(ticket, 1u);
-  __syncthreads();
-  const bool last = sm.ticket == gridDim.x - 1;
-  if (last) __threadfence();
-  return last;
 }
 
 __device__ __forceinline__ void add_hist(const SelectSmem<kSelThreads>& sm, uint32_t* row_hist, int bins) {
@@ -613,8 +567,10 @@ __device__ __forceinline__ void add_hist(const SelectSmem<kSelThreads>& sm, uint
   }
 }
 
-// e_j = p_j (and h_j) again at a candidate that is not kept.
+// e_j = p_j (and h_j) again at a candidate that is not kept (p_j = +0: they
+// hold it already).
 __device__ __forceinline__ void put_back(const SelectTask& s, uint2 c) {
+  if (c.y == 0) return;
   const float p = __uint_as_float(c.y);
   s.e[c.x] = p;
   if (s.h) s.h[c.x] = __fadd_rn(__fmul_rn(s.a.lr, s.g[c.x]), p);
@@ -644,12 +600,15 @@ __device__ __forceinline__ void count_second(SelectSmem<kSelThreads>& sm, const 
         const uint32_t b = first_bin(key, tau);
         above += valid && b > bin ? 1u : 0u;
         const bool in = valid && b == bin;
-        if (in) {  // rare: about one candidate in 500
-          atomicAdd(&sm.hist[(fine ? key - tau : key >> 11) & (kBins2 - 1)], 1u);
+        const uint32_t who = __ballot_sync(kFullMask, in);
+        if (who) {  // about one candidate in 500
+          if (in) atomicAdd(&sm.hist[(fine ? key - tau : key >> 11) & (kBins2 - 1)], 1u);
           if (listing) {
-            const uint32_t at = atomicAdd(&sm.listed, 1u);
-            if (at < (uint32_t)kOwnList) sm.list[at] = make_uint2(in_group, key);
-            else put_on_list(s, make_uint2(in_group, key));
+            uint32_t at = 0;
+            if (lane == 0) at = atomicAdd(&sm.listed, (uint32_t)__popc(who));
+            at = __shfl_sync(kFullMask, at, 0) + __popc(who & ((1u << lane) - 1u));
+            if (in && at < (uint32_t)kOwnList) sm.list[at] = make_uint2(in_group, key);
+            else if (in) put_on_list(s, make_uint2(in_group, key));
           }
         }
       },
@@ -660,11 +619,11 @@ __device__ __forceinline__ void count_second(SelectSmem<kSelThreads>& sm, const 
   __syncthreads();
   const uint32_t own = min(sm.listed, (uint32_t)kOwnList);
   if (!own) return;
-  if (threadIdx.x == 0) sm.ticket = atomicAdd(s.rs.state + ST_LISTED, own);
+  if (threadIdx.x == 0) sm.list_at = atomicAdd(s.rs.state + ST_LISTED, own);
   __syncthreads();
   const uint32_t cap = list_cap(s.a.d);
   for (uint32_t i = threadIdx.x; i < own; i += kSelThreads)
-    if (dq_in_bounds(sm.ticket + i < cap, s.a.err)) s.rs.list[sm.ticket + i] = sm.list[i];
+    if (dq_in_bounds(sm.list_at + i < cap, s.a.err)) s.rs.list[sm.list_at + i] = sm.list[i];
 }
 
 __device__ __forceinline__ void count_first(SelectSmem<kSelThreads>& sm, const SelectTask& s, const TileAhead& first,
@@ -678,91 +637,34 @@ __device__ __forceinline__ void count_first(SelectSmem<kSelThreads>& sm, const S
       [](int) {});
 }
 
-// One CTA, after the second round's counts of the whole row are in: T and the
-// number of keys equal to it that are kept (into the state), and for each
-// group the numbers of keys above and equal to T in the groups before it.
-template <bool GLOBAL>
-__device__ __forceinline__ void resolve_row(SelectSmem<kSelThreads>& sm, const SelectTask& s, uint32_t tau,
-                                            uint32_t bin, uint32_t k_rem, bool listing, const uint32_t* counts) {
-  find_bin<kSelThreads, kBins2, GLOBAL>(sm, counts, k_rem);
-  const uint32_t digit = sm.found[0];
-  k_rem = sm.found[1];
+// The exclusive prefix of gt[] and eq[] over the groups; an odd number of
+// groups per thread keeps the threads' shared-memory accesses on different
+// banks.
+__device__ __forceinline__ void group_places(SelectSmem<kSelThreads>& sm, int groups, uint32_t* gt, uint32_t* eq) {
   __syncthreads();
-  const uint32_t listed = listing ? __ldcg(s.rs.state + ST_LISTED) : 0u;
-  // body(group, key) over the row's keys in the bin: from the list, or (very
-  // many keys are nearly equal) from all candidates
-  auto for_listed = [&](auto&& body) {
-    if (listing) {
-      for (uint32_t i = threadIdx.x; i < listed; i += kSelThreads) {
-        const uint2 x = __ldcg(s.rs.list + i);
-        body((int)x.x, x.y);
-      }
-    } else {
-      SelectTask all = s;
-      all.warp0 = threadIdx.x >> 5;
-      all.nwarps = kSelWarps;
-      int in_group = 0;
-      walk(
-          all, load_first(all), [&](int group) { in_group = group; },
-          [&](uint2 c, bool valid) {
-            const uint32_t key = key_bits(c.y);
-            if (valid && first_bin(key, tau) == bin) body(in_group, key);
-          },
-          [](int) {});
-    }
-  };
-  uint32_t T;
-  if (bin < (uint32_t)kFineBins) {
-    T = tau + (bin << kFineShift) + digit;
-  } else {  // the last 11 bits
-    const uint32_t high = ((bin - kFineBins) << 12) | digit;
-    clear_hist(sm, 2048);
-    for_listed([&](int, uint32_t key) {
-      if ((key >> 11) == high) atomicAdd(&sm.hist[key & 2047u], 1u);
-    });
-    __syncthreads();
-    find_bin<kSelThreads, 2048, false>(sm, sm.hist, k_rem);
-    T = (high << 11) | sm.found[0];
-    k_rem = sm.found[1];
-  }
-  for_listed([&](int group, uint32_t key) {
-    if (key > T) atomicAdd(&s.rs.before[group].x, 1u);
-    if (key == T) atomicAdd(&s.rs.before[group].y, 1u);
-  });
-  __threadfence();
-  __syncthreads();
-  constexpr int kPer = kMaxGroups / kSelThreads;
+  const int per = ((groups + kSelThreads - 1) / kSelThreads) | 1;
+  const int i0 = min((int)threadIdx.x * per, groups), i1 = min(i0 + per, groups);
   uint64_t sum = 0, total;  // keys above T | keys equal to T << 32, both below 2^32
-  for (int q = 0; q < kPer; ++q) {
-    const int i = (int)threadIdx.x * kPer + q;
-    const uint2 v = i < s.groups ? __ldcg(s.rs.before + i) : make_uint2(0u, 0u);
-    sum += (uint64_t)v.x | (uint64_t)v.y << 32;
-  }
+  for (int i = i0; i < i1; ++i) sum += (uint64_t)gt[i] | (uint64_t)eq[i] << 32;
   uint64_t p = block_exclusive_scan<kSelThreads>(sum, &total, sm.scan);
-  for (int q = 0; q < kPer; ++q) {
-    const int i = (int)threadIdx.x * kPer + q;
-    if (i < s.groups) {
-      const uint2 v = __ldcg(s.rs.before + i);
-      s.rs.before[i] = make_uint2((uint32_t)p, (uint32_t)(p >> 32));
-      p += (uint64_t)v.x | (uint64_t)v.y << 32;
-    }
+  for (int i = i0; i < i1; ++i) {
+    const uint64_t v = (uint64_t)gt[i] | (uint64_t)eq[i] << 32;
+    gt[i] = (uint32_t)p;
+    eq[i] = (uint32_t)(p >> 32);
+    p += v;
   }
-  if (threadIdx.x == 0) {
-    s.rs.state[ST_T] = T;
-    s.rs.state[ST_NEED] = k_rem;
-  }
+  __syncthreads();
 }
 
 // The records of this task's groups, and e and h at the candidates not kept;
-// place(group): the numbers of keys above and equal to T before it.
-template <typename Place>
+// gt[], eq[]: the numbers of keys above and equal to T before each group.
 __device__ __forceinline__ void emit_groups(const SelectTask& s, const TileAhead& first, uint32_t T, uint32_t need,
-                                            Place&& place) {
+                                            const uint32_t* gt, const uint32_t* eq) {
   const int lane = threadIdx.x & 31;
   const uint32_t lt = (1u << lane) - 1u;
   uint2 before = make_uint2(0u, 0u);
   walk(
-      s, first, [&](int group) { before = place(group); },
+      s, first, [&](int group) { before = make_uint2(gt[group], eq[group]); },
       [&](uint2 c, bool valid) {
         const uint32_t key = key_bits(c.y);
         const uint32_t gts = __ballot_sync(kFullMask, valid && key > T);
@@ -786,148 +688,266 @@ __device__ __forceinline__ void emit_groups(const SelectTask& s, const TileAhead
 __global__ void __launch_bounds__(kSelThreads, 2) topk_count_kernel(const CompressArgs a, int rows, void* scratch) {
   dq_pdl_enter();
   __shared__ SelectSmem<kSelThreads> sm;
-  const SelectTask s = select_task(a, 0, rows, scratch);
+  const SelectTask s = select_task(a, 0, rows, scratch, blockIdx.y, blockIdx.x, gridDim.x);
   count_first(sm, s, load_first(s), call_tau(s.rs.state));
   add_hist(sm, s.rs.hist, kBins);
 }
 
-// 4. T's bin from the first-round counts, then the second round.  Where the
-// bin holds more keys than the list or T is far above tau, the row's last CTA
-// (a ticket counter; no CTA waits for another) goes on to T and the groups'
-// places; else every CTA of step 5 finds them.  For a row with too few
-// candidates instead: e as it is without any, and the top digit of all of p,
-// from which the last CTA takes a new tau.
+// 4. T's bin from the first-round counts, then the second round.  For a row
+// with too few candidates instead: nothing where they are all the non-zero
+// keys (T is 0); else every element becomes a candidate (as if kept), and the
+// first round is made again over all of them, from 0 up.
 __global__ void __launch_bounds__(kSelThreads, 2) topk_resolve_kernel(const CompressArgs a, int64_t k, int rows, void* scratch) {
   dq_pdl_enter();
   __shared__ SelectSmem<kSelThreads> sm;
-  const SelectTask s = select_task(a, k, rows, scratch);
+  const SelectTask s = select_task(a, k, rows, scratch, blockIdx.y, blockIdx.x, gridDim.x);
   const TileAhead first = load_first(s);
-  const uint32_t n = find_bin<kSelThreads, kBins, true>(sm, s.rs.hist, (uint32_t)k);
+  const uint32_t tau = call_tau(s.rs.state);
+  const uint32_t n = find_bin<kSelThreads, kBins>(sm, (uint32_t)k, RowCounts{s.rs.hist});
   const bool too_few = (int64_t)n < k;
   const uint32_t bin = sm.found[0], rest = sm.found[1];
   const bool listing = sm.found[2] <= list_cap(a.d);
-  const bool placed = bin >= (uint32_t)kFineBins || !listing;
   __syncthreads();
   if (blockIdx.x == 0 && threadIdx.x == 0) {
-    s.rs.state[ST_PLACED] = placed ? 1u : 0u;
-    s.rs.state[ST_SHORT] = too_few ? 1u : 0u;
+    s.rs.state[ST_ROUTE] = too_few ? (tau == 1 ? ROUTE_ZERO : ROUTE_SHORT) : listing ? ROUTE_LIST : ROUTE_BIN;
     s.rs.state[ST_BIN] = bin;
-    s.rs.state[ST_REST] = rest;
+    s.rs.state[ST_REST] = too_few ? (uint32_t)k - n : rest;
   }
   if (!too_few) {
-    const uint32_t tau = call_tau(s.rs.state);
     count_second(sm, s, first, tau, bin, listing);
     add_hist(sm, s.rs.hist2, kBins2);
-    if (!placed || !last_of_row(sm, s.rs.state + ST_TICKET)) return;
-    resolve_row<true>(sm, s, tau, bin, rest, listing, s.rs.hist2);
     return;
   }
-  clear_hist(sm, kTopBins);
+  if (tau == 1) return;
+  clear_hist(sm, kBins);
   for (int64_t t = blockIdx.x; t < s.nt; t += gridDim.x) {
     const uint32_t m = __ldcg(s.rs.cnt + t);
-    for (uint32_t i = threadIdx.x; i < m; i += kSelThreads) put_back(s, __ldcg(s.rs.cand + t * kTile + i));
+    uint2* slot = s.rs.cand + t * kTile;
+    for (uint32_t i = threadIdx.x; i < m; i += kSelThreads) put_back(s, __ldcg(slot + i));
     __syncthreads();
-    const int64_t end = min64((t + 1) * kTile, a.d);
-    for (int64_t j = t * kTile + threadIdx.x; j < end; j += kSelThreads) atomicAdd(&sm.hist[key_of(s.e[j]) >> 20], 1u);
+    const int64_t j0 = t * kTile;
+    const int n = (int)min64(kTile, a.d - j0);
+    for (int i = threadIdx.x; i < n; i += kSelThreads) {
+      const int64_t j = j0 + i;
+      const float p = s.e[j], en = __fsub_rn(p, p);
+      slot[i] = make_uint2((uint32_t)j, __float_as_uint(p));
+      if (__float_as_uint(p) != 0u) {
+        s.e[j] = en;
+        if (s.h) s.h[j] = __fadd_rn(__fmul_rn(a.lr, s.g[j]), en);
+      }
+      atomicAdd(&sm.hist[first_bin(key_of(p), 0)], 1u);
+    }
+    if (threadIdx.x == 0) s.rs.cnt[t] = (uint32_t)n;
   }
-  add_hist(sm, s.rs.hist2, kTopBins);
-  if (!last_of_row(sm, s.rs.state + ST_TICKET)) return;
-  find_bin<kSelThreads, kTopBins, true>(sm, s.rs.hist2, (uint32_t)k);
-  if (threadIdx.x == 0) s.rs.state[ST_TAU2] = sm.found[0] << 20;
+  add_hist(sm, s.rs.hist2, kBins);
 }
 
 // 5. T from the second-round counts, the groups' places from their counts and
-// the list, and the records.  For a row with too few candidates: the
-// candidates again, from the new tau up, and the last CTA selects among them
-// by itself.
-__global__ void __launch_bounds__(kSelThreads, 2) topk_emit_kernel(const CompressArgs a, int64_t k, int rows, void* scratch) {
+// the list, and the records.  Rows whose T is 0 need no counts at all.  Rows
+// that take further passes over the candidates (T's bin holds more keys than
+// the list: very many equal keys; or the sample was far off) are selected by a
+// cluster of CTAs each afterwards, since the others cannot wait for one
+// another.  Two: clusters of 4 or 8 made those rows up to 3 times as fast, but
+// every call slower, as fewer CTAs fit at once (dcgan-sized, 3.6M x 8, k = d /
+// 100: 80 us with 2, 82 with 4 or 8; 25M x 16 826 / 843 / 839).
+constexpr int kEmitCluster = 2;
+
+// T's last 11 bits where the second round has not settled them: the keys with
+// the leading bits `high`.
+__device__ __forceinline__ void third_round_add(uint32_t* hist, uint32_t key, uint32_t high) {
+  if ((key >> 11) == high) atomicAdd(hist + (key & 2047u), 1u);
+}
+
+// The records of a row with fewer than k non-zero keys, its candidates: all of
+// them, and the first `need` zeros in index order (their e = p - p is +0).
+// gt[], eq[]: the numbers of candidates and of zeros before each group.
+__device__ __forceinline__ void emit_with_zeros(SelectSmem<kSelThreads>& sm, const SelectTask& s, uint32_t need,
+                                                const uint32_t* gt, const uint32_t* eq) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t lt = (1u << lane) - 1u;
+  uint32_t* const bits = sm.hist + (threadIdx.x >> 5) * (kTile / 32);  // the tile's candidates, a bit each
+  static_assert(kSelWarps * (kTile / 32) <= kBins2, "bits of a tile per warp");
+  auto put = [&](uint32_t pos, uint2 x) {
+    if (dq_in_bounds(pos < (uint64_t)s.k, s.a.err)) s.rec[pos] = x;  // always true; keeps the write inside
+  };
+  for (int group = s.warp0; group < s.groups; group += s.nwarps) {
+    uint32_t above = gt[group], zeros = eq[group];
+    const int64_t t1 = min64(s.nt, (int64_t)(group + 1) << s.shift);
+    for (int64_t t = (int64_t)group << s.shift; t < t1; ++t) {
+      const uint32_t n = __ldcg(s.rs.cnt + t);
+      const uint2* slot = s.rs.cand + t * kTile;
+      const int64_t j0 = t * kTile;
+      const int size = (int)min64(kTile, s.a.d - j0);
+      const bool some = zeros < need;  // of this tile's zeros are kept
+      if (some) {
+        for (int i = lane; i < kTile / 32; i += 32) bits[i] = 0;
+        __syncwarp();
+      }
+      for (uint32_t o = lane; o < n; o += 32) {
+        const uint2 x = __ldcg(slot + o);
+        const uint32_t i = x.x - (uint32_t)j0;
+        put(above + o + min(zeros + (i - o), need), x);
+        if (some && dq_in_bounds(i < (uint32_t)kTile, s.a.err)) atomicOr(bits + (i >> 5), 1u << (i & 31));
+      }
+      __syncwarp();
+      uint32_t at = above, z = zeros;
+#pragma unroll 4
+      for (int r = 0; some && r < size; r += 32) {
+        const int64_t j = j0 + r + lane;
+        const uint32_t here = bits[r >> 5];
+        const uint32_t none = ~here & (size - r < 32 ? (1u << (size - r)) - 1u : kFullMask);
+        const uint32_t tie = z + __popc(none & lt);
+        if (((none >> lane) & 1u) && tie < need) {
+          put(at + __popc(here & lt) + tie, make_uint2((uint32_t)j, __float_as_uint(s.e[j])));
+          s.e[j] = 0.f;
+          if (s.h) s.h[j] = __fadd_rn(__fmul_rn(s.a.lr, s.g[j]), 0.f);
+        }
+        at += __popc(here);
+        z += __popc(none);
+      }
+      __syncwarp();
+      above += n;
+      zeros += (uint32_t)size - n;
+    }
+  }
+}
+
+// A ROUTE_BIN or ROUTE_SHORT row, by the CTAs of a cluster together.
+// (A call, so that its registers are no burden to the rows without it.)
+__device__ __noinline__ void select_by_cluster(SelectSmem<kSelThreads>& sm, const CompressArgs& a, int64_t k, int rows,
+                                               void* scratch, int row, uint32_t* places) {
+  cg::cluster_group cluster = cg::this_cluster();
+  const int rank = (int)cluster.block_rank();
+  const int lane = threadIdx.x & 31;
+  const SelectTask s = select_task(a, k, rows, scratch, row, rank, kEmitCluster);
+  auto cluster_counts = [&](int i) {  // of sm.hist
+    uint4 x = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+    for (int r = 0; r < kEmitCluster; ++r) {
+      const uint4 y = *cluster.map_shared_rank(reinterpret_cast<const uint4*>(sm.hist + i), r);
+      x.x += y.x;
+      x.y += y.y;
+      x.z += y.z;
+      x.w += y.w;
+    }
+    return x;
+  };
+  uint32_t tau, bin, rest;
+  if (__ldcg(s.rs.state + ST_ROUTE) == ROUTE_SHORT) {
+    tau = 0;
+    find_bin<kSelThreads, kBins>(sm, (uint32_t)k, RowCounts{s.rs.hist2});
+    bin = sm.found[0], rest = sm.found[1];
+    count_second(sm, s, load_first(s), tau, bin, false);
+    cluster.sync();
+    find_bin<kSelThreads, kBins2>(sm, rest, cluster_counts);
+  } else {
+    tau = call_tau(s.rs.state);
+    bin = __ldcg(s.rs.state + ST_BIN), rest = __ldcg(s.rs.state + ST_REST);
+    find_bin<kSelThreads, kBins2>(sm, rest, RowCounts{s.rs.hist2});
+  }
+  const uint32_t digit = sm.found[0];
+  uint32_t T = tau + (bin << kFineShift) + digit, need = sm.found[1];
+  cluster.sync();
+  if (bin >= (uint32_t)kFineBins) {
+    const uint32_t high = ((bin - kFineBins) << 12) | digit;
+    clear_hist(sm, 2048);
+    walk(
+        s, load_first(s), [](int) {},
+        [&](uint2 c, bool valid) {
+          if (valid) third_round_add(sm.hist, key_bits(c.y), high);
+        },
+        [](int) {});
+    cluster.sync();
+    find_bin<kSelThreads, 2048>(sm, need, cluster_counts);
+    T = (high << 11) | sm.found[0];
+    need = sm.found[1];
+    cluster.sync();  // nobody leaves, or counts anew, while its counts are read
+  }
+  uint32_t gt = 0, eq = 0;
+  walk(
+      s, load_first(s), [&](int) { gt = 0, eq = 0; },
+      [&](uint2 c, bool valid) {
+        const uint32_t key = key_bits(c.y);
+        gt += valid && key > T ? 1u : 0u;
+        eq += valid && key == T ? 1u : 0u;
+      },
+      [&](int group) {
+        gt = __reduce_add_sync(kFullMask, gt);
+        eq = __reduce_add_sync(kFullMask, eq);
+        if (lane == 0) s.rs.before[group] = make_uint2(gt, eq);
+      });
+  __threadfence();
+  cluster.sync();
+  for (int i = threadIdx.x; i < s.groups; i += kSelThreads) {
+    const uint2 n = __ldcg(s.rs.before + i);
+    places[i] = n.x;
+    places[s.groups + i] = n.y;
+  }
+  group_places(sm, s.groups, places, places + s.groups);
+  emit_groups(s, load_first(s), T, need, places, places + s.groups);
+  __syncthreads();
+}
+
+__global__ void __launch_bounds__(kSelThreads, 2)
+    topk_emit_kernel(const CompressArgs a, int64_t k, int rows, int ctas, void* scratch) {
   dq_pdl_enter();
   __shared__ SelectSmem<kSelThreads> sm;
   extern __shared__ uint32_t places[];
-  SelectTask s = select_task(a, k, rows, scratch);
-  const TileAhead first = load_first(s);
-  const uint32_t listed = s.rs.state[ST_LISTED];
-  const uint2 early = s.rs.list[threadIdx.x];  // (the list holds at least 8192)
-  auto placed = [&](int group) { return __ldcg(s.rs.before + group); };
-  if (!s.rs.state[ST_SHORT]) {
-    if (s.rs.state[ST_PLACED]) {
-      emit_groups(s, first, s.rs.state[ST_T], s.rs.state[ST_NEED], placed);
-      return;
-    }
+  const int row = (int)blockIdx.x / ctas;
+  if (row < a.nworkers) {
+    const SelectTask s = select_task(a, k, rows, scratch, row, (int)blockIdx.x - row * ctas, ctas);
+    const TileAhead first = load_first(s);
+    const uint32_t listed = s.rs.state[ST_LISTED], route = s.rs.state[ST_ROUTE];
     uint32_t* gt = places;
     uint32_t* eq = places + s.groups;
-    for (int i = threadIdx.x; i < s.groups; i += kSelThreads) {
-      gt[i] = s.rs.before[i].x;
-      eq[i] = 0;
-    }
-    find_bin<kSelThreads, kBins2, true>(sm, s.rs.hist2, s.rs.state[ST_REST]);
-    const uint32_t T = call_tau(s.rs.state) + (s.rs.state[ST_BIN] << kFineShift) + sm.found[0], need = sm.found[1];
-    for (uint32_t i = threadIdx.x; i < listed; i += kSelThreads) {
-      const uint2 x = i < (uint32_t)kSelThreads ? early : s.rs.list[i];
-      if (x.y > T) atomicAdd(gt + x.x, 1u);
-      if (x.y == T) atomicAdd(eq + x.x, 1u);
-    }
-    __syncthreads();
-    // exclusive prefix of both; an odd number of groups per thread keeps the
-    // threads' shared-memory accesses on different banks
-    const int per = ((s.groups + kSelThreads - 1) / kSelThreads) | 1;
-    const int i0 = min((int)threadIdx.x * per, s.groups), i1 = min(i0 + per, s.groups);
-    uint64_t sum = 0, total;  // keys above T | keys equal to T << 32, both below 2^32
-    for (int i = i0; i < i1; ++i) sum += (uint64_t)gt[i] | (uint64_t)eq[i] << 32;
-    uint64_t p = block_exclusive_scan<kSelThreads>(sum, &total, sm.scan);
-    for (int i = i0; i < i1; ++i) {
-      const uint64_t v = (uint64_t)gt[i] | (uint64_t)eq[i] << 32;
-      gt[i] = (uint32_t)p;
-      eq[i] = (uint32_t)(p >> 32);
-      p += v;
-    }
-    __syncthreads();
-    emit_groups(s, first, T, need, [&](int group) { return make_uint2(gt[group], eq[group]); });
-    return;
-  }
-  const uint32_t tau = s.rs.state[ST_TAU2];
-  for (int64_t t = blockIdx.x; t < s.nt; t += gridDim.x) {
-    constexpr int kRows = kTile / (4 * kSelThreads);
-    float v[kRows][4];
-    uint32_t cmask[kRows];
-#pragma unroll
-    for (int i = 0; i < kRows; ++i) {
-      const int64_t j = t * kTile + 4 * ((int64_t)i * kSelThreads + threadIdx.x);
-      cmask[i] = 0;
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        v[i][q] = 0.f;
-        if (j + q < a.d) {
-          v[i][q] = s.e[j + q];
-          if (key_of(v[i][q]) >= tau) {
-            cmask[i] |= 1u << q;
-            const float en = __fsub_rn(v[i][q], v[i][q]);
-            s.e[j + q] = en;
-            if (s.h) s.h[j + q] = __fadd_rn(__fmul_rn(a.lr, s.g[j + q]), en);
-          }
-        }
+    if (route == ROUTE_ZERO) {
+      for (int i = threadIdx.x; i < s.groups; i += kSelThreads) {
+        uint32_t n = 0;
+        const int64_t t0 = (int64_t)i << s.shift, t1 = min64(s.nt, (int64_t)(i + 1) << s.shift);
+        for (int64_t t = t0; t < t1; ++t) n += __ldcg(s.rs.cnt + t);
+        gt[i] = n;
+        eq[i] = (uint32_t)(min64(t1 * kTile, a.d) - t0 * kTile) - n;
       }
+      group_places(sm, s.groups, gt, eq);
+      emit_with_zeros(sm, s, s.rs.state[ST_REST], gt, eq);
+    } else if (route == ROUTE_LIST) {
+      for (int i = threadIdx.x; i < s.groups; i += kSelThreads) {
+        gt[i] = s.rs.before[i].x;
+        eq[i] = 0;
+      }
+      const uint2 early = s.rs.list[threadIdx.x];  // (the list holds at least 8192)
+      auto for_listed = [&](auto&& body) {
+        for (uint32_t i = threadIdx.x; i < listed; i += kSelThreads)
+          body(i < (uint32_t)kSelThreads ? early : s.rs.list[i]);
+      };
+      find_bin<kSelThreads, kBins2>(sm, s.rs.state[ST_REST], RowCounts{s.rs.hist2});
+      const uint32_t bin = s.rs.state[ST_BIN];
+      uint32_t T = call_tau(s.rs.state) + (bin << kFineShift) + sm.found[0], need = sm.found[1];
+      if (bin >= (uint32_t)kFineBins) {
+        const uint32_t high = ((bin - kFineBins) << 12) | sm.found[0];
+        __syncthreads();
+        clear_hist(sm, 2048);
+        for_listed([&](uint2 x) { third_round_add(sm.hist, x.y, high); });
+        __syncthreads();
+        find_bin<kSelThreads, 2048>(sm, need, OwnCounts{sm.hist});
+        T = (high << 11) | sm.found[0];
+        need = sm.found[1];
+      }
+      for_listed([&](uint2 x) {
+        if (x.y > T) atomicAdd(gt + x.x, 1u);
+        if (x.y == T) atomicAdd(eq + x.x, 1u);
+      });
+      group_places(sm, s.groups, gt, eq);
+      emit_groups(s, first, T, need, gt, eq);
     }
-    const uint32_t n = write_tile_candidates<kSelThreads, kRows>(v, cmask, t * kTile, s.rs.cand + t * kTile,
-                                                                 sm.warp_sums, a.err);
-    if (threadIdx.x == 0) s.rs.cnt[t] = n;
   }
-  if (!last_of_row(sm, s.rs.state + ST_TICKET + 1)) return;
-  s.warp0 = threadIdx.x >> 5;
-  s.nwarps = kSelWarps;
-  count_first(sm, s, load_first(s), tau);
-  __syncthreads();
-  find_bin<kSelThreads, kBins, false>(sm, sm.hist, (uint32_t)k);
-  const uint32_t bin = sm.found[0], rest = sm.found[1];
-  const bool listing = sm.found[2] <= list_cap(a.d);
-  __syncthreads();
-  count_second(sm, s, load_first(s), tau, bin, listing);
-  __threadfence();
-  __syncthreads();
-  resolve_row<false>(sm, s, tau, bin, rest, listing, sm.hist);
-  __threadfence();
-  __syncthreads();
-  emit_groups(s, load_first(s), __ldcg(s.rs.state + ST_T), __ldcg(s.rs.state + ST_NEED), placed);
+  for (int r = (int)blockIdx.x / kEmitCluster; r < a.nworkers; r += (int)gridDim.x / kEmitCluster) {
+    const uint32_t route = __ldcg(row_scratch(scratch, a.d, a.worker0 + r - a.row0).state + ST_ROUTE);
+    if (route == ROUTE_BIN || route == ROUTE_SHORT) {
+      __syncthreads();
+      select_by_cluster(sm, a, k, rows, scratch, r, places);
+    }
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -1703,6 +1723,9 @@ cudaError_t launch_topk_compress(const CompressArgs& a, int64_t k, bool keep_h, 
   const int64_t mean = 1 + 13 * k / (320 * tiles_of(a.d));
   const int ahead = (int)(mean < kFirst ? mean : kFirst);
   const size_t places = groups_of(a.d) * 2 * sizeof(uint32_t);
+  // (with a cluster for every row that needs one, where they fit at once)
+  const unsigned least = kEmitCluster * rows < 2 * 152 ? kEmitCluster * rows : 2 * 152;
+  const unsigned emit = ((select.x * rows > least ? select.x * rows : least) + kEmitCluster - 1) / kEmitCluster * kEmitCluster;
   if ((st = allow_smem(topk_emit_kernel, kMaxGroups * 2 * sizeof(uint32_t), 1, emit_done)) != cudaSuccess) return st;
   (void)(launched(launch_pdl(topk_sample_kernel, dim3(kSampBlocks, rows), dim3(kSampThreads), 0, stream, a,
                              sample_rank(a.d, k), scratch)) &&
@@ -1710,7 +1733,8 @@ cudaError_t launch_topk_compress(const CompressArgs& a, int64_t k, bool keep_h, 
                              stream, a, scratch)) &&
          launched(launch_pdl(topk_count_kernel, select, dim3(kSelThreads), 0, stream, a, ahead, scratch)) &&
          launched(launch_pdl(topk_resolve_kernel, select, dim3(kSelThreads), 0, stream, a, k, ahead, scratch)) &&
-         launched(launch_pdl(topk_emit_kernel, select, dim3(kSelThreads), places, stream, a, k, ahead, scratch)));
+         launched(launch_pdl_cluster(topk_emit_kernel, kEmitCluster, dim3(emit), dim3(kSelThreads), places, stream, a, k,
+                                     ahead, (int)select.x, scratch)));
   return st;
 }
 

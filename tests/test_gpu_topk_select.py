@@ -12,7 +12,12 @@ for bit with numpy on the same fp32 p:
   elements reach the threshold and the candidates are taken again;
 * a few dense tiles among thousands with one candidate each;
 * a k-th key far above the threshold, so many equal keys that their list
-  overflows, k = 1 and k = d.
+  overflows, k = 1 and k = d;
+* sparse gradients: fewer than k non-zero entries (the k-th key is 0 and
+  almost every element equals it) and a few more than k (every element is a
+  candidate and T far above the threshold 0), also with more workers than
+  there are clusters for them.  These are ordinary inputs, so their time is
+  held against a dense gradient's too.
 """
 from __future__ import annotations
 
@@ -40,7 +45,7 @@ def sampled(d):
     return (at[:, None] * 8 + np.arange(8, dtype=np.uint64)).ravel().astype(np.int64)
 
 
-def gradient(kind, d, rng):
+def gradient(kind, d, k, rng):
     g = rng.standard_normal(d).astype(np.float32)
     if kind == "trap":
         g *= np.float32(1e-3)
@@ -55,6 +60,10 @@ def gradient(kind, d, rng):
         g[rng.choice(d, 3, replace=False)] *= np.float32(1e25)
     elif kind == "ties":
         g = np.sign(g) * (rng.integers(1, 4, d) * 0.5).astype(np.float32)
+    elif kind == "zeros":
+        g[:] = 0
+    elif kind in ("sparse", "just enough"):  # -0 and +0 elsewhere
+        g[rng.random(d) >= (0.5 if kind == "sparse" else 1.1) * k / d] *= 0
     return g
 
 
@@ -63,7 +72,10 @@ CASES = [(1, 1, 2, "gauss"), (3, 2, 2, "gauss"), (2_049, 2_049, 2, "ties"), (20_
          (393_215, 4_000, 9, "gauss"), (65_535, 65_535, 20, "gauss"), (65_536, 300, 20, "gauss"),
          (200_003, 200_003, 9, "gauss"), (786_431, 9_000, 4, "ties"), (300_005, 2, 20, "outliers"),
          (300_005, 150_000, 20, "ties"), (1_000_003, 1, 2, "gauss"), (1_000_003, 990_000, 2, "gauss"),
-         (1_000_003, 200_000, 2, "trap"), (9_000_001, 400_000, 2, "ties"), (9_000_001, 21_000, 2, "sparse tiles")]
+         (1_000_003, 200_000, 2, "trap"), (9_000_001, 400_000, 2, "ties"), (9_000_001, 21_000, 2, "sparse tiles"),
+         (200_003, 9_000, 2, "sparse"), (1_000_003, 20_000, 3, "sparse"), (1_000_003, 20_000, 3, "just enough"),
+         (1_000_003, 300_000, 2, "just enough"), (90_001, 1_000, 64, "sparse"), (1_000_003, 60_000, 2, "zeros"), (35_000_001, 50_000, 1, "sparse"),
+         (35_000_001, 50_000, 1, "trap"), (90_001, 30_000, 64, "ties")]
 
 
 @pytest.mark.parametrize("keep", [False, True])
@@ -77,10 +89,13 @@ def test_records_residual_and_offsets(P, d, k, M, kind, keep):
     ld = (d + 3) // 4 * 4
     i = M - 1  # the worker looked at; the others get zeros
     e = np.zeros(d, np.float32)
+    if kind in ("sparse", "just enough"):
+        e = -e  # -0: with -0 in the gradient, p is -0 there
+        h.set_residual(i, e)
     g_dev = torch.zeros((M, ld), device="cuda")
     msgs = torch.zeros((M, h.message_bytes()), dtype=torch.uint8, device="cuda")
     for step in range(2):
-        g = gradient(kind, d, rng)
+        g = gradient(kind, d, k, rng)
         g_dev[i, :d] = torch.from_numpy(g)
         h.workers_compress_all(g_dev, ld, msgs)
         h.synchronize()
@@ -106,3 +121,32 @@ def test_records_residual_and_offsets(P, d, k, M, kind, keep):
             h.get_lookahead(i, got)
             assert np.array_equal(got.view(np.uint32), (s + e).view(np.uint32)), step
     h.destroy()
+
+
+@pytest.mark.parametrize("d,M", [(400_000, 4), (3_600_000, 8)])  # on chip; the sampled kernels
+def test_sparse_gradients_take_a_few_times_a_dense_one(P, d, M):
+    """Fewer than k non-zero entries, so that almost every element equals the k-th key: no
+    slower than a dense gradient but for a few passes.  Selected by one CTA per worker it
+    took 120 times a dense gradient's time."""
+    stream = torch.cuda.current_stream()
+    k, ld = d // 100, (d + 3) // 4 * 4
+    took = {}
+    for kind in ("gauss", "sparse"):
+        h = P.create(P.make_config(d=d, M=M, compressor=P.TOPK, lr=0.25, k=k, cuda_stream=stream.cuda_stream))
+        gen = torch.Generator(device="cuda").manual_seed(5)
+        g = torch.randn((M, ld), generator=gen, device="cuda")
+        if kind == "sparse":
+            g *= torch.rand((M, ld), generator=gen, device="cuda") < 0.005
+        msgs = torch.zeros((M, h.message_bytes()), dtype=torch.uint8, device="cuda")
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        times = []
+        for _ in range(5):
+            a.record()
+            for _ in range(4):
+                h.workers_compress_all(g, ld, msgs)
+            b.record()
+            torch.cuda.synchronize()
+            times.append(a.elapsed_time(b) / 4)
+        took[kind] = min(times)
+        h.destroy()
+    assert took["sparse"] < 5 * took["gauss"], took
