@@ -40,8 +40,9 @@
 // workers as +0, in the library's pairwise order) / M at the indices some
 // worker sent; elsewhere the sum is +0 and w is unchanged.  Where the records
 // are dense enough (tile_server), a first kernel finds where each worker's
-// records of each tile of indices start, and a CTA per tile merges the
-// workers' records of it in shared memory.  Sparse records of up to 64
+// records of each tile of indices start, a CTA per tile merges the workers'
+// records of it in shared memory, and tiles with very many are shared out in
+// parts by a third kernel.  Sparse records of up to 64
 // workers: one thread per record in two launches, which scatter the values
 // into a table and set the worker's bit in a per-index mask, then let the
 // lowest worker of each index sum the index's values and update w_j.  Above
@@ -1181,8 +1182,9 @@ __global__ void __launch_bounds__(kChipThreads, 1) topk_chip_kernel(const Compre
 // ---------------------------------------------------------------------------
 constexpr int kStartsPer = 4;
 
-__global__ void __launch_bounds__(256) topk_server_starts_kernel(const ServerArgs s, uint32_t* starts) {
+__global__ void __launch_bounds__(256) topk_server_starts_kernel(const ServerArgs s, uint32_t* starts, uint32_t* dense) {
   dq_pdl_enter();
+  if (dense && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *dense = 0;
   const int m = blockIdx.y;
   const int64_t r0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * kStartsPer;
   const int lane = threadIdx.x & 31;
@@ -1243,7 +1245,9 @@ __device__ __forceinline__ float srv_average(float acc, const ServerArgs& s) {
 // workers; all zero between calls) and M values per index (never cleared).
 //   1. scatter: record (m, r) with index j writes its value to entry (j, m)
 //      and sets bit m of j's mask.
-//   2. reduce: the record of the lowest worker in j's mask owns j.  It sums
+//   2. reduce: the record of the lowest worker in j's mask owns j.  It loads j's
+//      values 16 bytes at a time (one by one, M = 64, d = 100,000, k = d / 10,
+//      the same indices: 28 us from warm caches, 15 so) and sums
 //      the values of the workers in the mask, in worker order with the
 //      absent workers as +0 leaves (the library's pairwise order), updates
 //      w_j and clears j's mask.  The other records of j read its mask
@@ -1261,14 +1265,19 @@ constexpr int kSrvMaskMaxM = 64;
 template <typename Mask>
 struct SrvTables {
   Mask* mask;   // d masks
-  float* vals;  // worker m's value of index j at vals[j * M + m]
+  float* vals;  // worker m's value of index j at vals[j * srv_row(M) + m]
 };
+
+// Values per index in the table: whole 16-byte loads.
+__host__ __device__ constexpr int64_t srv_row(int32_t nworkers) {
+  return nworkers <= 2 ? nworkers : (nworkers + 3) / 4 * 4;
+}
 
 // Words of a mask: one bit per worker.
 __host__ __device__ constexpr int srv_mask_words(int32_t nworkers) { return nworkers <= 32 ? 1 : 2; }
 
 __host__ __device__ constexpr int64_t srv_mask_table_words(int64_t d, int32_t nworkers) {
-  return (srv_mask_words(nworkers) + (int64_t)nworkers) * round64(d);
+  return (srv_mask_words(nworkers) + srv_row(nworkers)) * round64(d);
 }
 
 template <typename Mask>
@@ -1296,29 +1305,31 @@ __global__ void __launch_bounds__(kSrvThreads) topk_server_scatter_kernel(const 
   const uint2 rec = reinterpret_cast<const uint2*>(s.msgs + (int64_t)m * s.msg_stride)[r];
   // records come from the compressor and are below d
   if (!dq_in_bounds((int64_t)rec.x < s.d, s.err)) return;
-  t.vals[(int64_t)rec.x * s.M + m] = __uint_as_float(rec.y);
+  t.vals[(int64_t)rec.x * srv_row(s.M) + m] = __uint_as_float(rec.y);
   atomicOr(t.mask + rec.x, (Mask)1 << m);
 }
 
-// The sum at an index whose mask of workers is `mask`, by the owner m with its
-// value v; value(who): another worker's.
-template <int P, typename Mask, typename Value>
-__device__ __forceinline__ float owner_sum(Mask mask, int m, float v, Value&& value) {
+// The sum at an index whose mask of workers is `mask`, by the owner with its
+// value v; four(w, x): the values of workers w .. w + 3 (w + 1 for two workers
+// in all; of those in the mask, anything for the others).
+template <int P, typename Mask, typename Four>
+__device__ __forceinline__ float owner_sum(Mask mask, float v, Four&& four) {
   if ((mask & (mask - 1u)) == 0u) return P == 1 ? v : __fadd_rn(v, 0.f);  // one value among +0 leaves
   // the padded tree itself: chunks of C leaves (workers), each summed
   // pairwise from its values (+0 where a worker is absent), then the
   // P / C chunk sums pairwise -- the chunks are the tree's subtrees
-  constexpr int C = P < 16 ? P : 16;
+  constexpr int C = P < 16 ? P : 16, Q = C < 4 ? C : 4;
   float part[P / C];
 #pragma unroll
   for (int c = 0; c < P / C; ++c) {
     const uint32_t bits = (uint32_t)(mask >> (C * c)) & (uint32_t)((1ull << C) - 1ull);
     float x[C];
 #pragma unroll
-    for (int u = 0; u < C; ++u) {
-      const int who = C * c + u;
-      x[u] = 0.f;
-      if ((bits >> u) & 1u) x[u] = who == m ? v : value(who);
+    for (int u = 0; u < C; u += Q) {
+      float y[4] = {};
+      if ((bits >> u) & ((1u << Q) - 1u)) four(C * c + u, y);
+#pragma unroll
+      for (int q = 0; q < Q; ++q) x[u + q] = (bits >> (u + q)) & 1u ? y[q] : 0.f;
     }
 #pragma unroll
     for (int width = C / 2; width >= 1; width /= 2)
@@ -1344,185 +1355,309 @@ __global__ void __launch_bounds__(kSrvThreads) topk_server_reduce_kernel(const S
   const Mask mask = t.mask[j];
   // the owner: bit m set and no bit below it
   if (!((mask >> m) & 1u) || (mask & (((Mask)1 << m) - 1u))) return;
-  const float sum = owner_sum<P>(mask, m, __uint_as_float(rec.y), [&](int who) { return t.vals[j * s.M + who]; });
+  const float* vals = t.vals + j * srv_row(s.M);
+  const float sum = owner_sum<P>(mask, __uint_as_float(rec.y), [&](int who, float (&x)[4]) {
+    if constexpr (P <= 2) {
+      x[0] = vals[0];
+      x[1] = vals[1];
+    } else {
+      const float4 v = *reinterpret_cast<const float4*>(vals + who);
+      x[0] = v.x;
+      x[1] = v.y;
+      x[2] = v.z;
+      x[3] = v.w;
+    }
+  });
   s.w[j] = server_out(s, s.w[j], srv_average<POW2>(sum, s));
   t.mask[j] = 0;
 }
 
-// Server for dense records (tile_server), M <= kSrvMaskMaxM: one CTA per
-// kMergeTile indices.  starts[m][t] tells where worker m's records of each run
-// of kSrvTile indices are.  Two ways to merge, by the tile's number of records:
-//   list (up to half a record per index): the records go to shared memory,
+// Server for dense records (tile_server), M <= kSrvMaskMaxM, in two kernels.
+// starts[m][t] tells where worker m's records of each run of kSrvTile indices
+// are.
+//   merge, a CTA per tile of kMergeRuns runs: up to kMergeCap records go to shared memory,
 //     worker after worker, and set their worker's bit in their index's mask;
 //     the record of the lowest worker of an index owns it.  A sole worker's
 //     record updates w; the indices of several workers get rows of M values in
 //     what the list leaves free, as many at a time as fit, which their records
-//     fill and their owners sum.
-//   table: a zeroed value per worker and index, as many runs of indices at a
-//     time as fit; the records set theirs and every index sums its column (+0
-//     where nobody sent it, which leaves w as it is).
-// Records and touched parameters are all it moves: against the tables of the
-// two kernels above, whose scattered sectors go through DRAM twice, 25M x 16,
-// k = d / 100: 453 -> 143 us (k = d / 20: 1611 -> 348), the starts included.
+//     fill and their owners sum.  A tile with more records goes on a list.
+//   dense, over the list: a zeroed value per worker and index of some runs; the
+//     records set theirs and every index sums its column (+0 where nobody sent
+//     it, which leaves w as it is).  Records gather where a layer's gradients
+//     are large, in a few tiles out of thousands, so those tiles are dealt out
+//     in runs to a grid of their own (524,288 x 64, k = d / 10 in a tenth of
+//     the vector: 392 us where the merge's CTAs did it themselves, 38 so).
+// Records and touched parameters are all they move, against the tables of the
+// two kernels above, whose scattered sectors go through DRAM twice.  Latency
+// bounds them: the loads of a thread's 8 records, and of the parameters it
+// owns, are in flight together (one after the other: 25M x 16, k = d / 100,
+// 143 us, 103 so).
 constexpr int kMergeThreads = 256;
-constexpr int kMergeRuns = 16;
-constexpr int kMergeTile = kMergeRuns * kSrvTile;  // indices per CTA
-constexpr int kMergeCap = 2048;                    // records in the list
-constexpr int kMergeRow = 2048;                    // words for the rows of shared indices
+constexpr int kMergeCap = 2048;  // records in the list
+constexpr int kMergeRuns = 16;   // runs per merge CTA
+// Words for the rows of shared indices (what leaves 4 or, above 32 workers, 3
+// CTAs per SM).
+constexpr int merge_row_words(size_t mask_bytes) { return mask_bytes == 4 ? 2048 : 4096; }
 
-// Shared memory: the list, the rows, the masks and the rows' numbers, or the
-// table (at least one run).
+// Shared memory of the merge kernel: the list, the rows, the masks and the rows'
+// numbers.
 constexpr size_t merge_smem(size_t mask_bytes) {
-  return kMergeCap * sizeof(uint2) + kMergeRow * sizeof(float) + kMergeTile * (mask_bytes + sizeof(uint16_t));
+  return kMergeCap * sizeof(uint2) + merge_row_words(mask_bytes) * sizeof(float) +
+         kMergeRuns * kSrvTile * (mask_bytes + sizeof(uint16_t));
 }
-static_assert(kSrvMaskMaxM * kSrvTile * sizeof(float) <= merge_smem(8) && 32 * kSrvTile * sizeof(float) <= merge_smem(4),
-              "a run of every worker fits");
+// Runs of an item of the dense kernel, at most, and its shared memory.
+constexpr int dense_runs(int P) { return P >= 32 ? 1 : P >= 4 ? 48 / P : 16; }
+constexpr size_t dense_smem(int M, int P) { return (size_t)M * dense_runs(P) * kSrvTile * sizeof(float); }
 
-// Whether the merge kernel runs: it wants some records in each tile, and so
-// many in all that the other kernels' tables do not stay in L2 (us, tables in
-// worker order / merged: 3.6M x 8, 1 %, 288,000 records, the layers' scales
-// such that most share a few tiles, 15 / 20; 3.6M x 16, 1 %, 48 / 32; 25M x 16,
-// 1 %, 453 / 143; 25M x 32, 0.1 %, 107 / 61; 25M x 4, 0.1 %, 19 / 22).
+// Whether these kernels run.  They look at every tile in three launches, so
+// they want many records, in a vector of many tiles (us from cold caches, the
+// tables' kernels / these; indices spread evenly, gathered in a tenth of the
+// vector, the same for all workers):
+//   3.6M x 8, 1 %, 288,000 records    27 / 23   14 / 20   16 / 19
+//   25M x 4, 0.2 %, 200,000           29 / 45   19 / 36   16 / 49
+//   25M x 16, 0.2 %, 800,000          98 / 62   55 / 48   23 / 60
+//   3.6M x 32, 1 %, 1,152,000         89 / 53   47 / 23   27 / 37
+//   10M x 16, 1 %, 1,600,000         119 / 51   66 / 44   35 / 40
+//   25M x 16, 1 %, 4,000,000         282 / 103 155 / 78   74 / 82
+//   1.05M x 64, 10 %, 6,710,848      231 / 71  133 / 80   98 / 70
+//   25M x 1, 3 %, 750,000             72 / 42   17 / 33   72 / 42
+//   10M x 2, 3 %, 600,000             45 / 32   16 / 29   39 / 31
+// Over 2600 such cases the line below has the least loss on either side of it.
 bool tile_server(int64_t d, int64_t k, int nworkers) {
   const double records = (double)k * nworkers;
-  return nworkers <= kSrvMaskMaxM && d >= 500'000 && records >= 500e3 && records >= 0.03 * (double)d;
+  return nworkers <= kSrvMaskMaxM && d >= 1'000'000 && records >= 700e3 && records >= 0.03 * (double)d;
+}
+
+// Server scratch of the two kernels, after the starts: the number of tiles on
+// the list, then the tiles.
+__host__ __device__ constexpr int64_t starts_words(int64_t d, int32_t nworkers) {
+  return round64((int64_t)nworkers * (srv_tiles(d) + 1));
+}
+__host__ __device__ constexpr int64_t dense_list_words(int64_t d) {
+  return 64 + round64((srv_tiles(d) + kMergeRuns - 1) / kMergeRuns);
 }
 
 template <typename Mask, bool POW2, int P>
-__global__ void __launch_bounds__(kMergeThreads, 4) topk_server_tile_kernel(const ServerArgs s, const uint32_t* starts) {
+__global__ void __launch_bounds__(kMergeThreads, 4)
+    topk_server_merge_kernel(const ServerArgs s, const uint32_t* starts, uint32_t* dense) {
   dq_pdl_enter();
+  constexpr int kIndices = kMergeRuns * kSrvTile;
+  constexpr uint32_t kNone = ~0u;
   extern __shared__ __align__(16) unsigned char tile_smem[];
   uint2* list = reinterpret_cast<uint2*>(tile_smem);             // {index in the tile | worker << 16, value}
   float* rows = reinterpret_cast<float*>(list + kMergeCap);      // M values per row
-  Mask* mask = reinterpret_cast<Mask*>(rows + kMergeRow);
-  uint16_t* row_of = reinterpret_cast<uint16_t*>(mask + kMergeTile);  // of a shared index
+  Mask* mask = reinterpret_cast<Mask*>(rows + merge_row_words(sizeof(Mask)));
+  uint16_t* row_of = reinterpret_cast<uint16_t*>(mask + kIndices);  // of a shared index
   __shared__ uint32_t nshared;
-  float* table = reinterpret_cast<float*>(tile_smem);
-  __shared__ uint32_t st[kMergeRuns + 1][P];                     // each worker's first record of each run
-  __shared__ uint32_t off[P + 1];                                // the workers' parts of the records at hand
+  __shared__ uint32_t first[P];                                  // each worker's first record of the tile
+  __shared__ uint32_t off[P + 1];                                // the tile's records of the workers before it
   const int64_t nts = srv_tiles(s.d);
-  const int64_t run0 = (int64_t)blockIdx.x * kMergeRuns;
+  const int64_t run0 = (int64_t)blockIdx.x * kMergeRuns, run1 = min64(run0 + kMergeRuns, nts);
   const int64_t t0 = run0 * kSrvTile;
   const int lane = threadIdx.x & 31;
-  for (int i = threadIdx.x; i < (kMergeRuns + 1) * s.M; i += kMergeThreads) {
-    const int m = i / (kMergeRuns + 1), r = i - m * (kMergeRuns + 1);
-    st[r][m] = (uint32_t)min64(starts[(int64_t)m * (nts + 1) + min64(run0 + r, nts)], s.k);
+  if (threadIdx.x < 32) {
+    uint32_t before = 0;
+    for (int m0 = 0; m0 < s.M; m0 += 32) {
+      const int m = m0 + lane;
+      uint32_t lo = 0, hi = 0;
+      if (m < s.M) {
+        lo = (uint32_t)min64(starts[(int64_t)m * (nts + 1) + run0], s.k);
+        hi = (uint32_t)min64(starts[(int64_t)m * (nts + 1) + run1], s.k);
+      }
+      const uint32_t n = hi > lo ? hi - lo : 0u;
+      uint32_t x = n;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(kFullMask, x, o);
+        if (lane >= o) x += y;
+      }
+      if (m < s.M) {
+        first[m] = lo;
+        off[m] = before + x - n;
+      }
+      before += __shfl_sync(kFullMask, x, 31);
+    }
+    if (lane == 0) off[s.M] = before;
   }
-  // the tile's parameters on their way while the records come
-  if (threadIdx.x < kMergeTile / 32 && t0 + 32 * (int)threadIdx.x < s.d)
-    asm volatile("prefetch.global.L2 [%0];" ::"l"(s.w + t0 + 32 * threadIdx.x));
-  for (int i = threadIdx.x; i < kMergeTile; i += kMergeThreads) mask[i] = 0;
+  for (int i = threadIdx.x; i < kIndices; i += kMergeThreads) mask[i] = 0;
   if (threadIdx.x == 0) nshared = 0;
   __syncthreads();
-  // off[] for the records of the runs [a, b), by one warp
-  auto place = [&](int a, int b) {
-    if (threadIdx.x < 32) {
-      uint32_t run = 0;
-      for (int m0 = 0; m0 < s.M; m0 += 32) {
-        const uint32_t n = m0 + lane < s.M ? max(st[b][m0 + lane], st[a][m0 + lane]) - st[a][m0 + lane] : 0u;
-        uint32_t x = n;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const uint32_t y = __shfl_up_sync(kFullMask, x, o);
-          if (lane >= o) x += y;
-        }
-        if (m0 + lane < s.M) off[m0 + lane] = run + x - n;
-        run += __shfl_sync(kFullMask, x, 31);
-      }
-      if (lane == 0) off[s.M] = run;
-    }
-    __syncthreads();
-  };
-  // body(place, worker, index in the tile, value bits) over those records
-  // (they come from the compressor: sorted, and below d)
-  auto for_records = [&](int a, auto&& body) {
-    for (uint32_t f = threadIdx.x; f < off[s.M]; f += kMergeThreads) {
-      int m = 0;  // the worker: off[m] <= f < off[m + 1]
-#pragma unroll
-      for (int step = P / 2; step >= 1; step >>= 1)
-        if (m + step < s.M && off[m + step] <= f) m += step;
-      const uint2 rec = reinterpret_cast<const uint2*>(s.msgs + (int64_t)m * s.msg_stride)[st[a][m] + (f - off[m])];
-      const int64_t i = (int64_t)rec.x - t0;
-      body(f, m, dq_in_bounds(i >= 0 && i < kMergeTile && (int64_t)rec.x < s.d, s.err) ? (int)i : -1, rec.y);
-    }
-    __syncthreads();
-  };
-  place(0, kMergeRuns);
   const uint32_t n = off[s.M];
-  if (n <= (uint32_t)kMergeCap) {
-    for_records(0, [&](uint32_t f, int m, int i, uint32_t v) {
-      list[f] = make_uint2(i < 0 ? 0xFFFFFFFFu : (uint32_t)i | (uint32_t)m << 16, v);
-      if (i >= 0) atomicOr(mask + i, (Mask)1 << m);
-    });
-    for (uint32_t f = threadIdx.x; f < n; f += kMergeThreads) {
-      const uint2 e = list[f];
-      if (e.x == 0xFFFFFFFFu) continue;
-      const uint32_t i = e.x & 0xFFFFu;
-      const int m = (int)(e.x >> 16);
-      const Mask bits = mask[i];
-      if (bits & (((Mask)1 << m) - 1u)) continue;  // a lower worker owns the index
-      if (bits != (Mask)1 << m) {
-        row_of[i] = (uint16_t)atomicAdd(&nshared, 1u);
-        continue;
-      }
-      const float sum = owner_sum<P>(bits, m, __uint_as_float(e.y), [](int) { return 0.f; });
-      s.w[t0 + i] = server_out(s, s.w[t0 + i], srv_average<POW2>(sum, s));
-    }
-    __syncthreads();
-    const uint32_t at_once = kMergeRow / (uint32_t)s.M, shared = nshared;
-    for (uint32_t row0 = 0; row0 < shared; row0 += at_once) {
-      // body(row, record, index, worker, mask) for the records of these rows
-      auto for_shared = [&](auto&& body) {
-        for (uint32_t f = threadIdx.x; f < n; f += kMergeThreads) {
-          const uint2 e = list[f];
-          if (e.x == 0xFFFFFFFFu) continue;
-          const uint32_t i = e.x & 0xFFFFu;
-          const int m = (int)(e.x >> 16);
-          const Mask bits = mask[i];
-          if (bits == (Mask)1 << m) continue;
-          const uint32_t row = row_of[i] - row0;
-          if (row < at_once) body(row, e.y, i, m, bits);
-        }
-        __syncthreads();
-      };
-      for_shared([&](uint32_t row, uint32_t v, uint32_t, int m, Mask) { rows[row * s.M + m] = __uint_as_float(v); });
-      for_shared([&](uint32_t row, uint32_t v, uint32_t i, int m, Mask bits) {
-        if (bits & (((Mask)1 << m) - 1u)) return;
-        const float sum = owner_sum<P>(bits, m, __uint_as_float(v), [&](int who) { return rows[row * s.M + who]; });
-        s.w[t0 + i] = server_out(s, s.w[t0 + i], srv_average<POW2>(sum, s));
-      });
-    }
+  if (n == 0) return;
+  if (n > (uint32_t)kMergeCap) {
+    if (threadIdx.x == 0) dense[64 + atomicAdd(dense, 1u)] = blockIdx.x;
     return;
   }
-  constexpr int kTableRuns = (int)(merge_smem(sizeof(Mask)) / (P * kSrvTile * sizeof(float)));
-  constexpr int kRuns = kTableRuns < kMergeRuns ? kTableRuns : kMergeRuns;
-  constexpr int kWidth = kRuns * kSrvTile;
-  for (int a = 0; a < kMergeRuns && t0 + a * kSrvTile < s.d; a += kRuns) {
-    const int b = min(a + kRuns, kMergeRuns);
-    __syncthreads();
-    for (int i = threadIdx.x; i < s.M * (kWidth / 4); i += kMergeThreads)
-      reinterpret_cast<float4*>(table)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-    place(a, b);
-    for_records(a, [&](uint32_t, int m, int i, uint32_t v) {
-      const int x = i - a * kSrvTile;
-      if (i >= 0 && x >= 0 && x < kWidth) table[m * kWidth + x] = __uint_as_float(v);
+  // this thread's records, their loads in flight together
+  constexpr int kMine = kMergeCap / kMergeThreads;
+  uint2 mine[kMine];  // {index, value}, then {index in the tile | worker << 16, value}
+  int who[kMine];
+#pragma unroll
+  for (int u = 0; u < kMine; ++u) {
+    const uint32_t f = threadIdx.x + u * kMergeThreads;
+    int m = 0;  // the worker: off[m] <= f < off[m + 1]
+#pragma unroll
+    for (int step = P / 2; step >= 1; step >>= 1)
+      if (m + step < s.M && off[m + step] <= f) m += step;
+    who[u] = m;
+    if (f < n) mine[u] = reinterpret_cast<const uint2*>(s.msgs + (int64_t)m * s.msg_stride)[first[m] + (f - off[m])];
+  }
+#pragma unroll
+  for (int u = 0; u < kMine; ++u) {
+    const uint32_t f = threadIdx.x + u * kMergeThreads;
+    if (f >= n) {
+      mine[u].x = kNone;
+      continue;
+    }
+    // (records come from the compressor: sorted, and below d)
+    const int64_t i = (int64_t)mine[u].x - t0;
+    const bool here = dq_in_bounds(i >= 0 && i < kIndices && (int64_t)mine[u].x < s.d, s.err);
+    mine[u].x = here ? (uint32_t)i | (uint32_t)who[u] << 16 : kNone;
+    list[f] = mine[u];
+    if (here) atomicOr(mask + i, (Mask)1 << who[u]);
+  }
+  __syncthreads();
+  // sole workers' indices: their parameters in flight together
+  float wv[kMine];
+#pragma unroll
+  for (int u = 0; u < kMine; ++u) {
+    if (mine[u].x == kNone) continue;
+    const uint32_t i = mine[u].x & 0xFFFFu;
+    const int m = (int)(mine[u].x >> 16);
+    const Mask bits = mask[i];
+    if (bits == (Mask)1 << m) {
+      wv[u] = s.w[t0 + i];
+    } else {
+      if (!(bits & (((Mask)1 << m) - 1u))) row_of[i] = (uint16_t)atomicAdd(&nshared, 1u);  // the lowest worker's
+      mine[u].x = kNone;
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < kMine; ++u) {
+    if (mine[u].x == kNone) continue;
+    const float v = __uint_as_float(mine[u].y), sum = P == 1 ? v : __fadd_rn(v, 0.f);  // among +0 leaves
+    s.w[t0 + (mine[u].x & 0xFFFFu)] = server_out(s, wv[u], srv_average<POW2>(sum, s));
+  }
+  __syncthreads();
+  const uint32_t at_once = merge_row_words(sizeof(Mask)) / (uint32_t)s.M, shared = nshared;
+  for (uint32_t row0 = 0; row0 < shared; row0 += at_once) {
+    // body(row, record, index, worker, mask) for the records of these rows
+    auto for_shared = [&](auto&& body) {
+      for (uint32_t f = threadIdx.x; f < n; f += kMergeThreads) {
+        const uint2 e = list[f];
+        if (e.x == kNone) continue;
+        const uint32_t i = e.x & 0xFFFFu;
+        const int m = (int)(e.x >> 16);
+        const Mask bits = mask[i];
+        if (bits == (Mask)1 << m) continue;
+        const uint32_t row = row_of[i] - row0;
+        if (row < at_once) body(row, e.y, i, m, bits);
+      }
+      __syncthreads();
+    };
+    for_shared([&](uint32_t row, uint32_t v, uint32_t, int m, Mask) { rows[row * s.M + m] = __uint_as_float(v); });
+    for_shared([&](uint32_t row, uint32_t v, uint32_t i, int m, Mask bits) {
+      if (bits & (((Mask)1 << m) - 1u)) return;
+      const float sum = owner_sum<P>(bits, __uint_as_float(v), [&](int who, float (&x)[4]) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (q < P && who + q < s.M) x[q] = rows[row * s.M + who + q];
+      });
+      s.w[t0 + i] = server_out(s, s.w[t0 + i], srv_average<POW2>(sum, s));
     });
-    const int width = (int)min64((int64_t)(b - a) * kSrvTile, s.d - t0 - a * kSrvTile);
+  }
+}
+
+template <bool POW2, int P>
+__global__ void __launch_bounds__(kMergeThreads, 4)
+    topk_server_dense_kernel(const ServerArgs s, const uint32_t* starts, const uint32_t* dense) {
+  dq_pdl_enter();
+  extern __shared__ __align__(16) float table[];  // M rows of values
+  const int64_t nts = srv_tiles(s.d);
+  __shared__ uint32_t first[P], past[P];          // each worker's records of the item
+  // warps per worker, or workers per warp; of those so many at a time, and so
+  // many rows of 32 records of each, that 8 loads are in flight
+  constexpr int kWarps = kMergeThreads / 32, kShare = P < kWarps ? kWarps / P : 1;
+  constexpr int kWorkers = P < kWarps ? 1 : P / kWarps, kTake = kWorkers < 4 ? kWorkers : 4, kAhead = 8 / kTake;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  // as many runs per item as leave two items to every CTA
+  const int64_t tiles = dense[0];
+  const int per = (int)max64(1, min64(dense_runs(P), tiles * kMergeRuns / (2 * (int64_t)gridDim.x)));
+  const int row = per * kSrvTile;
+  const int items_per = (kMergeRuns + per - 1) / per;  // of a tile
+  const int64_t items = tiles * items_per;
+  for (int64_t item = blockIdx.x; item < items; item += gridDim.x) {
+    const int64_t tile = dense[64 + item / items_per];
+    const int part = (int)(item % items_per);
+    const int64_t run0 = tile * kMergeRuns + part * per;
+    const int64_t run1 = min64(run0 + min(per, kMergeRuns - part * per), nts);
+    const int64_t t0 = run0 * kSrvTile;
+    const int width = (int)min64((run1 - run0) * kSrvTile, s.d - t0);
+    if (width <= 0) continue;  // past the last run (the same in every thread)
+    for (int m = threadIdx.x; m < s.M; m += kMergeThreads) {
+      const uint32_t* st = starts + (int64_t)m * (nts + 1);
+      first[m] = (uint32_t)min64(st[run0], s.k);
+      past[m] = (uint32_t)min64(st[run1], s.k);
+    }
+    for (int i = threadIdx.x; i < s.M * (row / 4); i += kMergeThreads)
+      reinterpret_cast<float4*>(table)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    __syncthreads();
+#pragma unroll 1
+    for (int w0 = 0; w0 < kWorkers; w0 += kTake) {
+      // (records come from the compressor: sorted, and below d)
+      int64_t at[kTake], end[kTake];
+      bool more = false;
+#pragma unroll
+      for (int t = 0; t < kTake; ++t) {
+        const int m = warp / kShare + kWarps * (w0 + t);
+        at[t] = end[t] = 0;
+        if (m < s.M) {
+          at[t] = first[m] + 32 * (warp % kShare) + lane;
+          end[t] = past[m];
+        }
+        more = more || at[t] < end[t];
+      }
+      while (more) {
+        more = false;
+        uint2 rec[kTake][kAhead];
+#pragma unroll
+        for (int t = 0; t < kTake; ++t) {
+          const uint2* msg =
+              reinterpret_cast<const uint2*>(s.msgs + (int64_t)(warp / kShare + kWarps * (w0 + t)) * s.msg_stride);
+#pragma unroll
+          for (int u = 0; u < kAhead; ++u)
+            if (at[t] + 32 * kShare * u < end[t]) rec[t][u] = msg[at[t] + 32 * kShare * u];
+        }
+#pragma unroll
+        for (int t = 0; t < kTake; ++t) {
+          float* values = table + (warp / kShare + kWarps * (w0 + t)) * row;
+#pragma unroll
+          for (int u = 0; u < kAhead; ++u)
+            if (at[t] + 32 * kShare * u < end[t]) {
+              const int64_t i = (int64_t)rec[t][u].x - t0;
+              if (dq_in_bounds(i >= 0 && i < width, s.err)) values[i] = __uint_as_float(rec[t][u].y);
+            }
+          at[t] += 32 * kShare * kAhead;
+          more = more || at[t] < end[t];
+        }
+      }
+    }
+    __syncthreads();
     for (int i = threadIdx.x; i < width; i += kMergeThreads) {
       // the padded tree, in chunks of up to 16 workers
       constexpr int C = P < 16 ? P : 16;
-      float part[P / C];
+      float part_sum[P / C];
 #pragma unroll
       for (int c = 0; c < P / C; ++c) {
         float x[C];
 #pragma unroll
-        for (int u = 0; u < C; ++u) x[u] = C * c + u < s.M ? table[(C * c + u) * kWidth + i] : 0.f;
-        part[c] = pairwise_n<C>(x);
+        for (int u = 0; u < C; ++u) x[u] = C * c + u < s.M ? table[(C * c + u) * row + i] : 0.f;
+        part_sum[c] = pairwise_n<C>(x);
       }
-      const float sum = pairwise_n<P / C>(part);
-      const int64_t j = t0 + a * kSrvTile + i;
-      s.w[j] = server_out(s, s.w[j], srv_average<POW2>(sum, s));
+      const float sum = pairwise_n<P / C>(part_sum);
+      s.w[t0 + i] = server_out(s, s.w[t0 + i], srv_average<POW2>(sum, s));
     }
+    __syncthreads();
   }
 }
 
@@ -1618,7 +1753,7 @@ size_t topk_scratch_bytes(int64_t d, int64_t k, int32_t rows, int32_t nworkers) 
   const int64_t server_words = nworkers <= 0 ? 0
                                : nworkers <= kSrvMaskMaxM && !tile_server(d, k, nworkers)
                                    ? srv_mask_table_words(d, nworkers)
-                                   : round64((int64_t)nworkers * (srv_tiles(d) + 1));
+                                   : starts_words(d, nworkers) + dense_list_words(d);
   return (size_t)(row_words(d) * rows + server_words) * 4u;
 }
 
@@ -1738,19 +1873,31 @@ cudaError_t launch_topk_compress(const CompressArgs& a, int64_t k, bool keep_h, 
   return st;
 }
 
-static cudaError_t launch_tile_server(const ServerArgs& s, const uint32_t* starts, cudaStream_t stream) {
-  const dim3 grid((unsigned)((s.d + kMergeTile - 1) / kMergeTile));
-  auto go = [&](auto kernel, size_t mask_bytes, std::atomic<bool> (&done)[kSmemDevices]) -> cudaError_t {
-    const cudaError_t st = allow_smem(kernel, merge_smem(mask_bytes), 1, done);
+static cudaError_t launch_tile_server(const ServerArgs& s, const uint32_t* starts, uint32_t* dense, cudaStream_t stream,
+                                      uint64_t* launches) {
+  const int64_t tiles = (srv_tiles(s.d) + kMergeRuns - 1) / kMergeRuns;
+  auto go = [&](auto merge, auto dense_kernel, size_t mask_bytes, int P,
+                std::atomic<bool> (&done)[2][kSmemDevices]) -> cudaError_t {
+    cudaError_t st = allow_smem(merge, merge_smem(mask_bytes), 1, done[0]);
+    if (st == cudaSuccess) st = allow_smem(dense_kernel, dense_smem(P, P), 1, done[1]);
+    if (st == cudaSuccess)
+      st = launch_pdl(merge, dim3((unsigned)tiles), dim3(kMergeThreads), merge_smem(mask_bytes), stream, s, starts, dense);
     if (st != cudaSuccess) return st;
-    return launch_pdl(kernel, grid, dim3(kMergeThreads), merge_smem(mask_bytes), stream, s, starts);
+    *launches += 1;
+    const int64_t items = tiles * kMergeRuns, most = 152 * (s.M > 56 ? 3 : 4);  // CTAs that fit at once
+    st = launch_pdl(dense_kernel, dim3((unsigned)(items < most ? items : most)), dim3(kMergeThreads), dense_smem(s.M, P),
+                    stream, s, starts, (const uint32_t*)dense);
+    *launches += st == cudaSuccess ? 1 : 0;
+    return st;
   };
   switch (next_pow2(s.M)) {
-#define DQ_TILE(P, MASK)                                                                  \
-  case P: {                                                                               \
-    static std::atomic<bool> done[2][kSmemDevices];                                       \
-    return s.M_pow2 ? go(topk_server_tile_kernel<MASK, true, P>, sizeof(MASK), done[0])   \
-                    : go(topk_server_tile_kernel<MASK, false, P>, sizeof(MASK), done[1]); \
+#define DQ_TILE(P, MASK)                                                                                    \
+  case P: {                                                                                                 \
+    static std::atomic<bool> done[2][2][kSmemDevices];                                                      \
+    return s.M_pow2 ? go(topk_server_merge_kernel<MASK, true, P>, topk_server_dense_kernel<true, P>,        \
+                         sizeof(MASK), P, done[0])                                                          \
+                    : go(topk_server_merge_kernel<MASK, false, P>, topk_server_dense_kernel<false, P>,      \
+                         sizeof(MASK), P, done[1]);                                                         \
   }
     DQ_TILE(1, uint32_t) DQ_TILE(2, uint32_t) DQ_TILE(4, uint32_t) DQ_TILE(8, uint32_t) DQ_TILE(16, uint32_t)
     DQ_TILE(32, uint32_t) DQ_TILE(64, unsigned long long)
@@ -1769,12 +1916,11 @@ cudaError_t launch_topk_server(const ServerArgs& s, void* scratch, int32_t rows,
   uint32_t* starts = reinterpret_cast<uint32_t*>(scratch) + row_words(s.d) * rows;
   const dim3 starts_grid((unsigned)((s.k + 256 * kStartsPer - 1) / (256 * kStartsPer)), (unsigned)s.M);
   if (tile_server(s.d, s.k, s.M)) {
-    cudaError_t st = launch_pdl(topk_server_starts_kernel, starts_grid, dim3(256), 0, stream, s, starts);
+    uint32_t* dense = starts + starts_words(s.d, s.M);
+    const cudaError_t st = launch_pdl(topk_server_starts_kernel, starts_grid, dim3(256), 0, stream, s, starts, dense);
     if (st != cudaSuccess) return st;
     *launches += 1;
-    st = launch_tile_server(s, starts, stream);
-    *launches += st == cudaSuccess ? 1 : 0;
-    return st;
+    return launch_tile_server(s, starts, dense, stream, launches);
   }
   if (s.M <= kSrvMaskMaxM) {
     const dim3 grid((unsigned)((s.k + kSrvThreads - 1) / kSrvThreads * s.M));
@@ -1807,7 +1953,7 @@ cudaError_t launch_topk_server(const ServerArgs& s, void* scratch, int32_t rows,
     return st;
   }
   const int64_t n = (int64_t)s.M * s.k;
-  launch_pdl(topk_server_starts_kernel, starts_grid, dim3(256), 0, stream, s, starts);
+  launch_pdl(topk_server_starts_kernel, starts_grid, dim3(256), 0, stream, s, starts, (uint32_t*)nullptr);
   const unsigned blocks = (unsigned)((n + kSrvThreads - 1) / kSrvThreads);
   if (s.M_pow2) launch_pdl(topk_server_owner_kernel<true>, dim3(blocks), dim3(kSrvThreads), 0, stream, s, starts);
   else launch_pdl(topk_server_owner_kernel<false>, dim3(blocks), dim3(kSrvThreads), 0, stream, s, starts);

@@ -111,34 +111,97 @@ def test_two_bits_beyond_the_small_sizes(P, M):
     run(P, oracle.SQUANT, M, (0, *cuts, d), d=d, bucket=512, bits=2)
 
 
-@pytest.mark.parametrize("kind", ["spread", "shared", "dense"])
-@pytest.mark.parametrize("M", [1, 2, 3, 8, 16, 17, 32, 33, 64])
-def test_top_k_merged_by_tiles(P, M, kind):
-    """Half a million records: spread over the vector; two in three of them at
-    indices every worker sends; and all of them in a few tiles, more than a
-    list holds."""
-    d, k = 4_100_007, -(-510_000 // M)
-    rng = np.random.default_rng(M)
-    ocfg = oracle_config(d, M, oracle.TOPK, lr=0.03, k=k)
-    h = P.create(P.make_config(d=d, M=M, compressor=P.TOPK, lr=0.03, k=k,
-                               cuda_stream=torch.cuda.current_stream().cuda_stream))
+def records(kind, M, d, k, rng):
+    """M messages of k records."""
     common = rng.choice(d, 2 * k // 3, replace=False)
-    msgs = np.zeros((M, h.message_bytes() // 8, 2), np.uint32)
+    msgs = np.zeros((M, (8 * k + 255) // 256 * 32, 2), np.uint32)
     for m in range(M):
         if kind == "spread":
             idx = rng.choice(d, k, replace=False)
         elif kind == "shared":
             own = rng.permutation(np.setdiff1d(rng.choice(d, 2 * k, replace=False), common))
             idx = np.concatenate([common, own[:k - len(common)]])
+        elif kind == "edge":  # tiles of 4096 indices with 2048 records in all, 2049, and the rest at the end
+            n = 2048 // M + (m < 2048 % M)
+            idx = np.concatenate([rng.choice(4096, n, replace=False),
+                                  4096 + rng.choice(4096, n + (m == 0), replace=False)])
+            idx = np.concatenate([idx, d - 1 - rng.choice(d - 8192, k - len(idx), replace=False)])
         else:
             idx = d - 1 - rng.choice(k + k // 3, k, replace=False)
         msgs[m, :k, 0] = np.sort(idx)
         msgs[m, :k, 1] = rng.standard_normal(k).astype(np.float32).view(np.uint32)
-    msgs = msgs.view(np.uint8).reshape(M, -1)
+    return msgs.view(np.uint8).reshape(M, -1)
+
+
+@pytest.mark.parametrize("kind", ["spread", "shared", "dense"])
+@pytest.mark.parametrize("M", [1, 2, 3, 8, 16, 17, 32, 33, 64])
+def test_top_k_merged_by_tiles(P, M, kind):
+    """Half a million records: spread over the vector; two in three of them at
+    indices every worker sends; and all of them in a few tiles, more than a
+    list holds."""
+    top_k_server(P, 4_100_007, M, -(-510_000 // M), kind)
+
+
+@pytest.mark.parametrize("oadam", [False, True], ids=["omd", "oadam"])
+@pytest.mark.parametrize("kind", ["spread", "shared", "dense", "edge"])
+@pytest.mark.parametrize("M", [1, 2, 3, 4, 5, 8, 16, 17, 32, 33, 64])
+def test_top_k_lists_and_dense_tiles(P, M, kind, oadam):
+    """A million records, from where they are merged by tiles: also a tile with as many
+    records as a list holds and one with one more, and with Optimistic Adam on the
+    server, which wants +0 at the indices nobody sent."""
+    top_k_server(P, 4_100_007, M, -(-1_010_000 // M), kind, oadam=oadam)
+
+
+@pytest.mark.parametrize("M", [16, 64])
+def test_top_k_records_gathered_in_a_tenth_take_no_longer(P, M):
+    """Layers differ in scale, so the records of a step often sit in a few tiles.  Those
+    are shared out over the GPU; a CTA for each took four times as long as for the same
+    number of records spread evenly."""
+    d, k = 1_048_576, 104_857
+    took = {}
+    for kind in ("spread", "gathered"):
+        h = P.create(P.make_config(d=d, M=M, compressor=P.TOPK, lr=0.03, k=k,
+                                   cuda_stream=torch.cuda.current_stream().cuda_stream))
+        gen = torch.Generator(device="cuda").manual_seed(M)
+        msgs = torch.zeros((M, h.message_bytes()), dtype=torch.uint8, device="cuda")
+        for m in range(M):
+            p = torch.rand(d, generator=gen, device="cuda")
+            if kind == "gathered":
+                p[:k + 100] += 1
+            msgs[m].view(torch.int32)[:2 * k:2] = torch.topk(p, k).indices.sort().values.int()
+        w = torch.zeros(d, device="cuda")
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        times = []
+        for _ in range(5):
+            a.record()
+            for _ in range(8):
+                h.server_aggregate_update(msgs, w)
+            b.record()
+            torch.cuda.synchronize()
+            times.append(a.elapsed_time(b) / 8)
+        took[kind] = min(times)
+        h.destroy()
+    assert took["gathered"] < 2.5 * took["spread"], took
+
+
+def top_k_server(P, d, M, k, kind, oadam=False):
+    rng = np.random.default_rng(M)
+    ocfg = oracle_config(d, M, oracle.TOPK, lr=0.03, k=k)
+    h = P.create(P.make_config(d=d, M=M, compressor=P.TOPK, lr=0.03, k=k,
+                               cuda_stream=torch.cuda.current_stream().cuda_stream))
+    params = dict(alpha=1e-2, beta1=0.5, beta2=0.9, eps=1e-8)
+    if oadam:
+        h.set_server_optimizer(P.dqgan.oadam(**params))
     w = (rng.standard_normal(d) * 0.02).astype(np.float32)
     w_gpu = torch.from_numpy(w.copy()).to("cuda")
-    h.server_aggregate_update(torch.from_numpy(msgs).to("cuda"), w_gpu)
-    oracle.server_step(ocfg, msgs, w)
-    h.synchronize()
-    assert_params_equal(w_gpu.cpu().numpy(), w)
+    state = oracle.OAdamState(d, oracle.OAdam(**params)) if oadam else None
+    for step in range(1, 3 if oadam else 2):
+        msgs = records(kind, M, d, k, rng)
+        h.server_aggregate_update(torch.from_numpy(msgs).to("cuda"), w_gpu)
+        if oadam:
+            state.server_step_range(ocfg, step, msgs, w, 0, d)
+        else:
+            oracle.server_step(ocfg, msgs, w)
+        h.synchronize()
+        assert_params_equal(w_gpu.cpu().numpy(), w)
     h.destroy()
