@@ -711,13 +711,9 @@ identity_compress_kernel(const CompressArgs a) {
 // CTAs of a persistent kernel per row: about four waves of resident CTAs in
 // all rows, no more than `need`.
 int64_t persistent_blocks(int64_t need, int threads, int nworkers) {
-  static int sms[64] = {0};
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return need;
-  if (sms[dev] == 0 && cudaDeviceGetAttribute(&sms[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-    sms[dev] = 0;
-  if (sms[dev] <= 0) return need;
-  const int64_t cap = ((int64_t)sms[dev] * 4 * (2048 / threads) + nworkers - 1) / nworkers;
+  const int sms = device_sms();
+  if (sms <= 0) return need;
+  const int64_t cap = ((int64_t)sms * 4 * (2048 / threads) + nworkers - 1) / nworkers;
   return need < cap ? need : max64(cap, 1);
 }
 

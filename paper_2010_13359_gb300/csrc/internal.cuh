@@ -11,6 +11,7 @@
 
 #include <cuda.h>
 
+#include <atomic>
 #include <utility>
 
 #include "dqgan.h"
@@ -156,6 +157,44 @@ template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
                               Args&&... args) {
   return launch_pdl_cluster(kern, 1, grid, block, smem, stream, std::forward<Args>(args)...);
+}
+
+// What is asked of the runtime once per device (attributes, occupancy) is kept
+// by device ordinal.  Handles may be used from several host threads, so what is
+// kept is atomic; two threads that ask at once store the same answer.
+constexpr int kKeptDevices = 64;
+
+// CTAs of `kern` with `smem` bytes of dynamic shared memory that fit on the
+// current device at once; `most`: what any launch of the kernel uses (the limit
+// belongs to the function, and the last call sets it).
+template <typename K>
+inline cudaError_t resident_ctas(K kern, int threads, int smem, int most, std::atomic<int> (&kept)[kKeptDevices],
+                                 int* ctas) {
+  int dev = 0;
+  cudaError_t st = cudaGetDevice(&dev);
+  if (st != cudaSuccess) return st;
+  if (dev < 0 || dev >= kKeptDevices) return cudaErrorInvalidDevice;
+  *ctas = kept[dev].load(std::memory_order_acquire);
+  if (*ctas != 0) return cudaSuccess;
+  int sms = 0, per_sm = 0;
+  if ((st = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most)) != cudaSuccess ||
+      (st = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess ||
+      (st = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem)) != cudaSuccess)
+    return st;
+  *ctas = sms * (per_sm > 0 ? per_sm : 1);
+  kept[dev].store(*ctas, std::memory_order_release);
+  return cudaSuccess;
+}
+
+// SMs of the current device; 0 if it cannot be asked.
+inline int device_sms() {
+  static std::atomic<int> kept[kKeptDevices];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kKeptDevices) return 0;
+  int sms = kept[dev].load(std::memory_order_acquire);
+  if (sms == 0 && cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess)
+    kept[dev].store(sms, std::memory_order_release);
+  return sms;
 }
 
 // Kernel launchers: each enqueues its kernels on `stream`, adds the number of

@@ -1592,23 +1592,13 @@ template <int NG, bool POW2, bool SEG>
 cudaError_t launch_sign_tma(const ServerArgs& s, const SignServerExtras& x, cudaStream_t stream) {
   auto kern = sign_server_tma_kernel<NG, POW2, SEG>;
   constexpr int smem = tma_sign_smem_bytes<SEG>();
-  int dev = 0;
-  cudaError_t st = cudaGetDevice(&dev);
+  static std::atomic<int> kept[kKeptDevices];
+  int cap = 0;
+  const cudaError_t st = resident_ctas(kern, 32 * kTmaWarps, smem, smem, kept, &cap);
   if (st != cudaSuccess) return st;
-  static int blocks_for[64] = {0};
-  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-  if (blocks_for[dev] == 0) {
-    if ((st = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess)
-      return st;
-    int sms = 0, per_sm = 0;
-    if ((st = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return st;
-    if ((st = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * kTmaWarps, smem)) != cudaSuccess)
-      return st;
-    blocks_for[dev] = sms * (per_sm > 0 ? per_sm : 1);
-  }
   const int64_t warps = SEG ? x.seg_nslices : ((s.d + s.bucket - 1) / s.bucket) * (s.bucket / 1024);
   const int64_t need = (warps + kTmaWarps - 1) / kTmaWarps;
-  const unsigned blocks = (unsigned)(need < blocks_for[dev] ? need : blocks_for[dev]);
+  const unsigned blocks = (unsigned)(need < cap ? need : cap);
   if (blocks == 0) return cudaSuccess;
   launch_pdl(kern, dim3(blocks), dim3(32 * kTmaWarps), smem, stream, s, SegSlices{x.seg_slices, x.seg_nslices},
              *s.sign_words_map);
@@ -1619,23 +1609,13 @@ template <int NG, bool POW2, bool SEG>
 cudaError_t launch_sign_col(const ServerArgs& s, const SignServerExtras& x, cudaStream_t stream) {
   auto kern = sign_server_col_kernel<NG, POW2, SEG>;
   constexpr int smem = ColLayout<SEG>::kSmem;
-  int dev = 0;
-  cudaError_t st = cudaGetDevice(&dev);
+  static std::atomic<int> kept[kKeptDevices];
+  int cap = 0;
+  const cudaError_t st = resident_ctas(kern, 32 * kColWarps, smem, smem, kept, &cap);
   if (st != cudaSuccess) return st;
-  static int blocks_for[64] = {0};
-  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-  if (blocks_for[dev] == 0) {
-    if ((st = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess)
-      return st;
-    int sms = 0, per_sm = 0;
-    if ((st = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return st;
-    if ((st = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * kColWarps, smem)) != cudaSuccess)
-      return st;
-    blocks_for[dev] = sms * (per_sm > 0 ? per_sm : 1);
-  }
   const int64_t nslices = SEG ? x.seg_nslices : ((s.d + s.bucket - 1) / s.bucket) * (s.bucket / 1024);
   const int64_t need = (nslices + kColWarps - 1) / kColWarps;
-  const unsigned blocks = (unsigned)(need < blocks_for[dev] ? need : blocks_for[dev]);
+  const unsigned blocks = (unsigned)(need < cap ? need : cap);
   if (blocks == 0) return cudaSuccess;
   launch_pdl(kern, dim3(blocks), dim3(32 * kColWarps), smem, stream, s, SegSlices{x.seg_slices, x.seg_nslices}, *s.sign_words_map,
                                                   *x.params_map);
@@ -1646,12 +1626,8 @@ cudaError_t launch_sign_col(const ServerArgs& s, const SignServerExtras& x, cuda
 // one or two the latency of a slice's chain (copies in, transpose, store)
 // shows and the bit-transpose kernel is as fast or faster.
 bool sign_col_pays(int64_t nslices) {
-  static int sms[64] = {0};
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
-  if (sms[dev] == 0 && cudaDeviceGetAttribute(&sms[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-    return false;
-  return nslices >= 4ll * sms[dev] * kColWarps;
+  const int sms = device_sms();
+  return sms > 0 && nslices >= 4ll * sms * kColWarps;
 }
 
 template <int BITS, bool POW2, bool SEG, int NSET, int FM = 0>
@@ -1659,25 +1635,12 @@ cudaError_t launch_squant_tma(const ServerArgs& s, const CUtensorMap* params_map
   auto kern = squant_server_tma_kernel<BITS, POW2, SEG, NSET, FM>;
   constexpr int pbox = sq_params_boxed(BITS) ? 32 * (32 / BITS) * 4 : 0;  // bytes of a parameter box
   const int smem = kTmaWarps * 2 * (pbox + s.M * 128) + 1024;  // + alignment slack
-  int dev = 0;
-  cudaError_t st = cudaGetDevice(&dev);
+  constexpr int most = kTmaWarps * 2 * (pbox + 32 * 128) + 1024;  // of any worker count
+  // kept by worker count (asking on every call took a quarter of a small call's time)
+  static std::atomic<int> kept[33][kKeptDevices];
+  int cap = 0;
+  const cudaError_t st = resident_ctas(kern, 32 * kTmaWarps, smem, most, kept[s.M], &cap);
   if (st != cudaSuccess) return st;
-  // resident CTAs on the device by worker count (asking on every call took a
-  // quarter of a small call's time)
-  static std::atomic<int> blocks_for[64][33];
-  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-  int cap = blocks_for[dev][s.M].load(std::memory_order_acquire);
-  if (cap == 0) {
-    constexpr int most = kTmaWarps * 2 * (pbox + 32 * 128) + 1024;  // of any worker count
-    if ((st = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most)) != cudaSuccess)
-      return st;
-    int sms = 0, per_sm = 0;
-    if ((st = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return st;
-    if ((st = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * kTmaWarps, smem)) != cudaSuccess)
-      return st;
-    cap = sms * (per_sm > 0 ? per_sm : 1);
-    blocks_for[dev][s.M].store(cap, std::memory_order_release);
-  }
   const int64_t nslices = SEG ? (s.d + 32 * (32 / BITS) - 1) / (32 * (32 / BITS))
                               : ((s.d + s.bucket - 1) / s.bucket) * (s.bucket / (32 * (32 / BITS)));
   const int64_t need = (nslices + kTmaWarps - 1) / kTmaWarps;
@@ -1692,22 +1655,12 @@ cudaError_t launch_squant_table(const ServerArgs& s, const SignServerExtras& x, 
   auto kern = squant_server_table_kernel<BITS, NG, FULL>;
   constexpr int box = (4 * NG * kSignSegBoxWords * 4 + 127) / 128 * 128;
   constexpr int smem = kTmaWarps * 2 * box + 128;  // + alignment slack
-  int dev = 0;
-  cudaError_t st = cudaGetDevice(&dev);
+  static std::atomic<int> kept[kKeptDevices];
+  int cap = 0;
+  const cudaError_t st = resident_ctas(kern, 32 * kTmaWarps, smem, smem, kept, &cap);
   if (st != cudaSuccess) return st;
-  static int blocks_for[64] = {0};
-  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-  if (blocks_for[dev] == 0) {
-    if ((st = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess)
-      return st;
-    int sms = 0, per_sm = 0;
-    if ((st = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return st;
-    if ((st = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * kTmaWarps, smem)) != cudaSuccess)
-      return st;
-    blocks_for[dev] = sms * (per_sm > 0 ? per_sm : 1);
-  }
   const int64_t need = (x.seg_nslices + kTmaWarps - 1) / kTmaWarps;
-  const unsigned blocks = (unsigned)(need < blocks_for[dev] ? need : blocks_for[dev]);
+  const unsigned blocks = (unsigned)(need < cap ? need : cap);
   return launch_pdl(kern, dim3(blocks), dim3(32 * kTmaWarps), smem, stream, s, SegSlices{x.seg_slices, x.seg_nslices},
                     *s.squant_words_map);
 }
@@ -1913,17 +1866,14 @@ using EncodeFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, voi
 // cuTensorMapEncodeTiled through the runtime's driver entry point (no link
 // against libcuda); nullptr if it is unavailable.
 EncodeFn tensor_map_encoder() {
-  static EncodeFn encode = nullptr;
-  static bool looked_up = false;
-  if (!looked_up) {
-    looked_up = true;
+  static const EncodeFn encode = []() -> EncodeFn {
     void* fn = nullptr;
     cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) ==
-            cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      encode = reinterpret_cast<EncodeFn>(fn);
-  }
+    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+        q != cudaDriverEntryPointSuccess)
+      return nullptr;
+    return reinterpret_cast<EncodeFn>(fn);
+  }();
   return encode;
 }
 

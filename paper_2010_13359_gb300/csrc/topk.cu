@@ -1779,14 +1779,12 @@ static unsigned select_blocks(int64_t d, int nworkers) {
 // more than 8 CTAs, their size).  The attributes belong to the function on the
 // current device, so that they were set is remembered per device ordinal.
 // Several host threads may race to set them; setting them twice is harmless.
-constexpr int kSmemDevices = 64;
-
 template <typename K>
-static cudaError_t allow_smem(K kernel, size_t bytes, int cluster, std::atomic<bool> (&done)[kSmemDevices]) {
+static cudaError_t allow_smem(K kernel, size_t bytes, int cluster, std::atomic<bool> (&done)[kKeptDevices]) {
   int dev = 0;
   cudaError_t st = cudaGetDevice(&dev);
   if (st != cudaSuccess) return st;
-  const bool known = dev >= 0 && dev < kSmemDevices;
+  const bool known = dev >= 0 && dev < kKeptDevices;
   if (known && done[dev].load(std::memory_order_acquire)) return cudaSuccess;
   st = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   if (st == cudaSuccess && cluster > 8)
@@ -1824,8 +1822,8 @@ static int chip_ctas(int64_t d, int nworkers) {
 }
 
 static cudaError_t launch_chip(int ctas, bool keep_h, const CompressArgs& a, int64_t k, cudaStream_t stream) {
-  static std::atomic<bool> done[3][2][kSmemDevices];
-  auto go = [&](auto kernel, int n, std::atomic<bool> (&set)[kSmemDevices]) -> cudaError_t {
+  static std::atomic<bool> done[3][2][kKeptDevices];
+  auto go = [&](auto kernel, int n, std::atomic<bool> (&set)[kKeptDevices]) -> cudaError_t {
     const cudaError_t st = allow_smem(kernel, kChipMax * sizeof(float), n, set);
     if (st != cudaSuccess) return st;
     const size_t need = (size_t)chip_part(a.d, n) * sizeof(float);
@@ -1841,7 +1839,7 @@ static cudaError_t launch_chip(int ctas, bool keep_h, const CompressArgs& a, int
 
 cudaError_t launch_topk_compress(const CompressArgs& a, int64_t k, bool keep_h, void* scratch,
                                  cudaStream_t stream, uint64_t* launches) {
-  static std::atomic<bool> emit_done[kSmemDevices];
+  static std::atomic<bool> emit_done[kKeptDevices];
   const unsigned rows = (unsigned)a.nworkers;
   cudaError_t st = cudaSuccess;
   auto launched = [&](cudaError_t r) {
@@ -1877,7 +1875,7 @@ static cudaError_t launch_tile_server(const ServerArgs& s, const uint32_t* start
                                       uint64_t* launches) {
   const int64_t tiles = (srv_tiles(s.d) + kMergeRuns - 1) / kMergeRuns;
   auto go = [&](auto merge, auto dense_kernel, size_t mask_bytes, int P,
-                std::atomic<bool> (&done)[2][kSmemDevices]) -> cudaError_t {
+                std::atomic<bool> (&done)[2][kKeptDevices]) -> cudaError_t {
     cudaError_t st = allow_smem(merge, merge_smem(mask_bytes), 1, done[0]);
     if (st == cudaSuccess) st = allow_smem(dense_kernel, dense_smem(P, P), 1, done[1]);
     if (st == cudaSuccess)
@@ -1893,7 +1891,7 @@ static cudaError_t launch_tile_server(const ServerArgs& s, const uint32_t* start
   switch (next_pow2(s.M)) {
 #define DQ_TILE(P, MASK)                                                                                    \
   case P: {                                                                                                 \
-    static std::atomic<bool> done[2][2][kSmemDevices];                                                      \
+    static std::atomic<bool> done[2][2][kKeptDevices];                                                      \
     return s.M_pow2 ? go(topk_server_merge_kernel<MASK, true, P>, topk_server_dense_kernel<true, P>,        \
                          sizeof(MASK), P, done[0])                                                          \
                     : go(topk_server_merge_kernel<MASK, false, P>, topk_server_dense_kernel<false, P>,      \
