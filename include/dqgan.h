@@ -146,7 +146,9 @@ DQGAN_API int dqgan_validate_config(const dqgan_config* cfg);
  * dqgan_last_error(NULL) holds the reason, and nothing stays allocated.
  * Test hook: with the environment variable DQGAN_TEST_FAIL_ALLOC=N set, the
  * N-th device allocation this thread makes from this call on (through later
- * calls as well) fails as out of memory, once.
+ * calls as well) fails as out of memory, once.  With DQGAN_TEST_NO_CLUSTERS
+ * set at the process's first top-k step, that and later steps take the forms
+ * for a device part on which no cluster of 8 or 16 blocks fits.
  */
 DQGAN_API int dqgan_create(const dqgan_config* cfg, dqgan_handle** out);
 

@@ -50,6 +50,7 @@
 // tile.
 #include <atomic>
 #include <cmath>
+#include <cstdlib>
 
 #include <cooperative_groups.h>
 
@@ -1758,10 +1759,11 @@ size_t topk_scratch_bytes(int64_t d, int64_t k, int32_t rows, int32_t nworkers) 
 }
 
 // Rank in a sample block that its estimate of tau has to reach, or 0 where
-// every element is a candidate instead: k is so near d that a sample rules
-// nothing out.
+// every non-zero element is a candidate instead: k is so near d that a sample
+// rules nothing out, or the vector is smaller than the sample.
 static uint32_t sample_rank(int64_t d, int64_t k) {
   const double expected = (double)k * kSamples / (double)d;
+  if (d < kSamples) return 0;
   const double rank = std::ceil((expected + 7.0 * std::sqrt(expected) + 12.0) / kSampBlocks);
   return rank < (double)(kSamples / kSampBlocks) ? (uint32_t)rank : 0u;
 }
@@ -1793,48 +1795,89 @@ static cudaError_t allow_smem(K kernel, size_t bytes, int cluster, std::atomic<b
   return st;
 }
 
+// The kernel that keeps p on chip in C CTAs, and the attributes it needs.
+template <int C>
+static cudaError_t launch_chip(bool keep_h, const CompressArgs& a, int64_t k, cudaStream_t stream) {
+  static std::atomic<bool> done[2][kKeptDevices];
+  auto go = [&](auto kernel, std::atomic<bool> (&set)[kKeptDevices]) -> cudaError_t {
+    const cudaError_t st = allow_smem(kernel, kChipMax * sizeof(float), C, set);
+    if (st != cudaSuccess) return st;
+    const size_t need = (size_t)chip_part(a.d, C) * sizeof(float);
+    return launch_pdl_cluster(kernel, C, dim3((unsigned)C, (unsigned)a.nworkers), dim3(kChipThreads), need, stream, a, k);
+  };
+  return keep_h ? go(topk_chip_kernel<C, true>, done[0]) : go(topk_chip_kernel<C, false>, done[1]);
+}
+
+// Workers whose C CTAs fit on the current device at once: 152, 15 and 7 for 1, 8
+// and 16 on a whole GB300; less, or 0, on a part of one, where the launch would
+// fail.  Asked once per device, with all the shared memory that a part may take.
+// (Test hook: DQGAN_TEST_NO_CLUSTERS in the environment then makes it 0 for
+// more than one CTA.)
+template <int C>
+static int chip_resident() {
+  static std::atomic<int> kept[kKeptDevices];  // plus 1
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kKeptDevices) return 0;
+  int n = kept[dev].load(std::memory_order_acquire);
+  if (n == 0) {
+    static std::atomic<bool> done[kKeptDevices];
+    const auto kernel = topk_chip_kernel<C, true>;
+    int fit = 0;
+    if (C > 1 && std::getenv("DQGAN_TEST_NO_CLUSTERS")) {
+      fit = 0;
+    } else if (allow_smem(kernel, kChipMax * sizeof(float), C, done) == cudaSuccess) {
+      if constexpr (C == 1) {
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, kernel, kChipThreads, kChipMax * sizeof(float)) !=
+            cudaSuccess)
+          fit = 0;
+        fit *= device_sms();
+      } else {
+        cudaLaunchConfig_t lc = {};
+        lc.gridDim = dim3(C);
+        lc.blockDim = dim3(kChipThreads);
+        lc.dynamicSmemBytes = kChipMax * sizeof(float);
+        cudaLaunchAttribute attr;
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = C;
+        attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+        lc.attrs = &attr;
+        lc.numAttrs = 1;
+        if (cudaOccupancyMaxActiveClusters(&fit, kernel, &lc) != cudaSuccess) fit = 0;
+      }
+    }
+    cudaGetLastError();  // a form that does not fit is not an error of the call
+    n = fit + 1;
+    kept[dev].store(n, std::memory_order_release);
+  }
+  return n - 1;
+}
+
 // CTAs per worker of the kernel that keeps p on chip, or 0 where the five
 // kernels are taken: the least of the times that fit what was measured (us,
 // k = d / 100, d from 4096 to 786,432, 1 to 64 workers).  On chip, a wave of
-// as many workers as are resident (152 SMs; 15 clusters of 8; 7 of 16) costs a
-// fixed latency and 0.45 per 1024 elements of a part; the five kernels cost
-// 20, their memory traffic, and a little for every worker's sample.  E.g. one
-// worker, d = 65,536: 9.1 with 16 CTAs (9.9 with 8, 21 with the five kernels);
-// 16 workers of 65,536: 24 with 8 CTAs, 31 with 16, 30 with the five; 64
-// workers of 32,768: 26 with 1, 50 with 8.  (Each with its server step.)
-// Below kSamples the five kernels have no sample, and 70 to 135.
+// as many workers as are resident costs a fixed latency and 0.45 per 1024
+// elements of a part; the five kernels cost 20, their memory traffic, and a
+// little for every worker's sample.  E.g. one worker, d = 65,536: 9.1 with 16
+// CTAs (9.9 with 8, 21 with the five kernels); 16 workers of 65,536: 24 with 8
+// CTAs, 31 with 16, 30 with the five; 64 workers of 32,768: 26 with 1, 50 with
+// 8.  (Each with its server step.)  Below kSamples the five kernels have no
+// sample, every non-zero element is a candidate, and they cost some 50 more.
 static int chip_ctas(int64_t d, int nworkers) {
-  double best = d < kSamples ? INFINITY : 20.0 + 2.2e-6 * (double)d * nworkers + 0.15 * nworkers;
+  double best = 20.0 + 2.2e-6 * (double)d * nworkers + 0.15 * nworkers + (d < kSamples ? 50.0 : 0.0);
   int ctas = 0;
   auto consider = [&](int n, int resident, double latency) {
     const int64_t part = chip_part(d, n);
-    if (part > kChipMax) return;
+    if (part > kChipMax || resident == 0) return;
     const double t = ((nworkers + resident - 1) / resident) * (latency + 0.45 * (double)part / 1024.0);
     if (t < best) {
       best = t;
       ctas = n;
     }
   };
-  consider(1, 152, 4.0);
-  consider(8, 15, 6.8);
-  consider(16, 7, 7.5);
+  consider(1, chip_resident<1>(), 4.0);
+  consider(8, chip_resident<8>(), 6.8);
+  consider(16, chip_resident<16>(), 7.5);
   return ctas;
-}
-
-static cudaError_t launch_chip(int ctas, bool keep_h, const CompressArgs& a, int64_t k, cudaStream_t stream) {
-  static std::atomic<bool> done[3][2][kKeptDevices];
-  auto go = [&](auto kernel, int n, std::atomic<bool> (&set)[kKeptDevices]) -> cudaError_t {
-    const cudaError_t st = allow_smem(kernel, kChipMax * sizeof(float), n, set);
-    if (st != cudaSuccess) return st;
-    const size_t need = (size_t)chip_part(a.d, n) * sizeof(float);
-    return launch_pdl_cluster(kernel, n, dim3((unsigned)n, (unsigned)a.nworkers), dim3(kChipThreads), need, stream, a, k);
-  };
-  const int h = keep_h ? 1 : 0;
-  switch (ctas) {
-    case 1: return go(keep_h ? topk_chip_kernel<1, true> : topk_chip_kernel<1, false>, 1, done[0][h]);
-    case 8: return go(keep_h ? topk_chip_kernel<8, true> : topk_chip_kernel<8, false>, 8, done[1][h]);
-    default: return go(keep_h ? topk_chip_kernel<16, true> : topk_chip_kernel<16, false>, 16, done[2][h]);
-  }
 }
 
 cudaError_t launch_topk_compress(const CompressArgs& a, int64_t k, bool keep_h, void* scratch,
@@ -1847,9 +1890,10 @@ cudaError_t launch_topk_compress(const CompressArgs& a, int64_t k, bool keep_h, 
     if (st == cudaSuccess) *launches += 1;
     return st == cudaSuccess;
   };
-  if (const int ctas = chip_ctas(a.d, a.nworkers)) {
-    launched(launch_chip(ctas, keep_h, a, k, stream));
-    return st;
+  switch (chip_ctas(a.d, a.nworkers)) {
+    case 1: launched(launch_chip<1>(keep_h, a, k, stream)); return st;
+    case 8: launched(launch_chip<8>(keep_h, a, k, stream)); return st;
+    case 16: launched(launch_chip<16>(keep_h, a, k, stream)); return st;
   }
   const dim3 tiles((unsigned)tiles_of(a.d), rows), select(select_blocks(a.d, a.nworkers), rows);
   // the rows that a tile with its share of 1.3 k candidates has

@@ -21,6 +21,10 @@ for bit with numpy on the same fp32 p:
 """
 from __future__ import annotations
 
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -150,3 +154,42 @@ def test_sparse_gradients_take_a_few_times_a_dense_one(P, d, M):
         took[kind] = min(times)
         h.destroy()
     assert took["sparse"] < 5 * took["gauss"], took
+
+
+# run by a child process: the sizes that take clusters of CTAs, and those that would take them
+NO_CLUSTERS = r"""
+import numpy as np, torch
+import paper_2010_13359_gb300 as P
+import oracle
+stream = torch.cuda.current_stream()
+for d, M, k, launches in ((300_007, 1, 3_000, 5), (65_535, 2, 700, 5), (49_153, 1, 20, 5), (786_431, 3, 8_000, 5),
+                          (65_536, 4, 60_000, 5), (40_000, 9, 400, 1), (33, 1, 3, 1)):
+    h = P.create(P.make_config(d=d, M=M, compressor=P.TOPK, lr=0.5, k=k, cuda_stream=stream.cuda_stream))
+    cfg = oracle.Config(d=d, M=M, compressor=oracle.TOPK, lr=0.5, k=k)
+    st = oracle.State(cfg)
+    ld = (d + 3) // 4 * 4
+    g_dev = torch.zeros((M, ld), device="cuda")
+    msgs = torch.zeros((M, h.message_bytes()), dtype=torch.uint8, device="cuda")
+    for step in range(2):
+        g = np.random.default_rng(step).standard_normal((M, d)).astype(np.float32)
+        g_dev[:, :d] = torch.from_numpy(g)
+        before = h.launch_count()
+        h.workers_compress_all(g_dev, ld, msgs)
+        assert h.launch_count() - before == launches, (d, M, h.launch_count() - before)
+        want = st.compress_all(g)
+        h.synchronize()
+        got = msgs.cpu().numpy()
+        for i in range(M):
+            assert np.array_equal(got[i, :8 * k], want[i][:8 * k]), (d, M, step, i)
+    h.destroy()
+print("no clusters: ok")
+"""
+
+
+def test_a_device_part_without_room_for_clusters(P):
+    """Where no cluster of 8 or 16 CTAs fits (a part of a device), their launch would fail;
+    those sizes take the five kernels then, below the sample's size too."""
+    env = dict(os.environ, DQGAN_TEST_NO_CLUSTERS="1")
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    res = subprocess.run([sys.executable, "-c", NO_CLUSTERS], cwd=root, env=env, capture_output=True, text=True, timeout=600)
+    assert res.returncode == 0 and "no clusters: ok" in res.stdout, res.stdout + res.stderr
