@@ -329,7 +329,7 @@ DQGAN_API int dqgan_set_segments(dqgan_handle* h, const int64_t* offsets, int32_
  *   else u = m_hat;
  *   w = w - alpha (2 u - u_prev);   u_prev = u.
  * m, v and u_prev start at 0 and are library-owned (with the q_hat buffer,
- * 4 x d fp32).  With
+ * 4 x d fp32; 3 x d with DQGAN_IDENTITY, which needs none).  With
  * b1 = 0, no DQGAN_OADAM_ADAPTIVE and alpha = 1 the update is
  * w_t = w_{t-1} - 2 q_hat_t + q_hat_{t-1}, the one-line OMD recurrence of
  * Section 2.2.  With top-k messages every parameter moves, not only the
@@ -352,7 +352,7 @@ typedef struct dqgan_server_optimizer {
 
 /* Choose the server update rule; only before the first step (step counter
  * 1, else DQGAN_ERR_INVALID_ARG).  DQGAN_SERVER_OADAM allocates m, v, u_prev
- * and the q_hat buffer (4 x d fp32, zero; DQGAN_ERR_OOM if that fails) and
+ * and the q_hat buffer (zero; DQGAN_ERR_OOM if that fails) and
  * adds m, v, u_prev to the
  * checkpoint state; DQGAN_SERVER_OMD frees them.  DQGAN_ERR_UNSUPPORTED for
  * DQGAN_TOPK with more than 64 workers.  Synchronous. */

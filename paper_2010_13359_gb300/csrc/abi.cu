@@ -39,8 +39,8 @@ struct dqgan_handle {
   bool params_map_ok = false;
   int32_t sign_path = 0;         // DQGAN_SIGN_SERVER at creation: 0 auto, 1 col, 2 tma
   dqgan_server_optimizer opt{};  // server update rule (kind DQGAN_SERVER_OMD: w = w - q_hat)
-  float* opt_m = nullptr;        // Optimistic Adam: m, v, u_prev and the server's q_hat
-  float* opt_v = nullptr;        // (d fp32 each, rows of one allocation)
+  float* opt_m = nullptr;        // Optimistic Adam: m, v, u_prev and (not identity, whose server
+  float* opt_v = nullptr;        // updates them itself) q_hat (d fp32 each, rows of one allocation)
   float* opt_u = nullptr;
   float* opt_q = nullptr;
   float pow1 = 1.f, pow2 = 1.f;  // b1^pow_t, b2^pow_t as fp32 running products
@@ -665,9 +665,10 @@ int dqgan_server_aggregate_update(dqgan_handle* h, const void* msgs_all, float* 
   s.sign_words_map = nullptr;
   s.squant_words_map = nullptr;
   // Optimistic Adam: the server kernel writes q_hat to the handle's buffer,
-  // then one dense pass updates m, v, u_prev and the parameters
+  // then one dense pass updates m, v, u_prev and the parameters (identity: the
+  // server kernel updates them)
   const bool oadam = h->opt_m != nullptr;
-  if (oadam) {
+  if (oadam && h->opt_q) {
     s.w = h->opt_q;
     s.store_q = 1;
   }
@@ -917,7 +918,9 @@ int dqgan_set_server_optimizer(dqgan_handle* h, const dqgan_server_optimizer* op
   h->pow_t = 0;
   if (opt->kind == DQGAN_SERVER_OMD) return DQGAN_OK;
   const int64_t ld = round_up(h->cfg.d, 64);
-  if ((st = dq_malloc(&h->opt_m, (size_t)(4 * ld) * 4)) != cudaSuccess) {
+  const bool q_row = h->cfg.compressor != DQGAN_IDENTITY;
+  const size_t bytes = (size_t)((q_row ? 4 : 3) * ld) * sizeof(float);
+  if ((st = dq_malloc(&h->opt_m, bytes)) != cudaSuccess) {
     cudaGetLastError();
     h->opt_m = nullptr;
     h->opt.kind = DQGAN_SERVER_OMD;
@@ -926,8 +929,8 @@ int dqgan_set_server_optimizer(dqgan_handle* h, const dqgan_server_optimizer* op
   }
   h->opt_v = h->opt_m + ld;
   h->opt_u = h->opt_v + ld;
-  h->opt_q = h->opt_u + ld;
-  if ((st = cudaMemset(h->opt_m, 0, (size_t)(4 * ld) * 4)) != cudaSuccess)
+  h->opt_q = q_row ? h->opt_u + ld : nullptr;
+  if ((st = cudaMemset(h->opt_m, 0, bytes)) != cudaSuccess)
     return cuda_fail(h, st, "zeroing the optimizer state");
   return DQGAN_OK;
 }

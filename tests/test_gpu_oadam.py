@@ -197,3 +197,16 @@ def test_oadam_argument_checks(P):
         h.set_server_optimizer(P.dqgan.oadam(**ADAM))
     assert ei.value.status == P.dqgan.ERR_UNSUPPORTED
     h.destroy()
+
+
+def test_identity_keeps_three_rows(P):
+    """The identity server updates m, v, u_prev and w where it forms q_hat: no row for q_hat."""
+    d = 16_000_000
+    for compressor, rows in ((oracle.IDENTITY, 3), (oracle.SIGN, 4)):
+        h = P.create(P.make_config(d=d, M=1, compressor=compressor, lr=0.1, bucket=1024,
+                                   cuda_stream=torch.cuda.current_stream().cuda_stream))
+        before = torch.cuda.mem_get_info()[0]
+        h.set_server_optimizer(P.dqgan.oadam(1e-3, 0.5, 0.999, 1e-8))
+        used = before - torch.cuda.mem_get_info()[0]
+        h.destroy()
+        assert abs(used - rows * 4 * d) <= 4 << 20, (compressor, used)
