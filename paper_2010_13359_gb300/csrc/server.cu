@@ -714,8 +714,12 @@ sign_server_col_kernel(const ServerArgs s, const SegSlices seg, const __grid_con
 // are decoded.  For b = 4, 8 V lives in shared memory replicated once per bank
 // (entry c of lane l at [c][l]), so the random code lookups of a warp never
 // conflict; for b = 2 (V in {-1, 0, +1}) the value is a select.
+// Above 64 workers the blocks' sums take registers too: held to the same 64 they
+// spill, and b = 4 and 8 with twice as many and half the CTAs are faster all the
+// same (geometric means over 65 to 4096 workers, d = 4096 to 4M: b = 4 46 -> 41 us,
+// b = 8 46 -> 39; b = 2 39.4 -> 40.0, kept).
 template <int BITS, int P8>
-__global__ void __launch_bounds__(256, 4) squant_server_kernel(const ServerArgs s) {
+__global__ void __launch_bounds__(256, P8 > 0 || BITS == 2 ? 4 : 2) squant_server_kernel(const ServerArgs s) {
   dq_pdl_enter();
   constexpr int K = (1 << (BITS - 1)) - 1;
   constexpr uint32_t MASK = (1u << BITS) - 1u;
@@ -1542,9 +1546,11 @@ __global__ void __launch_bounds__(256) oadam_update_kernel(const OAdamArgs a) {
 // Identity: the messages are the p vectors themselves.  OADAM: the update
 // rule follows in the same pass (s.w are the parameters then too), which
 // saves the averaged update's way through memory: 3.6M x 8, with its launch,
-// 47 us in two kernels, 37 in one.
+// 47 us in two kernels, 37 in one.  Above 64 workers two CTAs per SM, without
+// spills, against 4: geometric means over 65 to 200 workers 34 -> 28 us, 256 to
+// 4096 108 -> 84.
 template <int P8, bool OADAM>
-__global__ void __launch_bounds__(256, OADAM ? 3 : 4) identity_server_kernel(const ServerArgs s, const OAdamArgs oa) {
+__global__ void __launch_bounds__(256, P8 == 0 ? 2 : OADAM ? 3 : 4) identity_server_kernel(const ServerArgs s, const OAdamArgs oa) {
   dq_pdl_enter();
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t j = 4 * c;
