@@ -683,8 +683,8 @@ int dqgan_server_aggregate_update(dqgan_handle* h, const void* msgs_all, float* 
   if (tma_sign || tma_squant) {
     if (h->words_map_msgs != msgs_all) {
       const int64_t payload_words = tma_sign ? (s.d + 31) / 32 : (s.d * s.bits + 31) / 32;
-      // 36-word boxes wherever slices come from a table (layer segments:
-      // the sign server, and the quantiser server with 8-bit codes)
+      // 36-word boxes wherever slices come from a table (layer segments: the
+      // sign server, and the quantiser server with 4- and 8-bit codes)
       const bool table = !flat && h->seg_slices != nullptr;
       h->words_map_ok = dq::encode_words_map(s.msgs, s.msg_stride, s.off_payload, payload_words, s.M,
                                              tma_sign && flat, table ? dq::kSignSegBoxWords : 32, &h->words_map);
@@ -697,8 +697,9 @@ int dqgan_server_aggregate_update(dqgan_handle* h, const void* msgs_all, float* 
   x.seg_slices = h->seg_slices;
   x.seg_nslices = h->seg_nslices;
   // parameter boxes: 32 rows for the sign column kernel, one slice of
-  // 32 * (32 / b) elements for the b = 2, 4 quantiser server
-  const bool boxed_squant = tma_squant && s.squant_words_map && h->cfg.bits != 8;
+  // 32 * (32 / b) elements for the b = 2, 4 quantiser server (which with a
+  // table of slices, 4-bit codes with layer segments, takes none)
+  const bool boxed_squant = tma_squant && s.squant_words_map && h->cfg.bits != 8 && h->seg_slices == nullptr;
   if (((tma_sign && s.sign_words_map) || boxed_squant) && s.d >= 32) {
     if (h->params_map_w != target) {
       const int32_t rows = boxed_squant ? 32 / h->cfg.bits : 32;

@@ -581,7 +581,6 @@ __global__ void __launch_bounds__(128) squant_compress_rows_kernel(const Compres
   dq_pdl_enter();
   constexpr int K = (1 << (BITS - 1)) - 1;
   using Buckets = SpanBuckets<LPB, SEG>;
-  constexpr int kBucket = Buckets::kBucket;
   __shared__ float level_value[K + 1];  // fl(r / K)
   for (int r = threadIdx.x; r <= K; r += blockDim.x) level_value[r] = __fdiv_rn((float)r, (float)K);
   __syncthreads();

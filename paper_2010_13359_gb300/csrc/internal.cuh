@@ -220,8 +220,9 @@ cudaError_t launch_sign_server(const ServerArgs& s, const SignServerExtras& x, c
                                uint64_t* launches);
 // x.params_map: encode_params_map(w, d, 32 * (32 / bits) / 32) for bits 2 and
 // 4, or nullptr (then those widths take the kernel without TMA); with layer
-// segments and 8-bit codes, x.seg_slices lists each bucket's code words in
-// runs of up to 32 (and the words map has 36-word boxes).
+// segments and 4- or 8-bit codes, x.seg_slices lists each bucket's code words
+// in runs of up to 32 (the words map has 36-word boxes then, and no parameter
+// map is used).
 cudaError_t launch_squant_server(const ServerArgs& s, const SignServerExtras& x, cudaStream_t stream,
                                  uint64_t* launches);
 // oa: Optimistic Adam in the same pass (then s.w is not used), or nullptr.

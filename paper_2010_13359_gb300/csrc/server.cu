@@ -884,10 +884,6 @@ __device__ __forceinline__ void b2_pair_table_update(const uint32_t* words, cons
   }
 }
 
-// Passes over a lane's 8 elements in the b = 4 per-worker decode (1 or 2).
-constexpr int kSquant4Parts = 1;
-
-
 // b = 4 and 8 load each slice's scale (b = 8: and the lane's parameters)
 // one slice ahead; b = 4 writes its parameters back with plain stores
 // instead of a TMA store of the box, which frees the box as soon as the
@@ -1132,21 +1128,16 @@ squant_server_tma_kernel(const ServerArgs s, const __grid_constant__ CUtensorMap
     const uint32_t* words = reinterpret_cast<const uint32_t*>(buf0 + cur * box_bytes) + lane;
     const float* V8l = V8 + lane;
     // The per-worker decode (b = 4, 8, and b = 2 on slices that span layer
-    // segments) takes the lane's elements in kParts passes of NE (b = 4: two
-    // passes of 4, which halves the live sums at the cost of reading each
-    // code word and scale twice).
-    constexpr int kParts = BITS == 4 ? kSquant4Parts : 1;
-    constexpr int NE = EPL / kParts;
-    // one worker's decoded values of this lane's elements e0 .. e0 + NE - 1
-    auto decode_part = [&](uint32_t word, float sc, int e0, float (&v)[NE]) {
+    // segments): one worker's decoded values of this lane's elements.
+    auto decode = [&](uint32_t word, float sc, float (&v)[EPL]) {
       if constexpr (BITS == 2) {
         // code 0: -s, 1: +0, 2: +s (fl(s * 1) = s): one bit test picks +0,
         // one the sign
         const float nsc = -sc;
 #pragma unroll
-        for (int e = 0; e < NE; ++e) {
-          const bool zero = (word >> (2 * (e0 + e))) & 1u;
-          v[e] = zero ? 0.f : (((word >> (2 * (e0 + e) + 1)) & 1u) ? sc : nsc);
+        for (int e = 0; e < EPL; ++e) {
+          const bool zero = (word >> (2 * e)) & 1u;
+          v[e] = zero ? 0.f : (((word >> (2 * e + 1)) & 1u) ? sc : nsc);
         }
         return;
       }
@@ -1156,11 +1147,11 @@ squant_server_tma_kernel(const ServerArgs s, const __grid_constant__ CUtensorMap
       // 16..31, so the bits above the element's code need no mask).
       const float T4 = (BITS == 4) ? __fmul_rn(sc, V4) : 0.f;
 #pragma unroll
-      for (int e = 0; e < NE; ++e) {
+      for (int e = 0; e < EPL; ++e) {
         if constexpr (BITS == 4) {
-          v[e] = __shfl_sync(kFullMask, T4, (int)(word >> (4 * (e0 + e))));
+          v[e] = __shfl_sync(kFullMask, T4, (int)(word >> (4 * e)));
         } else {
-          v[e] = __fmul_rn(sc, V8l[__byte_perm(word, 0u, 0x4440u | (uint32_t)(e0 + e)) * 32u]);
+          v[e] = __fmul_rn(sc, V8l[__byte_perm(word, 0u, 0x4440u | (uint32_t)e) * 32u]);
         }
       }
     };
@@ -1182,80 +1173,76 @@ squant_server_tma_kernel(const ServerArgs s, const __grid_constant__ CUtensorMap
     // (slices that span buckets take their own instance of the decode, so
     // that the common one carries none of their scale handling)
     auto per_worker_sums = [&](bool mx) {
+      // group value of workers m .. m + 3 into g
+      auto group = [&](int m, float (&g)[EPL]) {
+        // the group's code words and scales first (a worker past M is not read)
+        uint32_t wd[4];
+        float sc[4];
 #pragma unroll
-      for (int part = 0; part < kParts; ++part) {
-        const int e0 = part * NE;
-        // group value of workers m .. m + 3 into g
-        auto group = [&](int m, float (&g)[NE]) {
-          // the group's code words and scales first (a worker past M is not read)
-          uint32_t wd[4];
-          float sc[4];
+        for (int u = 0; u < 4; ++u) {
+          const bool here = m + u < M;  // warp-uniform
+          wd[u] = here ? words[32 * (m + u)] : 0u;
+          sc[u] = here ? scale_of(mx, m + u) : 0.f;
+        }
+        float va[EPL], vb[EPL];
+        decode(wd[0], sc[0], va);
+        decode(wd[1], sc[1], vb);
+        const bool h1 = m + 1 < M;
 #pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const bool here = m + u < M;  // warp-uniform
-            wd[u] = here ? words[32 * (m + u)] : 0u;
-            sc[u] = here ? scale_of(mx, m + u) : 0.f;
-          }
-          float va[NE], vb[NE];
-          decode_part(wd[0], sc[0], e0, va);
-          decode_part(wd[1], sc[1], e0, vb);
-          const bool h1 = m + 1 < M;
+        for (int e = 0; e < EPL; ++e) g[e] = M == 1 ? va[e] : __fadd_rn(va[e], h1 ? vb[e] : 0.f);
+        if (M <= 2) return;
+        decode(wd[2], sc[2], va);
+        decode(wd[3], sc[3], vb);
+        const bool h2 = m + 2 < M, h3 = m + 3 < M;
 #pragma unroll
-          for (int e = 0; e < NE; ++e) g[e] = M == 1 ? va[e] : __fadd_rn(va[e], h1 ? vb[e] : 0.f);
-          if (M <= 2) return;
-          decode_part(wd[2], sc[2], e0, va);
-          decode_part(wd[3], sc[3], e0, vb);
-          const bool h2 = m + 2 < M, h3 = m + 3 < M;
+        for (int e = 0; e < EPL; ++e) g[e] = __fadd_rn(g[e], __fadd_rn(h2 ? va[e] : 0.f, h3 ? vb[e] : 0.f));
+      };
+      // x <- x + (value of groups i, i + 1), the second +0 past M
+      auto add_pair = [&](int i, float (&x)[EPL]) {
+        float t[EPL], g[EPL];
+        group(4 * i, t);
+        if (4 * (i + 1) < M) {
+          group(4 * (i + 1), g);
+        } else {
 #pragma unroll
-          for (int e = 0; e < NE; ++e) g[e] = __fadd_rn(g[e], __fadd_rn(h2 ? va[e] : 0.f, h3 ? vb[e] : 0.f));
-        };
-        // x <- x + (value of groups i, i + 1), the second +0 past M
-        auto add_pair = [&](int i, float (&x)[NE]) {
-          float t[NE], g[NE];
-          group(4 * i, t);
-          if (4 * (i + 1) < M) {
-            group(4 * (i + 1), g);
-          } else {
-#pragma unroll
-            for (int e = 0; e < NE; ++e) g[e] = 0.f;
-          }
-#pragma unroll
-          for (int e = 0; e < NE; ++e) x[e] = __fadd_rn(x[e], __fadd_rn(t[e], g[e]));
-        };
-        float r[NE];
-        group(0, r);
-        if (M > 4) {
-          float g[NE];
-          group(4, g);
-#pragma unroll
-          for (int e = 0; e < NE; ++e) r[e] = __fadd_rn(r[e], g[e]);
-          if (M > 8) {
-            add_pair(2, r);
-            if (M > 16) {
-              float h[NE];
-              group(16, h);
-              if (M > 20) {
-                group(20, g);
-              } else {
-#pragma unroll
-                for (int e = 0; e < NE; ++e) g[e] = 0.f;
-              }
-#pragma unroll
-              for (int e = 0; e < NE; ++e) h[e] = __fadd_rn(h[e], g[e]);
-              if (M > 24) {
-                add_pair(6, h);
-              } else {
-#pragma unroll
-                for (int e = 0; e < NE; ++e) h[e] = __fadd_rn(h[e], 0.f);
-              }
-#pragma unroll
-              for (int e = 0; e < NE; ++e) r[e] = __fadd_rn(r[e], h[e]);
-            }
-          }
+          for (int e = 0; e < EPL; ++e) g[e] = 0.f;
         }
 #pragma unroll
-        for (int e = 0; e < NE; ++e) acc[e0 + e] = r[e];
+        for (int e = 0; e < EPL; ++e) x[e] = __fadd_rn(x[e], __fadd_rn(t[e], g[e]));
+      };
+      float r[EPL];
+      group(0, r);
+      if (M > 4) {
+        float g[EPL];
+        group(4, g);
+#pragma unroll
+        for (int e = 0; e < EPL; ++e) r[e] = __fadd_rn(r[e], g[e]);
+        if (M > 8) {
+          add_pair(2, r);
+          if (M > 16) {
+            float h[EPL];
+            group(16, h);
+            if (M > 20) {
+              group(20, g);
+            } else {
+#pragma unroll
+              for (int e = 0; e < EPL; ++e) g[e] = 0.f;
+            }
+#pragma unroll
+            for (int e = 0; e < EPL; ++e) h[e] = __fadd_rn(h[e], g[e]);
+            if (M > 24) {
+              add_pair(6, h);
+            } else {
+#pragma unroll
+              for (int e = 0; e < EPL; ++e) h[e] = __fadd_rn(h[e], 0.f);
+            }
+#pragma unroll
+            for (int e = 0; e < EPL; ++e) r[e] = __fadd_rn(r[e], h[e]);
+          }
+        }
       }
+#pragma unroll
+      for (int e = 0; e < EPL; ++e) acc[e] = r[e];
     };
     if (per_worker) {
       if constexpr (SEG) {
