@@ -1388,6 +1388,9 @@ __global__ void __launch_bounds__(kSrvThreads) topk_server_reduce_kernel(const S
 //     are large, in a few tiles out of thousands, so those tiles are dealt out
 //     in runs to a grid of their own (524,288 x 64, k = d / 10 in a tenth of
 //     the vector: 392 us where the merge's CTAs did it themselves, 38 so).
+//     An item's parameters and the next one's place in the messages load with
+//     its records (25M x 16 in 64 layers, k = d / 100, some 560 dense tiles: 56
+//     us one after the other, 37 so).
 // Records and touched parameters are all they move, against the tables of the
 // two kernels above, whose scattered sectors go through DRAM twice.  Latency
 // bounds them: the loads of a thread's 8 records, and of the parameters it
@@ -1587,64 +1590,98 @@ __global__ void __launch_bounds__(kMergeThreads, 4)
   const int row = per * kSrvTile;
   const int items_per = (kMergeRuns + per - 1) / per;  // of a tile
   const int64_t items = tiles * items_per;
+  // the runs [run0, run1) of an item (empty past the vector's end)
+  struct Item {
+    int64_t run0, run1;
+  };
+  auto item_at = [&](int64_t item) {
+    const int64_t run0 = (int64_t)dense[64 + item / items_per] * kMergeRuns + (item % items_per) * per;
+    const int64_t tile_end = (run0 / kMergeRuns + 1) * kMergeRuns;
+    return Item{run0, max64(run0, min64(min64(run0 + per, tile_end), nts))};
+  };
+  // thread m's share of the next item's table of contents: worker m's records
+  uint32_t lo = 0, hi = 0;
+  auto load_records = [&](const Item& x) {
+    lo = hi = 0;
+    if ((int)threadIdx.x >= s.M || x.run0 >= nts) return;
+    const uint32_t* st = starts + (int64_t)threadIdx.x * (nts + 1);
+    lo = st[x.run0];
+    hi = st[x.run1];
+  };
+  if (blockIdx.x >= items) return;
+  Item next = item_at(blockIdx.x);
+  load_records(next);
   for (int64_t item = blockIdx.x; item < items; item += gridDim.x) {
-    const int64_t tile = dense[64 + item / items_per];
-    const int part = (int)(item % items_per);
-    const int64_t run0 = tile * kMergeRuns + part * per;
-    const int64_t run1 = min64(run0 + min(per, kMergeRuns - part * per), nts);
-    const int64_t t0 = run0 * kSrvTile;
-    const int width = (int)min64((run1 - run0) * kSrvTile, s.d - t0);
-    if (width <= 0) continue;  // past the last run (the same in every thread)
-    for (int m = threadIdx.x; m < s.M; m += kMergeThreads) {
-      const uint32_t* st = starts + (int64_t)m * (nts + 1);
-      first[m] = (uint32_t)min64(st[run0], s.k);
-      past[m] = (uint32_t)min64(st[run1], s.k);
+    const Item now = next;
+    const int64_t t0 = now.run0 * kSrvTile;
+    const int width = (int)max64(0, min64((now.run1 - now.run0) * kSrvTile, s.d - t0));
+    if ((int)threadIdx.x < s.M) {
+      first[threadIdx.x] = (uint32_t)min64(lo, s.k);
+      past[threadIdx.x] = (uint32_t)min64(hi, s.k);
     }
     for (int i = threadIdx.x; i < s.M * (row / 4); i += kMergeThreads)
       reinterpret_cast<float4*>(table)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     __syncthreads();
+    // the parameters, and the next item's, on their way with the records
+    float wv[dense_runs(P)];
+#pragma unroll
+    for (int u = 0; u < dense_runs(P); ++u) {
+      const int i = threadIdx.x + u * kMergeThreads;
+      wv[u] = i < width && !s.store_q ? s.w[t0 + i] : 0.f;
+    }
+    if (item + gridDim.x < items) {
+      next = item_at(item + gridDim.x);
+      load_records(next);
+    }
 #pragma unroll 1
     for (int w0 = 0; w0 < kWorkers; w0 += kTake) {
-      // (records come from the compressor: sorted, and below d)
-      int64_t at[kTake], end[kTake];
+      // (records come from the compressor: sorted, and below d, so that an item
+      // has no more of a worker's than indices)
+      uint32_t at[kTake];
+      int left[kTake];
       bool more = false;
 #pragma unroll
       for (int t = 0; t < kTake; ++t) {
-        const int m = warp / kShare + kWarps * (w0 + t);
-        at[t] = end[t] = 0;
-        if (m < s.M) {
-          at[t] = first[m] + 32 * (warp % kShare) + lane;
-          end[t] = past[m];
+        const int m = warp / kShare + kWarps * (w0 + t), skip = 32 * (warp % kShare) + lane;
+        at[t] = 0;
+        left[t] = 0;
+        if (m < s.M && past[m] > first[m]) {
+          at[t] = first[m] + skip;
+          left[t] = (int)min(past[m] - first[m], (uint32_t)row) - skip;
         }
-        more = more || at[t] < end[t];
+        more = more || left[t] > 0;
       }
       while (more) {
         more = false;
         uint2 rec[kTake][kAhead];
 #pragma unroll
         for (int t = 0; t < kTake; ++t) {
-          const uint2* msg =
-              reinterpret_cast<const uint2*>(s.msgs + (int64_t)(warp / kShare + kWarps * (w0 + t)) * s.msg_stride);
+          const uint2* msg = reinterpret_cast<const uint2*>(
+                                 s.msgs + (int64_t)(warp / kShare + kWarps * (w0 + t)) * s.msg_stride) + at[t];
 #pragma unroll
           for (int u = 0; u < kAhead; ++u)
-            if (at[t] + 32 * kShare * u < end[t]) rec[t][u] = msg[at[t] + 32 * kShare * u];
+            if (32 * kShare * u < left[t]) rec[t][u] = msg[32 * kShare * u];
         }
 #pragma unroll
         for (int t = 0; t < kTake; ++t) {
           float* values = table + (warp / kShare + kWarps * (w0 + t)) * row;
 #pragma unroll
           for (int u = 0; u < kAhead; ++u)
-            if (at[t] + 32 * kShare * u < end[t]) {
+            if (32 * kShare * u < left[t]) {
               const int64_t i = (int64_t)rec[t][u].x - t0;
               if (dq_in_bounds(i >= 0 && i < width, s.err)) values[i] = __uint_as_float(rec[t][u].y);
             }
           at[t] += 32 * kShare * kAhead;
-          more = more || at[t] < end[t];
+          left[t] -= 32 * kShare * kAhead;
+          more = more || left[t] > 0;
         }
       }
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < width; i += kMergeThreads) {
+#pragma unroll
+    for (int w = 0; w < dense_runs(P); ++w) {
+      const int i = threadIdx.x + w * kMergeThreads;
+      if (i >= width) break;
       // the padded tree, in chunks of up to 16 workers
       constexpr int C = P < 16 ? P : 16;
       float part_sum[P / C];
@@ -1656,7 +1693,7 @@ __global__ void __launch_bounds__(kMergeThreads, 4)
         part_sum[c] = pairwise_n<C>(x);
       }
       const float sum = pairwise_n<P / C>(part_sum);
-      s.w[t0 + i] = server_out(s, s.w[t0 + i], srv_average<POW2>(sum, s));
+      s.w[t0 + i] = server_out(s, wv[w], srv_average<POW2>(sum, s));
     }
     __syncthreads();
   }
