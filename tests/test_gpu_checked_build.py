@@ -4,7 +4,8 @@ computed stores and loads -- candidate slots, message records, the server's
 record offsets -- and skip an out-of-range access while setting a bit that
 dqgan_synchronize reports as DQGAN_ERR_BOUNDS; its top-k scratch sits
 between guard zones that dqgan_synchronize checks.  The guard-word tests and
-the top-k parity tests run again in a child process with that library
+the top-k tests (on chip and sampled, every route of the selection, the tables
+and the tiles of the server) run again in a child process with that library
 loaded (the binding loads the library DQGAN_LIBRARY names) and must report
 nothing; and a positive control -- a message whose last record lies past d,
 which the normal build skips silently -- must come back as DQGAN_ERR_BOUNDS
@@ -68,7 +69,8 @@ def test_checked_build_reports_an_out_of_range_record(checked_env):
 
 def test_guard_and_topk_tests_pass_under_the_checked_build(checked_env):
     cmd = [sys.executable, "-m", "pytest", "-q", "-x", "-m", "gpu", "-p", "no:cacheprovider",
-           "tests/test_gpu_guards.py", "tests/test_gpu_topk_paths.py", "tests/test_gpu_parity.py", "-k",
-           "guard or topk or Topk"]
+           "tests/test_gpu_guards.py", "tests/test_gpu_topk_paths.py", "tests/test_gpu_topk_select.py",
+           "tests/test_gpu_parity.py", "tests/test_gpu_server_workers.py", "-k",
+           "guard or topk or Topk or records_residual or (lists and (edge or shared))"]
     res = subprocess.run(cmd, cwd=ROOT, env=checked_env, capture_output=True, text=True, timeout=1500)
     assert res.returncode == 0, res.stdout[-4000:] + res.stderr[-2000:]

@@ -53,6 +53,8 @@ CASES = [
     ("topk", dict(d=300_007, M=8, compressor=oracle.TOPK, k=3_001)),
     ("topk_all", dict(d=4_099, M=3, compressor=oracle.TOPK, k=4_099)),
     ("topk_many", dict(d=20_000, M=70, compressor=oracle.TOPK, k=200)),
+    ("topk_sampled", dict(d=1_000_003, M=4, compressor=oracle.TOPK, k=10_001, keep_lookahead=True)),
+    ("topk_tiles", dict(d=1_100_003, M=8, compressor=oracle.TOPK, k=100_000)),
 ]
 
 
@@ -63,7 +65,8 @@ def test_guard_words_stay_intact(P, name, kw):
     ocfg = oracle.Config(lr=1e-2, seed=6, **kw)
     d, M = ocfg.d, ocfg.M
     h = P.create(P.make_config(d=d, M=M, compressor=ocfg.compressor, lr=ocfg.lr, bucket=ocfg.bucket, k=ocfg.k,
-                               bits=ocfg.bits, seed=ocfg.seed, cuda_stream=stream.cuda_stream))
+                               bits=ocfg.bits, seed=ocfg.seed, cuda_stream=stream.cuda_stream,
+                               flags=P.KEEP_LOOKAHEAD if ocfg.keep_lookahead else 0))
     mb = h.message_bytes()
     ld = (d + 3) // 4 * 4
     g_buf, g_view = guarded(M * ld * 4, dev)

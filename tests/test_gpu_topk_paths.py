@@ -1,21 +1,19 @@
-"""The top-k worker step's two routes to the same result, against the oracle.
+"""The top-k step's routes to the same result, against the oracle.
 
-The first pass writes, per tile, the elements whose top key digit reaches a
-threshold carried over from the worker's previous call; the second kernel
-uses them when the new top digit of the k-th largest key is not below that
-threshold, and otherwise re-extracts the candidates from p.  Whichever route
-a call takes, the records and residuals must be the oracle's bit for bit:
+Small vectors are selected on chip; larger ones through candidates at or above
+a threshold that a sample of the same call gives, counted in rounds.  Whichever
+route a call takes, the records and residuals must be the oracle's bit for bit:
 
-* a scale sequence that makes the threshold fall (re-extraction), rise far
-  (many candidates), land inside big groups of equal keys, and sit on an
-  all-zero p;
-* more candidates than a select CTA keeps on chip (k = d/2);
+* a scale sequence on one handle, on chip and with the sample: steady, falling
+  and rising by 10^3, big groups of equal keys, an all-zero p, denormal values
+  (nothing may carry over from call to call);
+* half of the elements kept (k = d/2);
 * server paths for up to 64 workers (per-index worker masks, one owner
   per index) and beyond (a thread per record);
-* at d = 7e7 the CTAs' tiles no longer fit one chunk of tile counts; there
-  the selection is checked by the properties that define it uniquely
-  (k records in index order holding p_j, no dropped key above the smallest
-  kept key, equal keys kept lowest index first, e = +0 exactly there).
+* at d = 7e7 tiles are taken in groups; there the selection is checked by the
+  properties that define it uniquely (k records in index order holding p_j, no
+  dropped key above the smallest kept key, equal keys kept lowest index first,
+  e = +0 exactly there).
 """
 from __future__ import annotations
 
@@ -86,19 +84,20 @@ def run_free(P, ocfg, kinds, seed=0):
     h.destroy()
 
 
-@pytest.mark.parametrize("d,k", [(200_003, 3_000), (40_000, 39_000), (5_000, 17)])
-def test_threshold_carry_routes(P, d, k):
+@pytest.mark.parametrize("d,k", [(200_003, 3_000), (40_000, 39_000), (5_000, 17), (1_000_003, 10_000)])
+def test_scale_sequence(P, d, k):
+    """On chip but for the last size, which takes the sampled kernels."""
     kinds = [1.0, 1.0, 1e-3, 1e-3, 1e3, "ties", "ties", "zeros", 1.0, 1e-30]
     ocfg = oracle_config(d, 2, oracle.TOPK, lr=0.5, k=k, seed=3, keep=True)
     run_free(P, ocfg, kinds, seed=d)
 
 
-def test_candidates_beyond_on_chip_copy(P):
+def test_half_of_the_elements_kept(P):
     ocfg = oracle_config(1_000_003, 1, oracle.TOPK, lr=0.1, k=500_000, seed=4, keep=False)
     run_free(P, ocfg, [1.0, 1.0, 0.5], seed=1)
 
 
-def test_many_tiles_per_cta_properties(P):
+def test_groups_of_tiles_by_properties(P):
     dev = torch.device("cuda:0")
     stream = torch.cuda.current_stream(dev)
     d, k, lr = 70_000_001, 700_000, 0.25

@@ -156,6 +156,47 @@ def test_sparse_gradients_take_a_few_times_a_dense_one(P, d, M):
     assert took["sparse"] < 5 * took["gauss"], took
 
 
+@pytest.mark.parametrize("d", [300_005, 1_000_003])  # on chip; the sampled kernels
+def test_gradients_from_another_stream(P, d):
+    """The gradients are still being written on another stream when the call is made; an event
+    orders the two."""
+    M, k, lr = 2, 5_000, np.float32(0.25)
+    mine, other = torch.cuda.Stream(), torch.cuda.Stream()
+    h = P.create(P.make_config(d=d, M=M, compressor=P.TOPK, lr=float(lr), k=k, cuda_stream=mine.cuda_stream))
+    ld = (d + 3) // 4 * 4
+    gen = torch.Generator(device="cuda").manual_seed(d)
+    sources = [torch.randn((M, ld), generator=gen, device="cuda") * 10.0 ** -step for step in range(4)]
+    g = torch.zeros((M, ld), device="cuda")
+    msgs = torch.zeros((M, h.message_bytes()), dtype=torch.uint8, device="cuda")
+    torch.cuda.synchronize()
+    got = []
+    for src in sources:
+        with torch.cuda.stream(other):
+            other.wait_stream(mine)
+            busy = torch.ones(1 << 24, device="cuda")
+            for _ in range(8):
+                busy = busy * 1.0001
+            g.copy_(src)
+            written = other.record_event()
+        mine.wait_event(written)
+        h.workers_compress_all(g, ld, msgs)
+        with torch.cuda.stream(mine):
+            got.append(msgs.clone())
+    h.synchronize()
+    torch.cuda.synchronize()
+    e = np.zeros((M, d), np.float32)
+    for step, src in enumerate(sources):
+        p = lr * src[:, :d].cpu().numpy() + e
+        for m in range(M):
+            rec = got[step][m, :8 * k].cpu().numpy().view(np.uint32).reshape(k, 2)
+            idx = np.sort(np.argpartition(np.abs(p[m]), d - k)[d - k:])  # no two keys are equal at the k-th
+            assert np.array_equal(rec[:, 0], idx.astype(np.uint32)), (step, m)
+            assert np.array_equal(rec[:, 1], p[m, idx].view(np.uint32)), (step, m)
+            e[m] = p[m]
+            e[m, idx] = 0
+    h.destroy()
+
+
 # run by a child process: the sizes that take clusters of CTAs, and those that would take them
 NO_CLUSTERS = r"""
 import numpy as np, torch

@@ -5,10 +5,11 @@ memory (and so cannot create a handle): it keeps its scratch in a fixed
 array inside the library and works on a residual the caller owns.  It must
 produce exactly the messages and residuals of dqgan_worker_compress with the
 top-k compressor.  Four calls in a row, the last two with the gradient
-scale dropped by 1e4 and then raised by 1e8, check that the shared scratch
-is cleared between calls, that the caller's residual carries over, and that
-the candidate threshold carried from call to call (also across the
-parametrised cases, which share the array) never changes a result.
+scale dropped by 1e4 and then raised by 1e8, check that the caller's residual
+carries over and that nothing else does; the last size is the largest, and with
+those of the second test the ones that use the array (smaller ones stay on
+chip).  Sizes taken in turn on the one array check that a call reads nothing
+there that a call of another size left.
 """
 from __future__ import annotations
 
@@ -54,6 +55,30 @@ def test_noalloc_topk_matches_handle_path(P, d, k):
         assert np.array_equal(got.view(np.uint32), e_ref.view(np.uint32)), f"call {call}: residuals differ"
         h.set_step(h.get_step() + 1)
     h.destroy()
+
+
+def test_noalloc_sizes_in_turn_share_the_array(P):
+    import oracle
+    dev = torch.device("cuda:0")
+    stream = torch.cuda.current_stream(dev)
+    rng = np.random.default_rng(11)
+    sizes = [(1 << 20, 10_486, 1.0), (800_001, 700_000, 1e3), (1 << 20, 100_000, 1e-3), (900_011, 9_000, 1e-3)]
+    e_dev = {d: torch.zeros((d + 3) // 4 * 4, device=dev) for d, _, _ in sizes}
+    e_orc = {d: np.zeros(d, np.float32) for d, _, _ in sizes}
+    for call, (d, k, scale) in enumerate(sizes * 2):
+        g = (rng.standard_normal(d) * scale).astype(np.float32)
+        if call == 5:  # fewer than k non-zero entries
+            g[rng.random(d) < 0.9] = 0
+        g_dev = torch.zeros((d + 3) // 4 * 4, device=dev)
+        g_dev[:d] = torch.from_numpy(g)
+        msg = torch.zeros(8 * k, dtype=torch.uint8, device=dev)
+        P.dqgan.topk_compress_noalloc(g_dev, e_dev[d], msg, d, k, 0.5, stream.cuda_stream)
+        torch.cuda.synchronize(dev)
+        cfg = oracle.Config(d=d, M=1, compressor=oracle.TOPK, lr=0.5, k=k)
+        want = oracle.worker_step(cfg, 0, call + 1, g, e_orc[d])
+        assert np.array_equal(msg.cpu().numpy(), want[:8 * k]), f"call {call}: records"
+        got = e_dev[d][:d].cpu().numpy()
+        assert np.array_equal(got.view(np.uint32), e_orc[d].view(np.uint32)), f"call {call}: residual"
 
 
 def test_noalloc_exact_size_views_odd_d(P):
