@@ -138,10 +138,12 @@ DQGAN_API int dqgan_validate_config(const dqgan_config* cfg);
  * compressors need).  Allocates on the current device: e (M x d fp32, zero:
  * e_0 = 0), h (M x d fp32, zero, only with DQGAN_KEEP_LOOKAHEAD: F(w_{-1/2})
  * is taken as 0 so that w_{1/2} = w_0), and top-k scratch (per worker row
- * about 8 bytes per parameter for the candidates; for the server, with M <= 64
- * and sparse records (M k below 3 % of d) per-index worker masks and values,
- * 4 + 4M bytes per parameter (8 + 4M above 32 workers), else a table of record
- * ranges).  Sets t = 1.
+ * about 8 bytes per parameter for the candidates; for the server, with
+ * M <= 64, per-index worker masks and values, 4 + 4M bytes per parameter
+ * (8 + 4M above 32 workers; M rounded up to a multiple of 4 from 3 on), unless
+ * the records are many: d >= 1,000,000, M k >= 700,000 and M k >= 3 % of d;
+ * then, and above 64 workers, a table of record ranges, M / 64 bytes per
+ * parameter).  Sets t = 1.
  * *out receives the handle; on error *out is NULL and
  * dqgan_last_error(NULL) holds the reason, and nothing stays allocated.
  * Test hook: with the environment variable DQGAN_TEST_FAIL_ALLOC=N set, the

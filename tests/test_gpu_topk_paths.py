@@ -143,3 +143,18 @@ def test_server_worker_counts(P, M):
     order, so w matches bit for bit."""
     ocfg = oracle_config(50_003, M, oracle.TOPK, lr=0.5, k=777, seed=M, keep=False)
     run_free(P, ocfg, [1.0, 1.0, "ties"], seed=M)
+
+
+@pytest.mark.parametrize("M,k,server", [(8, 25_000, 36), (8, 87_499, 36), (8, 87_500, 0.125), (5, 10_000, 36),
+                                        (40, 5_000, 168), (65, 5_000, 65 / 64)])
+def test_scratch_is_what_the_header_says(P, M, k, server):
+    """Bytes per parameter: 4 for each residual, about 8 for each worker's candidates, and the
+    server's tables or record ranges."""
+    d = 4_000_000
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    h = P.create(P.make_config(d=d, M=M, compressor=oracle.TOPK, lr=0.1, k=k,
+                               cuda_stream=torch.cuda.current_stream().cuda_stream))
+    used = (before - torch.cuda.mem_get_info()[0]) / d
+    h.destroy()
+    assert abs(used - (12 * M + server)) < 0.15 * M + 2, used
