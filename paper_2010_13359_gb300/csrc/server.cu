@@ -1752,10 +1752,16 @@ cudaError_t launch_squant_server(const ServerArgs& s, const SignServerExtras& x,
                                  uint64_t* launches) {
   const CUtensorMap* params_map = x.params_map;
   // The TMA kernels for 2-bit codes work on slices of 512 elements and wait
-  // for their copies; while there are few, a thread per 4 elements is faster
-  // (16 workers, flat, d = 131,072 / 524,288: 2.8 / 4.4 us against 3.4 / 3.5;
-  // layer segments, 524,288: 4.3 against 6.7).
-  const bool few = s.bits == 2 && s.d <= (s.word_bucket ? 524288 : 262144);
+  // for their copies; while there are few, a thread per 4 elements is faster,
+  // and its time grows with the workers.  Its time over theirs, flat: 0.87 at
+  // d = 1M with 1 worker; 0.89 / 1.07 at 700,000 / 1M with 4; 0.86 / 1.06 at
+  // 262,144 / 340,000 with 16; 0.94 / 1.21 with 32.  With layer segments their
+  // slices span buckets and the line lies far higher: 0.66 / 0.84 at 1.4M / 2M
+  // with 1 worker, 0.85 / 1.07 with 4, 0.80 / 0.88 at 8M / 11M with 12, 0.79 / 1.07
+  // with 16.
+  const int64_t few_to =
+      s.word_bucket ? (s.M > 4 ? 8'000'000 : 1'500'000) : max64(262'144, 5'000'000 / max64(s.M, 4));
+  const bool few = s.bits == 2 && s.d <= few_to;
   if (s.word_bucket && x.seg_slices && s.squant_words_map != nullptr) {
     // 4- and 8-bit codes, layer segments: slices from the per-bucket table
     const cudaError_t st = s.bits == 8 ? launch_squant_table<8>(s, x, stream) : launch_squant_table<4>(s, x, stream);

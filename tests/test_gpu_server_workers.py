@@ -111,6 +111,19 @@ def test_two_bits_beyond_the_small_sizes(P, M):
     run(P, oracle.SQUANT, M, (0, *cuts, d), d=d, bucket=512, bits=2)
 
 
+@pytest.mark.parametrize("M", [1, 3, 8, 16, 17, 32])
+def test_two_bits_past_the_line(P, M):
+    """Flat vectors just above the size from which slices are staged by TMA."""
+    run(P, oracle.SQUANT, M, d=max(262_144, 5_000_000 // max(M, 4)) + 519, bucket=512, bits=2)
+
+
+@pytest.mark.parametrize("M", [1, 3, 6, 17])
+def test_two_bits_with_layers_past_the_line(P, M):
+    d = (8_000_000 if M > 4 else 1_500_000) + 519
+    cuts = tuple(32 * c for c in np.sort(np.random.default_rng(M).choice(d // 32, 200, replace=False)) if c)
+    run(P, oracle.SQUANT, M, (0, *cuts, d), d=d, bucket=512, bits=2)
+
+
 def records(kind, M, d, k, rng):
     """M messages of k records."""
     common = rng.choice(d, 2 * k // 3, replace=False)
