@@ -763,10 +763,14 @@ cudaError_t squant_dispatch_bits(const CompressArgs& a, bool keep_h, bool l2, cu
 }
 
 // Whether a bucket of 128 goes to the rows kernels: a span per warp leaves a
-// quarter of the warps, and while those do not fill the GPU the latency counts
-// (12 workers, d = 65,536, sign: 2.9 us with a warp per bucket, 3.2 with a span
-// per warp, with layers 2.9 / 3.8; d = 5M: 112 / 108, with layers 114 / 111).
-bool rows_pay(const CompressArgs& a) { return a.nb * a.nworkers >= 32768; }
+// quarter of the warps, and while those do not fill the GPU the latency counts.
+// Time of the rows kernels over that of a warp per bucket, by buckets of all
+// workers (the same for 1 to 64 workers): sign 1.10 at 4096, 1.13 at 8192, 0.95
+// at 16,384, 1.00 at 24,576, 0.94 at 32,768 and 65,536 (with layers 1.25, 1.26, 1.03,
+// 1.08, 1.04, 1.00); quantisers 1.17 at 4096, 0.99 at 8192, 0.83 at 16,384, 0.82 at
+// 32,768, 0.90 at 65,536 (with layers 1.28, 1.02, 0.91, 0.86, 0.92).
+bool rows_pay(const CompressArgs& a, int64_t least) { return a.nb * a.nworkers >= least; }
+constexpr int64_t kSignRowsLeast = 32768, kQuantRowsLeast = 10240;
 
 // The grid of the rows kernels: 4 warps per CTA, a span per warp at a time.
 dim3 rows_grid(const CompressArgs& a) {
@@ -817,7 +821,8 @@ cudaError_t launch_sign_compress(const CompressArgs& a, bool keep_h, cudaStream_
     case 32: st = sign_rows_dispatch<8>(a, keep_h, stream); break;
     case 64: st = sign_rows_dispatch<16>(a, keep_h, stream); break;
     case 128:
-      st = rows_pay(a) ? sign_rows_dispatch<32>(a, keep_h, stream) : sign_dispatch_keep<1, 1>(a, keep_h, stream);
+      st = rows_pay(a, kSignRowsLeast) ? sign_rows_dispatch<32>(a, keep_h, stream)
+                                       : sign_dispatch_keep<1, 1>(a, keep_h, stream);
       break;
     case 256: st = sign_dispatch_keep<2, 1>(a, keep_h, stream); break;
     case 512: st = sign_dispatch_keep<4, 1>(a, keep_h, stream); break;
@@ -837,8 +842,8 @@ cudaError_t launch_squant_compress(const CompressArgs& a, bool keep_h, bool l2, 
     case 32: st = squant_rows_dispatch<8>(a, keep_h, l2, stream); break;
     case 64: st = squant_rows_dispatch<16>(a, keep_h, l2, stream); break;
     case 128:
-      st = rows_pay(a) ? squant_rows_dispatch<32>(a, keep_h, l2, stream)
-                       : squant_dispatch_bits<1, 1>(a, keep_h, l2, stream);
+      st = rows_pay(a, kQuantRowsLeast) ? squant_rows_dispatch<32>(a, keep_h, l2, stream)
+                                        : squant_dispatch_bits<1, 1>(a, keep_h, l2, stream);
       break;
     case 256: st = squant_dispatch_bits<2, 1>(a, keep_h, l2, stream); break;
     case 512: st = squant_dispatch_bits<4, 1>(a, keep_h, l2, stream); break;

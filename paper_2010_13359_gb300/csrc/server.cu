@@ -1714,8 +1714,10 @@ cudaError_t launch_sign_server(const ServerArgs& s, const SignServerExtras& x, c
   const int64_t nslices = seg ? x.seg_nslices : ((s.d + s.bucket - 1) / s.bucket) * (s.bucket / 1024);
   // Below some 600 slices of 1024 elements most SMs have a warp or two of the
   // TMA kernels, and the warp-per-chunk kernel, with four times the warps and
-  // no copy to wait for, is faster (8 workers, d = 65,536: 2.9 us against 3.8;
-  // 524,288: 3.0 / 3.9; 1,000,000: 3.8 / 3.9; 2,000,000: 5.6 / 5.1).
+  // no copy to wait for, is faster.  Its time over theirs, buckets of 1024 and
+  // 4096: 0.54 to 0.80 up to 524,288 elements with 1 to 32 workers, 0.86 to 0.97 at
+  // 786,432, 0.99 to 1.16 at 1M, 1.10 to 1.28 at 2M; with layer segments 0.64 to 0.99 up
+  // to 614,400, 0.92 to 1.13 at 786,432, 1.3 to 1.6 at 1M.
   const bool few = x.path == 0 && nslices <= 600;
   if (s.bucket >= 1024 && s.M <= 32 && !few && s.sign_words_map != nullptr && (!seg || x.seg_slices)) {
     const bool p2 = s.M_pow2 != 0;

@@ -71,3 +71,11 @@ def test_compress(P, comp, bits, bucket, keep):
 @pytest.mark.parametrize("comp,bits", FORMS)
 def test_compress_128_per_scale_with_a_span_per_warp(P, comp, bits, layers):
     run(P, comp, bits, 128, True, 2_097_152 + 677, layers)
+
+
+@pytest.mark.parametrize("layers", [0, 50])
+@pytest.mark.parametrize("comp,bits", FORMS[1:])
+def test_quantisers_128_per_scale_about_the_line(P, comp, bits, layers):
+    """A warp per bucket to 10,239 buckets of both workers, a span per warp from there."""
+    for d in (128 * 5119 + 5, 128 * 5120 + 37):
+        run(P, comp, bits, 128, True, d - 128 * layers, layers)
