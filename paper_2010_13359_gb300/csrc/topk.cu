@@ -8,7 +8,9 @@
 // without sorting.
 //
 // Small problems (chip_ctas): one kernel, 1, 8 or 16 CTAs per worker that keep
-// p on chip.  Large ones: five kernels, one pass over the dense vectors:
+// p on chip.  Large ones: five kernels (three where the candidates are few enough
+// for one launch to do steps 3 to 5, topk_pick_kernel), one pass over the dense
+// vectors:
 //   1. sample (16 blocks per worker): p at 65,536 elements spread over the
 //      vector; tau, a key that rather more than k of the d keys reach (1.3 k
 //      for k = d / 100), is read off their ranks.
@@ -427,13 +429,13 @@ struct SelectTask {
 
 // The CTA that is the `slot`-th of `ctas` that share row `row`.
 __device__ __forceinline__ SelectTask select_task(const CompressArgs& a, int64_t k, int rows, void* scratch, int row,
-                                                  int slot, int ctas) {
+                                                  int slot, int ctas, int warps = kSelWarps) {
   const int worker = a.worker0 + row;
   const int64_t at = (int64_t)(worker - a.row0) * a.ld;
   return SelectTask{a, row_scratch(scratch, a.d, worker - a.row0), k, tiles_of(a.d), groups_of(a.d), group_shift(a.d),
                     a.e + at, a.h ? a.h + at : nullptr, a.g + (int64_t)row * a.g_stride,
                     reinterpret_cast<uint2*>(a.msg + (int64_t)row * a.msg_stride),
-                    slot * kSelWarps + (int)(threadIdx.x >> 5), ctas * kSelWarps, rows};
+                    slot * warps + (int)(threadIdx.x >> 5), ctas * warps, rows};
 }
 
 // A tile's count and first rows of 32 candidates, loaded together (a slot has
@@ -686,6 +688,31 @@ __device__ __forceinline__ void emit_groups(const SelectTask& s, const TileAhead
       [](int) {});
 }
 
+// Every element of the tiles slot, slot + ctas, ... becomes a candidate, as if
+// kept (p from e, and from the candidates there were); body(p) for each.
+template <int NT, typename Body>
+__device__ __forceinline__ void all_as_candidates(const SelectTask& s, int slot, int ctas, Body&& body) {
+  for (int64_t t = slot; t < s.nt; t += ctas) {
+    const uint32_t m = __ldcg(s.rs.cnt + t);
+    uint2* tile = s.rs.cand + t * kTile;
+    for (uint32_t i = threadIdx.x; i < m; i += NT) put_back(s, __ldcg(tile + i));
+    __syncthreads();
+    const int64_t j0 = t * kTile;
+    const int n = (int)min64(kTile, s.a.d - j0);
+    for (int i = threadIdx.x; i < n; i += NT) {
+      const int64_t j = j0 + i;
+      const float p = s.e[j], en = __fsub_rn(p, p);
+      tile[i] = make_uint2((uint32_t)j, __float_as_uint(p));
+      if (__float_as_uint(p) != 0u) {
+        s.e[j] = en;
+        if (s.h) s.h[j] = __fadd_rn(__fmul_rn(s.a.lr, s.g[j]), en);
+      }
+      body(p);
+    }
+    if (threadIdx.x == 0) s.rs.cnt[t] = (uint32_t)n;
+  }
+}
+
 // 3. First round.
 __global__ void __launch_bounds__(kSelThreads, 2) topk_count_kernel(const CompressArgs a, int rows, void* scratch) {
   dq_pdl_enter();
@@ -722,25 +749,8 @@ __global__ void __launch_bounds__(kSelThreads, 2) topk_resolve_kernel(const Comp
   }
   if (tau == 1) return;
   clear_hist(sm, kBins);
-  for (int64_t t = blockIdx.x; t < s.nt; t += gridDim.x) {
-    const uint32_t m = __ldcg(s.rs.cnt + t);
-    uint2* slot = s.rs.cand + t * kTile;
-    for (uint32_t i = threadIdx.x; i < m; i += kSelThreads) put_back(s, __ldcg(slot + i));
-    __syncthreads();
-    const int64_t j0 = t * kTile;
-    const int n = (int)min64(kTile, a.d - j0);
-    for (int i = threadIdx.x; i < n; i += kSelThreads) {
-      const int64_t j = j0 + i;
-      const float p = s.e[j], en = __fsub_rn(p, p);
-      slot[i] = make_uint2((uint32_t)j, __float_as_uint(p));
-      if (__float_as_uint(p) != 0u) {
-        s.e[j] = en;
-        if (s.h) s.h[j] = __fadd_rn(__fmul_rn(a.lr, s.g[j]), en);
-      }
-      atomicAdd(&sm.hist[first_bin(key_of(p), 0)], 1u);
-    }
-    if (threadIdx.x == 0) s.rs.cnt[t] = (uint32_t)n;
-  }
+  all_as_candidates<kSelThreads>(s, blockIdx.x, gridDim.x,
+                                 [&](float p) { atomicAdd(&sm.hist[first_bin(key_of(p), 0)], 1u); });
   add_hist(sm, s.rs.hist2, kBins);
 }
 
@@ -762,18 +772,19 @@ __device__ __forceinline__ void third_round_add(uint32_t* hist, uint32_t key, ui
 
 // The records of a row with fewer than k non-zero keys, its candidates: all of
 // them, and the first `need` zeros in index order (their e = p - p is +0).
-// gt[], eq[]: the numbers of candidates and of zeros before each group.
-__device__ __forceinline__ void emit_with_zeros(SelectSmem<kSelThreads>& sm, const SelectTask& s, uint32_t need,
-                                                const uint32_t* gt, const uint32_t* eq) {
+// place(group): the numbers of candidates and of zeros before it; shared: kTile
+// / 32 words per warp.
+template <typename Place>
+__device__ __forceinline__ void emit_with_zeros(uint32_t* shared, const SelectTask& s, uint32_t need, Place&& place) {
   const int lane = threadIdx.x & 31;
   const uint32_t lt = (1u << lane) - 1u;
-  uint32_t* const bits = sm.hist + (threadIdx.x >> 5) * (kTile / 32);  // the tile's candidates, a bit each
-  static_assert(kSelWarps * (kTile / 32) <= kBins2, "bits of a tile per warp");
+  uint32_t* const bits = shared + (threadIdx.x >> 5) * (kTile / 32);  // the tile's candidates, a bit each
   auto put = [&](uint32_t pos, uint2 x) {
     if (dq_in_bounds(pos < (uint64_t)s.k, s.a.err)) s.rec[pos] = x;  // always true; keeps the write inside
   };
   for (int group = s.warp0; group < s.groups; group += s.nwarps) {
-    uint32_t above = gt[group], zeros = eq[group];
+    const uint2 before = place(group);
+    uint32_t above = before.x, zeros = before.y;
     const int64_t t1 = min64(s.nt, (int64_t)(group + 1) << s.shift);
     for (int64_t t = (int64_t)group << s.shift; t < t1; ++t) {
       const uint32_t n = __ldcg(s.rs.cnt + t);
@@ -911,7 +922,8 @@ __global__ void __launch_bounds__(kSelThreads, 2)
         eq[i] = (uint32_t)(min64(t1 * kTile, a.d) - t0 * kTile) - n;
       }
       group_places(sm, s.groups, gt, eq);
-      emit_with_zeros(sm, s, s.rs.state[ST_REST], gt, eq);
+      static_assert(kSelWarps * (kTile / 32) <= kBins2, "bits of a tile per warp");
+      emit_with_zeros(sm.hist, s, s.rs.state[ST_REST], [&](int group) { return make_uint2(gt[group], eq[group]); });
     } else if (route == ROUTE_LIST) {
       for (int i = threadIdx.x; i < s.groups; i += kSelThreads) {
         gt[i] = s.rs.before[i].x;
@@ -1038,6 +1050,47 @@ __device__ __forceinline__ void cluster_find(uint32_t* hist, uint32_t* coarse, u
   }
 }
 
+// T, the number of keys equal to it that are kept, and the numbers of keys above
+// and equal to T in the CTAs of lower rank, from keys spread over the cluster:
+// the top digits' counts are in sm.hist, each_key(body) calls body(key) for this
+// CTA's keys.  The caller arrives at a cluster barrier afterwards and waits at it
+// before it leaves: until then its counts may be read.
+struct Threshold {
+  uint32_t T, need, gt_before, eq_before;
+};
+template <int C, typename EachKey>
+__device__ __forceinline__ Threshold cluster_threshold(ChipSmem& sm, uint32_t k, int rank, EachKey&& each_key) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  Threshold t{0u, k, 0u, 0u};
+#pragma unroll
+  for (int round = 0; round < 3; ++round) {
+    uint32_t* hist = sm.hist + (round == 0 ? 0 : round == 1 ? 2048 : 3072);
+    uint32_t* coarse = sm.coarse + (round == 0 ? 0 : round == 1 ? 2048 : 3072) / kGroup;
+    const int low = 20 - 10 * round;  // key bits below this round's digit
+    if (round > 0)
+      each_key([&](uint32_t key) {
+        if ((key >> (low + 10)) == t.T) atomicAdd(&hist[(key >> low) & 1023u], 1u);
+      });
+    __syncthreads();
+    for (int group = warp; group < (round == 0 ? 2048 : 1024) / kGroup; group += kChipThreads / 32) {
+      const uint32_t n = __reduce_add_sync(kFullMask, hist[group * kGroup + lane] + hist[group * kGroup + 32 + lane]);
+      if (lane == 0) coarse[group] = n;
+    }
+    if constexpr (C > 1) cg::this_cluster().sync();
+    else __syncthreads();
+    if (warp == 0) {
+      if (round == 0) cluster_find<C, 2048>(hist, coarse, t.need, rank, sm.found[round]);
+      else cluster_find<C, 1024>(hist, coarse, t.need, rank, sm.found[round]);
+    }
+    __syncthreads();
+    t.T = round == 0 ? sm.found[0][0] : t.T << 10 | sm.found[round][0];
+    t.need = sm.found[round][1];
+    t.gt_before += sm.found[round][2];
+    t.eq_before = sm.found[round][3];
+  }
+  return t;
+}
+
 template <int C, bool KEEP_H>
 __global__ void __launch_bounds__(kChipThreads, 1) topk_chip_kernel(const CompressArgs a, int64_t k) {
   dq_pdl_enter();
@@ -1098,35 +1151,10 @@ __global__ void __launch_bounds__(kChipThreads, 1) topk_chip_kernel(const Compre
         if (j + q < d) atomicAdd(&sm.hist[key_of(v[q]) >> 20], 1u);
     }
   }
-  uint32_t T = 0, need = (uint32_t)k;
-  uint32_t gt_before = 0, eq_before = 0;  // keys above and equal to T in the parts before this one
-#pragma unroll
-  for (int round = 0; round < 3; ++round) {
-    uint32_t* hist = sm.hist + (round == 0 ? 0 : round == 1 ? 2048 : 3072);
-    uint32_t* coarse = sm.coarse + (round == 0 ? 0 : round == 1 ? 2048 : 3072) / kGroup;
-    const int low = 20 - 10 * round;  // key bits below this round's digit
-    if (round > 0)
-      for (int j = threadIdx.x; j < d; j += kChipThreads) {
-        const uint32_t key = key_of(p[j]);
-        if ((key >> (low + 10)) == T) atomicAdd(&hist[(key >> low) & 1023u], 1u);
-      }
-    __syncthreads();
-    for (int group = warp; group < (round == 0 ? 2048 : 1024) / kGroup; group += kWarps) {
-      const uint32_t n = __reduce_add_sync(kFullMask, hist[group * kGroup + lane] + hist[group * kGroup + 32 + lane]);
-      if (lane == 0) coarse[group] = n;
-    }
-    if constexpr (C > 1) cg::this_cluster().sync();
-    else __syncthreads();
-    if (warp == 0) {
-      if (round == 0) cluster_find<C, 2048>(hist, coarse, need, rank, sm.found[round]);
-      else cluster_find<C, 1024>(hist, coarse, need, rank, sm.found[round]);
-    }
-    __syncthreads();
-    T = round == 0 ? sm.found[0][0] : T << 10 | sm.found[round][0];
-    need = sm.found[round][1];
-    gt_before += sm.found[round][2];
-    eq_before = sm.found[round][3];
-  }
+  const Threshold th = cluster_threshold<C>(sm, (uint32_t)k, rank, [&](auto&& body) {
+    for (int j = threadIdx.x; j < d; j += kChipThreads) body(key_of(p[j]));
+  });
+  const uint32_t T = th.T, need = th.need;
   // every read of another CTA's shared memory is done: no CTA leaves before
   // all have said so
   if constexpr (C > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
@@ -1146,8 +1174,8 @@ __global__ void __launch_bounds__(kChipThreads, 1) topk_chip_kernel(const Compre
     sm.warp_eq[warp] = eq;
   }
   __syncthreads();
-  gt = gt_before + __reduce_add_sync(kFullMask, lane < warp ? sm.warp_gt[lane] : 0u);
-  eq = eq_before + __reduce_add_sync(kFullMask, lane < warp ? sm.warp_eq[lane] : 0u);
+  gt = th.gt_before + __reduce_add_sync(kFullMask, lane < warp ? sm.warp_gt[lane] : 0u);
+  eq = th.eq_before + __reduce_add_sync(kFullMask, lane < warp ? sm.warp_eq[lane] : 0u);
   const uint32_t lt = (1u << lane) - 1u;
   for (int base = j0; base < j1; base += 32) {
     const int j = base + lane;
@@ -1173,6 +1201,142 @@ __global__ void __launch_bounds__(kChipThreads, 1) topk_chip_kernel(const Compre
     eq += __popc(eqs);
   }
   if constexpr (C > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// ---------------------------------------------------------------------------
+// Steps 3 to 5 in one launch where a worker's candidates fit into the shared
+// memory of a cluster (picks): the cluster's CTAs share them evenly, in index
+// order, find T as above and write the records.  The three grids read the
+// candidates three times, and at these sizes each of them is launch, first loads
+// and barriers (3.6M x 8, k = d / 100, fresh gradients, the whole step: 101.5 us with
+// three launches, 86.5 so).  What does not fit after all (many
+// equal keys) is read from memory again in every round; with fewer than k
+// candidates the zeros fill the records, or all elements become candidates.
+// ---------------------------------------------------------------------------
+constexpr int kPickCtas = 8;
+constexpr int kPickTiles = 4096;  // tiles of a worker, at most
+constexpr int kPickCap = 14336;   // candidates of a CTA in shared memory
+static_assert(kPickCap * sizeof(uint2) + sizeof(ChipSmem) + (kPickTiles + 1 + kChipThreads / 32) * 4 < 227 * 1024, "fits");
+
+__global__ void __launch_bounds__(kChipThreads, 1) topk_pick_kernel(const CompressArgs a, int64_t k, void* scratch) {
+  dq_pdl_enter();
+  extern __shared__ __align__(16) uint2 cand[];  // this CTA's first kPickCap candidates
+  __shared__ __align__(16) ChipSmem sm;
+  __shared__ uint32_t pre[kPickTiles + 1];       // candidates before each tile
+  __shared__ uint32_t scan[kChipThreads / 32];
+  constexpr int kWarps = kChipThreads / 32;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int rank = blockIdx.x;
+  const SelectTask s = select_task(a, k, 0, scratch, blockIdx.y, rank, kPickCtas, kWarps);
+  const int nt = (int)s.nt;
+  // the tiles' places
+  auto place_tiles = [&]() -> uint32_t {
+    constexpr int kPer = kPickTiles / kChipThreads;
+    uint32_t c[kPer], sum = 0, total;
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) {
+      const int t = (int)threadIdx.x * kPer + q;
+      c[q] = t < nt ? __ldcg(s.rs.cnt + t) : 0u;
+      sum += c[q];
+    }
+    uint32_t at = block_exclusive_scan<kChipThreads>(sum, &total, scan);
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) {
+      const int t = (int)threadIdx.x * kPer + q;
+      if (t <= nt) pre[t] = at;
+      at += c[q];
+    }
+    if (threadIdx.x == 0) pre[nt] = total;
+    __syncthreads();
+    return total;
+  };
+  const bool zeros_left = call_tau(s.rs.state) == 1u;
+  for (int i = threadIdx.x; i < 4096; i += kChipThreads) sm.hist[i] = 0;
+  uint32_t n = place_tiles();
+  if ((int64_t)n < k && zeros_left) {  // the candidates are all non-zero keys: T is 0
+    static_assert(kWarps * (kTile / 32) <= 4096, "bits of a tile per warp");
+    emit_with_zeros(sm.hist, s, (uint32_t)k - n,
+                    [&](int t) { return make_uint2(pre[t], (uint32_t)((int64_t)t * kTile) - pre[t]); });
+    return;
+  }
+  if ((int64_t)n < k) {  // the sample was far off
+    all_as_candidates<kChipThreads>(s, rank, kPickCtas, [](float) {});
+    __threadfence();
+    cg::this_cluster().sync();
+    n = place_tiles();
+  }
+  const uint32_t lo = (uint32_t)((uint64_t)n * rank / kPickCtas), hi = (uint32_t)((uint64_t)n * (rank + 1) / kPickCtas);
+  const int m = (int)(hi - lo);
+  // the f-th candidate: of the last tile with no more than f before it
+  auto fetch = [&](uint32_t f) -> uint2 {
+    int t = 0;
+#pragma unroll
+    for (int step = kPickTiles / 2; step >= 1; step >>= 1)
+      if (t + step < nt && pre[t + step] <= f) t += step;
+    return __ldcg(s.rs.cand + (int64_t)t * kTile + (f - pre[t]));
+  };
+  const int own = min(m, kPickCap);
+  constexpr int kLoads = 4;
+  for (int i0 = threadIdx.x; i0 < m; i0 += kLoads * kChipThreads) {
+    uint2 x[kLoads];
+#pragma unroll
+    for (int u = 0; u < kLoads; ++u)
+      if (i0 + u * kChipThreads < m) x[u] = fetch(lo + i0 + u * kChipThreads);
+#pragma unroll
+    for (int u = 0; u < kLoads; ++u) {
+      const int i = i0 + u * kChipThreads;
+      if (i >= m) continue;
+      if (i < own) cand[i] = x[u];
+      atomicAdd(&sm.hist[key_bits(x[u].y) >> 20], 1u);
+    }
+  }
+  const Threshold th = cluster_threshold<kPickCtas>(sm, (uint32_t)k, rank, [&](auto&& body) {
+    for (int i = threadIdx.x; i < own; i += kChipThreads) body(key_bits(cand[i].y));
+    for (int i = own + (int)threadIdx.x; i < m; i += kChipThreads) body(key_bits(fetch(lo + i).y));
+  });
+  // no CTA leaves before all have read its counts
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  const uint32_t T = th.T, need = th.need;
+  // warp w takes the candidates [w, w + 1) * stretch, 32 at a time
+  const int stretch = (m + 32 * kWarps - 1) / (32 * kWarps) * 32;
+  const int i0 = min(warp * stretch, m), i1 = min(i0 + stretch, m);
+  uint32_t gt = 0, eq = 0;
+  for (int i = i0 + lane; i < i1; i += 32) {
+    const uint32_t key = key_bits(i < own ? cand[i].y : fetch(lo + i).y);
+    gt += key > T ? 1u : 0u;
+    eq += key == T ? 1u : 0u;
+  }
+  gt = __reduce_add_sync(kFullMask, gt);
+  eq = __reduce_add_sync(kFullMask, eq);
+  if (lane == 0) {
+    sm.warp_gt[warp] = gt;
+    sm.warp_eq[warp] = eq;
+  }
+  __syncthreads();
+  gt = th.gt_before + __reduce_add_sync(kFullMask, lane < warp ? sm.warp_gt[lane] : 0u);
+  eq = th.eq_before + __reduce_add_sync(kFullMask, lane < warp ? sm.warp_eq[lane] : 0u);
+  const uint32_t lt = (1u << lane) - 1u;
+  for (int base = i0; base < i1; base += 32) {
+    const int i = base + lane;
+    const bool valid = i < i1;
+    uint2 c = make_uint2(0u, 0u);
+    if (valid) c = i < own ? cand[i] : fetch(lo + i);
+    const uint32_t key = key_bits(c.y);
+    const uint32_t gts = __ballot_sync(kFullMask, valid && key > T);
+    const uint32_t eqs = __ballot_sync(kFullMask, valid && key == T);
+    const uint32_t tie = eq + __popc(eqs & lt);
+    if (valid) {
+      if (key > T || (key == T && tie < need)) {
+        const uint32_t pos = gt + __popc(gts & lt) + min(tie, need);
+        if (dq_in_bounds(pos < (uint64_t)k, a.err)) s.rec[pos] = c;  // always true; keeps the write inside
+      } else {
+        put_back(s, c);
+      }
+    }
+    gt += __popc(gts);
+    eq += __popc(eqs);
+  }
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
 // ---------------------------------------------------------------------------
@@ -1845,34 +2009,30 @@ static cudaError_t launch_chip(bool keep_h, const CompressArgs& a, int64_t k, cu
   return keep_h ? go(topk_chip_kernel<C, true>, done[0]) : go(topk_chip_kernel<C, false>, done[1]);
 }
 
-// Workers whose C CTAs fit on the current device at once: 152, 15 and 7 for 1, 8
-// and 16 on a whole GB300; less, or 0, on a part of one, where the launch would
-// fail.  Asked once per device, with all the shared memory that a part may take.
-// (Test hook: DQGAN_TEST_NO_CLUSTERS in the environment then makes it 0 for
-// more than one CTA.)
-template <int C>
-static int chip_resident() {
-  static std::atomic<int> kept[kKeptDevices];  // plus 1
+// Clusters of C CTAs of `kernel` that fit on the current device at once (for the
+// on-chip kernel 152, 15 and 7 of 1, 8 and 16 CTAs on a whole GB300); less, or 0,
+// on a part of one, where the launch would fail.  Asked once per device.  (Test
+// hook: DQGAN_TEST_NO_CLUSTERS in the environment then makes it 0 for more than
+// one CTA.)
+template <int C, typename K>
+static int resident_clusters(K kernel, size_t smem, std::atomic<bool> (&done)[kKeptDevices],
+                             std::atomic<int> (&kept)[kKeptDevices]) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kKeptDevices) return 0;
-  int n = kept[dev].load(std::memory_order_acquire);
+  int n = kept[dev].load(std::memory_order_acquire);  // plus 1
   if (n == 0) {
-    static std::atomic<bool> done[kKeptDevices];
-    const auto kernel = topk_chip_kernel<C, true>;
     int fit = 0;
     if (C > 1 && std::getenv("DQGAN_TEST_NO_CLUSTERS")) {
       fit = 0;
-    } else if (allow_smem(kernel, kChipMax * sizeof(float), C, done) == cudaSuccess) {
+    } else if (allow_smem(kernel, smem, C, done) == cudaSuccess) {
       if constexpr (C == 1) {
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, kernel, kChipThreads, kChipMax * sizeof(float)) !=
-            cudaSuccess)
-          fit = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, kernel, kChipThreads, smem) != cudaSuccess) fit = 0;
         fit *= device_sms();
       } else {
         cudaLaunchConfig_t lc = {};
         lc.gridDim = dim3(C);
         lc.blockDim = dim3(kChipThreads);
-        lc.dynamicSmemBytes = kChipMax * sizeof(float);
+        lc.dynamicSmemBytes = smem;
         cudaLaunchAttribute attr;
         attr.id = cudaLaunchAttributeClusterDimension;
         attr.val.clusterDim.x = C;
@@ -1887,6 +2047,13 @@ static int chip_resident() {
     kept[dev].store(n, std::memory_order_release);
   }
   return n - 1;
+}
+
+template <int C>
+static int chip_resident() {
+  static std::atomic<bool> done[kKeptDevices];
+  static std::atomic<int> kept[kKeptDevices];
+  return resident_clusters<C>(topk_chip_kernel<C, true>, kChipMax * sizeof(float), done, kept);
 }
 
 // CTAs per worker of the kernel that keeps p on chip, or 0 where the five
@@ -1917,6 +2084,25 @@ static int chip_ctas(int64_t d, int nworkers) {
   return ctas;
 }
 
+// Whether the selection is one launch (topk_pick_kernel): the candidates that
+// the sample leads one to expect fit on chip, with a tenth to spare, every
+// worker's cluster fits the device at once, and they are so few that 8 CTAs per
+// worker read them as fast as the grids of the three launches do.  Worker step,
+// one launch / three (us, layers of different scale; k: candidates): 600,000 x 1,
+// 6000: 18.2 / 21.2; 1M x 1, 10,000: 18.9 / 21.7, 100,000: 33.1 / 40.9; 1M x 8, 10,000:
+// 30.9 / 34.6; 1M x 16 (two waves) 57.1 / 54.0; 3.6M x 1, 18,000 (26,000): 24.9 / 25.5,
+// 36,000 (46,000): 28.5 / 26.4; 3.6M x 4, 36,000: 47.8 / 48.1; 3.6M x 8, 36,000: 77.0 / 79.9,
+// 72,000 (87,000): 84.8 / 84.8; 3.6M x 15, 72,000: 132 / 142; 14M x 2, 28,000: 74.2 / 75.5.
+static bool picks(const CompressArgs& a, int64_t k) {
+  static std::atomic<bool> done[kKeptDevices];
+  static std::atomic<int> kept[kKeptDevices];
+  const double candidates = (double)sample_rank(a.d, k) * kSampBlocks * (double)a.d / kSamples;
+  const double most = a.d <= 1'200'000 ? kPickCtas * kPickCap / 1.1
+                                       : fmin(kPickCtas * kPickCap / 1.1, 25e3 * (1.0 + 0.25 * a.nworkers));
+  return candidates > 0 && candidates <= most && tiles_of(a.d) <= kPickTiles &&
+         a.nworkers <= resident_clusters<kPickCtas>(topk_pick_kernel, kPickCap * sizeof(uint2), done, kept);
+}
+
 cudaError_t launch_topk_compress(const CompressArgs& a, int64_t k, bool keep_h, void* scratch,
                                  cudaStream_t stream, uint64_t* launches) {
   static std::atomic<bool> emit_done[kKeptDevices];
@@ -1933,6 +2119,18 @@ cudaError_t launch_topk_compress(const CompressArgs& a, int64_t k, bool keep_h, 
     case 16: launched(launch_chip<16>(keep_h, a, k, stream)); return st;
   }
   const dim3 tiles((unsigned)tiles_of(a.d), rows), select(select_blocks(a.d, a.nworkers), rows);
+  if (picks(a, k)) {
+    static std::atomic<bool> pick_done[kKeptDevices];
+    constexpr size_t smem = kPickCap * sizeof(uint2);
+    if ((st = allow_smem(topk_pick_kernel, smem, kPickCtas, pick_done)) != cudaSuccess) return st;
+    (void)(launched(launch_pdl(topk_sample_kernel, dim3(kSampBlocks, rows), dim3(kSampThreads), 0, stream, a,
+                               sample_rank(a.d, k), scratch)) &&
+           launched(launch_pdl(keep_h ? topk_form_kernel<true> : topk_form_kernel<false>, tiles, dim3(kFormThreads), 0,
+                               stream, a, scratch)) &&
+           launched(launch_pdl_cluster(topk_pick_kernel, kPickCtas, dim3(kPickCtas, rows), dim3(kChipThreads), smem, stream,
+                                       a, k, scratch)));
+    return st;
+  }
   // the rows that a tile with its share of 1.3 k candidates has
   const int64_t mean = 1 + 13 * k / (320 * tiles_of(a.d));
   const int ahead = (int)(mean < kFirst ? mean : kFirst);

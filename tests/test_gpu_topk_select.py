@@ -7,7 +7,8 @@ for bit with numpy on the same fp32 p:
 
 * few parameters (one CTA keeps them on chip), more (clusters of 8 and of 16
   CTAs do), parts that end in the last CTA, and d on both sides of the sizes
-  from which the sampled kernels run;
+  from which the sampled kernels run; few candidates (selected in one launch,
+  also where they turn out too many for its shared memory) and many;
 * a gradient that is large exactly at the sampled runs, so that too few
   elements reach the threshold and the candidates are taken again;
 * a few dense tiles among thousands with one candidate each;
@@ -79,7 +80,11 @@ CASES = [(1, 1, 2, "gauss"), (3, 2, 2, "gauss"), (2_049, 2_049, 2, "ties"), (20_
          (1_000_003, 200_000, 2, "trap"), (9_000_001, 400_000, 2, "ties"), (9_000_001, 21_000, 2, "sparse tiles"),
          (200_003, 9_000, 2, "sparse"), (1_000_003, 20_000, 3, "sparse"), (1_000_003, 20_000, 3, "just enough"),
          (1_000_003, 300_000, 2, "just enough"), (90_001, 1_000, 64, "sparse"), (1_000_003, 60_000, 2, "zeros"), (35_000_001, 50_000, 1, "sparse"),
-         (35_000_001, 50_000, 1, "trap"), (90_001, 30_000, 64, "ties")]
+         (35_000_001, 50_000, 1, "trap"), (90_001, 30_000, 64, "ties"),
+         # selected in one launch, up to its last size, and the next
+         (1_000_003, 20_000, 2, "trap"), (9_000_001, 20_000, 2, "ties"), (1_000_003, 500, 15, "gauss"),
+         (1_000_003, 500, 16, "gauss"), (1_000_003, 60_000, 2, "ties"), (1_000_003, 95_000, 3, "gauss"),
+         (4096 * 4096, 2_000, 1, "gauss"), (4096 * 4096 + 1, 2_000, 1, "gauss"), (600_001, 1, 3, "outliers")]
 
 
 @pytest.mark.parametrize("keep", [False, True])
