@@ -36,7 +36,7 @@
 //   Sparse gradients are ordinary input (frozen layers, rows nobody looked
 // up).  With tau = 0 for them and one CTA per worker for what the list does not
 // hold, 3.6M x 8, k = d / 100, k / 2 non-zero entries took 9.6 ms, 1.1 k 199 us;
-// now 139 and 79 (25M x 16: 64.8 ms and 2.19 ms; now 794 and 776 us).
+// now 135 and 73 (25M x 16: 64.8 ms and 2.19 ms; now 794 and 777 us).
 //
 // Server: w_j -= (sum over workers of the value recorded for j, absent
 // workers as +0, in the library's pairwise order) / M at the indices some
@@ -279,7 +279,7 @@ __global__ void __launch_bounds__(kSampThreads) topk_sample_kernel(const Compres
 
 // ---------------------------------------------------------------------------
 // 2. p = fl(fl(eta g) + e); e = p, or p - p at a candidate (key >= tau), and
-// h = fl(fl(eta g) + e); the select kernel corrects both at the candidates
+// h = fl(fl(eta g) + e); steps 3 to 5 correct both at the candidates
 // that are not kept, a fraction of them.  Element order in a tile: row i,
 // thread t, component q is tile offset 4 * (i * 256 + t) + q, so warp w of
 // row i covers the 128 consecutive offsets of group g = 8 i + w.  Candidate
@@ -408,10 +408,10 @@ __global__ void __launch_bounds__(kFormThreads, 4) topk_form_kernel(const Compre
 // the row's warps in turn (so that a stretch of the vector that holds most of
 // the candidates is shared by all of them).  What a step has to know of the
 // whole worker every CTA works out for itself from the counts of the step
-// before, which costs less than a step between them.  (A cluster of 8 or 16
-// CTAs per worker, with the counts summed through distributed shared memory,
-// took as long while the share of a CTA fits on chip, and twice as long for
-// 16 workers with 250,000 records each: 14 clusters of 16 fit at a time.)
+// before, which costs less than a step between them.  (One launch, by a
+// cluster of 8 CTAs per worker, is faster while a CTA's share fits on chip:
+// topk_pick_kernel.  With 250,000 records of each of 16 workers it took twice as
+// long.)
 // ---------------------------------------------------------------------------
 struct SelectTask {
   const CompressArgs& a;
