@@ -1260,6 +1260,7 @@ __global__ void __launch_bounds__(kChipThreads, 1) topk_pick_kernel(const Compre
     return;
   }
   if ((int64_t)n < k) {  // the sample was far off
+    cg::this_cluster().sync();  // every CTA has read the counts, and so comes here too, before one changes
     all_as_candidates<kChipThreads>(s, rank, kPickCtas, [](float) {});
     __threadfence();
     cg::this_cluster().sync();
