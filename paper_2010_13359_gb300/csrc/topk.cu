@@ -1591,10 +1591,14 @@ constexpr size_t dense_smem(int M, int P) { return (size_t)M * dense_runs(P) * k
 //   1.05M x 64, 10 %, 6,710,848      231 / 71  133 / 80   98 / 70
 //   25M x 1, 3 %, 750,000             72 / 42   17 / 33   72 / 42
 //   10M x 2, 3 %, 600,000             45 / 32   16 / 29   39 / 31
+// and from warm ones
+//   524,288 x 24, 10 %, 1,258,000     34 / 19   19 / 20   18 / 19
+//   524,288 x 48, 10 %, 2,516,000     82 / 29   38 / 45   35 / 29
+//   524,288 x 64, 10 %, 3,355,000    111 / 33   50 / 38   48 / 33
 // Over 2600 such cases the line below has the least loss on either side of it.
 bool tile_server(int64_t d, int64_t k, int nworkers) {
-  const double records = (double)k * nworkers;
-  return nworkers <= kSrvMaskMaxM && d >= 1'000'000 && records >= 700e3 && records >= 0.03 * (double)d;
+  const double records = (double)k * nworkers, least = d >= 1'000'000 ? 700e3 : 1e6;
+  return nworkers <= kSrvMaskMaxM && d >= 500'000 && records >= least && records >= 0.03 * (double)d;
 }
 
 // Server scratch of the two kernels, after the starts: the number of tiles on

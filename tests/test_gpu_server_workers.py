@@ -167,6 +167,13 @@ def test_top_k_lists_and_dense_tiles(P, M, kind, oadam):
     top_k_server(P, 4_100_007, M, -(-1_010_000 // M), kind, oadam=oadam)
 
 
+@pytest.mark.parametrize("kind", ["spread", "edge"])
+@pytest.mark.parametrize("d,M,k", [(500_000, 21, 47_620), (499_999, 21, 47_620), (999_999, 64, 15_624)])
+def test_top_k_at_the_smallest_merged(P, d, M, k, kind):
+    """The smallest vector that is merged by tiles, and one parameter or record less."""
+    top_k_server(P, d, M, k, kind)
+
+
 @pytest.mark.parametrize("M", [16, 64])
 def test_top_k_records_gathered_in_a_tenth_take_no_longer(P, M):
     """Layers differ in scale, so the records of a step often sit in a few tiles.  Those
