@@ -140,7 +140,7 @@ DQGAN_API int dqgan_validate_config(const dqgan_config* cfg);
  * is taken as 0 so that w_{1/2} = w_0), and top-k scratch (per worker row
  * about 8 bytes per parameter for the candidates; for the server, with
  * M <= 64, per-index worker masks and values, 4 + 4M bytes per parameter
- * (8 + 4M above 32 workers; M rounded up to a multiple of 4 from 3 on), unless
+ * (8 + 4M above 32 workers), unless
  * the records are many: d >= 500,000, M k >= 700,000 (below d = 1,000,000:
  * M k >= 1,000,000) and M k >= 3 % of d; then, and above 64 workers, a table
  * of record ranges, M / 64 bytes per parameter).  Sets t = 1.

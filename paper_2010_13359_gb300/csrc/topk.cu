@@ -1412,7 +1412,7 @@ __device__ __forceinline__ float srv_average(float acc, const ServerArgs& s) {
 //   1. scatter: record (m, r) with index j writes its value to entry (j, m)
 //      and sets bit m of j's mask.
 //   2. reduce: the record of the lowest worker in j's mask owns j.  It loads j's
-//      values 16 bytes at a time (one by one, M = 64, d = 100,000, k = d / 10,
+//      values 16 bytes at a time where M is a multiple of 4 (one by one, M = 64, d = 100,000, k = d / 10,
 //      the same indices: 28 us from warm caches, 15 so) and sums
 //      the values of the workers in the mask, in worker order with the
 //      absent workers as +0 leaves (the library's pairwise order), updates
@@ -1431,19 +1431,14 @@ constexpr int kSrvMaskMaxM = 64;
 template <typename Mask>
 struct SrvTables {
   Mask* mask;   // d masks
-  float* vals;  // worker m's value of index j at vals[j * srv_row(M) + m]
+  float* vals;  // worker m's value of index j at vals[j * M + m]
 };
-
-// Values per index in the table: whole 16-byte loads.
-__host__ __device__ constexpr int64_t srv_row(int32_t nworkers) {
-  return nworkers <= 2 ? nworkers : (nworkers + 3) / 4 * 4;
-}
 
 // Words of a mask: one bit per worker.
 __host__ __device__ constexpr int srv_mask_words(int32_t nworkers) { return nworkers <= 32 ? 1 : 2; }
 
 __host__ __device__ constexpr int64_t srv_mask_table_words(int64_t d, int32_t nworkers) {
-  return (srv_mask_words(nworkers) + srv_row(nworkers)) * round64(d);
+  return (srv_mask_words(nworkers) + (int64_t)nworkers) * round64(d);
 }
 
 template <typename Mask>
@@ -1471,7 +1466,7 @@ __global__ void __launch_bounds__(kSrvThreads) topk_server_scatter_kernel(const 
   const uint2 rec = reinterpret_cast<const uint2*>(s.msgs + (int64_t)m * s.msg_stride)[r];
   // records come from the compressor and are below d
   if (!dq_in_bounds((int64_t)rec.x < s.d, s.err)) return;
-  t.vals[(int64_t)rec.x * srv_row(s.M) + m] = __uint_as_float(rec.y);
+  t.vals[(int64_t)rec.x * s.M + m] = __uint_as_float(rec.y);
   atomicOr(t.mask + rec.x, (Mask)1 << m);
 }
 
@@ -1521,17 +1516,19 @@ __global__ void __launch_bounds__(kSrvThreads) topk_server_reduce_kernel(const S
   const Mask mask = t.mask[j];
   // the owner: bit m set and no bit below it
   if (!((mask >> m) & 1u) || (mask & (((Mask)1 << m) - 1u))) return;
-  const float* vals = t.vals + j * srv_row(s.M);
+  const float* vals = t.vals + j * s.M;
+  const bool whole = s.M % 4 == 0;  // rows of whole 16-byte words
   const float sum = owner_sum<P>(mask, __uint_as_float(rec.y), [&](int who, float (&x)[4]) {
-    if constexpr (P <= 2) {
-      x[0] = vals[0];
-      x[1] = vals[1];
-    } else {
+    if (P >= 4 && whole) {
       const float4 v = *reinterpret_cast<const float4*>(vals + who);
       x[0] = v.x;
       x[1] = v.y;
       x[2] = v.z;
       x[3] = v.w;
+    } else {
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (q < P && ((mask >> (who + q)) & 1u)) x[q] = vals[who + q];
     }
   });
   s.w[j] = server_out(s, s.w[j], srv_average<POW2>(sum, s));

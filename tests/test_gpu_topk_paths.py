@@ -145,7 +145,7 @@ def test_server_worker_counts(P, M):
     run_free(P, ocfg, [1.0, 1.0, "ties"], seed=M)
 
 
-@pytest.mark.parametrize("M,k,server", [(8, 25_000, 36), (8, 87_499, 36), (8, 87_500, 0.125), (5, 10_000, 36),
+@pytest.mark.parametrize("M,k,server", [(8, 25_000, 36), (8, 87_499, 36), (8, 87_500, 0.125), (5, 10_000, 24),
                                         (40, 5_000, 168), (65, 5_000, 65 / 64)])
 def test_scratch_is_what_the_header_says(P, M, k, server):
     """Bytes per parameter: 4 for each residual, about 8 for each worker's candidates, and the
